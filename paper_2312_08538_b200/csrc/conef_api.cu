@@ -1424,7 +1424,7 @@ int conef_apply_update(conef_ctx *ctx, float *x, const float *sum_values, const 
     if (n == 0)
         return CONEF_OK;
     const DevView V = current_view(ctx);
-    k_apply<<<n, 256, 0, (cudaStream_t)stream>>>(V, table_ptr(ctx, T_APPLY), x, sum_values, sum_dense1d);
+    apply_launch(ctx->q.kind, ctx->q.rank, V, table_ptr(ctx, T_APPLY), n, x, sum_values, sum_dense1d, (cudaStream_t)stream);
     LAUNCH_CHECK(ctx);
     return CONEF_OK;
 }

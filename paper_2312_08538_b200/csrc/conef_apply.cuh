@@ -6,67 +6,235 @@
 
 namespace conef {
 
-constexpr int kApplyTile = 4096;      // elements (or message values) per CTA, dense and sparse cases
-constexpr int kApplyRows = 16;        // low-rank: rows per CTA, one column per thread
+constexpr int kApplyThreads = 256;
+constexpr int kApplyTile = 4096;      // elements per CTA where the update is dense and elementwise
+constexpr int kApplySparse = 1024;    // message values per CTA where it is sparse: four per thread, all in flight
+
+// Low-rank tiles: a CTA's threads are laid out as ap_tx column groups (of ap_vec columns) by ap_ty
+// rows; a thread keeps its columns' rows of Q in registers and walks ap_rpt rows, ap_ty apart.
+inline void apply_classify(LayerDesc &L)
+{
+    L.ap_vec = (L.cols % 4 == 0 && L.g_off % 4 == 0) ? 4 : 1;
+    const int64_t ncg = (L.cols + L.ap_vec - 1) / L.ap_vec;
+    // column tiles of equal width: as few as leave at most 7 % of the threads idle, else the best of eight
+    const int64_t ct0 = (ncg + kApplyThreads - 1) / kApplyThreads;
+    double best = 0.0;
+    for (int64_t ct = ct0; ct < ct0 + 8 && best < 0.93; ++ct) {
+        const int64_t tx = (ncg + ct - 1) / ct, ty = kApplyThreads / tx;
+        const double used = (double)(tx * ty) / kApplyThreads * (double)ncg / (double)(ct * tx);
+        if (used > best && (tx >= 16 || ct == ct0)) {
+            best = used;
+            L.ap_tx = (int32_t)tx;
+            L.ap_ty = (int32_t)ty;
+            L.ap_ct = (int32_t)ct;
+        }
+    }
+    // a thread loads rank * 4 bytes per column before its first row: many rows amortise that on large
+    // tensors, few keep the SMs busy on small ones
+    L.ap_rpt = L.d >= (1 << 22) ? 64 : L.d >= (1 << 20) ? 32 : L.d >= (1 << 17) ? 16 : 8;
+}
 
 // tiles per tensor, in the order the kernel decodes them
-__host__ __device__ inline int64_t apply_tiles(const LayerDesc &L, int qkind)
+inline int64_t apply_tiles(LayerDesc &L, int qkind)
 {
     if (!L.compressed || qkind == CONEF_Q_IDENTITY)
         return (L.d + kApplyTile - 1) / kApplyTile;
     if (qkind == CONEF_Q_RANDK || qkind == CONEF_Q_RANDBLOCK)
-        return (L.k + kApplyTile - 1) / kApplyTile;
-    return ((L.rows + kApplyRows - 1) / kApplyRows) * ((L.cols + 255) / 256);
+        return (L.k + kApplySparse - 1) / kApplySparse;
+    apply_classify(L);
+    const int64_t rows = (int64_t)L.ap_ty * L.ap_rpt;
+    return L.ap_ct * ((L.rows + rows - 1) / rows);
 }
 
-__global__ void __launch_bounds__(256) k_apply(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
-                                               float *__restrict__ x, const float *__restrict__ sum_values,
-                                               const float *__restrict__ sum_dense1d)
+// x[a][b] -= sum_c P_hat[a][c] Qmean[b][c] (an fma chain over ascending c) on a tile.  RK: the rank, or
+// 0 for any rank; VEC columns per thread; B rows of x are loaded before the first is used; FV: rows
+// of the factors lie on 16-byte boundaries.  HBM-bound (8 bytes per element).  GPT-2-XL list, rank 4:
+// one column per thread and 16 rows one after the other took 3.76 ms (3.3 TB/s); four columns and
+// eight rows in flight take 2.09 ms (6.0 TB/s); four rows in flight 2.21 ms, eight under a
+// 64-register cap (spills) 3.1 ms.  GPT-2-small list, rank 8: 324 -> 193 us.
+template <int RK, int VEC, int B, bool FV>
+__device__ __forceinline__ void apply_lowrank(const DevView &V, const LayerDesc &L, uint32_t tile, float *__restrict__ xs,
+                                              bool aligned)
+{
+    constexpr int RM = RK ? RK : CONEF_MAX_RANK;
+    const int r = RK ? RK : L.rank;
+    const uint32_t gtx = L.ap_tx, gty = L.ap_ty, gct = L.ap_ct;
+    const uint32_t ty = threadIdx.x / gtx, tx = threadIdx.x - ty * gtx;
+    const uint32_t rt = tile / gct, ct = tile - rt * gct;
+    const uint32_t b = (ct * gtx + tx) * VEC, m = (uint32_t)L.cols;
+    if (ty >= gty || b >= m)
+        return;
+    const float *__restrict__ phat = V.phat + L.msgp_off;
+    auto load_row = [&](const float *p, float (&out)[RM]) {
+        if (FV) {
+#pragma unroll
+            for (int c = 0; c + 4 <= RM; c += 4) {
+                const float4 t = __ldg((const float4 *)(p + c));
+                out[c] = t.x; out[c + 1] = t.y; out[c + 2] = t.z; out[c + 3] = t.w;
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < RM; ++c)
+                out[c] = (RK || c < r) ? __ldg(p + c) : 0.f;
+        }
+    };
+    float q[VEC][RM];
+    {
+        const float *__restrict__ qm = V.qprev + L.msgq_off + (size_t)b * r;
+#pragma unroll
+        for (int v = 0; v < VEC; ++v)
+            load_row(qm + v * r, q[v]);
+    }
+    auto load = [&](const float *p, float (&xv)[VEC]) {
+        if (VEC == 4 && aligned) {
+            const float4 t = *(const float4 *)p;
+            xv[0] = t.x; xv[1 % VEC] = t.y; xv[2 % VEC] = t.z; xv[3 % VEC] = t.w;
+        } else {
+#pragma unroll
+            for (int v = 0; v < VEC; ++v)
+                xv[v] = p[v];
+        }
+    };
+    auto update_store = [&](float *p, const float (&ph)[RM], float (&xv)[VEC]) {
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+            float dl = 0.f;
+#pragma unroll
+            for (int c = 0; c < RM; ++c)
+                if (RK || c < r)
+                    dl = __fmaf_rn(ph[c], q[v][c], dl);
+            xv[v] = __fsub_rn(xv[v], dl);
+        }
+        if (VEC == 4 && aligned) {
+            *(float4 *)p = make_float4(xv[0], xv[1 % VEC], xv[2 % VEC], xv[3 % VEC]);
+        } else {
+#pragma unroll
+            for (int v = 0; v < VEC; ++v)
+                p[v] = xv[v];
+        }
+    };
+    const uint32_t rows = (uint32_t)L.rows, span = gty * (uint32_t)L.ap_rpt;
+    uint32_t a = rt * span + ty;
+    const uint32_t a1 = min(rows, (rt + 1) * span);
+    float *xp = xs + (size_t)a * m + b;
+    const float *pp = phat + (size_t)a * r;
+    const size_t step = (size_t)gty * m;
+    const uint32_t pstep = gty * r;
+    for (; a + (B - 1) * gty < a1; a += B * gty) {
+        float xv[B][VEC];
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            load(xp + u * step, xv[u]);
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            float ph[RM];
+            load_row(pp + u * pstep, ph);
+            update_store(xp + u * step, ph, xv[u]);
+        }
+        xp += B * step;
+        pp += B * pstep;
+    }
+    for (; a < a1; a += gty) {
+        float xv[VEC], ph[RM];
+        load(xp, xv);
+        load_row(pp, ph);
+        update_store(xp, ph, xv);
+        xp += step;
+        pp += pstep;
+    }
+}
+
+// R: the configured rank of a low-rank Q (1, 2, 4, 8; 0: another one), or -1 for the other compressors
+template <int R>
+__global__ void __launch_bounds__(kApplyThreads, R == 8 ? 2 : 3)
+k_apply(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, float *__restrict__ x,
+        const float *__restrict__ sum_values, const float *__restrict__ sum_dense1d)
 {
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
-    const int64_t tile = blockIdx.x - pfx[li];
+    const uint32_t tile = blockIdx.x - pfx[li];
     float *__restrict__ xs = x + L.g_off;
     const float nw = V.n_workers_f;
-    if (!L.compressed || V.qkind == CONEF_Q_IDENTITY) {
-        const float *__restrict__ sum = L.compressed ? sum_values + L.msgv_off : sum_dense1d + L.msg1d_off;
-        for (int q = threadIdx.x; q < kApplyTile; q += 256) {
-            const int64_t j = tile * kApplyTile + q;
-            if (j < L.d)
-                xs[j] = __fsub_rn(xs[j], __fdiv_rn(sum[j], nw));
+    if (!L.compressed || (R < 0 && V.qkind == CONEF_Q_IDENTITY)) {
+        const size_t at = (size_t)tile * kApplyTile;
+        const float *__restrict__ sum = (L.compressed ? sum_values + L.msgv_off : sum_dense1d + L.msg1d_off) + at;
+        float *__restrict__ xt = xs + at;
+        const int n = (int)min((int64_t)kApplyTile, L.d - (int64_t)at);
+        if (n == kApplyTile && (((uintptr_t)xt | (uintptr_t)sum) & 15) == 0) {
+            float4 xv[4], sv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                xv[u] = ((const float4 *)xt)[u * kApplyThreads + threadIdx.x];
+                sv[u] = ((const float4 *)sum)[u * kApplyThreads + threadIdx.x];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                ((float4 *)xt)[u * kApplyThreads + threadIdx.x] =
+                    make_float4(__fsub_rn(xv[u].x, __fdiv_rn(sv[u].x, nw)), __fsub_rn(xv[u].y, __fdiv_rn(sv[u].y, nw)),
+                                __fsub_rn(xv[u].z, __fdiv_rn(sv[u].z, nw)), __fsub_rn(xv[u].w, __fdiv_rn(sv[u].w, nw)));
+        } else {
+#pragma unroll 4
+            for (int q = threadIdx.x; q < n; q += kApplyThreads)
+                xt[q] = __fsub_rn(xt[q], __fdiv_rn(sum[q], nw));
         }
-    } else if (V.qkind == CONEF_Q_RANDK || V.qkind == CONEF_Q_RANDBLOCK) {
+        return;
+    }
+    if constexpr (R < 0) {
+        // indices are distinct: no race.  Bound by the 32-byte sectors of x that hold one value each
         const float *__restrict__ sum = sum_values + L.msgv_off;
         const uint32_t *__restrict__ idx = V.idx + L.idx_off;
-        for (int q = threadIdx.x; q < kApplyTile; q += 256) {
-            const int64_t s = tile * kApplyTile + q;
-            if (s < L.k) {
-                const uint32_t j = idx[s];
-                xs[j] = __fsub_rn(xs[j], __fdiv_rn(sum[s], nw));   // indices are distinct: no race
-            }
+        constexpr int B = kApplySparse / kApplyThreads;
+        uint32_t j[B];
+        float sv[B], xv[B];
+        bool in[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int64_t s = (int64_t)tile * kApplySparse + u * kApplyThreads + threadIdx.x;
+            in[u] = s < L.k;
+            j[u] = in[u] ? idx[s] : 0u;
+            sv[u] = in[u] ? sum[s] : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            xv[u] = in[u] ? xs[j[u]] : 0.f;
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (in[u])
+                xs[j[u]] = __fsub_rn(xv[u], __fdiv_rn(sv[u], nw));
     } else {
-        // Delta = P_hat Qmean^T, Qmean = the warm start left by the reduction of the Q messages
-        const int r = L.rank;
-        const int64_t ctiles = (L.cols + 255) / 256;
-        const int64_t b = (tile % ctiles) * 256 + threadIdx.x;
-        const int64_t a0 = (tile / ctiles) * kApplyRows;
-        if (b >= L.cols)
-            return;
-        const float *__restrict__ phat = V.phat + L.msgp_off;
-        const float *__restrict__ qm = V.qprev + L.msgq_off + b * r;
-        float qreg[CONEF_MAX_RANK];
-#pragma unroll
-        for (int c = 0; c < CONEF_MAX_RANK; ++c)
-            qreg[c] = c < r ? qm[c] : 0.f;
-        for (int64_t a = a0; a < min(L.rows, a0 + kApplyRows); ++a) {
-            float dl = 0.f;
-#pragma unroll
-            for (int c = 0; c < CONEF_MAX_RANK; ++c)
-                if (c < r)
-                    dl = __fmaf_rn(phat[a * r + c], qreg[c], dl);
-            xs[a * L.cols + b] = __fsub_rn(xs[a * L.cols + b], dl);
+        // Delta = P_hat Qmean^T, Qmean = the warm start left by the reduction of the Q messages.
+        // Tensors thinner than the configured rank take the run-time rank.
+        const bool exact = R > 0 && L.rank == R;
+        const bool fv = ((L.msgp_off | L.msgq_off) & 3) == 0;
+        const bool aligned = ((uintptr_t)xs & 15) == 0;
+        constexpr int RX = R > 0 ? R : 0;
+        if (L.ap_vec == 4) {
+            if (exact && R >= 4 && fv)
+                apply_lowrank<RX, 4, 8, (R >= 4)>(V, L, tile, xs, aligned);
+            else if (exact && R < 4)
+                apply_lowrank<RX, 4, 4, false>(V, L, tile, xs, aligned);
+            else
+                apply_lowrank<0, 4, 1, false>(V, L, tile, xs, aligned);
+        } else {
+            if (exact)
+                apply_lowrank<RX, 1, 8, false>(V, L, tile, xs, false);
+            else
+                apply_lowrank<0, 1, 8, false>(V, L, tile, xs, false);
         }
+    }
+}
+
+inline void apply_launch(int qkind, int rank, const DevView &V, const int32_t *pfx, int tiles, float *x, const float *sum_values,
+                         const float *sum_dense1d, cudaStream_t s)
+{
+    const int r = qkind != CONEF_Q_LOWRANK ? -1 : rank == 1 || rank == 2 || rank == 4 || rank == 8 ? rank : 0;
+    switch (r) {
+    case -1: k_apply<-1><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
+    case 1: k_apply<1><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
+    case 2: k_apply<2><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
+    case 4: k_apply<4><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
+    case 8: k_apply<8><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
+    default: k_apply<0><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d);
     }
 }
 

@@ -88,6 +88,9 @@ struct LayerDesc {
     int64_t rs_info_off; // [v][rows]: bucket of a row | sign << 31
     int64_t rs_ptr_off;  // [v][w + 1]: start of each bucket's row list
     int64_t rs_row_off;  // [v][rows]: rows by bucket, ascending within a bucket, | sign << 31
+    // model update of a low-rank tensor (conef_apply.cuh): columns per thread, threads across and down, rows
+    // per thread, column tiles
+    int32_t ap_vec, ap_tx, ap_ty, ap_rpt, ap_ct, ap_pad;
     int32_t rs_vec;      // columns per thread of the row-sketch kernel (4 or 1)
     int32_t rs_pad;
 };

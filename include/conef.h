@@ -306,14 +306,14 @@ const char *conef_error_string(int code);
  * tensor index and step) into idx_out (DEVICE, k uint32, caller-owned) and
  * allocates nothing: no cudaMalloc, no cudaFree, no allocating library call.
  *
- * Its scratch (radix histograms and one counter per 256 elements, about
- * 290 KB) is a fixed array in the library's device image; every GPU that loads
+ * Its scratch (one counter per 2048 elements and a list of the elements near
+ * the threshold, about 290 KB) is a fixed array in the library's device image; every GPU that loads
  * the library holds it until the process exits.  Hence the limit
  * d <= CONEF_NOALLOC_MAX_ELEMS; a larger d returns CONEF_ERR_TOO_LARGE and
  * launches nothing.  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress); make that first call before any stream
  * capture.  All calls share the one array and it keeps the last call's
- * contents (each call clears what it needs zeroed), so two calls whose work
+ * contents (each call leaves its counters zeroed), so two calls whose work
  * overlaps on the GPU -- different streams, or different host threads -- race:
  * issue them on one stream, or order them yourself.  Work is enqueued on
  * `stream`; the call does not synchronise, so a selection that fails on the

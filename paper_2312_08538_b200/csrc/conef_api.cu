@@ -13,6 +13,7 @@
 #include "conef_internal.h"
 #include "conef_kernels.cuh"
 #include "conef_hash.cuh"
+#include "conef_randk.cuh"
 #include "conef_rowsketch.cuh"
 #include "conef_apply.cuh"
 #include "conef_fast.cuh"
@@ -27,7 +28,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 26 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 27 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -36,6 +37,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_FV, T_NOFV,                                        // tuned fused step (identity / random-k Q, int8 / int4 C) and the rest
        T_CSK,                                               // count sketch applied run by run: one tile per run
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
+       T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -73,6 +75,7 @@ struct Plan {
     bool short_tiles = false;   // tile lengths of the tuned passes below their limits
     bool any_fv = false;        // some tensor takes the tuned fused step (conef_flatvec.cuh)
     int fv_tiles = 1;           // ... with this many selection tiles per CTA
+    int sel_tiles = 1;          // random-k selection: tiles hashed per CTA
     bool any_fused = false;     // some tensor takes the fused passes 2 + 3 (conef_fused.cu)
     int n_fused = 0;
     bool any_csk = false;       // some tensor takes the shared-memory step of the chunk-wise count sketch
@@ -82,15 +85,15 @@ struct Plan {
     int64_t state_stride = 0;  // bytes per worker
     int64_t part_stride = 0;   // floats per worker
     int64_t ppart_stride = 0;  // floats per worker: pass-1 partial rows
-    int64_t idx_words = 0, unitoff_words = 0, tileoff_words = 0, sel_words = 0, selbits_words = 0;
+    int64_t idx_words = 0, wordoff_halves = 0, tileoff_words = 0, sel_words = 0, selbits_words = 0;
     int64_t rs_words = 0;      // row sketch: uint32 words of bucket tables
     int64_t cand_pairs = 0;    // random-k selection: (hash, index) pairs of all candidate lists
     int n_comp = 0;
     // byte offsets in the workspace
-    size_t off_layers = 0, off_pfx = 0, off_status = 0, off_sel = 0, off_idx = 0, off_unitoff = 0, off_tileoff = 0, off_selbits = 0,
+    size_t off_layers = 0, off_pfx = 0, off_status = 0, off_sel = 0, off_idx = 0, off_wordoff = 0, off_tileoff = 0, off_selbits = 0,
            off_pbar = 0, off_phat = 0, off_qprev = 0, off_state = 0, off_state_new = 0,
            off_msgv = 0, off_msgp = 0, off_msgq = 0, off_msg1d = 0, off_part = 0, off_ppart = 0, off_rs = 0, off_cand = 0,
-           off_ev[2] = {0, 0}, off_unitoff2[2] = {0, 0}, off_tileoff2[2] = {0, 0}, off_selbits2[2] = {0, 0},   // iConEF-v2
+           off_ev[2] = {0, 0}, off_wordoff2[2] = {0, 0}, off_tileoff2[2] = {0, 0}, off_selbits2[2] = {0, 0},   // iConEF-v2
            off_fu_units = 0, off_fu_groups = 0, off_fu_hint = 0, off_fu_ctr = 0, off_fu_scratch = 0, off_fu_q = 0,   // fused passes 2 + 3
            total = 0;
     int64_t fu_units = 0;          // (tensor, worker) units of the fused kernel
@@ -164,6 +167,8 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
         for (int l = 0; l < n_tensors; ++l)
             if (tensors[l].rows > 0 && tensors[l].cols > 0 && tensors[l].rows <= 0xFFFFFFFFLL / tensors[l].cols)
                 total += tensors[l].rows * tensors[l].cols;
+        for (P.sel_tiles = 1; P.sel_tiles < 8 && total / (kHistTile * 2 * P.sel_tiles) >= kPlanSMs * 16; P.sel_tiles *= 2) {
+        }
         P.fv_tiles = total * n_workers / (kHistTile * kFvTiles) >= kPlanSMs * 16 ? kFvTiles : 1;
     }
     // tile lengths of the tuned low-rank passes from the model's size
@@ -233,9 +238,8 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 L.rs_ptr_off = L.rs_info_off + (int64_t)c->cs_rows * L.rows;
                 L.rs_row_off = L.rs_ptr_off + (int64_t)c->cs_rows * (L.w + 1);
                 P.rs_words = L.rs_row_off + (int64_t)c->cs_rows * L.rows;
-                // four columns per thread where 16-byte accesses line up (random-k also needs message
-                // units that do not straddle rows)
-                L.rs_vec = (L.cols % 4 == 0 && L.g_off % 4 == 0 && (q->kind != CONEF_Q_RANDK || L.cols % 32 == 0)) ? 4 : 1;
+                // four columns per thread where 16-byte accesses line up
+                L.rs_vec = (L.cols % 4 == 0 && L.g_off % 4 == 0) ? 4 : 1;
                 tiles[T_RS] = (int)(c->cs_rows * ceil_div(L.w, kRsBuckets) * ceil_div(L.cols, kRsThreads * L.rs_vec));
                 break;
             default:
@@ -271,19 +275,20 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 L.k = kk < 1 ? 1 : (int64_t)kk;
                 L.idx_off = P.idx_words;
                 P.idx_words += L.k;
-                L.unitoff_off = P.unitoff_words;
-                P.unitoff_words += L.nunits;
+                L.wordoff_off = P.wordoff_halves;
+                P.wordoff_halves += ceil_div(L.d, kHistTile) * (kHistTile / 32);   // whole tiles: read and written 16 bytes at a time
                 L.tileoff_off = P.tileoff_words;
                 P.tileoff_words += ceil_div(L.d, kHistTile);
                 L.selbits_off = P.selbits_words;
-                P.selbits_words += ceil_div(L.d, 32) + 8;   // whole 256-element groups may be read
+                P.selbits_words += ceil_div(L.d, kHistTile) * (kHistTile / 32);
                 L.sel_off = P.sel_words;
                 P.sel_words += kSelWords;
-                // candidates of the second selection level: d / 2048 expected; room for twice that and a margin
                 L.cand_off = P.cand_pairs;
-                L.cand_cap = L.d / 1024 + 1024;
+                select_window(L.d, L.k, L.sel_lo, L.sel_hi, L.cand_cap, L.sel_scale);
                 P.cand_pairs += L.cand_cap;
-                tiles[T_HIST] = (int)ceil_div(L.d, kHistTile);
+                if (ceil_div(L.d, kHistTile) > kSelTailTiles)
+                    tiles[T_SEL_OFFS] = (int)ceil_div(L.d, (int64_t)kHistTile * (kSelThreads / 32));
+                tiles[T_HIST] = (int)ceil_div(L.d, (int64_t)kHistTile * P.sel_tiles);
             }
             if (q->kind != CONEF_Q_LOWRANK) {
                 L.msgv_off = P.msg_elems[CONEF_MSG_VALUES];
@@ -420,7 +425,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     P.off_status = take(256);
     P.off_sel = take((size_t)P.sel_words * 4);
     P.off_idx = take((size_t)P.idx_words * 4);
-    P.off_unitoff = take((size_t)P.unitoff_words * 4);
+    P.off_wordoff = take((size_t)P.wordoff_halves * 2);
     P.off_tileoff = take((size_t)P.tileoff_words * 4);
     P.off_selbits = take((size_t)P.selbits_words * 4);
     P.off_pbar = take((size_t)P.msg_elems[CONEF_MSG_P] * 4);
@@ -441,7 +446,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     if (c->iconef == 2)   // two value buffers per worker and the structures of two more draws of Q
         for (int x = 0; x < 2; ++x) {
             P.off_ev[x] = take((size_t)P.msg_stride[CONEF_MSG_VALUES] * 4 * n_workers);
-            P.off_unitoff2[x] = take((size_t)P.unitoff_words * 4);
+            P.off_wordoff2[x] = take((size_t)P.wordoff_halves * 2);
             P.off_tileoff2[x] = take((size_t)P.tileoff_words * 4);
             P.off_selbits2[x] = take((size_t)P.selbits_words * 4);
         }
@@ -577,20 +582,21 @@ void fill_view(conef_ctx *ctx)
     V.phat = (float *)(ws + P.off_phat);
     V.qprev = (float *)(ws + P.off_qprev);
     V.idx = (uint32_t *)(ws + P.off_idx);
-    V.unitoff = (uint32_t *)(ws + P.off_unitoff);
+    V.wordoff = (uint16_t *)(ws + P.off_wordoff);
     V.tileoff = (uint32_t *)(ws + P.off_tileoff);
     V.selbits = (uint32_t *)(ws + P.off_selbits);
     V.fv_tiles = P.fv_tiles;
+    V.sel_tiles = P.sel_tiles;
     V.sel = (uint32_t *)(ws + P.off_sel);
     V.cand = (uint32_t *)(ws + P.off_cand);
     V.status = (int32_t *)(ws + P.off_status);
     V.rs = (const uint32_t *)(ws + P.off_rs);
     V.pfx_rs = table_ptr(ctx, T_RS);
     V.iconef = ctx->c.iconef;
-    V.unitoffA = (uint32_t *)(ws + P.off_unitoff2[0]);
+    V.wordoffA = (uint16_t *)(ws + P.off_wordoff2[0]);
     V.tileoffA = (uint32_t *)(ws + P.off_tileoff2[0]);
     V.selbitsA = (uint32_t *)(ws + P.off_selbits2[0]);
-    V.unitoffB = (uint32_t *)(ws + P.off_unitoff2[1]);
+    V.wordoffB = (uint16_t *)(ws + P.off_wordoff2[1]);
     V.tileoffB = (uint32_t *)(ws + P.off_tileoff2[1]);
     V.selbitsB = (uint32_t *)(ws + P.off_selbits2[1]);
     V.ev_old = V.ev_new = nullptr;
@@ -630,10 +636,10 @@ DevView current_view(const conef_ctx *ctx)
         // the structures of a draw live beside the values it stored
         const Plan &P = ctx->plan;
         const int a = ctx->ev_cur, b = ctx->ev_cur ^ 1;
-        V.unitoffA = (uint32_t *)(ctx->ws + P.off_unitoff2[a]);
+        V.wordoffA = (uint16_t *)(ctx->ws + P.off_wordoff2[a]);
         V.tileoffA = (uint32_t *)(ctx->ws + P.off_tileoff2[a]);
         V.selbitsA = (uint32_t *)(ctx->ws + P.off_selbits2[a]);
-        V.unitoffB = (uint32_t *)(ctx->ws + P.off_unitoff2[b]);
+        V.wordoffB = (uint16_t *)(ctx->ws + P.off_wordoff2[b]);
         V.tileoffB = (uint32_t *)(ctx->ws + P.off_tileoff2[b]);
         V.selbitsB = (uint32_t *)(ctx->ws + P.off_selbits2[b]);
     }
@@ -977,20 +983,15 @@ int launch_fused(conef_ctx *ctx, const DevView &V, cudaStream_t s, bool own_q)
 
 int launch_randk_select(conef_ctx *ctx, const DevView &V, cudaStream_t s)
 {
-    const int nh = tiles_of(ctx, T_HIST), nc = tiles_of(ctx, T_GS);
+    const int nh = tiles_of(ctx, T_HIST), no = tiles_of(ctx, T_SEL_OFFS);
     if (nh == 0)
         return CONEF_OK;
-    CK_CUDA(cudaMemsetAsync(V.sel, 0, (size_t)ctx->plan.sel_words * 4, s));
-    k_rk_hist<0><<<nh, 256, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_pick<0><<<nc, 1024, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_hist<1><<<nh, 256, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_pick<1><<<nc, 1024, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_hist<2><<<nh, 256, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_pick<2><<<nc, 1024, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_hist<3><<<nh, 256, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_pick<3><<<nc, 1024, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_count<<<nh, 256, 0, s>>>(V); LAUNCH_CHECK(ctx);
-    k_rk_scan<<<nc, 1024, 0, s>>>(V); LAUNCH_CHECK(ctx);
+    k_rk_select<<<nh, kSelThreads, 0, s>>>(V);
+    LAUNCH_CHECK(ctx);
+    if (no > 0) {
+        k_rk_offsets<<<no, kSelThreads, 0, s>>>(V, table_ptr(ctx, T_SEL_OFFS));
+        LAUNCH_CHECK(ctx);
+    }
     return CONEF_OK;
 }
 
@@ -1214,7 +1215,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                 continue;   // last step's draw B is this step's draw A
             DevView D = V;
             D.step = draw + kSecondDraw;
-            D.unitoff = x == 0 ? V.unitoffA : V.unitoffB;
+            D.wordoff = x == 0 ? V.wordoffA : V.wordoffB;
             D.tileoff = x == 0 ? V.tileoffA : V.tileoffB;
             D.selbits = x == 0 ? V.selbitsA : V.selbitsB;
             ctx->draw_step[set] = -1;
@@ -1471,7 +1472,7 @@ int conef_decompress_error(conef_ctx *ctx, int worker, float *out, conef_stream 
         // the index set of the draw that stored e~
         DevView D = V;
         D.step = V.ev_step + kSecondDraw;
-        D.unitoff = V.unitoffA;
+        D.wordoff = V.wordoffA;
         D.tileoff = V.tileoffA;
         D.selbits = V.selbitsA;
         ctx->draw_step[ctx->ev_cur] = -1;

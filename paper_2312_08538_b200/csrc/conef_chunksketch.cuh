@@ -53,8 +53,6 @@ __global__ void __launch_bounds__(kCsThreads) k_sketch_chunk(const __grid_consta
     uint32_t blk_start = 0;
     if (QK == CONEF_Q_RANDBLOCK)
         blk_start = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step), d, (uint32_t)L.k);
-    const int unit_shift = 31 - __clz(L.unit);          // message slots are handed out per unit of 32..256 elements
-    const uint32_t words_per_unit = (uint32_t)L.unit >> 5;
 
     // a warp takes 32 consecutive elements at a time (one word of the membership bitmap)
     for (uint32_t base = j_lo + warp * 32; base < j_hi; base += kCsThreads) {
@@ -97,20 +95,11 @@ __global__ void __launch_bounds__(kCsThreads) k_sketch_chunk(const __grid_consta
             }
         } else {
             sel = valid && ((word >> lane) & 1u);
-            if (word != 0) {   // (uniform over the warp)
-                // slot = tile offset + unit offset + selected elements before this one in its unit
-                const uint32_t wi = base >> 5, first = wi & ~(words_per_unit - 1);
-                uint32_t before = 0;
-                for (uint32_t x = first; x < wi; ++x)
-                    before += __popc(V.selbits[L.selbits_off + x]);
-                if (sel) {
-                    const uint32_t slot = V.tileoff[L.tileoff_off + base / kHistTile] +
-                                          V.unitoff[L.unitoff_off + (base >> unit_shift)] + before +
-                                          __popc(word & ((1u << lane) - 1u));
-                    msg[slot] = p;
-                    if (worker == 0)
-                        V.idx[L.idx_off + slot] = j;
-                }
+            if (sel) {
+                const uint32_t slot = draw_slot(L, V.wordoff, V.tileoff, word, j);
+                msg[slot] = p;
+                if (worker == 0)
+                    V.idx[L.idx_off + slot] = j;
             }
         }
         // r = p - Delta (zero on a transmitted coordinate); Alg. 4 line 9 keeps beta e as well

@@ -131,11 +131,17 @@ __device__ __forceinline__ bool has_second(const DevView &V)
 
 // iConEF-v2: the second application of Q in a step draws from the stream of step t + 2^62
 constexpr int64_t kSecondDraw = 1ll << 62;
-// Whether element j belongs to a stored draw of Q (membership bitmap, unit and tile offsets as the
-// selection kernels leave them; or the block of random-block-k), and its slot among the k values.
+// Message slot of member j of a random-k draw whose bitmap word is `word` (conef_select.cuh)
+__device__ __forceinline__ uint32_t draw_slot(const LayerDesc &L, const uint16_t *__restrict__ wordoff,
+                                              const uint32_t *__restrict__ tileoff, uint32_t word, uint32_t j)
+{
+    return tileoff[L.tileoff_off + j / kHistTile] + wordoff[L.wordoff_off + (j >> 5)] + __popc(word & ((1u << (j & 31u)) - 1u));
+}
+// Whether element j belongs to a stored draw of Q (the bitmap and offsets the selection leaves, or
+// the block of random-block-k), and its slot among the k values.
 template <int QK>
 __device__ __forceinline__ bool draw_member(const LayerDesc &L, const uint32_t *__restrict__ selbits,
-                                            const uint32_t *__restrict__ unitoff,
+                                            const uint16_t *__restrict__ wordoff,
                                             const uint32_t *__restrict__ tileoff, uint32_t blk_start, uint32_t j,
                                             uint32_t &slot)
 {
@@ -143,15 +149,10 @@ __device__ __forceinline__ bool draw_member(const LayerDesc &L, const uint32_t *
         slot = j - blk_start;   // wraps to a large value below the block
         return slot < (uint32_t)L.k;
     }
-    const uint32_t wi = j >> 5, word = selbits[L.selbits_off + wi];
+    const uint32_t word = selbits[L.selbits_off + (j >> 5)];
     if (!((word >> (j & 31u)) & 1u))
         return false;
-    const int unit_shift = 31 - __clz(L.unit);
-    const uint32_t first = (j >> unit_shift) << (unit_shift - 5);   // first bitmap word of the unit
-    uint32_t before = __popc(word & ((1u << (j & 31u)) - 1u));
-    for (uint32_t x = first; x < wi; ++x)
-        before += __popc(selbits[L.selbits_off + x]);
-    slot = tileoff[L.tileoff_off + j / kHistTile] + unitoff[L.unitoff_off + (j >> unit_shift)] + before;
+    slot = draw_slot(L, wordoff, tileoff, word, j);
     return true;
 }
 

@@ -44,14 +44,13 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
     uint8_t *scales = st + L.b_off;
     uint8_t *codes2 = st + L.a2_off, *scales2 = st + L.b2_off;   // the second state (ICO)
     float *__restrict__ msg = V.msgv + worker * V.msgv_stride + L.msgv_off;
-    const uint8_t *__restrict__ bits = (const uint8_t *)(V.selbits + L.selbits_off);
-    const uint32_t *__restrict__ tileoff = V.tileoff + L.tileoff_off;
+    const uint32_t *__restrict__ bits = V.selbits + L.selbits_off;
     uint32_t blk_start = 0;
     if (QK == CONEF_Q_RANDBLOCK)
         blk_start = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step), d, (uint32_t)L.k);
     // iConEF-v2: the draw that stored e~ (A) and this step's second draw (B)
-    const uint8_t *__restrict__ bitsA = (const uint8_t *)(V.selbitsA + L.selbits_off);
-    const uint8_t *__restrict__ bitsB = (const uint8_t *)(V.selbitsB + L.selbits_off);
+    const uint32_t *__restrict__ bitsA = V.selbitsA + L.selbits_off;
+    const uint32_t *__restrict__ bitsB = V.selbitsB + L.selbits_off;
     const float *__restrict__ ev_old = V.ev_old + worker * V.msgv_stride + L.msgv_off;
     float *__restrict__ ev_new = V.ev_new + worker * V.msgv_stride + L.msgv_off;
     uint32_t blk_startA = 0, blk_startB = 0;
@@ -89,15 +88,15 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
             cp_async_small<4 * CW>(r_cw + slot * T * CW, codes + (CW == 1 ? (j >> 1) : j));
             cp_async_small<4>(r_sc + slot * T, word_of(scales + (size_t)(j >> unit_shift) * SB));
             if (QK == CONEF_Q_RANDK)
-                cp_async_small<4>(r_sel + slot * T, word_of(bits + (j >> 3)));
+                cp_async_small<4>(r_sel + slot * T, bits + (j >> 5));
             if (ICO == 1) {
                 cp_async_small<4 * CW>(r_cv + slot * T * CW, codes2 + (CW == 1 ? (j >> 1) : j));
                 cp_async_small<4>(r_sc2 + slot * T, word_of(scales2 + (size_t)(j >> unit_shift) * SB));
             }
             if (ICO == 2 && QK == CONEF_Q_RANDK) {
                 if (V.ev_valid)
-                    cp_async_small<4>(r_selA + slot * T, word_of(bitsA + (j >> 3)));
-                cp_async_small<4>(r_selB + slot * T, word_of(bitsB + (j >> 3)));
+                    cp_async_small<4>(r_selA + slot * T, bitsA + (j >> 5));
+                cp_async_small<4>(r_selB + slot * T, bitsB + (j >> 5));
             }
         }
         cp_async_commit();
@@ -107,11 +106,10 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
             return __half2float(__ushort_as_half((unsigned short)((blk & 1u) ? word >> 16 : word & 0xFFFFu)));
         return __uint_as_float(word);
     };
-    auto byte_in = [](uint32_t word, const uint8_t *p) { return (word >> (8 * (uint32_t)((uintptr_t)p & 3))) & 0xFFu; };
+    auto byte_in = [](uint32_t word, uint32_t j) { return (word >> (j & 24u)) & 0xFFu; };   // this thread's 8 bits of a bitmap word
 #pragma unroll
     for (int s = 0; s < D - 1; ++s)
         issue(s, s);
-    uint32_t toff = 0;
     int rs = 0;
     // one chunk; CHECK is false where the warp's 256 elements all exist (no selects on `valid`)
     auto chunk = [&](int c, auto check_c) {
@@ -120,7 +118,7 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
         cp_async_wait<D - 1>();                          // this chunk's copies have landed
         constexpr int buf = 0;
         float4 g0[1], g1[1];
-        uint32_t w0[1], w1[1], v0[1], v1[1], sel[1], selA[1], selB[1];
+        uint32_t w0[1], w1[1], v0[1], v1[1], sel[1], selA[1], selB[1];   // sel: bitmap words
         float sc[1], sc2[1];
         {
             const uint32_t jj = elem(c);
@@ -131,7 +129,7 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
             w0[0] = have ? r_cw[rs * T * CW] : 0u;
             w1[0] = (have && CW == 2) ? r_cw[rs * T * CW + CW - 1] : 0u;
             sc[0] = have ? scale_in(r_sc[rs * T], jj >> unit_shift) : 0.f;
-            sel[0] = (have && QK == CONEF_Q_RANDK) ? byte_in(r_sel[rs * T], bits + (jj >> 3)) : 0u;
+            sel[0] = (have && QK == CONEF_Q_RANDK) ? r_sel[rs * T] : 0u;
             v0[0] = v1[0] = 0u;
             sc2[0] = 0.f;
             selA[0] = selB[0] = 0u;
@@ -141,22 +139,20 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
                 sc2[0] = have ? scale_in(r_sc2[rs * T], jj >> unit_shift) : 0.f;
             }
             if (ICO == 2 && QK == CONEF_Q_RANDK) {
-                selA[0] = (have && V.ev_valid) ? byte_in(r_selA[rs * T], bitsA + (jj >> 3)) : 0u;
-                selB[0] = have ? byte_in(r_selB[rs * T], bitsB + (jj >> 3)) : 0u;
+                selA[0] = (have && V.ev_valid) ? r_selA[rs * T] : 0u;
+                selB[0] = have ? r_selB[rs * T] : 0u;
             }
         }
         rs = rs + 1 == D ? 0 : rs + 1;
         const uint32_t j = elem(c);
         const bool valid = !CHECK || j < d;
-        if (QK == CONEF_Q_RANDK && c % kFvChunks == 0)
-            toff = tileoff[tile0 + c / kFvChunks];
         const float gv[8] = {g0[buf].x, g0[buf].y, g0[buf].z, g0[buf].w, g1[buf].x, g1[buf].y, g1[buf].z, g1[buf].w};
         float e[8], r[8];
         decode8<DK, HALF>(w0[buf], w1[buf], scale_const<DK, HALF>(sc[buf]), e);
         float qv[8];
         if (ICO == 1)
             decode8<DK, HALF>(v0[buf], v1[buf], scale_const<DK, HALF>(sc2[buf]), qv);
-        uint32_t mybits = sel[buf];
+        uint32_t mybits = byte_in(sel[buf], j);
         // iConEF-v2: the stored state is q; e~ comes from the values draw A kept
         uint32_t mA = 0, mB = 0, slotA = 0, slotB = 0;
         if (ICO == 2) {
@@ -164,23 +160,12 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
             for (int q = 0; q < 8; ++q)
                 qv[q] = e[q];
             if (QK == CONEF_Q_RANDK) {
-                mA = selA[buf];
-                mB = selB[buf];
-                const int cA = __popc(mA), cB = __popc(mB);
-                int incA = cA, incB = cB;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int tA = __shfl_up_sync(0xffffffffu, incA, o), tB = __shfl_up_sync(0xffffffffu, incB, o);
-                    if (o < lpb && (lane & (lpb - 1)) >= o) {
-                        incA += tA;
-                        incB += tB;
-                    }
-                }
-                const uint32_t tile = tile0 + (uint32_t)(c / kFvChunks), unit = j >> unit_shift;
-                if (cA)
-                    slotA = V.tileoffA[L.tileoff_off + tile] + V.unitoffA[L.unitoff_off + unit] + (uint32_t)(incA - cA);
-                if (cB)
-                    slotB = V.tileoffB[L.tileoff_off + tile] + V.unitoffB[L.unitoff_off + unit] + (uint32_t)(incB - cB);
+                mA = byte_in(selA[buf], j);
+                mB = byte_in(selB[buf], j);
+                if (mA)
+                    slotA = draw_slot(L, V.wordoffA, V.tileoffA, selA[buf], j);
+                if (mB)
+                    slotB = draw_slot(L, V.wordoffB, V.tileoffB, selB[buf], j);
             } else {
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
@@ -213,16 +198,8 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
         // message slot of this thread's first selected element
         uint32_t slot = 0;
         if (QK == CONEF_Q_RANDK) {
-            const int cnt = __popc(mybits);
-            int inc = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, inc, o);
-                if (o < lpb && (lane & (lpb - 1)) >= o)
-                    inc += t;
-            }
-            if (cnt)
-                slot = toff + V.unitoff[L.unitoff_off + (j >> unit_shift)] + (uint32_t)(inc - cnt);   // (a copy of this word in the ring cost more than the load)
+            if (mybits)
+                slot = draw_slot(L, V.wordoff, V.tileoff, sel[buf], j);
         } else if (QK == CONEF_Q_RANDBLOCK) {
             slot = j - blk_start + (uint32_t)__ffs(mybits) - 1u;   // the block is contiguous: first selected element
         }

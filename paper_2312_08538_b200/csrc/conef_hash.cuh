@@ -27,12 +27,30 @@ __host__ __device__ __forceinline__ uint64_t h64(uint64_t st, uint64_t j)
     return mix64(st + kGolden * (j + 1));
 }
 __device__ __forceinline__ uint32_t hash32(uint64_t st, uint64_t j) { return (uint32_t)(h64(st, j) >> 32); }
-
-
-// membership in S_t: key(j) = (hash32(j) << 32) | j is not above the threshold (tau_hi, tau_lo)
-__device__ __forceinline__ bool rk_selected(uint32_t h, uint32_t j, uint32_t tau_hi, uint32_t tau_lo)
+// hash32 without the mixer's last step, which can only flip the lowest bit: comparisons with an even
+// bound (x < even) come out the same
+__device__ __forceinline__ uint32_t hash32_but_lowest(uint64_t st, uint64_t j)
 {
-    return h < tau_hi || (h == tau_hi && j <= tau_lo);
+    uint64_t z = st + kGolden * (j + 1);
+    z ^= z >> 30;
+    z *= 0xBF58476D1CE4E5B9ULL;
+    z ^= z >> 27;
+    return (uint32_t)((z * 0x94D049BB133111EBULL) >> 32);
+}
+
+// Window [lo, hi] of hash values that holds the k-th smallest of d uniform 32-bit hashes: six
+// standard deviations of that rank, sqrt(k (1 - k/d)), and a margin for small k, to either side of
+// its expectation; cap: room for the elements inside (12 deviations and twice the margin expected);
+// scale: ((h - lo) * scale) >> 32 cuts the window into 256 equal bins
+inline void select_window(int64_t d, int64_t k, uint32_t &lo, uint32_t &hi, uint32_t &cap, uint64_t &scale)
+{
+    const double sd = __builtin_sqrt((double)k * (1.0 - (double)k / (double)d)), half = 6.0 * sd + 16.0;
+    const double per = 4294967296.0 / (double)d;   // hash values per rank
+    const double a = ((double)k - half) * per, b = ((double)k + half) * per;
+    lo = (a > 0.0 ? (uint32_t)a : 0u) & ~1u;                  // even, and hi odd: see hash32_but_lowest
+    hi = (b < 4294967295.0 ? (uint32_t)b : 0xFFFFFFFFu) | 1u;
+    cap = (uint32_t)(16.0 * sd + 256.0);
+    scale = (256ull << 32) / ((uint64_t)(hi - lo) + 1u);
 }
 
 // random-block-k: first index of the kept block, uniform on [0, d - k], from the shared stream

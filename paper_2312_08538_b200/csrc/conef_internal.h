@@ -23,21 +23,12 @@ constexpr int kP2RowsPerTile = 256;     // pass 2: rows reduced by one CTA befor
 constexpr int kRsThreads = 128;         // row sketch: threads per CTA (four columns each where 16-byte loads line up, else one)
 constexpr int kRsBuckets = 8;           // row sketch: buckets handled by one CTA
 constexpr int kHistTile = 8192;         // random-k selection: elements hashed per CTA
-constexpr int kHistBins = 2048;         // radix levels: 11 + 11 + 10 bits of the 32-bit hash
-constexpr int kMaxTies = 1024;          // elements that may share the threshold's 32-bit hash
-constexpr int kSelWords = 3 * kHistBins + 16 + kMaxTies;  // uint32 words of selection scratch per tensor
-
-// selection state words (after the three histograms)
-enum { SEL_PREFIX = 0, SEL_REMAIN = 1, SEL_TAU_HI = 2, SEL_TAU_LO = 3, SEL_NTIES = 4, SEL_NCAND = 5,
-       // used by the allocation-free selection only: radix levels that found their bin (bits 0-2),
-       // a failed tie-break, the number of coordinates counted
-       SEL_FOUND = 6, SEL_FAILED = 7, SEL_TOTAL = 8 };
+constexpr int kSelWords = 8;            // uint32 words of counters per tensor
 
 // status bits written by kernels (sticky, OR-ed)
 enum {
-    ST_TIE_OVERFLOW = 1,    // more elements share the threshold hash than the tie list holds
     ST_COUNT_MISMATCH = 2,  // the number of selected coordinates differs from k
-    ST_SELECT_FAILED = 4,   // a radix level found no bin holding the wanted rank
+    ST_SELECT_FAILED = 4,   // no threshold: a radix level without its bin, or too many keys on one 32-bit hash
     ST_FUSED_TIMEOUT = 8    // a bounded wait of the fused low-rank kernel ran out (a copy or a gang member never arrived)
 };
 
@@ -62,13 +53,15 @@ struct LayerDesc {
     int64_t msgq_off;    // floats, within a worker's Q message
     int64_t msg1d_off;   // floats, within a worker's DENSE1D message
     int64_t idx_off;     // uint32 words in the shared index buffer
-    int64_t unitoff_off; // uint32 words in the shared per-unit slot-offset buffer
+    int64_t wordoff_off; // uint16 entries in the shared slot offsets of bitmap words within their tile
     int64_t tileoff_off; // uint32 words in the shared per-tile (kHistTile elements) slot-offset buffer
     int64_t selbits_off; // uint32 words in the shared membership bitmap (bit i of word w: element 32 w + i is in S_t)
     int64_t part_off;    // floats, within a worker's pass-2 partial buffer
-    int64_t sel_off;     // uint32 words in the selection scratch
-    int64_t cand_off;    // uint32 words in the candidate list (pairs: hash, index)
-    int64_t cand_cap;    // pairs the list of this tensor holds
+    int64_t sel_off;     // uint32 words in the selection counters
+    int64_t cand_off;    // pairs (hash, index) in the list of the elements inside the selection window
+    uint32_t cand_cap;   // pairs the list of this tensor holds
+    uint32_t sel_lo, sel_hi, sel_pad;   // the window of hash values that holds the threshold
+    uint64_t sel_scale;                 // its bins
     int64_t p2_rows_generic;  // partial rows written by the generic pass 2
     int64_t p2_rows_fast;     // ... by the tuned pass 2
     // geometry of the tuned low-rank kernels (conef_fast.cuh); fast == 0: generic only
@@ -118,11 +111,13 @@ struct DevView {
     float *ppart;        int64_t ppart_stride;    // pass-1 partial rows per column segment
     // shared by all workers
     float *pbar, *phat, *qprev;                   // indexed by msgp_off / msgq_off
-    uint32_t *idx, *unitoff, *tileoff, *sel, *selbits;
-    uint32_t *cand;      // random-k selection: elements of the threshold's first-level bin, as (hash, index)
+    uint32_t *idx, *tileoff, *sel, *selbits;
+    uint16_t *wordoff;
+    uint32_t *cand;      // random-k selection: the elements inside the window, as (hash, index)
     // iConEF-v2 (Alg. 3 line 12): e~ = Q(p - Delta) kept as the k values of a second draw of Q.
     // Set A is the draw that stored the values being read (step ev_step), set B this step's.
-    uint32_t *unitoffA, *tileoffA, *selbitsA, *unitoffB, *tileoffB, *selbitsB;
+    uint32_t *tileoffA, *selbitsA, *tileoffB, *selbitsB;
+    uint16_t *wordoffA, *wordoffB;
     float *ev_old, *ev_new;      // per worker (msgv_stride apart), per tensor at msgv_off
     int64_t ev_step;
     int32_t ev_valid, ev_pad;    // 0: no e~ stored yet (e~_0 = 0)
@@ -131,6 +126,7 @@ struct DevView {
     const int32_t *pfx_rs;
     int32_t rs_vec_ok;   // this call's gradient pointers allow 16-byte loads
     int32_t fv_tiles;    // tuned fused step: selection tiles per CTA
+    int32_t sel_tiles, sel_pad;   // random-k selection: tiles per CTA
     // tile -> tensor prefix tables (n_layers + 1 entries each)
     const int32_t *pfx_flat, *pfx_pass, *pfx_p1, *pfx_p2, *pfx_q2, *pfx_hist, *pfx_gs;
     int32_t fast_on;     // the tuned kernels produced this step's pass-2 partials

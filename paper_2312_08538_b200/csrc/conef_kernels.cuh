@@ -27,284 +27,6 @@ __global__ void __launch_bounds__(256) k_passthrough(const __grid_constant__ Dev
     }
 }
 
-// ------------------------------------------------------------------ random-k selection (S3a)
-// The index set S_t = the k smallest keys (hash32(j) << 32 | j).  Membership
-// is "key(j) <= tau"; tau is found by a three-level radix select on the hash
-// (11 + 11 + 10 bits) followed by a tie-break on the index among the few
-// elements that share the threshold's hash.  No memory traffic: hashes are
-// recomputed.  All of it depends on (seed, tensor, step) only and is shared
-// by the N workers.
-
-template <int LEVEL>
-__global__ void __launch_bounds__(256) k_rk_hist(const __grid_constant__ DevView V)
-{
-    __shared__ uint32_t hist[kHistBins];
-    const int li = find_layer(V.pfx_hist, V.n_layers, blockIdx.x);
-    const LayerDesc &L = V.layers[li];
-    uint32_t *sel = V.sel + L.sel_off;
-    const uint32_t prefix = sel[3 * kHistBins + SEL_PREFIX];
-    for (int b = threadIdx.x; b < kHistBins; b += 256)
-        hist[b] = 0;
-    __syncthreads();
-    const uint64_t st = stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step);
-    const int64_t j0 = (int64_t)(blockIdx.x - V.pfx_hist[li]) * kHistTile;
-    uint32_t *stw = sel + 3 * kHistBins;
-    uint32_t *cand = V.cand + 2 * L.cand_off;
-    auto visit = [&](uint32_t h, uint32_t j) {
-        if (LEVEL == 0)
-            atomicAdd(&hist[h >> 21], 1u);
-        else if (LEVEL == 1) {
-            if ((h >> 21) == prefix) {
-                atomicAdd(&hist[(h >> 10) & 2047u], 1u);
-                // the later levels only look at these elements (one in 2048): keep them
-                const uint32_t pos = atomicAdd(&stw[SEL_NCAND], 1u);
-                if (pos < (uint32_t)L.cand_cap) {
-                    cand[2 * pos] = h;
-                    cand[2 * pos + 1] = j;
-                }
-            }
-        } else if (LEVEL == 2) {
-            if ((h >> 10) == prefix)
-                atomicAdd(&hist[h & 1023u], 1u);
-        } else {  // LEVEL 3: collect the elements whose hash equals the threshold's
-            if (h == stw[SEL_TAU_HI]) {
-                uint32_t pos = atomicAdd(&stw[SEL_NTIES], 1u);
-                if (pos < (uint32_t)kMaxTies)
-                    stw[16 + pos] = j;
-            }
-        }
-    };
-    // levels 2 and 3 read the candidate list where it held everything, and hash all elements again
-    // where it overflowed
-    const uint32_t ncand = LEVEL >= 2 ? stw[SEL_NCAND] : 0u;
-    if (LEVEL >= 2 && ncand <= (uint32_t)L.cand_cap) {
-        for (int q = threadIdx.x; q < kHistTile; q += 256) {
-            const int64_t x = j0 + q;
-            if (x >= (int64_t)ncand)
-                break;
-            visit(cand[2 * x], cand[2 * x + 1]);
-        }
-    } else {
-        for (int q = threadIdx.x; q < kHistTile; q += 256) {
-            int64_t j = j0 + q;
-            if (j >= L.d)
-                break;
-            visit(hash32(st, (uint64_t)j), (uint32_t)j);
-        }
-    }
-    if (LEVEL < 3) {
-        __syncthreads();
-        uint32_t *gh = sel + LEVEL * kHistBins;
-        for (int b = threadIdx.x; b < kHistBins; b += 256)
-            if (hist[b])
-                atomicAdd(&gh[b], hist[b]);
-    }
-}
-
-// one CTA of 1024 threads per random-k tensor: pick the bin that holds the
-// wanted rank, or (LEVEL 3) the tie-breaking index
-template <int LEVEL>
-__global__ void __launch_bounds__(1024) k_rk_pick(const __grid_constant__ DevView V)
-{
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t ties[kMaxTies];
-    const int li = find_layer(V.pfx_gs, V.n_layers, blockIdx.x);
-    const LayerDesc &L = V.layers[li];
-    uint32_t *sel = V.sel + L.sel_off;
-    uint32_t *stw = sel + 3 * kHistBins;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (LEVEL < 3) {
-        const uint32_t remain = (LEVEL == 0) ? (uint32_t)L.k : stw[SEL_REMAIN];
-        const uint32_t *gh = sel + LEVEL * kHistBins;
-        // each thread owns two adjacent bins; inclusive scan over threads
-        uint32_t c0 = gh[2 * tid], c1 = gh[2 * tid + 1];
-        uint32_t mine = c0 + c1, inc = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o)
-                inc += n;
-        }
-        if (lane == 31)
-            wsum[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t w = wsum[lane], winc = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                uint32_t n = __shfl_up_sync(0xffffffffu, winc, o);
-                if (lane >= o)
-                    winc += n;
-            }
-            wsum[lane] = winc - w;  // exclusive
-        }
-        __syncthreads();
-        const uint32_t before = wsum[warp] + inc - mine;  // elements in bins below 2*tid
-        __syncthreads();
-        if (tid == 0)
-            wsum[0] = 0xffffffffu;
-        __syncthreads();
-        // the wanted rank (1-based "remain") lies in the first bin whose inclusive count reaches it
-        if (before < remain && remain <= before + mine) {
-            uint32_t bin, rem;
-            if (remain <= before + c0) {
-                bin = 2 * tid;
-                rem = remain - before;
-            } else {
-                bin = 2 * tid + 1;
-                rem = remain - before - c0;
-            }
-            const uint32_t prefix = (LEVEL == 0) ? 0u : stw[SEL_PREFIX];
-            if (LEVEL == 0)
-                stw[SEL_PREFIX] = bin;
-            else if (LEVEL == 1)
-                stw[SEL_PREFIX] = (prefix << 11) | bin;
-            else
-                stw[SEL_TAU_HI] = (prefix << 10) | bin;
-            stw[SEL_REMAIN] = rem;
-            wsum[0] = 0;
-        }
-        __syncthreads();
-        if (tid == 0 && wsum[0] != 0)
-            atomicOr(V.status, ST_SELECT_FAILED);
-    } else {
-        const uint32_t n = stw[SEL_NTIES], remain = stw[SEL_REMAIN];
-        if (n > (uint32_t)kMaxTies || remain > n || remain == 0) {
-            if (tid == 0) {
-                atomicOr(V.status, ST_TIE_OVERFLOW);
-                stw[SEL_TAU_LO] = 0xffffffffu;
-            }
-            return;
-        }
-        if ((uint32_t)tid < n)
-            ties[tid] = stw[16 + tid];
-        __syncthreads();
-        if ((uint32_t)tid < n) {
-            uint32_t me = ties[tid], rank = 0;
-            for (uint32_t q = 0; q < n; ++q)
-                rank += ties[q] < me;
-            if (rank == remain - 1)
-                stw[SEL_TAU_LO] = me;  // the remain-th smallest index among the ties
-        }
-    }
-}
-
-
-// count the selected coordinates of every work unit; the exclusive prefix within the CTA's tile of
-// kHistTile elements goes to unitoff, the tile's total to tileoff (scanned by k_rk_scan):
-// message slot of an element = tileoff[tile] + unitoff[unit] + its rank within the unit
-__global__ void __launch_bounds__(256) k_rk_count(const __grid_constant__ DevView V)
-{
-    __shared__ uint32_t cnts[kHistTile / 32];
-    const int li = find_layer(V.pfx_hist, V.n_layers, blockIdx.x);
-    const LayerDesc &L = V.layers[li];
-    const uint32_t *stw = V.sel + L.sel_off + 3 * kHistBins;
-    const uint32_t tau_hi = stw[SEL_TAU_HI], tau_lo = stw[SEL_TAU_LO];
-    const uint64_t st = stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step);
-    const int64_t tile = blockIdx.x - V.pfx_hist[li];
-    const int64_t j0 = tile * kHistTile;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int U = L.unit, nu = kHistTile / U;   // units per tile: 32 .. 256
-    for (int u = warp; u < nu; u += 8) {
-        const int64_t base = j0 + (int64_t)u * U;
-        int cnt = 0;
-        if (base < L.d)
-            for (int q = lane; q < U; q += 32) {
-                const int64_t j = base + q;
-                const bool in = j < L.d && rk_selected(hash32(st, (uint64_t)j), (uint32_t)j, tau_hi, tau_lo);
-                // membership bitmap, read by the step kernels of all workers instead of hashing again
-                const uint32_t word = __ballot_sync(0xffffffffu, in);
-                if (lane == 0)
-                    V.selbits[L.selbits_off + ((base + q) >> 5)] = word;
-                cnt += in;
-            }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        if (lane == 0)
-            cnts[u] = (uint32_t)cnt;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        // exclusive scan of up to 256 counts: 8 per lane, then across lanes
-        const int per = nu / 32;   // 1 .. 8
-        uint32_t loc[8], sum = 0;
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            loc[x] = x < per ? cnts[lane * per + x] : 0u;
-            sum += loc[x];
-        }
-        uint32_t inc = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o)
-                inc += t;
-        }
-        uint32_t run = inc - sum;
-        const int64_t unit0 = j0 / U;
-#pragma unroll
-        for (int x = 0; x < 8; ++x)
-            if (x < per) {
-                if (unit0 + lane * per + x < L.nunits)
-                    V.unitoff[L.unitoff_off + unit0 + lane * per + x] = run;
-                run += loc[x];
-            }
-        if (lane == 31)
-            V.tileoff[L.tileoff_off + tile] = inc;
-    }
-}
-
-// exclusive scan of the per-tile totals, in place; one CTA per tensor
-__global__ void __launch_bounds__(1024) k_rk_scan(const __grid_constant__ DevView V)
-{
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t carry_s;
-    const int li = find_layer(V.pfx_gs, V.n_layers, blockIdx.x);
-    const LayerDesc &L = V.layers[li];
-    if (!L.compressed)
-        return;
-    uint32_t *cnt = V.tileoff + L.tileoff_off;
-    const int64_t ntiles = (L.d + kHistTile - 1) / kHistTile;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0)
-        carry_s = 0;
-    __syncthreads();
-    for (int64_t base = 0; base < ntiles; base += 1024) {
-        int64_t u = base + tid;
-        uint32_t v = u < ntiles ? cnt[u] : 0u, inc = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o)
-                inc += n;
-        }
-        if (lane == 31)
-            wsum[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t w = wsum[lane], winc = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                uint32_t n = __shfl_up_sync(0xffffffffu, winc, o);
-                if (lane >= o)
-                    winc += n;
-            }
-            wsum[lane] = winc - w;
-        }
-        __syncthreads();
-        const uint32_t carry = carry_s;
-        if (u < ntiles)
-            cnt[u] = carry + wsum[warp] + inc - v;
-        __syncthreads();
-        if (tid == 1023)
-            carry_s = carry + wsum[31] + inc;
-        __syncthreads();
-    }
-    if (tid == 0 && carry_s != (uint32_t)L.k)
-        atomicOr(V.status, ST_COUNT_MISMATCH);
-}
-
 // ------------------------------------------------------------------ quantiser (S5, C1)
 // scale and reciprocal of one block from its absmax; zero block when the
 // stored scale is not >= FLT_MIN
@@ -377,33 +99,23 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat(const __grid_constant__ D
             break;
         const uint32_t base = (uint32_t)(unit * U) + lane * E;
         // iConEF-v2 with random-k: membership bits of this thread's elements in the two second draws
-        // (a thread's E <= 8 elements share one bitmap word) and the slot of its first member, by
-        // the same prefix over the unit's lanes as the message slots below
+        // (a thread's E <= 8 elements share one bitmap word) and the slot of its first member
         uint32_t bitsA = 0, bitsB = 0, slotA = 0, slotB = 0;
         if (QK == CONEF_Q_RANDK && v2) {
             if (base < d) {
                 const uint32_t emask = (1u << E) - 1u, wi = L.selbits_off + (base >> 5), sh = base & 31u;
-                bitsA = V.ev_valid ? (V.selbitsA[wi] >> sh) & emask : 0u;
-                bitsB = (V.selbitsB[wi] >> sh) & emask;
+                const uint32_t wA = V.ev_valid ? V.selbitsA[wi] : 0u, wB = V.selbitsB[wi];
+                bitsA = (wA >> sh) & emask;
+                bitsB = (wB >> sh) & emask;
+                if (bitsA)
+                    slotA = draw_slot(L, V.wordoffA, V.tileoffA, wA, base);
+                if (bitsB)
+                    slotB = draw_slot(L, V.wordoffB, V.tileoffB, wB, base);
             }
-            const int cA = __popc(bitsA), cB = __popc(bitsB);
-            int incA = cA, incB = cB;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int nA = __shfl_up_sync(0xffffffffu, incA, o), nB = __shfl_up_sync(0xffffffffu, incB, o);
-                if (lane >= o) {
-                    incA += nA;
-                    incB += nB;
-                }
-            }
-            const int64_t tile = (unit * U) / kHistTile;
-            if (V.ev_valid)
-                slotA = V.tileoffA[L.tileoff_off + tile] + V.unitoffA[L.unitoff_off + unit] + (uint32_t)(incA - cA);
-            slotB = V.tileoffB[L.tileoff_off + tile] + V.unitoffB[L.unitoff_off + unit] + (uint32_t)(incB - cB);
         }
         float val[8], ekeep[8];
         bool selq[8];
-        int nsel = 0;
+        const uint32_t selword = (QK == CONEF_Q_RANDK && base < d) ? V.selbits[L.selbits_off + (base >> 5)] : 0u;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             val[q] = 0.f;
@@ -419,7 +131,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat(const __grid_constant__ D
                             e = ev_old[slotA + (uint32_t)__popc(bitsA & ((1u << q) - 1u))];
                     } else {
                         uint32_t sl;
-                        if (V.ev_valid && draw_member<QD>(L, V.selbitsA, V.unitoffA, V.tileoffA, blk_startA, j, sl))
+                        if (V.ev_valid && draw_member<QD>(L, V.selbitsA, V.wordoffA, V.tileoffA, blk_startA, j, sl))
                             e = ev_old[sl];
                     }
                 } else
@@ -434,8 +146,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat(const __grid_constant__ D
                     msg[j] = p;
                     val[q] = 0.f;
                 } else if (QK == CONEF_Q_RANDK) {
-                    selq[q] = (V.selbits[L.selbits_off + (j >> 5)] >> (j & 31u)) & 1u;   // bitmap left by the selection
-                    nsel += selq[q];
+                    selq[q] = (selword >> (j & 31u)) & 1u;   // bitmap left by the selection
                     val[q] = p;
                 } else if (QK == CONEF_Q_RANDBLOCK) {
                     const uint32_t slot = j - blk_start;   // wraps to a large value below the block
@@ -455,16 +166,8 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat(const __grid_constant__ D
                 }
             }
         }
-        if (QK == CONEF_Q_RANDK) {
-            int inc = nsel;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int n = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o)
-                    inc += n;
-            }
-            uint32_t slot = V.tileoff[L.tileoff_off + (unit * U) / kHistTile] + V.unitoff[L.unitoff_off + unit] +
-                            (uint32_t)(inc - nsel);
+        if (QK == CONEF_Q_RANDK && ((selword >> (base & 31u)) & ((1u << E) - 1u))) {
+            uint32_t slot = draw_slot(L, V.wordoff, V.tileoff, selword, base);
 #pragma unroll
             for (int q = 0; q < 8; ++q)
                 if (selq[q]) {
@@ -487,7 +190,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_flat(const __grid_constant__ D
                         ev_new[slotB + (uint32_t)__popc(bitsB & ((1u << q) - 1u))] = val[q];
                         val[q] = 0.f;
                     }
-                } else if (q < E && j < d && draw_member<QD>(L, V.selbitsB, V.unitoffB, V.tileoffB, blk_startB, j, sl)) {
+                } else if (q < E && j < d && draw_member<QD>(L, V.selbitsB, V.wordoffB, V.tileoffB, blk_startB, j, sl)) {
                     ev_new[sl] = val[q];
                     val[q] = 0.f;
                 }
@@ -859,9 +562,9 @@ __global__ void __launch_bounds__(256) k_decompress(const __grid_constant__ DevV
                 if (V.qkind == CONEF_Q_RANDBLOCK) {
                     const uint32_t bs = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)(V.ev_step + kSecondDraw)),
                                                         (uint32_t)L.d, (uint32_t)L.k);
-                    if (draw_member<CONEF_Q_RANDBLOCK>(L, V.selbitsA, V.unitoffA, V.tileoffA, bs, (uint32_t)j, sl))
+                    if (draw_member<CONEF_Q_RANDBLOCK>(L, V.selbitsA, V.wordoffA, V.tileoffA, bs, (uint32_t)j, sl))
                         ev = evp[sl];
-                } else if (draw_member<CONEF_Q_RANDK>(L, V.selbitsA, V.unitoffA, V.tileoffA, 0u, (uint32_t)j, sl))
+                } else if (draw_member<CONEF_Q_RANDK>(L, V.selbitsA, V.wordoffA, V.tileoffA, 0u, (uint32_t)j, sl))
                     ev = evp[sl];
             }
             e = __fadd_rn(ev, e);

@@ -7,258 +7,170 @@
 // framework's step) often holds no ConEF context and is not allowed to touch
 // the device allocator: its memory pool is fixed up front, and a cudaMalloc in
 // the middle of a step would synchronise the device or fail under memory
-// pressure.  The selection needs scratch (radix histograms, per-block counts);
+// pressure.  The selection needs scratch (a count per tile, the elements near the threshold);
 // here that scratch is a fixed array that lives in the library's device image.
 #include <cuda_runtime.h>
 
 #include <mutex>
 
-#include "conef_hash.cuh"
-#include "conef_internal.h"
+#include "conef_select.cuh"
 
 using namespace conef;
 
 namespace {
 
-constexpr int kNaUnit = 256;                                        // elements per counted block
+constexpr int kNaPer = 8;                                           // consecutive elements per thread
+constexpr int kNaTile = kSelThreads * kNaPer;                       // elements per CTA
 constexpr int64_t kNaMaxElems = CONEF_NOALLOC_MAX_ELEMS;
-constexpr int kNaSelWords = kSelWords;                              // histograms, state, tie list
-constexpr int64_t kNaWords = kNaSelWords + kNaMaxElems / kNaUnit;   // + one count per block
+constexpr int64_t kNaTiles = kNaMaxElems / kNaTile;
+constexpr int64_t kNaList = 16 * 2048 + 256;                        // select_window's room at its largest: d = 2^24, k = d / 2
+constexpr int64_t kNaWords = 8 + kNaTiles + 2 * kNaList;            // counters, a count per tile, the window's elements
 
 // The scratch itself.  Every GPU that loads the library holds these ~290 KB
 // until the process exits.  In host code the name below is only a handle for
 // cudaGetSymbolAddress; it is not a device address.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNaWords];
 
+// counter words: CTAs that have finished, elements listed (both zero between calls), then what the
+// first kernel leaves for the second: threshold key, whether the selection failed
+enum { NA_DONE = 0, NA_LISTED = 1, NA_TAU_LO = 2, NA_TAU_HI = 3, NA_FAILED = 4 };
+
 struct NaArgs {
-    uint32_t *sel;     // selection scratch (kNaSelWords words)
-    uint32_t *cnt;     // per-block counts, then offsets
+    uint32_t *ctr, *cnt;
+    uint2 *list;
     uint64_t stream;   // hash stream key of (seed, tensor, step)
-    uint32_t d, k;
+    uint32_t d, k, lo, hi, cap, ntiles;
+    uint64_t scale;
 };
 
-template <int LEVEL>
-__global__ void __launch_bounds__(256) k_na_hist(NaArgs a)
+// The context's selection (conef_select.cuh) without its bitmap: one pass counts each tile's elements
+// below the window and lists those inside; the last CTA finds the threshold and the tiles' offsets.
+__global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
 {
-    __shared__ uint32_t hist[kHistBins];
-    uint32_t *stw = a.sel + 3 * kHistBins;
-    const uint32_t prefix = stw[SEL_PREFIX];
-    for (int b = threadIdx.x; b < kHistBins; b += 256)
-        hist[b] = 0;
+    __shared__ SelectShared S;
+    __shared__ uint32_t s_n, s_base, s_cnt, s_last;
+    const int tid = threadIdx.x;
+    const bool windowed = a.d > (uint32_t)kSelShortTensor;
+    S.hist[tid] = 0;   // the bins of select_threshold
+    if (tid == 0)
+        s_n = s_cnt = 0;
     __syncthreads();
-    const int64_t j0 = (int64_t)blockIdx.x * kHistTile;
-    for (int q = threadIdx.x; q < kHistTile; q += 256) {
-        const int64_t j = j0 + q;
-        if (j >= a.d)
-            break;
-        const uint32_t h = hash32(a.stream, (uint64_t)j);
-        if (LEVEL == 0)
-            atomicAdd(&hist[h >> 21], 1u);
-        else if (LEVEL == 1) {
-            if ((h >> 21) == prefix)
-                atomicAdd(&hist[(h >> 10) & 2047u], 1u);
-        } else if (LEVEL == 2) {
-            if ((h >> 10) == prefix)
-                atomicAdd(&hist[h & 1023u], 1u);
-        } else if (h == stw[SEL_TAU_HI]) {
-            const uint32_t pos = atomicAdd(&stw[SEL_NTIES], 1u);
-            if (pos < (uint32_t)kMaxTies)
-                stw[16 + pos] = (uint32_t)j;
-        }
-    }
-    if (LEVEL < 3) {
-        __syncthreads();
-        uint32_t *gh = a.sel + LEVEL * kHistBins;
-        for (int b = threadIdx.x; b < kHistBins; b += 256)
-            if (hist[b])
-                atomicAdd(&gh[b], hist[b]);
-    }
-}
-
-// one CTA: the bin that holds the wanted rank (levels 0-2), the tie-breaking index (level 3)
-template <int LEVEL>
-__global__ void __launch_bounds__(1024) k_na_pick(NaArgs a, int32_t *status)
-{
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t ties[kMaxTies];
-    uint32_t *stw = a.sel + 3 * kHistBins;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (LEVEL < 3) {
-        const uint32_t remain = (LEVEL == 0) ? a.k : stw[SEL_REMAIN];
-        const uint32_t *gh = a.sel + LEVEL * kHistBins;
-        const uint32_t c0 = gh[2 * tid], c1 = gh[2 * tid + 1];
-        const uint32_t mine = c0 + c1;
-        uint32_t inc = mine;
+    if (windowed) {
+        const uint32_t j0 = blockIdx.x * kNaTile + tid * kNaPer;
+        uint32_t below = 0, upto = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o)
-                inc += n;
+        for (uint32_t q = 0; q < kNaPer; ++q) {
+            const uint32_t h = hash32_but_lowest(a.stream, j0 + q);
+            below |= h < a.lo ? 1u << q : 0u;
+            upto |= h <= a.hi ? 1u << q : 0u;
         }
-        if (lane == 31)
-            wsum[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t w = wsum[lane];
-            uint32_t winc = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t n = __shfl_up_sync(0xffffffffu, winc, o);
-                if (lane >= o)
-                    winc += n;
-            }
-            wsum[lane] = winc - w;
-        }
-        __syncthreads();
-        const uint32_t before = wsum[warp] + inc - mine;
-        if (before < remain && remain <= before + mine) {
-            uint32_t bin, rem;
-            if (remain <= before + c0) {
-                bin = 2 * tid;
-                rem = remain - before;
+        const uint32_t exist = j0 >= a.d ? 0u : a.d - j0 >= kNaPer ? (1u << kNaPer) - 1u : (1u << (a.d - j0)) - 1u;
+        for (uint32_t m = upto & ~below & exist; m; m &= m - 1) {
+            const uint32_t j = j0 + (uint32_t)__ffs(m) - 1u;
+            const uint2 e = make_uint2(hash32(a.stream, j), j);
+            const uint32_t pos = atomicAdd(&s_n, 1u);
+            if (pos < (uint32_t)kSelList) {
+                ((uint2 *)S.keys)[pos] = e;
             } else {
-                bin = 2 * tid + 1;
-                rem = remain - before - c0;
+                const uint32_t g = atomicAdd(&a.ctr[NA_LISTED], 1u);
+                if (g < a.cap)
+                    a.list[g] = e;
             }
-            const uint32_t prefix = (LEVEL == 0) ? 0u : stw[SEL_PREFIX];
-            if (LEVEL == 0)
-                stw[SEL_PREFIX] = bin;
-            else if (LEVEL == 1)
-                stw[SEL_PREFIX] = (prefix << 11) | bin;
-            else
-                stw[SEL_TAU_HI] = (prefix << 10) | bin;
-            stw[SEL_REMAIN] = rem;
-            atomicOr(&stw[SEL_FOUND], 1u << LEVEL);
         }
-    } else {
-        const uint32_t n = stw[SEL_NTIES], remain = stw[SEL_REMAIN];
-        if (n > (uint32_t)kMaxTies || remain > n || remain == 0) {
-            if (tid == 0) {
-                if (status)
-                    atomicOr(status, ST_TIE_OVERFLOW);
-                stw[SEL_TAU_LO] = 0xffffffffu;
-                stw[SEL_FAILED] = 1u;
-            }
-            return;
-        }
-        if ((uint32_t)tid < n)
-            ties[tid] = stw[16 + tid];
+        below = __popc(below & exist);
+        below = __reduce_add_sync(0xffffffffu, below);
+        if ((tid & 31) == 0 && below)
+            atomicAdd(&s_cnt, below);
         __syncthreads();
-        if ((uint32_t)tid < n) {
-            const uint32_t me = ties[tid];
-            uint32_t rank = 0;
-            for (uint32_t q = 0; q < n; ++q)
-                rank += ties[q] < me;
-            if (rank == remain - 1)
-                stw[SEL_TAU_LO] = me;
+        const uint32_t n = min(s_n, (uint32_t)kSelList);
+        if (tid == 0) {
+            s_base = n ? atomicAdd(&a.ctr[NA_LISTED], n) : 0u;
+            a.cnt[blockIdx.x] = s_cnt;
         }
+        __syncthreads();
+        for (uint32_t x = tid; x < n; x += kSelThreads)
+            if (s_base + x < a.cap)
+                a.list[s_base + x] = ((uint2 *)S.keys)[x];
     }
-}
-
-// WRITE == 0: count the selected coordinates of each block of 256 elements;
-// WRITE == 1: write them, in ascending order, at the block's offset
-template <int WRITE>
-__global__ void __launch_bounds__(256) k_na_count(NaArgs a, uint32_t *__restrict__ idx_out)
-{
-    const uint32_t *stw = a.sel + 3 * kHistBins;
-    const uint32_t tau_hi = stw[SEL_TAU_HI], tau_lo = stw[SEL_TAU_LO];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nblocks = ((int64_t)a.d + kNaUnit - 1) / kNaUnit;
-    for (int64_t blk = (int64_t)blockIdx.x * 8 + warp; blk < nblocks; blk += (int64_t)gridDim.x * 8) {
-        const uint32_t base = (uint32_t)blk * kNaUnit + lane * 8;   // a lane owns 8 consecutive elements
-        bool sel[8];
-        int n = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const uint32_t j = base + q;
-            sel[q] = j < a.d && rk_selected(hash32(a.stream, j), j, tau_hi, tau_lo);
-            n += sel[q];
-        }
-        int inc = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o)
-                inc += t;
-        }
-        if (!WRITE) {
-            if (lane == 31)
-                a.cnt[blk] = (uint32_t)inc;
-        } else {
-            uint32_t slot = a.cnt[blk] + (uint32_t)(inc - n);
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (sel[q]) {
-                    if (slot < a.k)   // never past the caller's k entries, whatever went wrong before
-                        idx_out[slot] = base + q;
-                    ++slot;
-                }
-        }
-    }
-}
-
-// exclusive scan of the block counts, in place (one CTA)
-__global__ void __launch_bounds__(1024) k_na_scan(NaArgs a)
-{
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t carry_s;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t nblocks = ((int64_t)a.d + kNaUnit - 1) / kNaUnit;
-    if (tid == 0)
-        carry_s = 0;
+    __threadfence();
     __syncthreads();
-    for (int64_t base = 0; base < nblocks; base += 1024) {
-        const int64_t u = base + tid;
-        const uint32_t v = u < nblocks ? a.cnt[u] : 0u;
-        uint32_t inc = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o)
-                inc += n;
-        }
-        if (lane == 31)
-            wsum[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t w = wsum[lane];
-            uint32_t winc = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t n = __shfl_up_sync(0xffffffffu, winc, o);
-                if (lane >= o)
-                    winc += n;
-            }
-            wsum[lane] = winc - w;
-        }
-        __syncthreads();
-        const uint32_t carry = carry_s;
-        if (u < nblocks)
-            a.cnt[u] = carry + wsum[warp] + inc - v;
-        __syncthreads();
-        if (tid == 1023)
-            carry_s = carry + wsum[31] + inc;
-        __syncthreads();
-    }
     if (tid == 0)
-        a.sel[3 * kHistBins + SEL_TOTAL] = carry_s;   // coordinates selected in all
+        s_last = atomicAdd(&a.ctr[NA_DONE], 1u) == a.ntiles - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_last)
+        return;
+    __threadfence();
+    const uint32_t nlist = load_cg(&a.ctr[NA_LISTED]);
+    uint32_t total = 0xFFFFFFFFu;
+    if (windowed && nlist <= a.cap)
+        total = select_finish<kNaTile>(S, a.list, nlist, a.lo, a.scale, a.k, a.cnt, a.ntiles, [](uint32_t) {});
+    bool failed = false;
+    // no listed element belongs: the members are the elements below the window (lo > 0 then)
+    if (total != 0xFFFFFFFFu && S.tau == 0 && tid == 0)
+        S.tau = ((uint64_t)a.lo << 32) - 1u;
+    if (total == 0xFFFFFFFFu) {
+        __syncthreads();
+        select_exact(S, a.stream, a.d, a.k);
+        failed = S.bad != 0;
+        const uint64_t tau = failed ? 0 : S.tau;
+        for (uint32_t t = 0; t < a.ntiles; ++t) {
+            __syncthreads();
+            if (tid == 0)
+                s_cnt = 0;
+            __syncthreads();
+            uint32_t c = 0;
+            for (uint32_t q = tid; q < kNaTile; q += kSelThreads) {
+                const uint32_t j = t * kNaTile + q;
+                c += j < a.d && (((uint64_t)hash32(a.stream, j) << 32) | j) <= tau;
+            }
+            c = __reduce_add_sync(0xffffffffu, c);
+            if ((tid & 31) == 0 && c)
+                atomicAdd(&s_cnt, c);
+            __syncthreads();
+            if (tid == 0)
+                a.cnt[t] = s_cnt;
+        }
+        __threadfence();
+        __syncthreads();
+        total = scan_counts(a.cnt, a.ntiles, S.wsum);
+    }
+    if (tid == 0) {
+        a.ctr[NA_DONE] = a.ctr[NA_LISTED] = 0;
+        a.ctr[NA_TAU_LO] = (uint32_t)S.tau;
+        a.ctr[NA_TAU_HI] = (uint32_t)(S.tau >> 32);
+        a.ctr[NA_FAILED] = failed || total != a.k;
+    }
 }
 
-// A selection that did not come out as exactly k coordinates (a radix level without its bin, more
-// ties on the threshold hash than the tie list holds, a count other than k) is made visible in
-// the output itself, since this entry point neither synchronises nor owns a status buffer:
-// idx_out[0] = 0xFFFFFFFF, a value no index can take.
-__global__ void k_na_finish(NaArgs a, uint32_t *__restrict__ idx_out)
+// The members in ascending order, hashed once more.  A selection that did not come out as exactly k
+// coordinates is made visible in the output itself, since this entry point neither synchronises nor
+// owns a status buffer: nothing is written but idx_out[0] = 0xFFFFFFFF, a value no index can take.
+__global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32_t *__restrict__ idx_out)
 {
-    const uint32_t *stw = a.sel + 3 * kHistBins;
-    if (threadIdx.x == 0 && (stw[SEL_FOUND] != 7u || stw[SEL_FAILED] != 0u || stw[SEL_TOTAL] != a.k))
-        idx_out[0] = 0xFFFFFFFFu;
+    __shared__ uint32_t wsum[kSelThreads / 32];
+    if (a.ctr[NA_FAILED]) {
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            idx_out[0] = 0xFFFFFFFFu;
+        return;
+    }
+    const uint64_t tau = ((uint64_t)a.ctr[NA_TAU_HI] << 32) | a.ctr[NA_TAU_LO];
+    const uint32_t j0 = blockIdx.x * kNaTile + threadIdx.x * kNaPer;
+    uint32_t in = 0, total;
+#pragma unroll
+    for (uint32_t q = 0; q < kNaPer; ++q) {
+        const uint32_t j = j0 + q;
+        if ((((uint64_t)hash32(a.stream, j) << 32) | j) <= tau && j < a.d)
+            in |= 1u << q;
+    }
+    uint32_t slot = a.cnt[blockIdx.x] + block_exclusive(__popc(in), wsum, total);
+    for (; in; in &= in - 1, ++slot)
+        if (slot < a.k)   // never past the caller's k entries, whatever went wrong before
+            idx_out[slot] = j0 + (uint32_t)__ffs(in) - 1u;
 }
 
 // device address of the scratch on each device, resolved once per device
 std::mutex g_mu;
 uint32_t *g_scratch_ptr[64] = {nullptr};
-int g_sm_count[64] = {0};
 
 }  // namespace
 
@@ -280,10 +192,6 @@ extern "C" int conef_randk_indices_noalloc(uint64_t seed, int64_t tensor, int64_
             void *p = nullptr;
             if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p)
                 return CONEF_ERR_CUDA;
-            int sms = 0;
-            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-                return CONEF_ERR_CUDA;
-            g_sm_count[dev] = sms;
             g_scratch_ptr[dev] = (uint32_t *)p;
         }
         scratch = g_scratch_ptr[dev];
@@ -292,29 +200,15 @@ extern "C" int conef_randk_indices_noalloc(uint64_t seed, int64_t tensor, int64_
         return CONEF_ERR_CUDA;   // an error from before this call is pending: nothing is launched on top of it
     cudaStream_t s = (cudaStream_t)stream;
     NaArgs a;
-    a.sel = scratch;
-    a.cnt = scratch + kNaSelWords;
+    a.ctr = scratch;
+    a.cnt = scratch + 8;
+    a.list = (uint2 *)(scratch + 8 + kNaTiles);
     a.stream = stream_key(seed, (uint64_t)tensor, (uint64_t)step);
     a.d = (uint32_t)d;
     a.k = (uint32_t)k;
-    // the array keeps the previous call's contents: histograms and state must start at zero
-    if (cudaMemsetAsync(a.sel, 0, sizeof(uint32_t) * kNaSelWords, s) != cudaSuccess)
-        return CONEF_ERR_CUDA;
-    const int nh = (int)((d + kHistTile - 1) / kHistTile);
-    const int64_t nblocks = (d + kNaUnit - 1) / kNaUnit;
-    const int64_t nc_cap = (int64_t)g_sm_count[dev] * 8;
-    const int nc = (int)((nblocks + 7) / 8 < nc_cap ? (nblocks + 7) / 8 : nc_cap);
-    k_na_hist<0><<<nh, 256, 0, s>>>(a);
-    k_na_pick<0><<<1, 1024, 0, s>>>(a, nullptr);
-    k_na_hist<1><<<nh, 256, 0, s>>>(a);
-    k_na_pick<1><<<1, 1024, 0, s>>>(a, nullptr);
-    k_na_hist<2><<<nh, 256, 0, s>>>(a);
-    k_na_pick<2><<<1, 1024, 0, s>>>(a, nullptr);
-    k_na_hist<3><<<nh, 256, 0, s>>>(a);
-    k_na_pick<3><<<1, 1024, 0, s>>>(a, nullptr);
-    k_na_count<0><<<nc, 256, 0, s>>>(a, idx_out);
-    k_na_scan<<<1, 1024, 0, s>>>(a);
-    k_na_count<1><<<nc, 256, 0, s>>>(a, idx_out);
-    k_na_finish<<<1, 32, 0, s>>>(a, idx_out);
+    select_window(d, k, a.lo, a.hi, a.cap, a.scale);
+    a.ntiles = (uint32_t)((d + kNaTile - 1) / kNaTile);
+    k_na_select<<<a.ntiles, kSelThreads, 0, s>>>(a);
+    k_na_write<<<a.ntiles, kSelThreads, 0, s>>>(a, idx_out);
     return cudaGetLastError() == cudaSuccess ? CONEF_OK : CONEF_ERR_CUDA;
 }

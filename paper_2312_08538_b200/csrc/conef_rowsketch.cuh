@@ -33,8 +33,7 @@ namespace conef {
 // the instructions, so the simple form stays.
 constexpr int kRsRows = CONEF_RS_ROWS;
 
-// VEC columns per thread (4: 16-byte loads; needs cols % 4 == 0, for random-k cols % 32 == 0, and
-// 16-byte aligned gradients; 1: any shape).  The CTA covers kRsThreads * VEC columns of kRsBuckets
+// VEC columns per thread (4: 16-byte loads; needs cols % 4 == 0 and 16-byte aligned gradients; 1: any shape).  The CTA covers kRsThreads * VEC columns of kRsBuckets
 // buckets of one sketch row.
 // RK: 4 when the tensor's rank is exactly 4 (one 16-byte load per row of P_hat), else 8 (any rank).
 template <int QK, int VEC, bool V1, int RK>
@@ -50,7 +49,6 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
     local /= slabs;
     const uint32_t grp = local % groups;
     const uint32_t i = local / groups;                      // sketch row this CTA builds
-    const int lane = threadIdx.x & 31;
     const uint32_t b = slab * CW + threadIdx.x * VEC;       // this thread's first column
     const bool colok = b < m;                               // VEC divides cols: all or none of the thread's columns exist
 
@@ -64,8 +62,6 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
     float *__restrict__ msg = V.msgv + worker * V.msgv_stride + L.msgv_off;
 
     const uint32_t *__restrict__ selbits = V.selbits + L.selbits_off;
-    const uint32_t *__restrict__ uoff = V.unitoff + L.unitoff_off;
-    const uint32_t *__restrict__ toff = V.tileoff + L.tileoff_off;   // slot = toff[tile] + uoff[unit] + rank
     uint32_t blk_start = 0;
     if (QK == CONEF_Q_RANDBLOCK)
         blk_start = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step), d, (uint32_t)L.k);
@@ -195,23 +191,7 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
                         nsel += sel[x];
                     }
                     if (i == 0) {   // the CTAs of sketch row 0 meet every matrix row once: they write the message
-                        uint32_t slot = 0;
-                        if (VEC == 4) {
-                            // cols % 32 == 0: a message unit is 8 consecutive lanes; exclusive prefix within them
-                            int inc = nsel;
-#pragma unroll
-                            for (int o = 1; o < 8; o <<= 1) {
-                                const int t = __shfl_up_sync(0xffffffffu, inc, o, 8);
-                                if ((lane & 7) >= o)
-                                    inc += t;
-                            }
-                            if (nsel)
-                                slot = toff[j / kHistTile] + uoff[j >> 5] + (uint32_t)(inc - nsel);
-                        } else {
-                            // one element per thread: its rank within the unit from the unit's bitmap word
-                            if (sel[0])
-                                slot = toff[j / kHistTile] + uoff[j >> 5] + __popc(word & ((1u << (j & 31u)) - 1u));
-                        }
+                        uint32_t slot = nsel ? draw_slot(L, V.wordoff, V.tileoff, word, j) : 0u;
 #pragma unroll
                         for (int x = 0; x < VEC; ++x)
                             if (sel[x]) {

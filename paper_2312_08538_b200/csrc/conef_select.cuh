@@ -1,0 +1,414 @@
+// Random-k selection (S3a): the shared index set S_t = the k smallest keys (hash32(j) << 32 | j) of a
+// tensor, which depends on (seed, tensor, step) only.
+//
+// Every element is hashed ONCE.  The k-th smallest of d uniform hashes lies within a few standard
+// deviations, sqrt(k (1 - k/d)) ranks, of rank k, so the window [lo, hi] of hash values that holds it
+// is known before anything is hashed (select_window; six deviations and a margin: missed with
+// probability below 1e-8 per tensor and step).  The hashing pass marks the elements below the window
+// in a bitmap and lists the few inside it (about 12 sqrt(k)); the CTA that finishes a tensor last
+// picks the exact threshold key among those, marks the members of the list, and turns the tiles' counts
+// into message offsets.  Where the window missed, and for tensors so short that it would hold most
+// of the tensor, that CTA finds the threshold by a radix select that hashes the tensor again.
+//
+// Consumers read the bitmap (bit i of word w: element 32 w + i is a member) and
+//   slot(j) = tileoff[j / 8192] + wordoff[j / 32] + members of j's word below j.
+//
+// Bound by the integer pipe: about 25 instructions per element, eight of them multiplies, no memory
+// traffic to speak of.  Transformer-big list (210 M elements): a three-level radix select that hashed
+// everything three times took 1.26 ms in ten launches; this takes 0.25 ms in two (the hashing loop
+// alone, without anything around it, 0.17 ms).  One 256 x 512 matrix: 35 us in eleven launches -> 11 us.
+#pragma once
+#include "conef_common.cuh"
+
+namespace conef {
+
+constexpr int kSelThreads = 256;
+constexpr int kSelBins = 2048;
+constexpr int kSelShortTensor = 1024;   // up to here the window is not used
+constexpr int kSelTailTiles = 16;       // tensors of at most this many tiles: the last CTA also writes the offsets
+constexpr int kSelList = 2304;          // window entries a CTA holds in shared memory (enough for any tensor of kSelTailTiles)
+constexpr int kSelTiles = 1280;         // tile counts it holds there
+constexpr int kSelTailWords = kSelTailTiles * kHistTile / 32;
+
+// shared memory of the CTA that finishes a tensor
+struct SelectShared {
+    uint32_t hist[kSelBins];
+    uint64_t keys[kSelList];
+    union {
+        uint32_t tiles[kSelTiles];
+        uint32_t words[kSelTailWords];
+    };
+    uint32_t wsum[kSelThreads / 32], wsum2[kSelThreads / 32];
+    uint64_t tau;
+    uint32_t bin, rem, n, bad;
+};
+
+// Loads of what other CTAs of the same launch wrote before their ticket: past L1, and volatile, so that
+// the compiler keeps them behind the ticket (__ldcg is free to move; it read the list before it was
+// complete).
+__device__ __forceinline__ uint32_t load_cg(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 load_cg(const uint2 *p)
+{
+    uint2 v;
+    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void load_cg(const uint32_t *p, uint32_t (&v)[8])   // 32 bytes, 16-byte aligned
+{
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p) : "memory");
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p + 4) : "memory");
+}
+
+// exclusive prefix over the CTA's threads of v; total: the sum over all threads
+__device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *wsum, uint32_t &total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o)
+            inc += n;
+    }
+    __syncthreads();   // wsum may still be read from the previous call
+    if (lane == 31)
+        wsum[warp] = inc;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kSelThreads / 32; ++w) {
+        const uint32_t t = wsum[w];
+        before += w < warp ? t : 0u;
+        all += t;
+    }
+    total = all;
+    return before + inc - v;
+}
+
+// The bin of the histogram that holds rank `rank` (1-based) and the rank within it; S.bad when none does.
+__device__ __forceinline__ void select_bin(SelectShared &S, uint32_t rank)
+{
+    constexpr int PER = kSelBins / kSelThreads;
+    const int tid = threadIdx.x;
+    if (tid == 0)
+        S.bad = 1u;
+    uint32_t c[PER], sum = 0, total;
+#pragma unroll
+    for (int x = 0; x < PER; ++x)
+        sum += c[x] = S.hist[tid * PER + x];
+    uint32_t before = block_exclusive(sum, S.wsum, total);
+    if (before < rank && rank <= before + sum) {
+#pragma unroll
+        for (int x = 0; x < PER; ++x) {
+            if (before < rank && rank <= before + c[x]) {
+                S.bin = tid * PER + x;
+                S.rem = rank - before;
+                S.bad = 0u;
+            }
+            before += c[x];
+        }
+    }
+    __syncthreads();
+}
+
+// S.tau = the key of rank `rank` (1-based) among the S.n keys in S.keys
+__device__ __forceinline__ void select_key(SelectShared &S, uint32_t rank)
+{
+    const uint32_t n = S.n;
+    if (n > (uint32_t)kSelList || rank == 0 || rank > n) {
+        if (threadIdx.x == 0)
+            S.bad = 1u;
+    } else {
+        for (uint32_t x = threadIdx.x; x < n; x += kSelThreads) {
+            const uint64_t me = S.keys[x];
+            uint32_t below = 0;
+            for (uint32_t y = 0; y < n; ++y)
+                below += S.keys[y] < me;
+            if (below == rank - 1)   // keys are distinct
+                S.tau = me;
+        }
+    }
+    __syncthreads();
+}
+
+// The threshold among the window's elements.  `below_mine`: the calling thread's share of the number of
+// elements below the window; scale: see select_window.  The caller has zeroed S.hist[0 .. kSelThreads)
+// and synchronised.  Returns the number of elements below the window, or 0xFFFFFFFF where the window
+// does not hold the threshold; S.tau is the threshold key (0 when no listed element belongs).
+__device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const uint2 *list, uint32_t nlist, uint32_t lo, uint64_t scale,
+                                                     uint32_t k, uint32_t below_mine)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool shared = nlist <= (uint32_t)kSelList;
+    if (shared) {
+        // one linear bin per thread; the few keys of the bin that holds the rank are compared
+        auto bin_of = [&](uint32_t h) { return min((uint32_t)(((uint64_t)(h - lo) * scale) >> 32), (uint32_t)kSelThreads - 1u); };
+#pragma unroll 4
+        for (uint32_t x = tid; x < nlist; x += kSelThreads) {
+            const uint2 e = load_cg(&list[x]);
+            S.keys[x] = ((uint64_t)e.x << 32) | e.y;
+            atomicAdd(&S.hist[bin_of(e.x)], 1u);
+        }
+        if (tid == 0) {
+            S.n = 0;
+            S.bad = 1u;
+            S.tau = 0;
+        }
+        __syncthreads();
+        const uint32_t c = S.hist[tid];
+        uint32_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o)
+                inc += n;
+        }
+        below_mine = __reduce_add_sync(0xffffffffu, below_mine);
+        if (lane == 31) {
+            S.wsum[warp] = inc;
+            S.wsum2[warp] = below_mine;
+        }
+        __syncthreads();
+        uint32_t before = inc - c, below = 0;
+#pragma unroll
+        for (int w = 0; w < kSelThreads / 32; ++w) {
+            before += w < warp ? S.wsum[w] : 0u;
+            below += S.wsum2[w];
+        }
+        if (below > k || k - below > nlist)
+            return 0xFFFFFFFFu;
+        const uint32_t rank = k - below;
+        if (rank == 0)
+            return below;
+        if (before < rank && rank <= before + c) {
+            S.bin = tid;
+            S.rem = rank - before;
+        }
+        __syncthreads();
+        const uint32_t bin = S.bin;
+        for (uint32_t x = tid; x < nlist; x += kSelThreads) {
+            const uint64_t key = S.keys[x];
+            if (bin_of((uint32_t)(key >> 32)) == bin)
+                S.hist[kSelThreads + min(atomicAdd(&S.n, 1u), (uint32_t)(kSelBins - kSelThreads - 1))] = x;   // (its place, not its count)
+        }
+        __syncthreads();
+        const uint32_t np = S.n;
+        if (np > (uint32_t)(kSelBins - kSelThreads - 1))
+            return 0xFFFFFFFFu;
+        for (uint32_t x = tid; x < np; x += kSelThreads) {
+            const uint64_t me = S.keys[S.hist[kSelThreads + x]];
+            uint32_t smaller = 0;
+            for (uint32_t y = 0; y < np; ++y)
+                smaller += S.keys[S.hist[kSelThreads + y]] < me;
+            if (smaller == S.rem - 1) {   // keys are distinct
+                S.tau = me;
+                S.bad = 0u;
+            }
+        }
+        __syncthreads();
+        return S.bad ? 0xFFFFFFFFu : below;
+    }
+    // a longer list stays in L2: two passes over it, 2048 bins
+    const uint64_t scale8 = scale * (kSelBins / kSelThreads);
+    auto bin_of = [&](uint32_t h) { return min((uint32_t)(((uint64_t)(h - lo) * scale8) >> 32), (uint32_t)kSelBins - 1u); };
+    for (int b = kSelThreads + tid; b < kSelBins; b += kSelThreads)
+        S.hist[b] = 0;
+    if (tid == 0)
+        S.tau = 0;
+    uint32_t below;
+    block_exclusive(below_mine, S.wsum, below);   // (synchronises)
+    if (below > k || k - below > nlist)
+        return 0xFFFFFFFFu;
+    if (below == k)
+        return below;
+#pragma unroll 8
+    for (uint32_t x = tid; x < nlist; x += kSelThreads)
+        atomicAdd(&S.hist[bin_of(load_cg(&list[x]).x)], 1u);
+    __syncthreads();
+    select_bin(S, k - below);
+    if (S.bad)
+        return 0xFFFFFFFFu;
+    const uint32_t bin = S.bin;
+    if (tid == 0)
+        S.n = 0;
+    __syncthreads();
+#pragma unroll 8
+    for (uint32_t x = tid; x < nlist; x += kSelThreads) {
+        const uint2 e = load_cg(&list[x]);
+        if (bin_of(e.x) == bin) {
+            const uint32_t pos = atomicAdd(&S.n, 1u);
+            if (pos < (uint32_t)kSelList)
+                S.keys[pos] = ((uint64_t)e.x << 32) | e.y;
+        }
+    }
+    __syncthreads();
+    select_key(S, S.rem);
+    return S.bad ? 0xFFFFFFFFu : below;
+}
+
+// calls f(j) for the listed elements that belong to the set
+template <class F>
+__device__ __forceinline__ void select_listed(SelectShared &S, const uint2 *list, uint32_t nlist, F f)
+{
+    const uint64_t tau = S.tau;
+    if (nlist <= (uint32_t)kSelList) {
+        for (uint32_t x = threadIdx.x; x < nlist; x += kSelThreads)
+            if (S.keys[x] <= tau)
+                f((uint32_t)S.keys[x]);
+    } else {
+#pragma unroll 4
+        for (uint32_t x = threadIdx.x; x < nlist; x += kSelThreads) {
+            const uint2 e = load_cg(&list[x]);
+            if ((((uint64_t)e.x << 32) | e.y) <= tau)
+                f(e.y);
+        }
+    }
+}
+
+// The threshold key of rank k over all d elements by one CTA: 11 + 11 + 10 bits of the hash, then the
+// index among the elements that share the threshold's hash.
+static __device__ __noinline__ void select_exact(SelectShared &S, uint64_t st, uint32_t d, uint32_t k)
+{
+    const int tid = threadIdx.x;
+    uint32_t prefix = 0, rank = k;
+#pragma unroll 1
+    for (int level = 0; level < 3; ++level) {
+        for (int b = tid; b < kSelBins; b += kSelThreads)
+            S.hist[b] = 0;
+        __syncthreads();
+        for (uint64_t j = tid; j < d; j += kSelThreads) {
+            const uint32_t h = hash32(st, j);
+            if (level == 0)
+                atomicAdd(&S.hist[h >> 21], 1u);
+            else if (level == 1) {
+                if ((h >> 21) == prefix)
+                    atomicAdd(&S.hist[(h >> 10) & 2047u], 1u);
+            } else if ((h >> 10) == prefix)
+                atomicAdd(&S.hist[h & 1023u], 1u);
+        }
+        __syncthreads();
+        select_bin(S, rank);
+        if (S.bad)
+            return;
+        prefix = level == 0 ? S.bin : level == 1 ? (prefix << 11) | S.bin : (prefix << 10) | S.bin;
+        rank = S.rem;
+        __syncthreads();
+    }
+    if (tid == 0)
+        S.n = 0;
+    __syncthreads();
+    for (uint64_t j = tid; j < d; j += kSelThreads)
+        if (hash32(st, j) == prefix) {
+            const uint32_t pos = atomicAdd(&S.n, 1u);
+            if (pos < (uint32_t)kSelList)
+                S.keys[pos] = ((uint64_t)prefix << 32) | (uint32_t)j;
+        }
+    __syncthreads();
+    select_key(S, rank);
+}
+
+// exclusive scan of n counts in place by the CTA; returns the total
+__device__ __forceinline__ uint32_t scan_counts(uint32_t *cnt, int64_t n, uint32_t *wsum)
+{
+    constexpr int PER = 4;
+    uint32_t carry = 0;
+    for (int64_t base = 0; base < n; base += kSelThreads * PER) {
+        const int64_t at = base + (int64_t)threadIdx.x * PER;
+        uint32_t c[PER], sum = 0, total;
+#pragma unroll
+        for (int x = 0; x < PER; ++x)
+            sum += c[x] = at + x < n ? load_cg(cnt + at + x) : 0u;
+        uint32_t run = carry + block_exclusive(sum, wsum, total);
+#pragma unroll
+        for (int x = 0; x < PER; ++x) {
+            if (at + x < n)
+                cnt[at + x] = run;
+            run += c[x];
+        }
+        carry += total;
+    }
+    __syncthreads();
+    return carry;
+}
+
+// What the last CTA of a tensor does with the window's elements: finds the threshold, calls mark(j) for
+// the listed members and adds them to their tiles' counts (tile = j / TILE), and turns the counts
+// into exclusive offsets, in place.  Returns the number of members, or 0xFFFFFFFF where the window
+// does not hold the threshold (nothing is marked then).
+template <uint32_t TILE, class Mark>
+__device__ __forceinline__ uint32_t select_finish(SelectShared &S, const uint2 *list, uint32_t nlist, uint32_t lo, uint64_t scale,
+                                                  uint32_t k, uint32_t *cnt, uint32_t ntiles, Mark mark)
+{
+    const int tid = threadIdx.x;
+    const bool shared = ntiles <= (uint32_t)kSelTiles;
+    uint32_t mine = 0;
+#pragma unroll 4
+    for (uint32_t t = tid; t < ntiles; t += kSelThreads) {
+        const uint32_t c = load_cg(cnt + t);
+        if (shared)
+            S.tiles[t] = c;
+        mine += c;
+    }
+    if (select_threshold(S, list, nlist, lo, scale, k, mine) == 0xFFFFFFFFu)
+        return 0xFFFFFFFFu;
+    select_listed(S, list, nlist, [&](uint32_t j) {
+        mark(j);
+        atomicAdd(shared ? &S.tiles[j / TILE] : &cnt[j / TILE], 1u);
+    });
+    if (!shared) {
+        __threadfence();
+        __syncthreads();
+        return scan_counts(cnt, ntiles, S.wsum);
+    }
+    __syncthreads();
+    constexpr uint32_t PER = (kSelTiles + kSelThreads - 1) / kSelThreads;
+    uint32_t c[PER], sum = 0, total;
+#pragma unroll
+    for (uint32_t x = 0; x < PER; ++x)
+        sum += c[x] = tid * PER + x < ntiles ? S.tiles[tid * PER + x] : 0u;
+    uint32_t run = block_exclusive(sum, S.wsum, total);
+#pragma unroll
+    for (uint32_t x = 0; x < PER; ++x) {
+        if (tid * PER + x < ntiles)
+            cnt[tid * PER + x] = run;
+        run += c[x];
+    }
+    return total;
+}
+
+// Offsets of the words of one tile of 8192 elements (a warp; 8 words per lane).
+__device__ __forceinline__ void select_offsets(const uint32_t *bits, uint16_t *wordoff, uint32_t tile)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t w0 = tile * (kHistTile / 32) + lane * 8;
+    uint32_t word[8], cnt = 0;   // (the arrays cover whole tiles; words past the tensor are zero)
+    load_cg(bits + w0, word);
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+        cnt += __popc(word[x]);
+    uint32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o)
+            inc += n;
+    }
+    uint32_t run = inc - cnt;
+    uint32_t pair[4];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        pair[x / 2] = x % 2 ? pair[x / 2] | (run << 16) : run;
+        run += __popc(word[x]);
+    }
+    *(uint4 *)(wordoff + w0) = make_uint4(pair[0], pair[1], pair[2], pair[3]);
+}
+
+}  // namespace conef

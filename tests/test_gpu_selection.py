@@ -1,0 +1,45 @@
+"""The random-k selection at its edges: tensors around the size that skips the hash window, around a
+tile, around the number of tiles the last CTA finishes alone; one, half and all coordinates kept; a
+window too long for shared memory; a model large enough for several tiles per CTA."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import conef_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [(1, 2), (32, 32), (5, 205), (1, 8191), (2, 4096), (1, 8193), (16, 8192), (1, 16 * 8192 + 1), (3, 999)]
+
+
+def _check(shapes, k_num, k_den, steps=(0, 1)):
+    from paper_2312_08538_b200 import binding as b
+    seed = 77
+    eng = b.ConEF([(r, c, 1) for r, c in shapes], 1, dict(kind="randk", k_num=k_num, k_den=k_den, seed=seed),
+                  dict(kind="int8", block=256), 0.1)
+    g = [torch.ones(sum(r * c for r, c in shapes), device="cuda")]
+    for step in steps:
+        eng.step(step, g, 0)
+        for l, (r, c) in enumerate(shapes):
+            d = r * c
+            k = max(1, d * k_num // k_den)
+            want = orc.randk_indices(seed, l, step, d, k)
+            assert np.array_equal(eng.indices(l).cpu().numpy().view(np.uint32), want), (step, r, c)
+            if d <= b.NOALLOC_MAX_ELEMS:
+                out = torch.empty(k, dtype=torch.int32, device="cuda")
+                b.conef_randk_indices_noalloc(seed, l, step, d, k, out)
+                assert np.array_equal(out.cpu().numpy().view(np.uint32), want), (step, r, c)
+    assert eng.last_status() == 0
+
+
+@pytest.mark.parametrize("k_num,k_den", [(1, 1000000), (1, 100), (1, 2), (1, 1)])
+def test_edges_of_tiles_and_windows(k_num, k_den):
+    _check(EDGES, k_num, k_den)
+
+
+def test_window_longer_than_shared_memory():
+    _check([(1000, 1600), (7, 9)], 1, 3)
+
+
+def test_several_tiles_per_cta():
+    _check([(5000, 8100), (33, 77), (2, 8192), (1200, 1111)], 1, 1000, steps=(5,))

@@ -16,6 +16,7 @@
 #include "conef_randk.cuh"
 #include "conef_rowsketch.cuh"
 #include "conef_apply.cuh"
+#include "conef_decode.cuh"
 #include "conef_fast.cuh"
 #include "conef_gs.cuh"
 #include "conef_flatvec.cuh"
@@ -28,7 +29,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 27 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 28 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -38,6 +39,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_CSK,                                               // count sketch applied run by run: one tile per run
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
        T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
+       T_DECODE,                                            // stored error expanded: tiles of kDecTile elements
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -260,6 +262,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             }
             tiles[T_FLAT] = (int)ceil_div(L.nunits, kFlatUnitsPerCta);
             tiles[T_GS] = 1;
+            tiles[T_DECODE] = (int)ceil_div(L.d, kDecTile);
             if (q->kind == CONEF_Q_IDENTITY) {
                 L.k = L.d;
             } else if (q->kind == CONEF_Q_RANDBLOCK) {
@@ -1481,7 +1484,13 @@ int conef_decompress_error(conef_ctx *ctx, int worker, float *out, conef_stream 
             return rc;
         ctx->draw_step[ctx->ev_cur] = V.ev_step;
     }
-    switch (ctx->c.kind) {
+    const int ck = ctx->c.kind;
+    if (ctx->c.iconef != 2 && (ck == CONEF_C_INT8 || ck == CONEF_C_INT4 || (ck == CONEF_C_STOCHQUANT && ctx->c.levels <= 127))) {
+        decode_launch(ck == CONEF_C_INT4, ctx->c.iconef == 1, V, table_ptr(ctx, T_DECODE), tiles_of(ctx, T_DECODE), worker, out, s);
+        LAUNCH_CHECK(ctx);
+        return CONEF_OK;
+    }
+    switch (ck) {
     case CONEF_C_IDENTITY: k_decompress<CONEF_C_IDENTITY><<<n, 256, 0, s>>>(V, worker, out); break;
     case CONEF_C_INT8: k_decompress<CONEF_C_INT8><<<n, 256, 0, s>>>(V, worker, out); break;
     case CONEF_C_INT4: k_decompress<CONEF_C_INT4><<<n, 256, 0, s>>>(V, worker, out); break;

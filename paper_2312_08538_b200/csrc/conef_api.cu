@@ -17,8 +17,10 @@
 #include "conef_rowsketch.cuh"
 #include "conef_apply.cuh"
 #include "conef_decode.cuh"
+#include "conef_dense.cuh"
 #include "conef_fast.cuh"
 #include "conef_gs.cuh"
+#include "conef_flat16.cuh"
 #include "conef_flatvec.cuh"
 #include "conef_chunksketch.cuh"
 #include "conef_rowsp1.cuh"
@@ -39,7 +41,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_CSK,                                               // count sketch applied run by run: one tile per run
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
        T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
-       T_DECODE,                                            // stored error expanded: tiles of kDecTile elements
+       T_DECODE,                                            // tiles of kDecTile elements: stored error expanded; the step on a dense error
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -296,12 +298,12 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             if (q->kind != CONEF_Q_LOWRANK) {
                 L.msgv_off = P.msg_elems[CONEF_MSG_VALUES];
                 P.msg_elems[CONEF_MSG_VALUES] += L.k;
-                // the tuned fused step: whole 8-element groups, 16-byte accesses, Alg. 2 proper
+                // the tuned fused step: Alg. 2 and iConEF-v1 on every shape; iConEF-v2 on whole 8-element
+                // groups with 16-byte accesses
                 const bool fv = (c->kind == CONEF_C_INT8 || c->kind == CONEF_C_INT4 ||
                                  (c->kind == CONEF_C_STOCHQUANT && c->levels <= 127)) && c->beta == 0.f &&
-                                (c->iconef == 0 || c->kind != CONEF_C_STOCHQUANT) &&
-                                L.d % 8 == 0 && L.g_off % 4 == 0 && L.d < (1ll << 31) &&
-                                (q->kind != CONEF_Q_IDENTITY || L.msgv_off % 4 == 0);
+                                (c->iconef == 0 || c->kind != CONEF_C_STOCHQUANT) && L.d < (1ll << 31) &&
+                                (c->iconef != 2 || (L.d % 8 == 0 && L.g_off % 4 == 0));
                 // the chunk-wise count sketch: a run's two windows in shared memory
                 const int64_t csk_floats = c->kind == CONEF_C_COUNTSKETCH && c->cs_chunk > 0
                                                ? 2 * c->cs_rows * chunk_window_max(L.d, L.w, c->cs_chunk) : 0;
@@ -1188,15 +1190,24 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
         LAUNCH_CHECK(ctx);
     }
     // single-phase compressors: the tuned fused step where a tensor allows it, the generic kernel elsewhere
-    const bool fv = ctx->fast && V.rs_vec_ok && ctx->plan.any_fv;
+    const bool fv = ctx->fast && ctx->plan.any_fv && (ctx->c.iconef != 2 || V.rs_vec_ok);
     const bool csk = ctx->fast && ctx->plan.any_csk;
     auto flat_step = [&](auto qk) -> int {
         constexpr int QK = decltype(qk)::value;
+        if (ctx->fast && ctx->c.kind == CONEF_C_IDENTITY && ctx->c.iconef == 0) {
+            const int n = tiles_of(ctx, T_DECODE);
+            if (n > 0) {
+                k_flat_dense<QK><<<dim3(n, ctx->n_workers), kDecThreads, 0, s>>>(V, table_ptr(ctx, T_DECODE));
+                LAUNCH_CHECK(ctx);
+            }
+            return CONEF_OK;
+        }
         if (!fv && !csk)
             return launch_flat<QK>(ctx, V, s);
         if (fv) {
-            CK_CUDA(flatvec_launch(QK, ctx->c.kind, ctx->c.kind == CONEF_C_STOCHQUANT ? 0 : V.scale_half, V,
-                                   table_ptr(ctx, T_FV), tiles_of(ctx, T_FV), s));
+            const int half = ctx->c.kind == CONEF_C_STOCHQUANT ? 0 : V.scale_half;
+            CK_CUDA(ctx->c.iconef == 2 ? flatvec_launch(QK, ctx->c.kind, half, V, table_ptr(ctx, T_FV), tiles_of(ctx, T_FV), s)
+                                       : flat16_launch(QK, ctx->c.kind, half, V, table_ptr(ctx, T_FV), tiles_of(ctx, T_FV), s));
             LAUNCH_CHECK(ctx);
         }
         if (csk) {

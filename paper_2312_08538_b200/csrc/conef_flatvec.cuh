@@ -1,19 +1,13 @@
-// Tuned fused step for Q in {identity, random-k, random-block-k} with an int8 / int4 error state,
-// or the stochastic quantiser of Eq. 6 with at most 127 levels (signed levels in one byte, fp32 scale)
-// (Alg. 2 lines 5, 6, 9 in one kernel): decode, p = eta g + e, message, residual, block absmax,
-// requantise, store in place.  A thread owns 8 consecutive elements (two 16-byte copies of the
-// gradient, one 8- or 4-byte copy of the codes, through a ring of asynchronous copies), a warp 256, so that every
-// quantisation block (32..256 elements) is an aligned group of lanes and its absmax a few
-// shuffles.  Membership in the shared random-k index set comes from the bitmap that the
-// selection kernels leave (one byte per thread), not from hashing every element again for every
-// worker; message slots are tile offset + block offset + a prefix over the block's lanes.
-// ICO = 1 is iConEF-v1 (Alg. 3) on an int8 / int4 state: a second state q of the same kind is decoded
-// beside the first, p = (eta g + e~) + q, and the store has a second round, q = C(r - decode(e~)).
-// ICO = 2 is iConEF-v2 (Alg. 3 line 12) with a sparsifying Q: e~ is the k values a second draw of Q
-// kept at the step that stored them (gathered through that draw's bitmap and slot offsets), the
-// stored state is q, p = (eta g + e~) + q; this step's second draw takes its members' residuals as
-// the next e~ and the rest is stored as q = C(r - e~).
-// Takes tensors with d % 8 == 0 and 16-byte aligned gradients; the generic kernel does the rest.
+// Tuned fused step of iConEF-v2 (Alg. 3 line 12) with a sparsifying Q on an int8 / int4 state: decode,
+// p = (eta g + e~) + q, message, residual, block absmax, requantise, store in place.  e~ is the k values
+// a second draw of Q kept at the step that stored them (gathered through that draw's bitmap and slot
+// offsets), the stored state is q; this step's second draw takes its members' residuals as the next e~
+// and the rest is stored as q = C(r - e~).  A thread owns 8 consecutive elements (two 16-byte copies of
+// the gradient, one 8- or 4-byte copy of the codes, through a ring of asynchronous copies), a warp
+// 256, so that every quantisation block (32..256 elements) is an aligned group of lanes and its absmax
+// a few shuffles.  Takes tensors with d % 8 == 0 and 16-byte aligned gradients; the generic kernel does
+// the rest.  (The other compressors take conef_flat16.cuh, whose zeroing of the transmitted coordinates
+// before the arithmetic does not carry over to e~.)
 #pragma once
 #include "conef_fast.cuh"
 
@@ -24,8 +18,8 @@ constexpr int kFvChunks = kHistTile / (kFvThreads * 8);   // 256-element chunks 
 constexpr int kFvRing = 3;                                // stages of the per-thread copy ring
 constexpr int kFvTiles = 4;                               // selection tiles (8192 elements) per CTA for large models (V.fv_tiles; 1 for small ones)
 
-template <int QK, int CK, bool HALF, int ICO = 0>
-__global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+template <int QK, int CK, bool HALF>   // QK: random-k or random-block-k
+__global__ void __launch_bounds__(kFvThreads, 3) k_flat_vec2(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
@@ -36,13 +30,10 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
     const int unit_shift = 31 - __clz(L.unit);
     const int lpb = L.unit >> 3;                       // lanes per quantisation block
     constexpr int CW = (CK == CONEF_C_INT4) ? 1 : 2;   // code words per thread
-    // signed levels of the stochastic quantiser decode like int8 codes with an fp32 scale
-    constexpr int DK = (CK == CONEF_C_STOCHQUANT) ? CONEF_C_INT8 : CK;
     uint8_t *st = V.state + worker * V.state_stride;
     const float *__restrict__ g = V.grads[worker] + L.g_off;
     uint8_t *codes = st + L.a_off;
     uint8_t *scales = st + L.b_off;
-    uint8_t *codes2 = st + L.a2_off, *scales2 = st + L.b2_off;   // the second state (ICO)
     float *__restrict__ msg = V.msgv + worker * V.msgv_stride + L.msgv_off;
     const uint32_t *__restrict__ bits = V.selbits + L.selbits_off;
     uint32_t blk_start = 0;
@@ -54,7 +45,7 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
     const float *__restrict__ ev_old = V.ev_old + worker * V.msgv_stride + L.msgv_off;
     float *__restrict__ ev_new = V.ev_new + worker * V.msgv_stride + L.msgv_off;
     uint32_t blk_startA = 0, blk_startB = 0;
-    if (ICO == 2 && QK == CONEF_Q_RANDBLOCK) {
+    if (QK == CONEF_Q_RANDBLOCK) {
         blk_startA = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)(V.ev_step + kSecondDraw)), d, (uint32_t)L.k);
         blk_startB = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)(V.step + kSecondDraw)), d, (uint32_t)L.k);
     }
@@ -68,8 +59,7 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
     // A ring of kFvRing stages of asynchronous copies per thread (a thread only reads what it
     // copied, so no barrier): the gradient, the code words, and 4-byte words that hold the block's
     // scale and the thread's membership byte(s).  Stage s of thread t: lo[s][t], hi[s][t] (16 bytes
-    // each), then 4-byte arrays [s][t] in the order codes, scale, membership, and with Alg. 3 the
-    // second state's codes and scale (version 1) or the two second draws' membership (version 2).
+    // each), then 4-byte arrays [s][t] in the order codes, scale, membership, the two second draws' membership.
     extern __shared__ __align__(128) uint8_t fv_smem[];
     constexpr int D = kFvRing, T = kFvThreads;
     constexpr int SB = HALF ? 2 : 4;
@@ -77,8 +67,7 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
     float4 *r_lo = (float4 *)fv_smem + tid, *r_hi = r_lo + D * T;
     uint32_t *r32 = (uint32_t *)((float4 *)fv_smem + 2 * D * T);
     uint32_t *r_cw = r32 + tid * CW, *r_sc = r32 + D * T * CW + tid, *r_sel = r32 + D * T * (CW + 1) + tid;
-    uint32_t *r_cv = r32 + D * T * (CW + 2) + tid * CW, *r_sc2 = r32 + D * T * (2 * CW + 2) + tid;   // ICO = 1
-    uint32_t *r_selA = r32 + D * T * (CW + 2) + tid, *r_selB = r32 + D * T * (CW + 3) + tid;         // ICO = 2
+    uint32_t *r_selA = r32 + D * T * (CW + 2) + tid, *r_selB = r32 + D * T * (CW + 3) + tid;
     auto word_of = [](const void *p) { return (const void *)((uintptr_t)p & ~(uintptr_t)3); };   // the aligned 4 bytes that hold *p
     auto issue = [&](int c, int slot) {
         const uint32_t j = elem(c);
@@ -89,11 +78,7 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
             cp_async_small<4>(r_sc + slot * T, word_of(scales + (size_t)(j >> unit_shift) * SB));
             if (QK == CONEF_Q_RANDK)
                 cp_async_small<4>(r_sel + slot * T, bits + (j >> 5));
-            if (ICO == 1) {
-                cp_async_small<4 * CW>(r_cv + slot * T * CW, codes2 + (CW == 1 ? (j >> 1) : j));
-                cp_async_small<4>(r_sc2 + slot * T, word_of(scales2 + (size_t)(j >> unit_shift) * SB));
-            }
-            if (ICO == 2 && QK == CONEF_Q_RANDK) {
+            if (QK == CONEF_Q_RANDK) {
                 if (V.ev_valid)
                     cp_async_small<4>(r_selA + slot * T, bitsA + (j >> 5));
                 cp_async_small<4>(r_selB + slot * T, bitsB + (j >> 5));
@@ -118,8 +103,8 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
         cp_async_wait<D - 1>();                          // this chunk's copies have landed
         constexpr int buf = 0;
         float4 g0[1], g1[1];
-        uint32_t w0[1], w1[1], v0[1], v1[1], sel[1], selA[1], selB[1];   // sel: bitmap words
-        float sc[1], sc2[1];
+        uint32_t w0[1], w1[1], sel[1], selA[1], selB[1];   // sel: bitmap words
+        float sc[1];
         {
             const uint32_t jj = elem(c);
             const bool have = !CHECK || jj < d;   // a stage that was not filled holds stale data
@@ -130,15 +115,8 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
             w1[0] = (have && CW == 2) ? r_cw[rs * T * CW + CW - 1] : 0u;
             sc[0] = have ? scale_in(r_sc[rs * T], jj >> unit_shift) : 0.f;
             sel[0] = (have && QK == CONEF_Q_RANDK) ? r_sel[rs * T] : 0u;
-            v0[0] = v1[0] = 0u;
-            sc2[0] = 0.f;
             selA[0] = selB[0] = 0u;
-            if (ICO == 1) {
-                v0[0] = have ? r_cv[rs * T * CW] : 0u;
-                v1[0] = (have && CW == 2) ? r_cv[rs * T * CW + CW - 1] : 0u;
-                sc2[0] = have ? scale_in(r_sc2[rs * T], jj >> unit_shift) : 0.f;
-            }
-            if (ICO == 2 && QK == CONEF_Q_RANDK) {
+            if (QK == CONEF_Q_RANDK) {
                 selA[0] = (have && V.ev_valid) ? r_selA[rs * T] : 0u;
                 selB[0] = have ? r_selB[rs * T] : 0u;
             }
@@ -148,14 +126,12 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
         const bool valid = !CHECK || j < d;
         const float gv[8] = {g0[buf].x, g0[buf].y, g0[buf].z, g0[buf].w, g1[buf].x, g1[buf].y, g1[buf].z, g1[buf].w};
         float e[8], r[8];
-        decode8<DK, HALF>(w0[buf], w1[buf], scale_const<DK, HALF>(sc[buf]), e);
+        decode8<CK, HALF>(w0[buf], w1[buf], scale_const<CK, HALF>(sc[buf]), e);
         float qv[8];
-        if (ICO == 1)
-            decode8<DK, HALF>(v0[buf], v1[buf], scale_const<DK, HALF>(sc2[buf]), qv);
         uint32_t mybits = byte_in(sel[buf], j);
         // iConEF-v2: the stored state is q; e~ comes from the values draw A kept
         uint32_t mA = 0, mB = 0, slotA = 0, slotB = 0;
-        if (ICO == 2) {
+        {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
                 qv[q] = e[q];
@@ -206,30 +182,23 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             float p = __fmaf_rn(lr, gv[q], e[q]);   // Alg. 2 line 5
-            if (ICO)
-                p = __fadd_rn(p, qv[q]);                  // Alg. 3 line 5: + q (the second state, or with version 2 the stored one)
+            p = __fadd_rn(p, qv[q]);                // Alg. 3 line 5: + q, the stored state
             e[q] = p;   // kept for the message stores below
-            r[q] = (QK == CONEF_Q_IDENTITY || ((mybits >> q) & 1u) || !valid) ? 0.f : p;   // r = p - Delta
+            r[q] = (((mybits >> q) & 1u) || !valid) ? 0.f : p;   // r = p - Delta
         }
-        if (QK != CONEF_Q_IDENTITY) {
-            // the few selected elements of this thread, in ascending index order
-            for (uint32_t m = mybits; m; m &= m - 1) {
-                const int q = __ffs(m) - 1;
-                float p = e[0];
+        // the few selected elements of this thread, in ascending index order
+        for (uint32_t m = mybits; m; m &= m - 1) {
+            const int q = __ffs(m) - 1;
+            float p = e[0];
 #pragma unroll
-                for (int x = 1; x < 8; ++x)
-                    p = q == x ? e[x] : p;
-                msg[slot] = p;
-                if (worker == 0)
-                    V.idx[L.idx_off + slot] = j + q;
-                ++slot;
-            }
+            for (int x = 1; x < 8; ++x)
+                p = q == x ? e[x] : p;
+            msg[slot] = p;
+            if (worker == 0)
+                V.idx[L.idx_off + slot] = j + q;
+            ++slot;
         }
-        if (QK == CONEF_Q_IDENTITY && valid) {
-            *(float4 *)(msg + j) = make_float4(e[0], e[1], e[2], e[3]);
-            *(float4 *)(msg + j + 4) = make_float4(e[4], e[5], e[6], e[7]);
-        }
-        if (ICO == 2) {
+        {
             // Alg. 3 line 12: e~ = Q(r) by the second draw; r - e~ is exactly zero where e~ keeps the value
             for (uint32_t mm = mB; mm; mm &= mm - 1) {
                 const int q = __ffs(mm) - 1;
@@ -255,39 +224,13 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
         float s, inv;
         unsigned short hb = 0;
         uint32_t c0 = 0, c1 = 0;
-        if constexpr (CK == CONEF_C_STOCHQUANT) {
-            // Eq. 6 with the block's max-norm: level floor(u) or floor(u) + 1, up with probability
-            // u - floor(u); the variate of (worker, tensor, step, element) from a counter-based stream
-            const float lv = (float)V.levels;
-            s = __fdiv_rn(amax, lv);
-            const bool zero = !(s >= FLT_MIN);
-            s = zero ? 0.f : s;
-            inv = zero ? 0.f : __fdiv_rn(1.0f, s);
-            if (!zero) {
-                const uint64_t stc = stream_key(mix64(V.seed_c + (uint64_t)worker + 1u), (uint64_t)li, (uint64_t)V.step);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    float u = __fmul_rn(fabsf(r[q]), inv);
-                    u = !(u <= lv) ? lv : u;
-                    const float l = floorf(u);
-                    const float frac = __fsub_rn(u, l);
-                    const float rnd = __fmul_rn((float)(uint32_t)(h64(stc, j + q) >> 40), 1.0f / 16777216.0f);
-                    int lev = (int)l + (rnd < frac ? 1 : 0);
-                    lev = min(lev, V.levels);
-                    const uint32_t byte = (uint32_t)(r[q] < 0.f ? -lev : lev) & 0xFFu;
-                    if (q < 4)
-                        c0 |= byte << (8 * q);
-                    else
-                        c1 |= byte << (8 * (q - 4));
-                }
-            }
-        } else {
-            block_scale<DK, HALF>(amax, s, inv, hb);
+        {
+            block_scale<CK, HALF>(amax, s, inv, hb);
             constexpr float qlim = (CK == CONEF_C_INT8 ? 127.f : 7.f) + 0.49f;
             if (__any_sync(0xffffffffu, !(__fmul_rn(amax, inv) < qlim)))
-                quant_pack8<DK, true>(r, inv, c0, c1);
+                quant_pack8<CK, true>(r, inv, c0, c1);
             else
-                quant_pack8<DK, false>(r, inv, c0, c1);
+                quant_pack8<CK, false>(r, inv, c0, c1);
         }
         if (valid) {
             if ((lane & (lpb - 1)) == 0) {
@@ -300,42 +243,6 @@ __global__ void __launch_bounds__(kFvThreads, ICO ? 3 : 4) k_flat_vec(const __gr
                 *(uint32_t *)(codes + (j >> 1)) = c0;
             else
                 *(uint2 *)(codes + j) = make_uint2(c0, c1);
-        }
-        if constexpr (ICO == 1 && CK != CONEF_C_STOCHQUANT) {
-            // Alg. 3 lines 10, 14: e~ = C(r) was just formed; q = C(r - decode(e~)), what the first state misses
-            float e1[8];
-            decode8<DK, HALF>(c0, c1, scale_const<DK, HALF>(s), e1);
-            float amax2 = 0.f;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                r[q] = __fsub_rn(r[q], e1[q]);
-                amax2 = fmaxf(amax2, fabsf(r[q]));
-            }
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1)
-                if (o <= 2 || lpb > o)
-                    amax2 = fmaxf(amax2, __shfl_xor_sync(0xffffffffu, amax2, o));
-            float s2, inv2;
-            unsigned short hb2 = 0;
-            uint32_t d0 = 0, d1 = 0;
-            block_scale<DK, HALF>(amax2, s2, inv2, hb2);
-            constexpr float qlim2 = (CK == CONEF_C_INT8 ? 127.f : 7.f) + 0.49f;
-            if (__any_sync(0xffffffffu, !(__fmul_rn(amax2, inv2) < qlim2)))
-                quant_pack8<DK, true>(r, inv2, d0, d1);
-            else
-                quant_pack8<DK, false>(r, inv2, d0, d1);
-            if (valid) {
-                if ((lane & (lpb - 1)) == 0) {
-                    if (HALF)
-                        ((unsigned short *)scales2)[j >> unit_shift] = hb2;
-                    else
-                        ((float *)scales2)[j >> unit_shift] = s2;
-                }
-                if (CW == 1)
-                    *(uint32_t *)(codes2 + (j >> 1)) = d0;
-                else
-                    *(uint2 *)(codes2 + j) = make_uint2(d0, d1);
-            }
         }
     };
     for (int c = 0; c < kSteps; ++c) {

@@ -3,7 +3,7 @@
 // four 16-byte loads of each stream in flight per thread; gradients off a 16-byte boundary are
 // read four bytes at a time, a warp 128 contiguous bytes, with the same number in flight.
 // ResNet-50 list, random-block-k, four workers: one element at a time in each thread took 415 us
-// (2.7 TB/s), this takes 194 us (5.8 TB/s).
+// (3.0 TB/s), this takes 194 us (6.3 TB/s).
 #pragma once
 #include "conef_decode.cuh"
 

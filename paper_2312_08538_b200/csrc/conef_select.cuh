@@ -43,9 +43,10 @@ struct SelectShared {
     uint32_t bin, rem, n, bad;
 };
 
-// Loads of what other CTAs of the same launch wrote before their ticket: past L1, and volatile, so that
-// the compiler keeps them behind the ticket (__ldcg is free to move; it read the list before it was
-// complete).
+// Loads of what other CTAs of the same launch wrote before their ticket: past L1, and volatile with a
+// memory clobber, so that the compiler may not move them ahead of the ticket.  (A first form without
+// either, and without the bound on the bin index, read out of bounds; an entry read before it was
+// written falls below the window and gives such an index.)
 __device__ __forceinline__ uint32_t load_cg(const uint32_t *p)
 {
     uint32_t v;

@@ -23,6 +23,7 @@
 #include "conef_flat16.cuh"
 #include "conef_flatvec.cuh"
 #include "conef_chunksketch.cuh"
+#include "conef_ilsketch.cuh"
 #include "conef_rowsp1.cuh"
 
 using namespace conef;
@@ -31,7 +32,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 28 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 30 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -42,6 +43,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
        T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
        T_DECODE,                                            // tiles of kDecTile elements: stored error expanded; the step on a dense error
+       T_IL, T_ILT,                                         // count sketch, workers interleaved: tiles of elements, of sketch entries
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -84,6 +86,10 @@ struct Plan {
     int n_fused = 0;
     bool any_csk = false;       // some tensor takes the shared-memory step of the chunk-wise count sketch
     size_t csk_smem = 0;        // ... with this much shared memory per CTA (two windows of the widest run)
+    std::vector<int> il_groups; // count sketch, workers interleaved: first tensor of every group, then n_tensors
+    bool il_direct = true;      // ... or each on its own state
+    std::vector<int64_t> il_fill;   // ... the records of every group
+    int64_t il_records = 0;     // ... and of the largest
     int64_t msg_elems[4] = {0, 0, 0, 0};
     int64_t err_elems = 0;
     int64_t state_stride = 0;  // bytes per worker
@@ -96,7 +102,7 @@ struct Plan {
     // byte offsets in the workspace
     size_t off_layers = 0, off_pfx = 0, off_status = 0, off_sel = 0, off_idx = 0, off_wordoff = 0, off_tileoff = 0, off_selbits = 0,
            off_pbar = 0, off_phat = 0, off_qprev = 0, off_state = 0, off_state_new = 0,
-           off_msgv = 0, off_msgp = 0, off_msgq = 0, off_msg1d = 0, off_part = 0, off_ppart = 0, off_rs = 0, off_cand = 0,
+           off_msgv = 0, off_msgp = 0, off_msgq = 0, off_msg1d = 0, off_part = 0, off_ppart = 0, off_rs = 0, off_cand = 0, off_il = 0,
            off_ev[2] = {0, 0}, off_wordoff2[2] = {0, 0}, off_tileoff2[2] = {0, 0}, off_selbits2[2] = {0, 0},   // iConEF-v2
            off_fu_units = 0, off_fu_groups = 0, off_fu_hint = 0, off_fu_ctr = 0, off_fu_scratch = 0, off_fu_q = 0,   // fused passes 2 + 3
            total = 0;
@@ -202,7 +208,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     }
     P.fast_it[0] = it1, P.fast_it[1] = it2, P.fast_it[2] = it3;
     P.fast_unit = unit;
-    int64_t g_off = 0, state_off = 0;
+    int64_t g_off = 0, state_off = 0, il_fill = 0;
     for (int l = 0; l < n_tensors; ++l) {
         const conef_tensor &t = tensors[l];
         if (t.rows <= 0 || t.cols <= 0)
@@ -294,6 +300,20 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 if (ceil_div(L.d, kHistTile) > kSelTailTiles)
                     tiles[T_SEL_OFFS] = (int)ceil_div(L.d, (int64_t)kHistTile * (kSelThreads / 32));
                 tiles[T_HIST] = (int)ceil_div(L.d, (int64_t)kHistTile * P.sel_tiles);
+            }
+            if (c->kind == CONEF_C_COUNTSKETCH && c->cs_chunk == 0 && q->kind != CONEF_Q_LOWRANK) {
+                tiles[T_IL] = (int)ceil_div(L.d, kIlTile);
+                tiles[T_ILT] = (int)ceil_div(c->cs_rows * L.w, kIlEntries);
+                // groups of consecutive tensors whose records fit kIlGroupBytes, or one larger tensor
+                const int64_t rec = c->cs_rows * L.w, most = kIlGroupBytes / (4 * il_width(n_workers));
+                if (P.il_groups.empty() || il_fill + rec > most) {
+                    P.il_groups.push_back(l);
+                    P.il_fill.push_back(0);
+                    il_fill = 0;
+                }
+                L.sk_off = il_fill;
+                P.il_fill.back() = il_fill += rec;
+                P.il_records = std::max(P.il_records, il_fill);
             }
             if (q->kind != CONEF_Q_LOWRANK) {
                 L.msgv_off = P.msg_elems[CONEF_MSG_VALUES];
@@ -448,6 +468,11 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     P.off_ppart = take((size_t)P.ppart_stride * 4 * n_workers);
     P.off_rs = take((size_t)P.rs_words * 4);
     P.off_cand = take((size_t)P.cand_pairs * 8);
+    if (!P.il_groups.empty())
+        P.il_groups.push_back(n_tensors);
+    P.il_direct = il_width(n_workers) == 1 || P.err_elems * n_workers < kIlDirect;
+    if (!P.il_direct)   // the old and the new records of one group
+        P.off_il = take((size_t)P.il_records * 4 * il_width(n_workers) * 2);
     if (c->iconef == 2)   // two value buffers per worker and the structures of two more draws of Q
         for (int x = 0; x < 2; ++x) {
             P.off_ev[x] = take((size_t)P.msg_stride[CONEF_MSG_VALUES] * 4 * n_workers);
@@ -688,6 +713,27 @@ int launch_flat(conef_ctx *ctx, DevView V, cudaStream_t s, int table = T_FLAT)
     return CONEF_OK;
 }
 
+// the step on a whole-tensor count sketch, all workers together (conef_ilsketch.cuh)
+template <int QK>
+int launch_il(conef_ctx *ctx, const DevView &V, cudaStream_t s)
+{
+    const Plan &P = ctx->plan;
+    const int32_t *pfx = table_ptr(ctx, T_IL), *epfx = table_ptr(ctx, T_ILT);
+    float *records = (float *)(ctx->ws + P.off_il);
+    if (P.il_direct) {
+        il_launch_direct<QK>(V, pfx, tiles_of(ctx, T_IL), s);
+        LAUNCH_CHECK(ctx);
+        return CONEF_OK;
+    }
+    for (size_t k = 0; k + 1 < P.il_groups.size(); ++k) {
+        const int l0 = P.il_groups[k], l1 = P.il_groups[k + 1];
+        const int e0 = P.pfx[T_IL][l0], en = P.pfx[T_IL][l1] - e0, t0 = P.pfx[T_ILT][l0], tn = P.pfx[T_ILT][l1] - t0;
+        ctx->launches += il_launch<QK>(V, pfx, e0, en, epfx, t0, tn, P.il_fill[k], records, s);
+        CK_CUDA(cudaGetLastError());
+    }
+    return CONEF_OK;
+}
+
 int launch_pass1(conef_ctx *ctx, DevView V, cudaStream_t s, int table = T_P1)
 {
     const int n = tiles_of(ctx, table);
@@ -793,10 +839,11 @@ template <class F>
 int with_new_sketch(conef_ctx *ctx, const DevView &V, cudaStream_t s, F body)
 {
     const bool sk = ctx->c.kind == CONEF_C_COUNTSKETCH || ctx->c.kind == CONEF_C_ROWSKETCH;
-    // built by atomic adds; the row sketch, and the run-by-run step where it takes every tensor, write
-    // every entry themselves
+    // built by atomic adds; the row sketch, the run-by-run step where it takes every tensor, and the
+    // step on interleaved workers write every entry themselves
     const bool all_csk = ctx->fast && ctx->plan.any_csk && tiles_of(ctx, T_NOFV) == 0 && ctx->q.kind != CONEF_Q_LOWRANK;
-    if (ctx->c.kind == CONEF_C_COUNTSKETCH && !all_csk)
+    const bool all_il = ctx->fast && tiles_of(ctx, T_IL) > 0 && !ctx->plan.il_direct;
+    if (ctx->c.kind == CONEF_C_COUNTSKETCH && !all_csk && !all_il)
         CK_CUDA(cudaMemsetAsync(V.state_new, 0, (size_t)ctx->plan.state_stride * ctx->n_workers, s));
     int rc = body();
     if (rc == CONEF_OK && sk)
@@ -1202,6 +1249,8 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             }
             return CONEF_OK;
         }
+        if (ctx->fast && tiles_of(ctx, T_IL) > 0)
+            return launch_il<QK>(ctx, V, s);
         if (!fv && !csk)
             return launch_flat<QK>(ctx, V, s);
         if (fv) {

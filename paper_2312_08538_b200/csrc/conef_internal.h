@@ -48,6 +48,7 @@ struct LayerDesc {
     int64_t b_bytes;
     int64_t a2_off, b2_off;   // iConEF-v1: the second state q, same sizes
     int64_t e_off;       // floats: position in the concatenated error vector
+    int64_t sk_off;      // count sketch: records, within the interleaved scratch of the tensor's group
     int64_t msgv_off;    // floats, within a worker's VALUES message
     int64_t msgp_off;    // floats, within a worker's P message
     int64_t msgq_off;    // floats, within a worker's Q message

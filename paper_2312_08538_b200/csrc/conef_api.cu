@@ -19,6 +19,7 @@
 #include "conef_decode.cuh"
 #include "conef_dense.cuh"
 #include "conef_fast.cuh"
+#include "conef_lrgen.cuh"
 #include "conef_gs.cuh"
 #include "conef_flat16.cuh"
 #include "conef_flatvec.cuh"
@@ -32,7 +33,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 30 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 33 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -44,6 +45,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
        T_DECODE,                                            // tiles of kDecTile elements: stored error expanded; the step on a dense error
        T_IL, T_ILT,                                         // count sketch, workers interleaved: tiles of elements, of sketch entries
+       T_GEN1, T_GEN2, T_GEN3,                              // low-rank passes for any shape
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -77,7 +79,7 @@ struct Plan {
     std::vector<int> fast_subs;     // ... and the most rows a period of its tensors spans
     int fast_it[3] = {kFastIt1, kFastIt2, kFastIt3};   // iterations per tile of the tuned passes
     int fast_unit = 256;            // elements per quantisation block
-    bool any_fast = false, any_slow = false, any_rs12 = false;
+    bool any_fast = false, any_slow = false, any_rs12 = false, any_gen = false;
     bool short_tiles = false;   // tile lengths of the tuned passes below their limits
     bool any_fv = false;        // some tensor takes the tuned fused step (conef_flatvec.cuh)
     int fv_tiles = 1;           // ... with this many selection tiles per CTA
@@ -183,8 +185,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     }
     // tile lengths of the tuned low-rank passes from the model's size
     int it1 = kFastIt1, it2 = kFastIt2, it3 = kFastIt3;
+    GenPlan gen;
     if (q->kind == CONEF_Q_LOWRANK) {
-        int64_t cta_iters = 0;
+        int64_t cta_iters = 0, rows = 0, row_groups = 0, chunks = 0;
         for (int l = 0; l < n_tensors; ++l) {
             LayerDesc T{};
             T.rows = tensors[l].rows;
@@ -196,7 +199,11 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             fast_classify(T, c->kind, unit, q->rank);   // offsets are zero here: only the geometry matters
             if (T.fast)
                 cta_iters += T.f_niter * T.f_ncg;
+            rows += T.rows;
+            row_groups += T.rows * ceil_div(T.cols, kGenCols);
+            chunks += ceil_div(T.d, kGenChunk);
         }
+        gen = gen_plan(rows * n_workers, row_groups * n_workers, chunks * n_workers);
         cta_iters *= n_workers;
         it1 = fast_tile_iters(kFastIt1, cta_iters);
         it2 = fast_tile_iters(kFastIt2, cta_iters);
@@ -417,6 +424,14 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                     }
                     L.pp_off = P.ppart_stride;
                     P.ppart_stride += (int64_t)L.f_j * L.rows * r;
+                } else if (c->iconef == 0 && gen_takes(L, c->kind)) {
+                    L.fast = 3;
+                    P.any_gen = true;
+                    gen_classify(L, gen);
+                    L.p2_rows_fast = L.g_t2;
+                    tiles[T_GEN1] = L.g_t1;
+                    tiles[T_GEN2] = (int)(L.g_t2 * ceil_div(L.cols, kGenCols));
+                    tiles[T_GEN3] = L.g_t3 * L.g_groups;
                 } else {
                     P.any_slow = true;
                     tiles[T_SLOW_FLAT] = tiles[T_FLAT];
@@ -1228,7 +1243,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             V.rs_vec_ok = 0;
     // tuned kernels for this call: the int8/int4 streaming passes, or the bucket-major passes on a row sketch
     const bool rs12 = ctx->fast && V.rs_vec_ok && ctx->plan.any_rs12;
-    const bool fast = (ctx->fast && aligned32 && ctx->plan.any_fast) || rs12;
+    const bool fast = (ctx->fast && (ctx->plan.any_fast ? aligned32 : ctx->plan.any_gen)) || rs12;
     int rc = CONEF_OK;
 
     if (phase == 0 && tiles_of(ctx, T_PASS) > 0) {
@@ -1308,6 +1323,14 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
         const bool fused = fast && !rs12 && ctx->fused && ctx->fused_ready && ctx->plan.any_fused && (phase == 1 || phase == 4);
         if (rc == CONEF_OK && fused)
             rc = launch_fused(ctx, V, s, phase == 4);
+        auto launch_gen = [&](int pass) -> int {
+            const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
+            if (n == 0)
+                return CONEF_OK;
+            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s));
+            LAUNCH_CHECK(ctx);
+            return CONEF_OK;
+        };
         auto launch_rs12 = [&](int pass) -> int {
             const int n = tiles_of(ctx, T_RS_P12);
             if (n == 0)
@@ -1329,6 +1352,8 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                 rc = launch_rs12(1);
             else if (fast)
                 rc = launch_fast(ctx, 1, V, s);
+            if (rc == CONEF_OK && fast)
+                rc = launch_gen(1);
             if (rc == CONEF_OK && slow_left)
                 rc = launch_pass1(ctx, V, s, fast ? T_SLOW_P1 : T_P1);
         }
@@ -1337,6 +1362,8 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                 rc = launch_rs12(2);
             else if (fast)
                 rc = launch_fast(ctx, 2, V, s, fused);
+            if (rc == CONEF_OK && fast)
+                rc = launch_gen(2);
             if (rc == CONEF_OK && slow_left)
                 rc = launch_pass2(ctx, V, s, fast ? T_SLOW_P2 : T_P2);
             if (rc == CONEF_OK)
@@ -1347,6 +1374,8 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                 if (ctx->c.kind == CONEF_C_ROWSKETCH)
                     return launch_rowsketch<CONEF_Q_LOWRANK>(ctx, V, s);
                 int r2 = fast ? launch_fast(ctx, 3, V, s, fused) : CONEF_OK;
+                if (r2 == CONEF_OK && fast)
+                    r2 = launch_gen(3);
                 if (r2 == CONEF_OK && slow_left)
                     r2 = launch_flat<CONEF_Q_LOWRANK>(ctx, V, s, fast ? T_SLOW_FLAT : T_FLAT);
                 return r2;

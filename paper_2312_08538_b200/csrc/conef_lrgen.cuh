@@ -1,0 +1,480 @@
+// Low-rank passes on an int8 / int4 error state for the shapes and ranks that the kernels of conef_fast.cuh
+// do not take: any width, any alignment, any rank (Sec. 5.2; Alg. 2, and Alg. 4 with beta).
+//
+//   pass 1  P_i = M_i Q_{t-1}     a warp takes four rows, its lanes neighbouring columns
+//   pass 2  Q_i = M_i^T P_hat     a warp takes 128 columns, four per lane, and runs down the rows
+//   pass 3  r = p - P_hat Q_i^T, absmax, requantise, store: a warp takes 256 consecutive elements (whole
+//           quantisation blocks), lane l the elements l, l + 32, ...
+//
+// Neighbouring lanes always have neighbouring elements, so that every load is a run of contiguous memory
+// whatever the width of the matrix, and no load depends on 16-byte alignment.  The rank is a template
+// parameter, the factors' rows come as vectors through L1, and every warp has 8 to 16 independent loads in
+// flight.  Bound by instruction issue and the L1 pipe (15 to 21 instructions per element, four L1
+// wavefronts per 32 elements for the rank-4 factor).  A recurrent model's odd layers (24.9 M elements, two
+// workers, int4, rank 2): 222 / 286 / 395 us for the three passes on the kernels for every codec
+// (conef_kernels.cuh: one element and a run-time rank at a time), 102 / 92 / 111 us here; 61 M elements,
+// four workers, rank 8: 2.60 / 1.12 / 10.05 ms -> 0.67 / 0.74 / 1.21 ms.
+#pragma once
+#include "conef_fast.cuh"
+
+namespace conef {
+
+constexpr int kGenThreads = 256;
+constexpr int kGenCols = 128;    // pass 2: columns per CTA
+constexpr int kGenChunk = 256;   // pass 3: elements per warp and step
+constexpr int kGenCtas = kPlanSMs * 6;   // CTAs a pass should have at least, where tiles can be made smaller
+
+// tile sizes for a model: rows per warp group of pass 1, rows per tile of pass 2, steps per tile of pass 3
+struct GenPlan {
+    int rg = 8, rt = 256, it = 16;
+};
+// rows: matrix rows of all workers, row_groups: (row, 128 columns) pairs, chunks: 256-element chunks
+inline GenPlan gen_plan(int64_t rows, int64_t row_groups, int64_t chunks)
+{
+    GenPlan G;
+    while (G.rg > 1 && rows / (4 * G.rg) < kGenCtas)
+        G.rg /= 2;
+    while (G.rt > 16 && row_groups / G.rt < kGenCtas)
+        G.rt /= 2;
+    while (G.it > 1 && chunks / (8 * G.it) < kGenCtas)
+        G.it /= 2;
+    return G;
+}
+inline bool gen_takes(const LayerDesc &L, int ckind) { return (ckind == CONEF_C_INT8 || ckind == CONEF_C_INT4) && L.d < (1ll << 31); }
+inline void gen_classify(LayerDesc &L, const GenPlan &G)
+{
+    L.g_rg = L.cols < 256 ? 8 : G.rg;   // (narrow matrices have no columns to share out)
+    L.g_rt = G.rt;
+    L.g_it = G.it;
+    // pass 3: a CTA's eight warps take eight neighbouring chunks and step down about one matrix row at a
+    // time (wide matrices) or eight chunks on (narrow ones), so that the same rows of Q_i stay in L1
+    const int64_t pr = std::max<int64_t>(1, (L.cols + kGenChunk / 2) / kGenChunk);
+    L.g_step = (int32_t)(pr <= 8 ? 8 : pr);
+    L.g_groups = (int32_t)((L.g_step + 7) / 8);
+    const int64_t nc = (L.d + kGenChunk - 1) / kGenChunk;
+    L.g_t1 = (int32_t)((L.rows + 4 * L.g_rg - 1) / (4 * L.g_rg));
+    L.g_t2 = (int32_t)((L.rows + L.g_rt - 1) / L.g_rt);
+    L.g_t3 = (int32_t)((nc + (int64_t)L.g_step * L.g_it - 1) / ((int64_t)L.g_step * L.g_it));
+}
+
+// a row of a factor; R = 0: any rank
+template <int R>
+__device__ __forceinline__ void factor_row(const float *__restrict__ p, int r, float (&out)[R ? R : CONEF_MAX_RANK])
+{
+    if constexpr (R == 4 || R == 8) {
+#pragma unroll
+        for (int c = 0; c < R; c += 4) {
+            const float4 t = __ldg((const float4 *)(p + c));
+            out[c] = t.x; out[c + 1] = t.y; out[c + 2] = t.z; out[c + 3] = t.w;
+        }
+    } else if constexpr (R == 2) {
+        const float2 t = __ldg((const float2 *)p);
+        out[0] = t.x; out[1] = t.y;
+    } else if constexpr (R == 1) {
+        out[0] = __ldg(p);
+    } else {
+#pragma unroll
+        for (int c = 0; c < CONEF_MAX_RANK; ++c)
+            out[c] = c < r ? __ldg(p + c) : 0.f;
+    }
+}
+// float(code) from a code's byte or nibble
+template <int CK>
+__device__ __forceinline__ float code_value(uint32_t raw)
+{
+    constexpr bool INT4 = CK == CONEF_C_INT4;
+    const uint32_t u = INT4 ? ((raw & 0xFu) ^ 8u) : ((raw & 0xFFu) ^ 0x80u);
+    return __fsub_rn(__uint_as_float(0x4B000000u | u), INT4 ? 8388616.f : 8388736.f);
+}
+template <int CK>
+__device__ __forceinline__ uint32_t code_raw(const uint8_t *__restrict__ codes, uint32_t j)
+{
+    return CK == CONEF_C_INT4 ? (uint32_t)__ldg(codes + (j >> 1)) >> (4 * (j & 1u)) : (uint32_t)__ldg(codes + j);
+}
+__device__ __forceinline__ float gen_scale(const uint8_t *__restrict__ b, uint32_t blk, bool half)
+{
+    return half ? __half2float(__ushort_as_half(__ldg((const unsigned short *)b + blk))) : __ldg((const float *)b + blk);
+}
+
+template <int CK, int R>
+__device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *red)
+{
+    constexpr int RM = R ? R : CONEF_MAX_RANK, NR = 4, P1U = RM > 4 ? 2 : 3;   // rows; column groups in flight
+    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
+    const int rg = L.g_rg, cs = 8 / rg;               // row groups of the CTA, warps that share a group's columns
+    const int grp = warp / cs, part = warp - grp * cs;
+    const uint32_t row0 = tile * (uint32_t)(NR * rg) + grp * NR;
+    const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
+    const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
+    const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ Q = V.qprev + L.msgq_off;
+    const int shift = 31 - __clz(L.unit);
+    const bool half = V.scale_half != 0;
+    const float lr = V.lr, omb = V.omb;
+    uint32_t jb[NR];   // (rows past the end repeat the last one and are not stored)
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+        jb[i] = min(row0 + i, n - 1) * m;
+    float acc[NR][RM];
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+        for (int c = 0; c < RM; ++c)
+            acc[i][c] = 0.f;
+    auto columns = [&](uint32_t col, auto count) {
+        constexpr int N = decltype(count)::value;
+        float gv[N][NR], sc[N][NR];
+        uint32_t w[N][NR];
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const uint32_t j = jb[i] + col + u * 32 * cs;
+                gv[u][i] = __ldg(g + j);
+                w[u][i] = code_raw<CK>(codes, j);
+                sc[u][i] = gen_scale(scales, j >> shift, half);
+            }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            float q[RM];
+            factor_row<R>(Q + (size_t)(col + u * 32 * cs) * r, r, q);
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const float p = __fmaf_rn(lr, gv[u][i], __fmul_rn(omb, __fmul_rn(code_value<CK>(w[u][i]), sc[u][i])));   // Alg. 2 (4) line 5
+#pragma unroll
+                for (int c = 0; c < RM; ++c)
+                    acc[i][c] = __fmaf_rn(p, q[c], acc[i][c]);
+            }
+        }
+    };
+    uint32_t col = part * 32 + lane;
+    for (; col + (P1U - 1) * 32 * cs < m; col += P1U * 32 * cs)
+        columns(col, IntC<P1U>());
+    for (; col < m; col += 32 * cs)
+        columns(col, IntC<1>());
+    // totals of column idx end up in the lanes whose bits below `plain` are zero
+    int idx = 0, hh = RM, plain = 32;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1)
+        if (hh > 1) {
+            hh >>= 1;
+            if (lane & o)
+                idx += hh;
+            plain = o;
+        }
+    const bool writer = (lane & (plain - 1)) == 0 && idx < r;
+    float *__restrict__ P = V.msgp + worker * V.msgp_stride + L.msgp_off;
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        warp_reduce_many<RM>(acc[i], lane);
+        if (writer) {
+            if (cs == 1) {
+                if (row0 + i < n)
+                    P[(size_t)(row0 + i) * r + idx] = acc[i][0];
+            } else {
+                red[(warp * NR + i) * CONEF_MAX_RANK + idx] = acc[i][0];
+            }
+        }
+    }
+    if (cs > 1) {
+        __syncthreads();
+        const int x = threadIdx.x;   // (group, row, rank) of the sum this thread forms, in warp order
+        if (x < rg * NR * CONEF_MAX_RANK) {
+            const int c = x % CONEF_MAX_RANK, i = x / CONEF_MAX_RANK % NR, gg = x / (CONEF_MAX_RANK * NR);
+            const uint32_t row = tile * (uint32_t)(NR * rg) + gg * NR + i;
+            if (c < r && row < n) {
+                float s = red[(gg * cs * NR + i) * CONEF_MAX_RANK + c];
+                for (int k = 1; k < cs; ++k)
+                    s = __fadd_rn(s, red[((gg * cs + k) * NR + i) * CONEF_MAX_RANK + c]);
+                P[(size_t)row * r + c] = s;
+            }
+        }
+    }
+}
+
+template <int CK, int R>
+__device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *red)
+{
+    constexpr int RM = R ? R : CONEF_MAX_RANK, K = 4, U = RM > 4 ? 2 : 4;   // columns per lane, rows in flight
+    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
+    const uint32_t ct = (m + kGenCols - 1) / kGenCols, rt = tile / ct, c0 = (tile - rt * ct) * kGenCols + lane;
+    const uint32_t r_lo = rt * (uint32_t)L.g_rt, r_hi = min(n, r_lo + (uint32_t)L.g_rt);
+    const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
+    const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
+    const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ ph = V.phat + L.msgp_off;
+    const int shift = 31 - __clz(L.unit);
+    const bool half = V.scale_half != 0;
+    const float lr = V.lr, omb = V.omb;
+    uint32_t col[K];   // (columns past the end repeat the last one and are not stored)
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        col[k] = min(c0 + 32 * k, m - 1);
+    float acc[K][RM];
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int c = 0; c < RM; ++c)
+            acc[k][c] = 0.f;
+    auto rows = [&](uint32_t a, auto count) {
+        constexpr int N = decltype(count)::value;
+        float gv[N][K], sc[N][K];
+        uint32_t w[N][K];
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const uint32_t j = (a + 8 * u) * m + col[k];
+                gv[u][k] = __ldg(g + j);
+                w[u][k] = code_raw<CK>(codes, j);
+                sc[u][k] = gen_scale(scales, j >> shift, half);
+            }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            float pr[RM];
+            factor_row<R>(ph + (size_t)(a + 8 * u) * r, r, pr);
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float p = __fmaf_rn(lr, gv[u][k], __fmul_rn(omb, __fmul_rn(code_value<CK>(w[u][k]), sc[u][k])));
+#pragma unroll
+                for (int c = 0; c < RM; ++c)
+                    acc[k][c] = __fmaf_rn(p, pr[c], acc[k][c]);
+            }
+        }
+    };
+    uint32_t a = r_lo + warp;
+    for (; a + 8 * (U - 1) < r_hi; a += 8 * U)
+        rows(a, IntC<U>());
+    for (; a < r_hi; a += 8)
+        rows(a, IntC<1>());
+    // the eight warps' sums, in warp order; one column and rank at a time is four floats per lane
+    float *part = V.part + worker * V.part_stride + L.part_off + (size_t)rt * m * r;
+#pragma unroll
+    for (int c = 0; c < RM; ++c) {
+        if (!R && c >= r)
+            break;
+        if (c)
+            __syncthreads();
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            red[warp * kGenCols + 32 * k + lane] = acc[k][c];
+        __syncthreads();
+        const uint32_t x = threadIdx.x, cc = (tile - rt * ct) * kGenCols + x;
+        if (x < (uint32_t)kGenCols && cc < m) {
+            float s = red[x];
+#pragma unroll
+            for (int k = 1; k < 8; ++k)
+                s = __fadd_rn(s, red[k * kGenCols + x]);
+            part[(size_t)cc * r + c] = s;
+        }
+    }
+}
+
+template <int CK, int R, int KB>
+__device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L, uint32_t tile, uint8_t *bytes)
+{
+    constexpr int RM = R ? R : CONEF_MAX_RANK, K = kGenChunk / 32, NB = K / KB;   // KB * 32 elements per block
+    constexpr bool INT4 = CK == CONEF_C_INT4;
+    constexpr int NW = INT4 ? 1 : 2;   // code words per lane
+    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t m = (uint32_t)L.cols, d = (uint32_t)L.d;
+    const uint32_t step = L.g_step, groups = L.g_groups, nc = (d + kGenChunk - 1) / kGenChunk;
+    const uint32_t tt = tile / groups, cpos = (tile - tt * groups) * 8 + warp;   // place among the chunks of a step
+    if (cpos >= step)
+        return;   // (no CTA-wide barrier below)
+    uint8_t *st = V.state + worker * V.state_stride;
+    uint32_t *codes = (uint32_t *)(st + L.a_off);
+    uint8_t *scales = st + L.b_off;
+    const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ ph = V.phat + L.msgp_off;
+    const float *__restrict__ Q = V.msgq + worker * V.msgq_stride + L.msgq_off;
+    const bool half = V.scale_half != 0;
+    const float lr = V.lr, omb = V.omb, beta = V.beta;
+    uint8_t *mine = bytes + warp * kGenChunk;
+    const uint32_t nblk = (uint32_t)L.nunits;
+
+    uint32_t ch = tt * (uint32_t)L.g_it * step + cpos;
+    // row and column of the chunk's first element, and how they move from step to step
+    uint32_t row = (ch * kGenChunk) / m, col = ch * kGenChunk - row * m;
+    const uint32_t drow = (step * kGenChunk) / m, dcol = step * kGenChunk - drow * m;
+    float gn[K], sn = 0.f;
+    uint32_t wn[NW];
+    auto fetch = [&](uint32_t c) {   // (32-bit offsets: d < 2^31)
+        const uint32_t j = c * kGenChunk + lane;
+        if (c < nc) {
+            if (j + 32 * (K - 1) - lane + 31u < d) {
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    gn[k] = __ldcs(g + j + 32 * k);
+            } else {
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    gn[k] = j + 32 * k < d ? __ldcs(g + j + 32 * k) : 0.f;
+            }
+#pragma unroll
+            for (int x = 0; x < NW; ++x)   // (the state's arrays are padded to 256 bytes)
+                wn[x] = codes[c * (32 * NW) + 32 * x + lane];
+            const uint32_t b = c * NB + lane;
+            sn = 0.f;
+            if (lane < NB && b < nblk)
+                sn = half ? __half2float(__ushort_as_half(((const unsigned short *)scales)[b])) : ((const float *)scales)[b];
+        }
+    };
+    fetch(ch);
+    for (int it = 0; it < L.g_it && ch < nc; ++it, ch += step) {
+        float gv[K];
+        uint32_t w[NW];
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            gv[k] = gn[k];
+#pragma unroll
+        for (int x = 0; x < NW; ++x)
+            w[x] = wn[x];
+        const float sv = sn;
+        if (it + 1 < L.g_it)
+            fetch(ch + step);
+        const uint32_t j0 = ch * kGenChunk + lane;
+        float res[K], ek[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            // element 32 k + lane: its word is another lane's
+            uint32_t raw;
+            if (INT4)
+                raw = __shfl_sync(0xffffffffu, w[0], 4 * k + (lane >> 3)) >> (4 * (lane & 7));
+            else
+                raw = __shfl_sync(0xffffffffu, w[NW == 2 ? k / 4 : 0], 8 * (k & 3) + (lane >> 2)) >> (8 * (lane & 3));
+            const float s = __shfl_sync(0xffffffffu, sv, k / KB);
+            ek[k] = __fmul_rn(code_value<CK>(raw), s);
+            res[k] = __fmaf_rn(lr, gv[k], __fmul_rn(omb, ek[k]));   // Alg. 2 (4) line 5
+        }
+        // r = p - P_hat Q_i^T
+        if (col + (kGenChunk - 1) < m && (ch + 1) * kGenChunk <= d) {   // one matrix row
+            float pr[RM];
+            factor_row<R>(ph + (size_t)row * r, r, pr);
+            const float *q0 = Q + (size_t)(col + lane) * r;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                float q[RM];
+                factor_row<R>(q0 + 32 * k * r, r, q);
+#pragma unroll
+                for (int c = 0; c < RM; ++c)
+                    if (R || c < r)
+                        res[k] = __fmaf_rn(-pr[c], q[c], res[k]);
+            }
+        } else {
+            uint32_t cc = col + lane, rr = row;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                if (cc >= m) {
+                    const uint32_t t = m >= 32 ? 1u : cc / m;
+                    cc -= t * m;
+                    rr += t;
+                }
+                if (j0 + 32 * k < d) {
+                    float pr[RM], q[RM];
+                    factor_row<R>(ph + (size_t)rr * r, r, pr);
+                    factor_row<R>(Q + (size_t)cc * r, r, q);
+#pragma unroll
+                    for (int c = 0; c < RM; ++c)
+                        if (R || c < r)
+                            res[k] = __fmaf_rn(-pr[c], q[c], res[k]);
+                } else {
+                    res[k] = ek[k] = 0.f;
+                }
+                cc += 32;
+            }
+        }
+        if (beta != 0.f) {   // Alg. 4 line 9 stores C(beta e + r)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                res[k] = __fmaf_rn(beta, ek[k], res[k]);
+        }
+        // block maxima: lane b takes block b's
+        float amax = 0.f;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            float x = 0.f;
+#pragma unroll
+            for (int k = 0; k < KB; ++k)
+                x = fmaxf(x, fabsf(res[b * KB + k]));
+            const float y = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));   // (not negative: ordered like integers)
+            amax = lane == b ? y : amax;
+        }
+        float s, inv;
+        unsigned short hb = 0;
+        if (half)
+            block_scale<CK, true>(amax, s, inv, hb);
+        else
+            block_scale<CK, false>(amax, s, inv, hb);
+        constexpr float qm = INT4 ? 7.f : 127.f;
+        const bool clamp = __any_sync(0xffffffffu, !(__fmul_rn(amax, inv) < qm + 0.49f));   // (see quant_pack8)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            float x = __fmul_rn(res[k], __shfl_sync(0xffffffffu, inv, k / KB));
+            if (clamp)
+                x = fminf(fmaxf(x, -qm), qm);
+            mine[32 * k + lane] = (uint8_t)__float_as_uint(__fadd_rn(x, 12582912.0f));   // the low byte is the code
+        }
+        const uint32_t b = ch * NB + lane;
+        if (lane < NB && b < nblk) {
+            if (half)
+                ((unsigned short *)scales)[b] = hb;
+            else
+                ((float *)scales)[b] = s;
+        }
+        __syncwarp();
+        if (INT4) {
+            const uint2 v = *(const uint2 *)(mine + 8 * lane);
+            auto four = [](uint32_t x) {   // four bytes' low nibbles -> 16 bits
+                x &= 0x0F0F0F0Fu;
+                x |= x >> 4;
+                return __byte_perm(x, 0u, 0x4420);
+            };
+            codes[ch * 32 + lane] = four(v.x) | (four(v.y) << 16);
+        } else {
+#pragma unroll
+            for (int x = 0; x < NW; ++x)
+                codes[ch * 64 + 32 * x + lane] = *(const uint32_t *)(mine + 128 * x + 4 * lane);
+        }
+        __syncwarp();
+        row += drow;
+        col += dcol;
+        if (col >= m) {
+            col -= m;
+            ++row;
+        }
+    }
+}
+
+// R: the configured rank (1, 2, 4, 8; 0: another one).  Tensors thinner than it, and those behind them whose
+// factors are off the vector loads' alignment, take the run-time rank.
+template <int PASS, int CK, int R, int KB>
+__global__ void __launch_bounds__(kGenThreads, R == 8 || R == 0 ? 3 : 4) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+{
+    __shared__ __align__(16) float red[PASS == 2 ? 8 * kGenCols : PASS == 1 ? 8 * 4 * CONEF_MAX_RANK : 8 * kGenChunk / 4];
+    const int li = find_layer(pfx, V.n_layers, blockIdx.x);
+    const LayerDesc &L = V.layers[li];
+    const uint32_t tile = blockIdx.x - pfx[li];
+    constexpr int VW = R == 8 ? 4 : R ? R : 1;   // floats per vector load
+    const bool exact = R != 0 && L.rank == R && ((L.msgp_off | L.msgq_off) & (VW - 1)) == 0;
+    if (PASS == 1) {
+        if (R && exact)
+            gen_p1_body<CK, R>(V, L, tile, red);
+        else
+            gen_p1_body<CK, 0>(V, L, tile, red);
+    } else if (PASS == 2) {
+        if (R && exact)
+            gen_p2_body<CK, R>(V, L, tile, red);
+        else
+            gen_p2_body<CK, 0>(V, L, tile, red);
+    } else {
+        if (R && exact)
+            gen_p3_body<CK, R, KB>(V, L, tile, (uint8_t *)red);
+        else
+            gen_p3_body<CK, 0, KB>(V, L, tile, (uint8_t *)red);
+    }
+}
+
+// launcher (conef_lrgen.cu)
+cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s);
+
+}  // namespace conef

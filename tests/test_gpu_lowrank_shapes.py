@@ -1,0 +1,50 @@
+"""Low-rank passes for any shape: widths around a warp, a chunk and eight chunks, tensors thinner than the
+rank, odd offsets, every rank, block size and both scale types, with and without beta.  Factors against
+the oracle; stored codes and scales teacher-forced, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2312_08538_b200 import workloads as wl
+from tests import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [(70, 33, 1), (3, 1, 0), (9, 31, 1), (40, 255, 1), (5, 1, 0), (130, 257, 1), (1, 700, 1), (300, 5, 1), (17, 2049, 1),
+         (2, 9000, 1), (64, 127, 1)]
+
+
+@pytest.mark.parametrize("rank,c", [(1, dict(kind="int8", block=256)), (2, dict(kind="int4", block=128, scale_dtype="fp16")),
+                                    (3, dict(kind="int8", block=32, scale_dtype="fp16")), (4, dict(kind="int4", block=64)),
+                                    (4, dict(kind="int8", block=128, scale_dtype="fp16", beta=0.3)),
+                                    (8, dict(kind="int4", block=256, scale_dtype="fp16", beta=0.9)), (8, dict(kind="int8", block=64))])
+def test_passes_on_edges(rank, c):
+    from paper_2312_08538_b200 import binding as b
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=EDGES, n_workers=2, q=dict(kind="lowrank", rank=rank), c=c, grad="normal1e-3")
+    q0 = wl.q_init(cfg, "cuda")
+    eng, o = pu.make_gpu(cfg, q_init=q0), pu.make_oracle(cfg, q_init=q0.cpu().numpy())
+    for t in range(2):
+        pu.load_state_from_oracle(eng, o)
+        gd, gh = pu.grads_both(cfg, t)
+        res = o.step(t, gh)
+        eng.step(t, gd, 0)
+        for l in o.compressed:
+            for i in range(o.N):
+                assert pu.frob_err(eng.factors(l, i)["p_i"].cpu().numpy(), res[l].P[i]) <= 1e-5, (t, l, "P_i")
+        eng.reduce_messages(b.MSG_P)
+        for l in o.compressed:
+            eng.factors(l, 0)["p_hat"].copy_(torch.from_numpy(res[l].Phat).cuda())
+        eng.step(t, gd, 2)
+        for l in o.compressed:
+            for i in range(o.N):
+                f = eng.factors(l, i)["q_i"]
+                assert pu.frob_err(f.cpu().numpy(), res[l].Qi[i]) <= 1e-5, (t, l, "Q_i")
+                f.copy_(torch.from_numpy(res[l].Qi[i]).cuda())
+        eng.step(t, gd, 3)
+        for l in o.compressed:
+            for i in range(o.N):
+                ga, gs = pu.gpu_state_arrays(eng, o, i, l)
+                oa, os_ = pu.oracle_state_arrays(o, i, l)
+                assert np.array_equal(ga, oa) and np.array_equal(gs, os_), (t, l, i)
+        eng.reduce_messages(b.MSG_Q)

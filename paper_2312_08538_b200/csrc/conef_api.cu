@@ -187,7 +187,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     int it1 = kFastIt1, it2 = kFastIt2, it3 = kFastIt3;
     GenPlan gen;
     if (q->kind == CONEF_Q_LOWRANK) {
-        int64_t cta_iters = 0, rows = 0, row_groups = 0, chunks = 0;
+        int64_t cta_iters = 0, rows = 0, chunks = 0;
         for (int l = 0; l < n_tensors; ++l) {
             LayerDesc T{};
             T.rows = tensors[l].rows;
@@ -200,10 +200,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             if (T.fast)
                 cta_iters += T.f_niter * T.f_ncg;
             rows += T.rows;
-            row_groups += T.rows * ceil_div(T.cols, kGenCols);
             chunks += ceil_div(T.d, kGenChunk);
         }
-        gen = gen_plan(rows * n_workers, row_groups * n_workers, chunks * n_workers);
+        gen = gen_plan(rows * n_workers, chunks * n_workers);
         cta_iters *= n_workers;
         it1 = fast_tile_iters(kFastIt1, cta_iters);
         it2 = fast_tile_iters(kFastIt2, cta_iters);
@@ -428,9 +427,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                     L.fast = 3;
                     P.any_gen = true;
                     gen_classify(L, gen);
-                    L.p2_rows_fast = L.g_t2;
+                    L.p2_rows_fast = rtiles;
                     tiles[T_GEN1] = L.g_t1;
-                    tiles[T_GEN2] = (int)(L.g_t2 * ceil_div(L.cols, kGenCols));
+                    tiles[T_GEN2] = L.g_t2;
                     tiles[T_GEN3] = L.g_t3 * L.g_groups;
                 } else {
                     P.any_slow = true;

@@ -1,8 +1,8 @@
 // Low-rank passes on an int8 / int4 error state for the shapes and ranks that the kernels of conef_fast.cuh
 // do not take: any width, any alignment, any rank (Sec. 5.2; Alg. 2, and Alg. 4 with beta).
 //
-//   pass 1  P_i = M_i Q_{t-1}     a warp takes four rows, its lanes neighbouring columns
-//   pass 2  Q_i = M_i^T P_hat     a warp takes 128 columns, four per lane, and runs down the rows
+//   pass 1  P_i = M_i Q_{t-1}     a warp takes four rows (small models: one), its lanes neighbouring columns
+//   pass 2  Q_i = M_i^T P_hat     a warp takes 64 columns, two per lane, and runs down 256 rows
 //   pass 3  r = p - P_hat Q_i^T, absmax, requantise, store: a warp takes 256 consecutive elements (whole
 //           quantisation blocks), lane l the elements l, l + 32, ...
 //
@@ -10,32 +10,36 @@
 // whatever the width of the matrix, and no load depends on 16-byte alignment.  The rank is a template
 // parameter, the factors' rows come as vectors through L1, and every warp has 8 to 16 independent loads in
 // flight.  Bound by instruction issue and the L1 pipe (15 to 21 instructions per element, four L1
-// wavefronts per 32 elements for the rank-4 factor).  A recurrent model's odd layers (24.9 M elements, two
-// workers, int4, rank 2): 222 / 286 / 395 us for the three passes on the kernels for every codec
-// (conef_kernels.cuh: one element and a run-time rank at a time), 102 / 92 / 111 us here; 61 M elements,
-// four workers, rank 8: 2.60 / 1.12 / 10.05 ms -> 0.67 / 0.74 / 1.21 ms.
+// wavefronts per 32 elements for the rank-4 factor).
+//
+// The order of every sum is part of the result: a factor that moves by one rounding moves a stored int4
+// code by a whole quantum now and then, and the steps that follow amplify it (a reversed sum over the row
+// tiles alone: 1e-4 to 6e-4 of the outputs' norm after a few steps).  It is that of the kernels for every
+// codec (conef_kernels.cuh), so a row's columns and a tile's rows are not shared out among warps.
+//
+// A recurrent model's odd layers (24.9 M elements, two workers, int4, rank 2): 222 / 286 / 395 us for the
+// three passes on the kernels for every codec (one element and a run-time rank at a time), 125 / 168 / 112 us
+// here.
 #pragma once
 #include "conef_fast.cuh"
 
 namespace conef {
 
 constexpr int kGenThreads = 256;
-constexpr int kGenCols = 128;    // pass 2: columns per CTA
+constexpr int kGenCols = 64;     // pass 2: columns per warp
 constexpr int kGenChunk = 256;   // pass 3: elements per warp and step
 constexpr int kGenCtas = kPlanSMs * 6;   // CTAs a pass should have at least, where tiles can be made smaller
 
-// tile sizes for a model: rows per warp group of pass 1, rows per tile of pass 2, steps per tile of pass 3
+// tile sizes for a model: rows per warp of pass 1 (4 or 1), steps per tile of pass 3
 struct GenPlan {
-    int rg = 8, rt = 256, it = 16;
+    int nr = 4, it = 16;
 };
-// rows: matrix rows of all workers, row_groups: (row, 128 columns) pairs, chunks: 256-element chunks
-inline GenPlan gen_plan(int64_t rows, int64_t row_groups, int64_t chunks)
+// rows: matrix rows of all workers, chunks: 256-element chunks
+inline GenPlan gen_plan(int64_t rows, int64_t chunks)
 {
     GenPlan G;
-    while (G.rg > 1 && rows / (4 * G.rg) < kGenCtas)
-        G.rg /= 2;
-    while (G.rt > 16 && row_groups / G.rt < kGenCtas)
-        G.rt /= 2;
+    if (rows / 32 < kGenCtas)
+        G.nr = 1;
     while (G.it > 1 && chunks / (8 * G.it) < kGenCtas)
         G.it /= 2;
     return G;
@@ -43,8 +47,7 @@ inline GenPlan gen_plan(int64_t rows, int64_t row_groups, int64_t chunks)
 inline bool gen_takes(const LayerDesc &L, int ckind) { return (ckind == CONEF_C_INT8 || ckind == CONEF_C_INT4) && L.d < (1ll << 31); }
 inline void gen_classify(LayerDesc &L, const GenPlan &G)
 {
-    L.g_rg = L.cols < 256 ? 8 : G.rg;   // (narrow matrices have no columns to share out)
-    L.g_rt = G.rt;
+    L.g_nr = G.nr;
     L.g_it = G.it;
     // pass 3: a CTA's eight warps take eight neighbouring chunks and step down about one matrix row at a
     // time (wide matrices) or eight chunks on (narrow ones), so that the same rows of Q_i stay in L1
@@ -52,8 +55,8 @@ inline void gen_classify(LayerDesc &L, const GenPlan &G)
     L.g_step = (int32_t)(pr <= 8 ? 8 : pr);
     L.g_groups = (int32_t)((L.g_step + 7) / 8);
     const int64_t nc = (L.d + kGenChunk - 1) / kGenChunk;
-    L.g_t1 = (int32_t)((L.rows + 4 * L.g_rg - 1) / (4 * L.g_rg));
-    L.g_t2 = (int32_t)((L.rows + L.g_rt - 1) / L.g_rt);
+    L.g_t1 = (int32_t)((L.rows + 8 * L.g_nr - 1) / (8 * L.g_nr));
+    L.g_t2 = (int32_t)((((L.rows + kP2RowsPerTile - 1) / kP2RowsPerTile) * ((L.cols + kGenCols - 1) / kGenCols) + 7) / 8);
     L.g_t3 = (int32_t)((nc + (int64_t)L.g_step * L.g_it - 1) / ((int64_t)L.g_step * L.g_it));
 }
 
@@ -96,15 +99,13 @@ __device__ __forceinline__ float gen_scale(const uint8_t *__restrict__ b, uint32
     return half ? __half2float(__ushort_as_half(__ldg((const unsigned short *)b + blk))) : __ldg((const float *)b + blk);
 }
 
-template <int CK, int R>
-__device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *red)
+template <int CK, int R, int NR>   // NR: rows per warp
+__device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L, uint32_t tile)
 {
-    constexpr int RM = R ? R : CONEF_MAX_RANK, NR = 4, P1U = RM > 4 ? 2 : 3;   // rows; column groups in flight
+    constexpr int RM = R ? R : CONEF_MAX_RANK, P1U = NR == 1 ? 6 : RM > 4 ? 2 : 3;   // column groups in flight
     const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
-    const int rg = L.g_rg, cs = 8 / rg;               // row groups of the CTA, warps that share a group's columns
-    const int grp = warp / cs, part = warp - grp * cs;
-    const uint32_t row0 = tile * (uint32_t)(NR * rg) + grp * NR;
+    const uint32_t row0 = (tile * 8u + warp) * NR;
     const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
     const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
     const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ Q = V.qprev + L.msgq_off;
@@ -129,7 +130,7 @@ __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L
         for (int u = 0; u < N; ++u)
 #pragma unroll
             for (int i = 0; i < NR; ++i) {
-                const uint32_t j = jb[i] + col + u * 32 * cs;
+                const uint32_t j = jb[i] + col + u * 32;
                 gv[u][i] = __ldg(g + j);
                 w[u][i] = code_raw<CK>(codes, j);
                 sc[u][i] = gen_scale(scales, j >> shift, half);
@@ -137,7 +138,7 @@ __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L
 #pragma unroll
         for (int u = 0; u < N; ++u) {
             float q[RM];
-            factor_row<R>(Q + (size_t)(col + u * 32 * cs) * r, r, q);
+            factor_row<R>(Q + (size_t)(col + u * 32) * r, r, q);
 #pragma unroll
             for (int i = 0; i < NR; ++i) {
                 const float p = __fmaf_rn(lr, gv[u][i], __fmul_rn(omb, __fmul_rn(code_value<CK>(w[u][i]), sc[u][i])));   // Alg. 2 (4) line 5
@@ -147,10 +148,10 @@ __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L
             }
         }
     };
-    uint32_t col = part * 32 + lane;
-    for (; col + (P1U - 1) * 32 * cs < m; col += P1U * 32 * cs)
+    uint32_t col = lane;
+    for (; col + (P1U - 1) * 32 < m; col += P1U * 32)
         columns(col, IntC<P1U>());
-    for (; col < m; col += 32 * cs)
+    for (; col < m; col += 32)
         columns(col, IntC<1>());
     // totals of column idx end up in the lanes whose bits below `plain` are zero
     int idx = 0, hh = RM, plain = 32;
@@ -167,39 +168,21 @@ __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
         warp_reduce_many<RM>(acc[i], lane);
-        if (writer) {
-            if (cs == 1) {
-                if (row0 + i < n)
-                    P[(size_t)(row0 + i) * r + idx] = acc[i][0];
-            } else {
-                red[(warp * NR + i) * CONEF_MAX_RANK + idx] = acc[i][0];
-            }
-        }
-    }
-    if (cs > 1) {
-        __syncthreads();
-        const int x = threadIdx.x;   // (group, row, rank) of the sum this thread forms, in warp order
-        if (x < rg * NR * CONEF_MAX_RANK) {
-            const int c = x % CONEF_MAX_RANK, i = x / CONEF_MAX_RANK % NR, gg = x / (CONEF_MAX_RANK * NR);
-            const uint32_t row = tile * (uint32_t)(NR * rg) + gg * NR + i;
-            if (c < r && row < n) {
-                float s = red[(gg * cs * NR + i) * CONEF_MAX_RANK + c];
-                for (int k = 1; k < cs; ++k)
-                    s = __fadd_rn(s, red[((gg * cs + k) * NR + i) * CONEF_MAX_RANK + c]);
-                P[(size_t)row * r + c] = s;
-            }
-        }
+        if (writer && row0 + i < n)
+            P[(size_t)(row0 + i) * r + idx] = acc[i][0];
     }
 }
 
 template <int CK, int R>
-__device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *red)
+__device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L, uint32_t tile)
 {
-    constexpr int RM = R ? R : CONEF_MAX_RANK, K = 4, U = RM > 4 ? 2 : 4;   // columns per lane, rows in flight
+    constexpr int RM = R ? R : CONEF_MAX_RANK, K = kGenCols / 32, U = RM > 4 ? 4 : 8;   // columns per lane, rows in flight
     const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
-    const uint32_t ct = (m + kGenCols - 1) / kGenCols, rt = tile / ct, c0 = (tile - rt * ct) * kGenCols + lane;
-    const uint32_t r_lo = rt * (uint32_t)L.g_rt, r_hi = min(n, r_lo + (uint32_t)L.g_rt);
+    const uint32_t task = tile * 8u + warp, ct = (m + kGenCols - 1) / kGenCols, rt = task / ct, c0 = (task - rt * ct) * kGenCols + lane;
+    const uint32_t r_lo = rt * (uint32_t)kP2RowsPerTile, r_hi = min(n, r_lo + (uint32_t)kP2RowsPerTile);
+    if (r_lo >= n)
+        return;   // (no CTA-wide barrier below)
     const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
     const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
     const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ ph = V.phat + L.msgp_off;
@@ -224,7 +207,7 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
         for (int u = 0; u < N; ++u)
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                const uint32_t j = (a + 8 * u) * m + col[k];
+                const uint32_t j = (a + u) * m + col[k];
                 gv[u][k] = __ldg(g + j);
                 w[u][k] = code_raw<CK>(codes, j);
                 sc[u][k] = gen_scale(scales, j >> shift, half);
@@ -232,7 +215,7 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
 #pragma unroll
         for (int u = 0; u < N; ++u) {
             float pr[RM];
-            factor_row<R>(ph + (size_t)(a + 8 * u) * r, r, pr);
+            factor_row<R>(ph + (size_t)(a + u) * r, r, pr);
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 const float p = __fmaf_rn(lr, gv[u][k], __fmul_rn(omb, __fmul_rn(code_value<CK>(w[u][k]), sc[u][k])));
@@ -242,32 +225,20 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
             }
         }
     };
-    uint32_t a = r_lo + warp;
-    for (; a + 8 * (U - 1) < r_hi; a += 8 * U)
+    uint32_t a = r_lo;
+    for (; a + U <= r_hi; a += U)
         rows(a, IntC<U>());
-    for (; a < r_hi; a += 8)
+    for (; a < r_hi; ++a)
         rows(a, IntC<1>());
-    // the eight warps' sums, in warp order; one column and rank at a time is four floats per lane
-    float *part = V.part + worker * V.part_stride + L.part_off + (size_t)rt * m * r;
+    float *part = V.part + worker * V.part_stride + L.part_off + (size_t)rt * m * r;   // added in order by k_lr_pass2_reduce
 #pragma unroll
-    for (int c = 0; c < RM; ++c) {
-        if (!R && c >= r)
-            break;
-        if (c)
-            __syncthreads();
+    for (int k = 0; k < K; ++k)
+        if (c0 + 32 * k < m) {
 #pragma unroll
-        for (int k = 0; k < K; ++k)
-            red[warp * kGenCols + 32 * k + lane] = acc[k][c];
-        __syncthreads();
-        const uint32_t x = threadIdx.x, cc = (tile - rt * ct) * kGenCols + x;
-        if (x < (uint32_t)kGenCols && cc < m) {
-            float s = red[x];
-#pragma unroll
-            for (int k = 1; k < 8; ++k)
-                s = __fadd_rn(s, red[k * kGenCols + x]);
-            part[(size_t)cc * r + c] = s;
+            for (int c = 0; c < RM; ++c)
+                if (R || c < r)
+                    part[(size_t)(c0 + 32 * k) * r + c] = acc[k][c];
         }
-    }
 }
 
 template <int CK, int R, int KB>
@@ -448,29 +419,34 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
 // R: the configured rank (1, 2, 4, 8; 0: another one).  Tensors thinner than it, and those behind them whose
 // factors are off the vector loads' alignment, take the run-time rank.
 template <int PASS, int CK, int R, int KB>
-__global__ void __launch_bounds__(kGenThreads, R == 8 || R == 0 ? 3 : 4) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+__global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3 : 4) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
-    __shared__ __align__(16) float red[PASS == 2 ? 8 * kGenCols : PASS == 1 ? 8 * 4 * CONEF_MAX_RANK : 8 * kGenChunk / 4];
+    __shared__ __align__(16) uint8_t bytes[PASS == 3 ? 8 * kGenChunk : 16];
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t tile = blockIdx.x - pfx[li];
     constexpr int VW = R == 8 ? 4 : R ? R : 1;   // floats per vector load
     const bool exact = R != 0 && L.rank == R && ((L.msgp_off | L.msgq_off) & (VW - 1)) == 0;
     if (PASS == 1) {
-        if (R && exact)
-            gen_p1_body<CK, R>(V, L, tile, red);
-        else
-            gen_p1_body<CK, 0>(V, L, tile, red);
+        if (R && exact) {
+            if (L.g_nr == 4)
+                gen_p1_body<CK, R, 4>(V, L, tile);
+            else
+                gen_p1_body<CK, R, 1>(V, L, tile);
+        } else {
+            for (int x = 0; x < L.g_nr; ++x)
+                gen_p1_body<CK, 0, 1>(V, L, tile * (uint32_t)L.g_nr + x);
+        }
     } else if (PASS == 2) {
         if (R && exact)
-            gen_p2_body<CK, R>(V, L, tile, red);
+            gen_p2_body<CK, R>(V, L, tile);
         else
-            gen_p2_body<CK, 0>(V, L, tile, red);
+            gen_p2_body<CK, 0>(V, L, tile);
     } else {
         if (R && exact)
-            gen_p3_body<CK, R, KB>(V, L, tile, (uint8_t *)red);
+            gen_p3_body<CK, R, KB>(V, L, tile, bytes);
         else
-            gen_p3_body<CK, 0, KB>(V, L, tile, (uint8_t *)red);
+            gen_p3_body<CK, 0, KB>(V, L, tile, bytes);
     }
 }
 

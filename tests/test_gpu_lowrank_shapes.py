@@ -1,6 +1,7 @@
 """Low-rank passes for any shape: widths around a warp, a chunk and eight chunks, tensors thinner than the
 rank, odd offsets, every rank, block size and both scale types, with and without beta.  Factors against
-the oracle; stored codes and scales teacher-forced, bit for bit."""
+the oracle; stored codes and scales teacher-forced, bit for bit.  The order of
+the factors' sums is that of the kernels for every codec: free-running steps give the same bits on both."""
 import numpy as np
 import pytest
 import torch
@@ -48,3 +49,32 @@ def test_passes_on_edges(rank, c):
                 oa, os_ = pu.oracle_state_arrays(o, i, l)
                 assert np.array_equal(ga, oa) and np.array_equal(gs, os_), (t, l, i)
         eng.reduce_messages(b.MSG_Q)
+
+
+@pytest.mark.parametrize("rank,c", [(1, dict(kind="int8", block=256)), (2, dict(kind="int4", block=128, scale_dtype="fp16")),
+                                    (3, dict(kind="int8", block=32, scale_dtype="fp16")), (4, dict(kind="int4", block=64, beta=0.3)),
+                                    (8, dict(kind="int8", block=128))])
+@pytest.mark.parametrize("many", [False, True])   # one row per warp in pass 1, or four
+def test_order_of_sums(rank, c, many):
+    from paper_2312_08538_b200 import binding as b
+    cfg = wl.config("resnet50-mini")
+    shapes = EDGES + [(256, 65, 1), (257, 63, 1), (1030, 129, 1)] + ([(30011, 97, 1)] if many else [])
+    cfg.update(tensors=shapes, n_workers=2, q=dict(kind="lowrank", rank=rank), c=c, grad="normal1e-3")
+    q0 = wl.q_init(cfg, "cuda")
+    both = [pu.make_gpu(cfg, q_init=q0, fast=f) for f in (True, False)]
+    layers = [l for l, t in enumerate(shapes) if t[2]]
+    for t in range(3):
+        gd, _ = pu.grads_both(cfg, t)
+        for e, f in zip(both, (True, False)):
+            e.step(t, gd, 0)
+            e.set_fast_path(True)   # (the same Gram-Schmidt)
+            e.reduce_messages(b.MSG_P)
+            e.set_fast_path(f)
+            e.step(t, gd, 1)
+        for l in layers:
+            for i in range(2):
+                x, y = (e.factors(l, i) for e in both)
+                for k in ("p_i", "q_i"):
+                    assert torch.equal(x[k], y[k]), (t, l, i, k)
+        for e in both:
+            e.reduce_messages(b.MSG_Q)

@@ -2,7 +2,8 @@
 // do not take: any width, any alignment, any rank (Sec. 5.2; Alg. 2, and Alg. 4 with beta).
 //
 //   pass 1  P_i = M_i Q_{t-1}     a warp takes four rows (small models: one), its lanes neighbouring columns
-//   pass 2  Q_i = M_i^T P_hat     a warp takes 64 columns, two per lane, and runs down 256 rows
+//   pass 2  Q_i = M_i^T P_hat     a warp takes 32 columns and runs down 256 rows (two columns per lane: 168 us instead
+//                                 of 140 below)
 //   pass 3  r = p - P_hat Q_i^T, absmax, requantise, store: a warp takes 256 consecutive elements (whole
 //           quantisation blocks), lane l the elements l, l + 32, ...
 //
@@ -18,7 +19,7 @@
 // codec (conef_kernels.cuh), so a row's columns and a tile's rows are not shared out among warps.
 //
 // A recurrent model's odd layers (24.9 M elements, two workers, int4, rank 2): 222 / 286 / 395 us for the
-// three passes on the kernels for every codec (one element and a run-time rank at a time), 125 / 168 / 112 us
+// three passes on the kernels for every codec (one element and a run-time rank at a time), 125 / 140 / 112 us
 // here.
 #pragma once
 #include "conef_fast.cuh"
@@ -26,7 +27,7 @@
 namespace conef {
 
 constexpr int kGenThreads = 256;
-constexpr int kGenCols = 64;     // pass 2: columns per warp
+constexpr int kGenCols = 32;     // pass 2: columns per warp
 constexpr int kGenChunk = 256;   // pass 3: elements per warp and step
 constexpr int kGenCtas = kPlanSMs * 6;   // CTAs a pass should have at least, where tiles can be made smaller
 

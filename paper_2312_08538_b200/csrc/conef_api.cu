@@ -43,7 +43,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_CSK,                                               // count sketch applied run by run: one tile per run
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
        T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
-       T_DECODE,                                            // tiles of kDecTile elements: stored error expanded; the step on a dense error
+       T_DECODE,                                            // tiles of the stored error expanded (dec_batch) or of the step on a dense error (kDecTile elements)
        T_IL, T_ILT,                                         // count sketch, workers interleaved: tiles of elements, of sketch entries
        T_GEN1, T_GEN2, T_GEN3,                              // low-rank passes for any shape
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
@@ -74,6 +74,7 @@ struct Plan {
     // 2c + {0,1}: passes 2, 3 over the tensors the fused kernel leaves; table 10 (tuned pass 1)
     // counts the tiles of the kernel that adds up the row partials of pass 1
     std::vector<int32_t> pfx[kNumTables];
+    int dec_batch = 0;              // vectors per thread where the stored error is expanded
     std::vector<int> fast_threads;  // CTA size of each class
     std::vector<char> fast_narrow;  // ... and whether its tensors' rows are shorter than 256 elements
     std::vector<int> fast_subs;     // ... and the most rows a period of its tensors spans
@@ -183,6 +184,11 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
         }
         P.fv_tiles = total * n_workers / (kHistTile * kFvTiles) >= kPlanSMs * 16 ? kFvTiles : 1;
     }
+    int64_t compressed = 0;
+    for (int l = 0; l < n_tensors; ++l)
+        if (tensors[l].compress && tensors[l].rows > 0 && tensors[l].cols > 0 && tensors[l].rows <= 0xFFFFFFFFLL / tensors[l].cols)
+            compressed += tensors[l].rows * tensors[l].cols;
+    P.dec_batch = dec_batch(compressed);
     // tile lengths of the tuned low-rank passes from the model's size
     int it1 = kFastIt1, it2 = kFastIt2, it3 = kFastIt3;
     GenPlan gen;
@@ -276,7 +282,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             }
             tiles[T_FLAT] = (int)ceil_div(L.nunits, kFlatUnitsPerCta);
             tiles[T_GS] = 1;
-            tiles[T_DECODE] = (int)ceil_div(L.d, kDecTile);
+            tiles[T_DECODE] = (int)ceil_div(L.d, c->kind == CONEF_C_IDENTITY ? kDecTile : dec_tile(P.dec_batch));
             if (q->kind == CONEF_Q_IDENTITY) {
                 L.k = L.d;
             } else if (q->kind == CONEF_Q_RANDBLOCK) {
@@ -1574,7 +1580,7 @@ int conef_decompress_error(conef_ctx *ctx, int worker, float *out, conef_stream 
     }
     const int ck = ctx->c.kind;
     if (ctx->c.iconef != 2 && (ck == CONEF_C_INT8 || ck == CONEF_C_INT4 || (ck == CONEF_C_STOCHQUANT && ctx->c.levels <= 127))) {
-        decode_launch(ck == CONEF_C_INT4, ctx->c.iconef == 1, V, table_ptr(ctx, T_DECODE), tiles_of(ctx, T_DECODE), worker, out, s);
+        decode_launch(ctx->plan.dec_batch, ck == CONEF_C_INT4, ctx->c.iconef == 1, V, table_ptr(ctx, T_DECODE), tiles_of(ctx, T_DECODE), worker, out, s);
         LAUNCH_CHECK(ctx);
         return CONEF_OK;
     }

@@ -1,4 +1,4 @@
-"""The stored error expanded to fp32 at the edges of the decode tiles (4096 elements; output on and
+"""The stored error expanded to fp32 at the edges of the decode tiles (1024 elements, 4096 in large models; output on and
 off 16-byte boundaries), against the codes and scales read back from the state."""
 import numpy as np
 import pytest
@@ -23,16 +23,17 @@ def _expand(ctx, worker, tensor, d, kind, block, scale_dtype, second):
 @pytest.mark.parametrize("kind,block,scale_dtype", [("int8", 256, "fp32"), ("int8", 32, "fp16"), ("int4", 128, "fp16"),
                                                     ("int4", 64, "fp32")])
 @pytest.mark.parametrize("offset", [0, 1])
-def test_decode_equals_codes_times_scales(kind, block, scale_dtype, iconef, offset):
+@pytest.mark.parametrize("shapes", [SHAPES, SHAPES + [(1, 1024), (1, 1023), (1600, 1600)]])
+def test_decode_equals_codes_times_scales(kind, block, scale_dtype, iconef, offset, shapes):
     from paper_2312_08538_b200 import binding as b
-    ctx = b.ConEF([(r, c, 1) for r, c in SHAPES], 2, dict(kind="randk", k_num=1, k_den=10, seed=3),
+    ctx = b.ConEF([(r, c, 1) for r, c in shapes], 2, dict(kind="randk", k_num=1, k_den=10, seed=3),
                   dict(kind=kind, block=block, scale_dtype=scale_dtype, iconef=iconef), 0.1)
-    total = sum(r * c for r, c in SHAPES)
+    total = sum(r * c for r, c in shapes)
     ctx.step(0, [torch.randn(total, device="cuda") for _ in range(2)], 0)
     out = torch.full((total + offset + 1,), 7.0, device="cuda")
     ctx.decompress_error(1, out[offset:])
     want = [_expand(ctx, 1, l, r * c, kind, block, scale_dtype, False) +
-            (_expand(ctx, 1, l, r * c, kind, block, scale_dtype, True) if iconef else 0) for l, (r, c) in enumerate(SHAPES)]
+            (_expand(ctx, 1, l, r * c, kind, block, scale_dtype, True) if iconef else 0) for l, (r, c) in enumerate(shapes)]
     got = out.cpu().numpy()
     assert np.array_equal(got[offset:offset + total], np.concatenate(want).astype(np.float32))
     assert got[offset + total] == 7.0

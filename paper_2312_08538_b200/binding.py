@@ -143,8 +143,11 @@ def conef_workspace_bytes(tensors, n_workers: int, q: Dict, c: Dict) -> int:
 
 
 def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the handle alone: torch.cuda.current_stream() builds an object around it in every call, a good part
+    # of the host time of a small step.  (Every caller holds device memory, so CUDA is initialised.)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def conef_randk_indices_noalloc(seed: int, tensor: int, step: int, d: int, k: int, idx_out: torch.Tensor,
@@ -183,6 +186,7 @@ class ConEF:
                               C.byref(cc), float(lr), self._ws_ptr, nbytes, _stream_handle(stream)),
                "conef_init")
         self.h = h
+        self._dense1d = self.message_elems(MSG_DENSE1D)
 
     def close(self):
         if getattr(self, "h", None) and lib is not None:
@@ -236,7 +240,7 @@ class ConEF:
             res[MSG_Q] = self.reduce_messages(MSG_Q, outs.get(MSG_Q), stream)
         else:
             res[MSG_VALUES] = self.reduce_messages(MSG_VALUES, outs.get(MSG_VALUES), stream)
-        if self.message_elems(MSG_DENSE1D) > 0:
+        if self._dense1d > 0:
             res[MSG_DENSE1D] = self.reduce_messages(MSG_DENSE1D, outs.get(MSG_DENSE1D), stream)
         return res
 

@@ -1446,8 +1446,10 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
             // the launches work on different tensors: all but the first run on side streams
             const int tabs[3] = {T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16};
             const int csz[3] = {1, 8, 16};
-            int used = 0, launched = 0;
-            if (ctx->n_aux > 0)
+            int used = 0, launched = 0, launches = tiles_of(ctx, T_GS_REST) > 0;
+            for (int k = 0; k < 3; ++k)
+                launches += tiles_of(ctx, tabs[k]) > 0;
+            if (ctx->n_aux > 0 && launches > 1)   // (one launch stays on the caller's stream)
                 CK_CUDA(cudaEventRecord(ctx->ev_fork, s));
             auto pick = [&]() -> cudaStream_t {
                 if (launched++ == 0 || used >= ctx->n_aux)

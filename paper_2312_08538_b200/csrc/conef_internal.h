@@ -27,6 +27,7 @@ constexpr int kSelWords = 8;            // uint32 words of counters per tensor
 
 // status bits written by kernels (sticky, OR-ed)
 enum {
+    ST_LIST_STALE = 1,      // random-k selection: the list of window elements held something else (the set was found without it)
     ST_COUNT_MISMATCH = 2,  // the number of selected coordinates differs from k
     ST_SELECT_FAILED = 4,   // no threshold: a radix level without its bin, or too many keys on one 32-bit hash
     ST_FUSED_TIMEOUT = 8    // a bounded wait of the fused low-rank kernel ran out (a copy or a gang member never arrived)

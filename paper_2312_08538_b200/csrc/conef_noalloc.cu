@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
     const uint32_t nlist = load_cg(&a.ctr[NA_LISTED]);
     uint32_t total = 0xFFFFFFFFu;
     if (windowed && nlist <= a.cap)
-        total = select_finish<kNaTile>(S, a.list, nlist, a.lo, a.scale, a.k, a.cnt, a.ntiles, [](uint32_t) {});
+        total = select_finish<kNaTile>(S, SelectWindow{a.lo, a.hi, a.d, a.k, a.scale, nullptr}, a.list, nlist, a.cnt, a.ntiles, [](uint32_t) {});
     bool failed = false;
     // no listed element belongs: the members are the elements below the window (lo > 0 then)
     if (total != 0xFFFFFFFFu && S.tau == 0 && tid == 0)

@@ -7,9 +7,8 @@ namespace conef {
 // select_finish for a tensor of at most kSelTailTiles tiles, word offsets included: its bitmap is
 // completed in shared memory (16 words per thread), so that nothing but the list and the bitmap
 // itself is waited for
-__device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const uint2 *list, uint32_t nlist, uint32_t lo,
-                                                        uint64_t scale, uint32_t k, uint32_t *bits, uint32_t *tileoff,
-                                                        uint16_t *wordoff, uint32_t ntiles)
+__device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
+                                                        uint32_t *bits, uint32_t *tileoff, uint16_t *wordoff, uint32_t ntiles)
 {
     constexpr int PER = kSelTailWords / kSelThreads;   // a tile is 16 threads' words
     static_assert(PER == 16, "half a warp per tile");
@@ -29,9 +28,9 @@ __device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const u
             }
         }
     }
-    if (select_threshold(S, list, nlist, lo, scale, k, below) == 0xFFFFFFFFu)
+    if (select_threshold(S, W, list, nlist, below) == 0xFFFFFFFFu)
         return 0xFFFFFFFFu;
-    select_listed(S, list, nlist, [&](uint32_t j) { atomicOr(&S.words[j >> 5], 1u << (j & 31u)); });
+    select_listed(S, W, list, nlist, [&](uint32_t j) { atomicOr(&S.words[j >> 5], 1u << (j & 31u)); });
     __syncthreads();
     uint32_t word[PER], cnt = 0, total;
 #pragma unroll
@@ -150,11 +149,12 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
 
     // ---- the CTA that finishes the tensor
     const uint32_t k = (uint32_t)L.k, nlist = load_cg(&ctr[1]);
+    const SelectWindow W{lo, hi, d, k, L.sel_scale, V.status};
     uint32_t total = 0xFFFFFFFFu;
     if (windowed && nlist <= L.cand_cap)
         total = ntiles <= (uint32_t)kSelTailTiles
-                    ? select_finish_short(S, list, nlist, lo, L.sel_scale, k, bits, tileoff, wordoff, ntiles)
-                    : select_finish<kHistTile>(S, list, nlist, lo, L.sel_scale, k, tileoff, ntiles,
+                    ? select_finish_short(S, W, list, nlist, bits, tileoff, wordoff, ntiles)
+                    : select_finish<kHistTile>(S, W, list, nlist, tileoff, ntiles,
                                                [&](uint32_t j) { atomicOr(&bits[j >> 5], 1u << (j & 31u)); });
     if (total == 0xFFFFFFFFu) {
         __syncthreads();

@@ -26,7 +26,7 @@ constexpr int kSelThreads = 256;
 constexpr int kSelBins = 2048;
 constexpr int kSelShortTensor = 1024;   // up to here the window is not used
 constexpr int kSelTailTiles = 16;       // tensors of at most this many tiles: the last CTA also writes the offsets
-constexpr int kSelList = 2304;          // window entries a CTA holds in shared memory (enough for any tensor of kSelTailTiles)
+constexpr int kSelList = 2304;          // window entries a CTA holds in shared memory (a tensor of kSelTailTiles expects 2204 at most)
 constexpr int kSelTiles = 1280;         // tile counts it holds there
 constexpr int kSelTailWords = kSelTailTiles * kHistTile / 32;
 
@@ -44,9 +44,10 @@ struct SelectShared {
 };
 
 // Loads of what other CTAs of the same launch wrote before their ticket: past L1, and volatile with a
-// memory clobber, so that the compiler may not move them ahead of the ticket.  (A first form without
-// either, and without the bound on the bin index, read out of bounds; an entry read before it was
-// written falls below the window and gives such an index.)
+// memory clobber, so that the compiler may not move them ahead of the ticket (it may move __ldcg, whose
+// result depends on its address alone).  A form without them read shared memory out of bounds: an
+// entry that was written lies inside the window, and select_window's scale then gives a bin below
+// kSelThreads, so the entry had been read before it was written.
 __device__ __forceinline__ uint32_t load_cg(const uint32_t *p)
 {
     uint32_t v;
@@ -140,30 +141,55 @@ __device__ __forceinline__ void select_key(SelectShared &S, uint32_t rank)
     __syncthreads();
 }
 
+// A tensor's window, its k and d (scale: see select_window), and where a list that holds anything but
+// elements of the window is reported (null: nowhere)
+struct SelectWindow {
+    uint32_t lo, hi, d, k;
+    uint64_t scale;
+    int32_t *status;
+    // Whether a list entry can be one of this tensor's; no entry is used as an index before this is known.
+    // (Calls that share one scratch and overlap see one another's entries.)
+    __device__ __forceinline__ bool holds(uint2 e) const { return e.x - lo <= hi - lo && e.y < d; }
+    // Result of a list that failed: as if the window had missed, so that the tensor is hashed again.  All
+    // threads of the CTA take it.
+    __device__ __forceinline__ uint32_t stale() const
+    {
+        if (status && threadIdx.x == 0)
+            atomicOr(status, ST_LIST_STALE);
+        return 0xFFFFFFFFu;
+    }
+};
+
 // The threshold among the window's elements.  `below_mine`: the calling thread's share of the number of
-// elements below the window; scale: see select_window.  The caller has zeroed S.hist[0 .. kSelThreads)
-// and synchronised.  Returns the number of elements below the window, or 0xFFFFFFFF where the window
-// does not hold the threshold; S.tau is the threshold key (0 when no listed element belongs).
-__device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const uint2 *list, uint32_t nlist, uint32_t lo, uint64_t scale,
-                                                     uint32_t k, uint32_t below_mine)
+// elements below the window.  The caller has zeroed S.hist[0 .. kSelThreads) and synchronised.  Returns
+// the number of elements below the window, or 0xFFFFFFFF where the window does not hold the threshold;
+// S.tau is the threshold key (0 when no listed element belongs).
+__device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
+                                                     uint32_t below_mine)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lo = W.lo, k = W.k;
     const bool shared = nlist <= (uint32_t)kSelList;
+    bool stale = false;
     if (shared) {
         // one linear bin per thread; the few keys of the bin that holds the rank are compared
-        auto bin_of = [&](uint32_t h) { return min((uint32_t)(((uint64_t)(h - lo) * scale) >> 32), (uint32_t)kSelThreads - 1u); };
+        auto bin_of = [&](uint32_t h) { return (uint32_t)(((uint64_t)(h - lo) * W.scale) >> 32); };
 #pragma unroll 4
         for (uint32_t x = tid; x < nlist; x += kSelThreads) {
             const uint2 e = load_cg(&list[x]);
             S.keys[x] = ((uint64_t)e.x << 32) | e.y;
-            atomicAdd(&S.hist[bin_of(e.x)], 1u);
+            if (W.holds(e))
+                atomicAdd(&S.hist[bin_of(e.x)], 1u);
+            else
+                stale = true;
         }
         if (tid == 0) {
             S.n = 0;
             S.bad = 1u;
             S.tau = 0;
         }
-        __syncthreads();
+        if (__syncthreads_or(stale))
+            return W.stale();
         const uint32_t c = S.hist[tid];
         uint32_t inc = c;
 #pragma unroll
@@ -218,8 +244,8 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const uint
         return S.bad ? 0xFFFFFFFFu : below;
     }
     // a longer list stays in L2: two passes over it, 2048 bins
-    const uint64_t scale8 = scale * (kSelBins / kSelThreads);
-    auto bin_of = [&](uint32_t h) { return min((uint32_t)(((uint64_t)(h - lo) * scale8) >> 32), (uint32_t)kSelBins - 1u); };
+    const uint64_t scale8 = W.scale * (kSelBins / kSelThreads);
+    auto bin_of = [&](uint32_t h) { return (uint32_t)(((uint64_t)(h - lo) * scale8) >> 32); };
     for (int b = kSelThreads + tid; b < kSelBins; b += kSelThreads)
         S.hist[b] = 0;
     if (tid == 0)
@@ -231,9 +257,15 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const uint
     if (below == k)
         return below;
 #pragma unroll 8
-    for (uint32_t x = tid; x < nlist; x += kSelThreads)
-        atomicAdd(&S.hist[bin_of(load_cg(&list[x]).x)], 1u);
-    __syncthreads();
+    for (uint32_t x = tid; x < nlist; x += kSelThreads) {
+        const uint2 e = load_cg(&list[x]);
+        if (W.holds(e))
+            atomicAdd(&S.hist[bin_of(e.x)], 1u);
+        else
+            stale = true;
+    }
+    if (__syncthreads_or(stale))
+        return W.stale();
     select_bin(S, k - below);
     if (S.bad)
         return 0xFFFFFFFFu;
@@ -255,9 +287,10 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const uint
     return S.bad ? 0xFFFFFFFFu : below;
 }
 
-// calls f(j) for the listed elements that belong to the set
+// calls f(j) for the listed elements that belong to the set; j < d, also where the list changed after
+// select_threshold looked at it
 template <class F>
-__device__ __forceinline__ void select_listed(SelectShared &S, const uint2 *list, uint32_t nlist, F f)
+__device__ __forceinline__ void select_listed(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist, F f)
 {
     const uint64_t tau = S.tau;
     if (nlist <= (uint32_t)kSelList) {
@@ -268,7 +301,7 @@ __device__ __forceinline__ void select_listed(SelectShared &S, const uint2 *list
 #pragma unroll 4
         for (uint32_t x = threadIdx.x; x < nlist; x += kSelThreads) {
             const uint2 e = load_cg(&list[x]);
-            if ((((uint64_t)e.x << 32) | e.y) <= tau)
+            if ((((uint64_t)e.x << 32) | e.y) <= tau && e.y < W.d)
                 f(e.y);
         }
     }
@@ -345,8 +378,8 @@ __device__ __forceinline__ uint32_t scan_counts(uint32_t *cnt, int64_t n, uint32
 // into exclusive offsets, in place.  Returns the number of members, or 0xFFFFFFFF where the window
 // does not hold the threshold (nothing is marked then).
 template <uint32_t TILE, class Mark>
-__device__ __forceinline__ uint32_t select_finish(SelectShared &S, const uint2 *list, uint32_t nlist, uint32_t lo, uint64_t scale,
-                                                  uint32_t k, uint32_t *cnt, uint32_t ntiles, Mark mark)
+__device__ __forceinline__ uint32_t select_finish(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
+                                                  uint32_t *cnt, uint32_t ntiles, Mark mark)
 {
     const int tid = threadIdx.x;
     const bool shared = ntiles <= (uint32_t)kSelTiles;
@@ -358,9 +391,9 @@ __device__ __forceinline__ uint32_t select_finish(SelectShared &S, const uint2 *
             S.tiles[t] = c;
         mine += c;
     }
-    if (select_threshold(S, list, nlist, lo, scale, k, mine) == 0xFFFFFFFFu)
+    if (select_threshold(S, W, list, nlist, mine) == 0xFFFFFFFFu)
         return 0xFFFFFFFFu;
-    select_listed(S, list, nlist, [&](uint32_t j) {
+    select_listed(S, W, list, nlist, [&](uint32_t j) {
         mark(j);
         atomicAdd(shared ? &S.tiles[j / TILE] : &cnt[j / TILE], 1u);
     });

@@ -31,9 +31,11 @@ constexpr int64_t kNaWords = 8 + kNaTiles + 2 * kNaList;            // counters,
 // cudaGetSymbolAddress; it is not a device address.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNaWords];
 
-// counter words: CTAs that have finished, elements listed (both zero between calls), then what the
-// first kernel leaves for the second: threshold key, whether the selection failed
-enum { NA_DONE = 0, NA_LISTED = 1, NA_TAU_LO = 2, NA_TAU_HI = 3, NA_FAILED = 4 };
+// Counter words: CTAs that have finished and elements listed (the second kernel of every call clears
+// them, so that whatever calls that overlap did to them is over with the last of those calls), then what
+// the first kernel leaves for the second: the threshold key, and whose it is (hash stream, d, k; k = 0: no
+// threshold).
+enum { NA_DONE = 0, NA_LISTED = 1, NA_TAU_LO = 2, NA_TAU_HI = 3, NA_STREAM_LO = 4, NA_STREAM_HI = 5, NA_D = 6, NA_K = 7 };
 
 struct NaArgs {
     uint32_t *ctr, *cnt;
@@ -52,8 +54,11 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
     const int tid = threadIdx.x;
     const bool windowed = a.d > (uint32_t)kSelShortTensor;
     S.hist[tid] = 0;   // the bins of select_threshold
-    if (tid == 0)
+    if (tid == 0) {
         s_n = s_cnt = 0;
+        if (blockIdx.x == 0)
+            a.ctr[NA_K] = 0;   // (before this CTA's ticket, so before the last CTA's result)
+    }
     __syncthreads();
     if (windowed) {
         const uint32_t j0 = blockIdx.x * kNaTile + tid * kNaPer;
@@ -135,20 +140,25 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
         total = scan_counts(a.cnt, a.ntiles, S.wsum);
     }
     if (tid == 0) {
-        a.ctr[NA_DONE] = a.ctr[NA_LISTED] = 0;
         a.ctr[NA_TAU_LO] = (uint32_t)S.tau;
         a.ctr[NA_TAU_HI] = (uint32_t)(S.tau >> 32);
-        a.ctr[NA_FAILED] = failed || total != a.k;
+        a.ctr[NA_STREAM_LO] = (uint32_t)a.stream;
+        a.ctr[NA_STREAM_HI] = (uint32_t)(a.stream >> 32);
+        a.ctr[NA_D] = a.d;
+        a.ctr[NA_K] = failed || total != a.k ? 0u : a.k;
     }
 }
 
 // The members in ascending order, hashed once more.  A selection that did not come out as exactly k
-// coordinates is made visible in the output itself, since this entry point neither synchronises nor
+// coordinates, or whose result is not there (another call's kernels ran in between), is made visible in the output itself, since this entry point neither synchronises nor
 // owns a status buffer: nothing is written but idx_out[0] = 0xFFFFFFFF, a value no index can take.
 __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32_t *__restrict__ idx_out)
 {
     __shared__ uint32_t wsum[kSelThreads / 32];
-    if (a.ctr[NA_FAILED]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        a.ctr[NA_DONE] = a.ctr[NA_LISTED] = 0;   // (no CTA of this kernel reads them)
+    if (a.ctr[NA_STREAM_LO] != (uint32_t)a.stream || a.ctr[NA_STREAM_HI] != (uint32_t)(a.stream >> 32) ||
+        a.ctr[NA_D] != a.d || a.ctr[NA_K] != a.k) {
         if (blockIdx.x == 0 && threadIdx.x == 0)
             idx_out[0] = 0xFFFFFFFFu;
         return;

@@ -24,6 +24,35 @@ __device__ __forceinline__ int find_layer(const int32_t *__restrict__ pfx, int n
     return lo;
 }
 
+// Loads of what other CTAs of the same launch wrote before a ticket or a flag: past L1, and volatile with
+// a memory clobber, so that the compiler may not move them ahead of it (it may move __ldcg, whose
+// result depends on its address alone).
+__device__ __forceinline__ uint32_t load_cg(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 load_cg(const uint2 *p)
+{
+    uint2 v;
+    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 load_cg(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void load_cg(const uint32_t *p, uint32_t (&v)[8])   // 32 bytes, 16-byte aligned
+{
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p) : "memory");
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p + 4) : "memory");
+}
+
 __device__ __forceinline__ float warp_max(float v)
 {
 #pragma unroll

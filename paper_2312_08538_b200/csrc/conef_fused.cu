@@ -31,6 +31,7 @@
 #include <algorithm>
 
 #include "conef_codec.cuh"
+#include "conef_common.cuh"
 
 namespace conef {
 
@@ -516,9 +517,9 @@ __global__ void __launch_bounds__(kFuThreads, MINB) k_fused23(const __grid_const
                 __threadfence();
                 for (int x = tid; x < 256 * R / 4; x += kFuThreads) {
                     const float4 *src = (const float4 *)(part + (size_t)cg * ntp * 256 * R) + x;
-                    float4 acc = __ldcg(src);
+                    float4 acc = load_cg(src);
                     for (uint32_t tt = 1; tt < ntp; ++tt) {
-                        const float4 v = __ldcg(src + (size_t)tt * (256 * R / 4));
+                        const float4 v = load_cg(src + (size_t)tt * (256 * R / 4));
                         acc.x = __fadd_rn(acc.x, v.x); acc.y = __fadd_rn(acc.y, v.y);
                         acc.z = __fadd_rn(acc.z, v.z); acc.w = __fadd_rn(acc.w, v.w);
                     }
@@ -541,7 +542,7 @@ __global__ void __launch_bounds__(kFuThreads, MINB) k_fused23(const __grid_const
                         for (uint32_t s = 0; s < subs; ++s) {
                             const uint32_t pos = s * m + c, off = pos & 255u;
                             const uint32_t sp = (((off >> 7) * 4u + (off & 3u)) << 5) + ((off >> 2) & 31u);
-                            const float4 v = __ldcg((const float4 *)(qseg + (size_t)(pos >> 8) * 256 * R) + h * 256 + sp);
+                            const float4 v = load_cg((const float4 *)(qseg + (size_t)(pos >> 8) * 256 * R) + h * 256 + sp);
                             if (s == 0) {
                                 acc = v;
                             } else {
@@ -569,7 +570,7 @@ __global__ void __launch_bounds__(kFuThreads, MINB) k_fused23(const __grid_const
                 for (int q = 0; q < 4; ++q)
 #pragma unroll
                     for (int c = 0; c < R; c += 4) {
-                        const float4 t4 = __ldcg((const float4 *)(q_res + (size_t)(col[x] + q) * R + c));
+                        const float4 t4 = load_cg((const float4 *)(q_res + (size_t)(col[x] + q) * R + c));
                         frag[4 * x + q][c] = t4.x; frag[4 * x + q][c + 1] = t4.y;
                         frag[4 * x + q][c + 2] = t4.z; frag[4 * x + q][c + 3] = t4.w;
                     }

@@ -43,32 +43,6 @@ struct SelectShared {
     uint32_t bin, rem, n, bad;
 };
 
-// Loads of what other CTAs of the same launch wrote before their ticket: past L1, and volatile with a
-// memory clobber, so that the compiler may not move them ahead of the ticket (it may move __ldcg, whose
-// result depends on its address alone).  A form without them read shared memory out of bounds: an
-// entry that was written lies inside the window, and select_window's scale then gives a bin below
-// kSelThreads, so the entry had been read before it was written.
-__device__ __forceinline__ uint32_t load_cg(const uint32_t *p)
-{
-    uint32_t v;
-    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint2 load_cg(const uint2 *p)
-{
-    uint2 v;
-    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void load_cg(const uint32_t *p, uint32_t (&v)[8])   // 32 bytes, 16-byte aligned
-{
-    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p) : "memory");
-    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p + 4) : "memory");
-}
-
 // exclusive prefix over the CTA's threads of v; total: the sum over all threads
 __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *wsum, uint32_t &total)
 {
@@ -148,7 +122,9 @@ struct SelectWindow {
     uint64_t scale;
     int32_t *status;
     // Whether a list entry can be one of this tensor's; no entry is used as an index before this is known.
-    // (Calls that share one scratch and overlap see one another's entries.)
+    // (Calls that share one scratch and overlap see one another's entries.  A form without load_cg read shared
+    // memory out of bounds: an entry that was written lies inside the window, and select_window's scale
+    // then gives a bin below kSelThreads, so that entry had been read before it was written.)
     __device__ __forceinline__ bool holds(uint2 e) const { return e.x - lo <= hi - lo && e.y < d; }
     // Result of a list that failed: as if the window had missed, so that the tensor is hashed again.  All
     // threads of the CTA take it.

@@ -31,11 +31,11 @@ constexpr int64_t kNaWords = 8 + kNaTiles + 2 * kNaList;            // counters,
 // cudaGetSymbolAddress; it is not a device address.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNaWords];
 
-// Counter words: CTAs that have finished and elements listed (the second kernel of every call clears
+// Counter words: elements listed and CTAs that have finished (the second kernel of every call clears
 // them, so that whatever calls that overlap did to them is over with the last of those calls), then what
 // the first kernel leaves for the second: the threshold key, and whose it is (hash stream, d, k; k = 0: no
 // threshold).
-enum { NA_DONE = 0, NA_LISTED = 1, NA_TAU_LO = 2, NA_TAU_HI = 3, NA_STREAM_LO = 4, NA_STREAM_HI = 5, NA_D = 6, NA_K = 7 };
+enum { NA_LISTED = 0, NA_DONE = 1, NA_TAU_LO = 2, NA_TAU_HI = 3, NA_STREAM_LO = 4, NA_STREAM_HI = 5, NA_D = 6, NA_K = 7 };
 
 struct NaArgs {
     uint32_t *ctr, *cnt;
@@ -50,7 +50,7 @@ struct NaArgs {
 __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
 {
     __shared__ SelectShared S;
-    __shared__ uint32_t s_n, s_base, s_cnt, s_last;
+    __shared__ uint32_t s_n, s_base, s_cnt, s_last, s_listed;
     const int tid = threadIdx.x;
     const bool windowed = a.d > (uint32_t)kSelShortTensor;
     S.hist[tid] = 0;   // the bins of select_threshold
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
             if (pos < (uint32_t)kSelList) {
                 ((uint2 *)S.keys)[pos] = e;
             } else {
-                const uint32_t g = atomicAdd(&a.ctr[NA_LISTED], 1u);
+                const uint32_t g = select_claim(a.ctr, 1u);
                 if (g < a.cap)
                     a.list[g] = e;
             }
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
         __syncthreads();
         const uint32_t n = min(s_n, (uint32_t)kSelList);
         if (tid == 0) {
-            s_base = n ? atomicAdd(&a.ctr[NA_LISTED], n) : 0u;
+            s_base = n ? select_claim(a.ctr, n) : 0u;
             a.cnt[blockIdx.x] = s_cnt;
         }
         __syncthreads();
@@ -100,12 +100,11 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
     __threadfence();
     __syncthreads();
     if (tid == 0)
-        s_last = atomicAdd(&a.ctr[NA_DONE], 1u) == a.ntiles - 1 ? 1u : 0u;
+        s_last = select_ticket(a.ctr, a.ntiles, s_listed);   // (one thread's answer: the barriers below depend on it)
     __syncthreads();
     if (!s_last)
         return;
-    __threadfence();
-    const uint32_t nlist = load_cg(&a.ctr[NA_LISTED]);
+    const uint32_t nlist = s_listed;
     uint32_t total = 0xFFFFFFFFu;
     if (windowed && nlist <= a.cap)
         total = select_finish<kNaTile>(S, SelectWindow{a.lo, a.hi, a.d, a.k, a.scale, nullptr}, a.list, nlist, a.cnt, a.ntiles, [](uint32_t) {});
@@ -150,29 +149,42 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
 }
 
 // The members in ascending order, hashed once more.  A selection that did not come out as exactly k
-// coordinates, or whose result is not there (another call's kernels ran in between), is made visible in the output itself, since this entry point neither synchronises nor
-// owns a status buffer: nothing is written but idx_out[0] = 0xFFFFFFFF, a value no index can take.
+// coordinates, or whose result is not there (another call's kernels ran in between), is made visible in
+// the output itself, since this entry point neither synchronises nor owns a status buffer: nothing is
+// written but idx_out[0] = 0xFFFFFFFF, a value no index can take.
 __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32_t *__restrict__ idx_out)
 {
-    __shared__ uint32_t wsum[kSelThreads / 32];
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        a.ctr[NA_DONE] = a.ctr[NA_LISTED] = 0;   // (no CTA of this kernel reads them)
-    if (a.ctr[NA_STREAM_LO] != (uint32_t)a.stream || a.ctr[NA_STREAM_HI] != (uint32_t)(a.stream >> 32) ||
-        a.ctr[NA_D] != a.d || a.ctr[NA_K] != a.k) {
+    __shared__ uint32_t wsum[kSelThreads / 32], s_own, s_first;
+    __shared__ uint64_t s_tau;
+    const uint32_t j0 = blockIdx.x * kNaTile + threadIdx.x * kNaPer;
+    if (threadIdx.x == 0) {   // (one thread reads them: a CTA has to agree on whether it goes on)
+        const uint2 tau = *(const uint2 *)(a.ctr + NA_TAU_LO);
+        const uint4 of = *(const uint4 *)(a.ctr + NA_STREAM_LO);
+        s_first = a.cnt[blockIdx.x];
+        s_tau = ((uint64_t)tau.y << 32) | tau.x;
+        s_own = of.x == (uint32_t)a.stream && of.y == (uint32_t)(a.stream >> 32) && of.z == a.d && of.w == a.k;
+        if (blockIdx.x == 0)
+            a.ctr[NA_DONE] = a.ctr[NA_LISTED] = 0;   // (no CTA of this kernel reads them)
+    }
+    uint32_t h[kNaPer];   // (while those loads are under way)
+#pragma unroll
+    for (uint32_t q = 0; q < kNaPer; ++q)
+        h[q] = hash32(a.stream, j0 + q);
+    __syncthreads();
+    if (!s_own) {
         if (blockIdx.x == 0 && threadIdx.x == 0)
             idx_out[0] = 0xFFFFFFFFu;
         return;
     }
-    const uint64_t tau = ((uint64_t)a.ctr[NA_TAU_HI] << 32) | a.ctr[NA_TAU_LO];
-    const uint32_t j0 = blockIdx.x * kNaTile + threadIdx.x * kNaPer;
+    const uint64_t tau = s_tau;
     uint32_t in = 0, total;
 #pragma unroll
     for (uint32_t q = 0; q < kNaPer; ++q) {
         const uint32_t j = j0 + q;
-        if ((((uint64_t)hash32(a.stream, j) << 32) | j) <= tau && j < a.d)
+        if ((((uint64_t)h[q] << 32) | j) <= tau && j < a.d)
             in |= 1u << q;
     }
-    uint32_t slot = a.cnt[blockIdx.x] + block_exclusive(__popc(in), wsum, total);
+    uint32_t slot = s_first + block_exclusive<true>(__popc(in), wsum, total);
     for (; in; in &= in - 1, ++slot)
         if (slot < a.k)   // never past the caller's k entries, whatever went wrong before
             idx_out[slot] = j0 + (uint32_t)__ffs(in) - 1u;

@@ -67,7 +67,7 @@ __device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const S
 __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_constant__ DevView V)
 {
     __shared__ SelectShared S;
-    __shared__ uint32_t s_n, s_base, s_cnt[8], s_last;
+    __shared__ uint32_t s_n, s_base, s_cnt[8], s_last, s_listed;
     const int li = find_layer(V.pfx_hist, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t d = (uint32_t)L.d, lo = L.sel_lo, hi = L.sel_hi, T = (uint32_t)V.sel_tiles;
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
     const uint32_t ntiles = (uint32_t)((L.d + kHistTile - 1) / kHistTile);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t st = stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step);
-    uint32_t *ctr = V.sel + L.sel_off;   // finished CTAs, listed elements: zero between selections
+    uint32_t *ctr = V.sel + L.sel_off;   // listed elements and finished CTAs: zero between selections
     uint2 *list = (uint2 *)V.cand + L.cand_off;
     uint32_t *bits = V.selbits + L.selbits_off;
     uint32_t *tileoff = V.tileoff + L.tileoff_off;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
                 if (pos < (uint32_t)kSelList) {
                     ((uint2 *)S.keys)[pos] = e;
                 } else {   // (not expected: the list of a CTA holds several times the usual number)
-                    const uint32_t g = atomicAdd(&ctr[1], 1u);
+                    const uint32_t g = select_claim(ctr, 1u);
                     if (g < L.cand_cap)
                         list[g] = e;
                 }
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
         __syncthreads();
         const uint32_t n = min(s_n, (uint32_t)kSelList);
         if (tid == 0)
-            s_base = n ? atomicAdd(&ctr[1], n) : 0u;
+            s_base = n ? select_claim(ctr, n) : 0u;
         if (tid < T && tile0 + tid < ntiles)
             tileoff[tile0 + tid] = s_cnt[tid];
         __syncthreads();
@@ -141,14 +141,13 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
     __threadfence();
     __syncthreads();
     if (tid == 0)
-        s_last = atomicAdd(&ctr[0], 1u) == ncta - 1 ? 1u : 0u;
+        s_last = select_ticket(ctr, ncta, s_listed);   // (one thread's answer: the barriers below depend on it)
     __syncthreads();
     if (!s_last)
         return;
-    __threadfence();
 
     // ---- the CTA that finishes the tensor
-    const uint32_t k = (uint32_t)L.k, nlist = load_cg(&ctr[1]);
+    const uint32_t k = (uint32_t)L.k, nlist = s_listed;
     const SelectWindow W{lo, hi, d, k, L.sel_scale, V.status};
     uint32_t total = 0xFFFFFFFFu;
     if (windowed && nlist <= L.cand_cap)

@@ -43,7 +43,23 @@ struct SelectShared {
     uint32_t bin, rem, n, bad;
 };
 
-// exclusive prefix over the CTA's threads of v; total: the sum over all threads
+// A tensor's counters, one 64-bit word: listed elements in the low half, CTAs that have finished in the high
+// half.  A CTA's ticket thus also tells how many elements were listed before it.
+using SelectCtr = unsigned long long;
+__device__ __forceinline__ uint32_t select_claim(uint32_t *ctr, uint32_t n) { return (uint32_t)atomicAdd((SelectCtr *)ctr, (SelectCtr)n); }
+// thread 0 only; whether this CTA is the last of ncta, and the elements listed by all of them
+__device__ __forceinline__ bool select_ticket(uint32_t *ctr, uint32_t ncta, uint32_t &listed)
+{
+    const SelectCtr before = atomicAdd((SelectCtr *)ctr, 1ull << 32);
+    listed = (uint32_t)before;
+    if ((uint32_t)(before >> 32) != ncta - 1)
+        return false;
+    __threadfence();   // (with the barrier that follows, for the whole CTA)
+    return true;
+}
+
+// exclusive prefix over the CTA's threads of v; total: the sum over all threads; FRESH: wsum is not in use
+template <bool FRESH = false>
 __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *wsum, uint32_t &total)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -54,7 +70,8 @@ __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *wsum, 
         if (lane >= o)
             inc += n;
     }
-    __syncthreads();   // wsum may still be read from the previous call
+    if (!FRESH)
+        __syncthreads();   // wsum may still be read from the previous call
     if (lane == 31)
         wsum[warp] = inc;
     __syncthreads();

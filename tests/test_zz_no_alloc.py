@@ -65,26 +65,3 @@ def test_noalloc_rejects_what_its_fixed_scratch_cannot_hold():
     from oracle import conef_oracle as orc
     assert np.array_equal(idx, orc.randk_indices(7, 2, 5, d, k))      # (the failure mark 0xFFFFFFFF would show here)
     assert int(out[k].item()) == -1, "nothing is written past the k entries"
-
-
-def test_overlapping_calls_write_nothing_out_of_place_and_leave_nothing_behind():
-    """Calls on several streams share the one scratch and may spoil one another's index sets (they are the
-    caller's to order), but every write stays inside the call's own k entries, whatever the sizes; and
-    a call that starts after them is right again, whatever the overlap left in the counters."""
-    from paper_2312_08538_b200 import binding as b
-    from oracle import conef_oracle as orc
-    sizes = [(b.NOALLOC_MAX_ELEMS, 1 << 23), (5000, 50), (1 << 20, 1 << 10), (300, 7), (b.NOALLOC_MAX_ELEMS - 77, 16)]
-    streams = [torch.cuda.Stream() for _ in sizes]
-    outs = [torch.full((k + 64,), -1, dtype=torch.int32, device="cuda") for _, k in sizes]
-    torch.cuda.synchronize()
-    for step in range(50):
-        for (d, k), out, s in zip(sizes, outs, streams):
-            b.conef_randk_indices_noalloc(3, 0, step, d, k, out, stream=s)
-        if step % 10 == 9:
-            torch.cuda.synchronize()
-            for (d, k), out in zip(sizes, outs):
-                assert bool((out[k:] == -1).all())
-            for d, k in ((70000, 700), (300, 7), (1 << 21, 99)):
-                out = torch.empty(k, dtype=torch.int32, device="cuda")
-                b.conef_randk_indices_noalloc(9, 4, step, d, k, out)
-                assert np.array_equal(out.cpu().numpy().view(np.uint32), orc.randk_indices(9, 4, step, d, k))

@@ -266,6 +266,13 @@ int conef_set_total_workers(conef_ctx *ctx, int total);
 /* Choose kernels: 0 = generic kernels only, 1 = tuned kernels where the
  * tensor's shape and alignment allow (default). */
 int conef_set_fast_path(conef_ctx *ctx, int enable);
+/* For tests: has the random-k selection of every tensor above 1024 elements end as it otherwise does
+ * for one tensor and step in 1e8: the window of hash values does not hold the threshold
+ * (CONEF_SELECT_MISS), more elements lie inside it than its list has room for (CONEF_SELECT_FULL), or
+ * the list holds something else (CONEF_SELECT_STALE, which conef_last_status reports as bit 0).
+ * The index sets are the same.  CONEF_SELECT_NORMAL is the default.  Nothing is launched. */
+enum { CONEF_SELECT_NORMAL = 0, CONEF_SELECT_MISS = 1, CONEF_SELECT_FULL = 2, CONEF_SELECT_STALE = 3 };
+int conef_set_select(conef_ctx *ctx, int how);
 /* Low-rank Q, phase 1 (Sec. 5.2; Alg. 2 line 9): on tensors whose shape allows it (rank 4 or 8,
  * cols a multiple of 32 and at least 256, int4 blocks of 128 or int8 blocks of 256) the two
  * halves of phase 1, Q_i = M_i^T P_hat and state = C(p - P_hat Q_i^T), run in ONE persistent
@@ -328,6 +335,12 @@ const char *conef_error_string(int code);
 #define CONEF_NOALLOC_MAX_ELEMS (1 << 24)
 int conef_randk_indices_noalloc(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_t k,
                                 uint32_t *idx_out /* DEVICE */, conef_stream stream);
+/* For tests: the same call ending as `how` says (see conef_set_select), or with the second of its two
+ * kernels left out (CONEF_SELECT_HALF): what a call finds behind it is then what another's kernels
+ * leave that ran between its own. */
+enum { CONEF_SELECT_HALF = 4 };
+int conef_randk_indices_noalloc_select(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_t k,
+                                       int how, uint32_t *idx_out /* DEVICE */, conef_stream stream);
 
 #ifdef __cplusplus
 }

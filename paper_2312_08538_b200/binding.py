@@ -24,13 +24,15 @@ Q_IDENTITY, Q_RANDK, Q_LOWRANK, Q_RANDBLOCK = 0, 1, 2, 3
 C_IDENTITY, C_INT8, C_INT4, C_COUNTSKETCH, C_ROWSKETCH, C_STOCHQUANT = 0, 1, 2, 3, 4, 5
 SCALE_FP32, SCALE_FP16 = 0, 1
 MSG_VALUES, MSG_P, MSG_Q, MSG_DENSE1D = 0, 1, 2, 3
+SELECT_NORMAL, SELECT_MISS, SELECT_FULL, SELECT_STALE, SELECT_HALF = 0, 1, 2, 3, 4
 MAX_WORKERS, MAX_RANK = 64, 8
 
 EXPORTS = ["conef_workspace_bytes", "conef_init", "conef_step", "conef_reduce_messages",
            "conef_decompress_error", "conef_apply_update", "conef_error_reset", "conef_destroy", "conef_message_elems", "conef_error_elems",
            "conef_state_bytes_per_worker", "conef_get_message", "conef_get_state", "conef_get_state2",
            "conef_get_indices", "conef_get_factors", "conef_last_status", "conef_launch_count",
-           "conef_set_fast_path", "conef_set_total_workers", "conef_error_string", "conef_randk_indices_noalloc",
+           "conef_set_fast_path", "conef_set_select", "conef_set_total_workers", "conef_error_string", "conef_randk_indices_noalloc",
+           "conef_randk_indices_noalloc_select",
            "conef_get_error_step", "conef_set_error_step", "conef_set_fused", "conef_fused_info",
            "conef_get_fused_q"]
 
@@ -84,11 +86,13 @@ def _load() -> C.CDLL:
                                     C.POINTER(vp), C.POINTER(i32)]
     L.conef_last_status.argtypes = [vp, vp, C.POINTER(i32)]
     L.conef_set_fast_path.argtypes = [vp, i32]
+    L.conef_set_select.argtypes = [vp, i32]
     L.conef_set_total_workers.argtypes = [vp, i32]
     L.conef_set_fused.argtypes = [vp, i32, i32, i32]
     L.conef_fused_info.argtypes = [vp] + [C.POINTER(i32)] * 5
     L.conef_get_fused_q.argtypes = [vp, i32, i32, C.POINTER(vp)]
     L.conef_randk_indices_noalloc.argtypes = [C.c_uint64, i64, i64, i64, i64, vp, vp]
+    L.conef_randk_indices_noalloc_select.argtypes = [C.c_uint64, i64, i64, i64, i64, i32, vp, vp]
     L.conef_error_string.argtypes = [i32]
     L.conef_error_string.restype = C.c_char_p
     return L
@@ -159,6 +163,14 @@ def conef_randk_indices_noalloc(seed: int, tensor: int, step: int, d: int, k: in
     assert idx_out.is_cuda and idx_out.element_size() == 4 and idx_out.numel() >= k and idx_out.is_contiguous()
     _check(lib.conef_randk_indices_noalloc(int(seed), int(tensor), int(step), int(d), int(k), idx_out.data_ptr(),
                                            _stream_handle(stream)), "conef_randk_indices_noalloc")
+
+
+def conef_randk_indices_noalloc_select(seed: int, tensor: int, step: int, d: int, k: int, how: int, idx_out: torch.Tensor,
+                                       stream=None) -> None:
+    """The same call ending as `how` (SELECT_*) says (tests)."""
+    assert idx_out.is_cuda and idx_out.element_size() == 4 and idx_out.numel() >= k and idx_out.is_contiguous()
+    _check(lib.conef_randk_indices_noalloc_select(int(seed), int(tensor), int(step), int(d), int(k), int(how), idx_out.data_ptr(),
+                                                  _stream_handle(stream)), "conef_randk_indices_noalloc_select")
 
 
 class ConEF:
@@ -263,6 +275,10 @@ class ConEF:
 
     def set_fast_path(self, enable: bool) -> None:
         _check(lib.conef_set_fast_path(self.h, int(enable)), "conef_set_fast_path")
+
+    def set_select(self, how: int) -> None:
+        """How the random-k selection ends (SELECT_*; tests): the index sets are the same."""
+        _check(lib.conef_set_select(self.h, int(how)), "conef_set_select")
 
     def set_fused(self, enable: bool, tile_periods: int = 0, ctas_per_sm: int = 0) -> None:
         """Low-rank phase 1 in one persistent kernel (default on); tile_periods = 0: default tile

@@ -1789,6 +1789,14 @@ int conef_set_fast_path(conef_ctx *ctx, int enable)
     return CONEF_OK;
 }
 
+int conef_set_select(conef_ctx *ctx, int how)
+{
+    if (!ctx || how < CONEF_SELECT_NORMAL || how > CONEF_SELECT_STALE)
+        return CONEF_ERR_INVALID_ARG;
+    ctx->view.sel_how = how;
+    return CONEF_OK;
+}
+
 const char *conef_error_string(int code)
 {
     switch (code) {

@@ -131,7 +131,7 @@ struct DevView {
     const int32_t *pfx_rs;
     int32_t rs_vec_ok;   // this call's gradient pointers allow 16-byte loads
     int32_t fv_tiles;    // tuned fused step: selection tiles per CTA
-    int32_t sel_tiles, sel_pad;   // random-k selection: tiles per CTA
+    int32_t sel_tiles, sel_how;   // random-k selection: tiles per CTA, CONEF_SELECT_*
     // tile -> tensor prefix tables (n_layers + 1 entries each)
     const int32_t *pfx_flat, *pfx_pass, *pfx_p1, *pfx_p2, *pfx_q2, *pfx_hist, *pfx_gs;
     int32_t fast_on;     // the tuned kernels produced this step's pass-2 partials

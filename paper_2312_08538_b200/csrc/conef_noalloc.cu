@@ -41,7 +41,7 @@ struct NaArgs {
     uint32_t *ctr, *cnt;
     uint2 *list;
     uint64_t stream;   // hash stream key of (seed, tensor, step)
-    uint32_t d, k, lo, hi, cap, ntiles;
+    uint32_t d, k, lo, hi, cap, ntiles, how;   // how: CONEF_SELECT_*
     uint64_t scale;
 };
 
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
         const uint32_t exist = j0 >= a.d ? 0u : a.d - j0 >= kNaPer ? (1u << kNaPer) - 1u : (1u << (a.d - j0)) - 1u;
         for (uint32_t m = upto & ~below & exist; m; m &= m - 1) {
             const uint32_t j = j0 + (uint32_t)__ffs(m) - 1u;
-            const uint2 e = make_uint2(hash32(a.stream, j), j);
+            const uint2 e = make_uint2(hash32(a.stream, j), a.how == CONEF_SELECT_STALE ? 0xFFFFFFFFu : j);
             const uint32_t pos = atomicAdd(&s_n, 1u);
             if (pos < (uint32_t)kSelList) {
                 ((uint2 *)S.keys)[pos] = e;
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
         return;
     const uint32_t nlist = s_listed;
     uint32_t total = 0xFFFFFFFFu;
-    if (windowed && nlist <= a.cap)
+    if (windowed && nlist <= a.cap && a.how != CONEF_SELECT_MISS)
         total = select_finish<kNaTile>(S, SelectWindow{a.lo, a.hi, a.d, a.k, a.scale, nullptr}, a.list, nlist, a.cnt, a.ntiles, [](uint32_t) {});
     bool failed = false;
     // no listed element belongs: the members are the elements below the window (lo > 0 then)
@@ -194,10 +194,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32
 std::mutex g_mu;
 uint32_t *g_scratch_ptr[64] = {nullptr};
 
-}  // namespace
-
-extern "C" int conef_randk_indices_noalloc(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_t k,
-                                           uint32_t *idx_out, conef_stream stream)
+int write_indices(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_t k, int how, uint32_t *idx_out, conef_stream stream)
 {
     if (d <= 0 || k <= 0 || k > d || tensor < 0 || step < 0 || !idx_out)
         return CONEF_ERR_INVALID_ARG;
@@ -229,8 +226,27 @@ extern "C" int conef_randk_indices_noalloc(uint64_t seed, int64_t tensor, int64_
     a.d = (uint32_t)d;
     a.k = (uint32_t)k;
     select_window(d, k, a.lo, a.hi, a.cap, a.scale);
+    a.how = (uint32_t)how;
+    if (how == CONEF_SELECT_FULL)
+        a.cap = 1;
     a.ntiles = (uint32_t)((d + kNaTile - 1) / kNaTile);
     k_na_select<<<a.ntiles, kSelThreads, 0, s>>>(a);
-    k_na_write<<<a.ntiles, kSelThreads, 0, s>>>(a, idx_out);
+    if (how != CONEF_SELECT_HALF)
+        k_na_write<<<a.ntiles, kSelThreads, 0, s>>>(a, idx_out);
     return cudaGetLastError() == cudaSuccess ? CONEF_OK : CONEF_ERR_CUDA;
+}
+
+}  // namespace
+
+extern "C" int conef_randk_indices_noalloc(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_t k,
+                                           uint32_t *idx_out, conef_stream stream)
+{
+    return write_indices(seed, tensor, step, d, k, CONEF_SELECT_NORMAL, idx_out, stream);
+}
+extern "C" int conef_randk_indices_noalloc_select(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_t k,
+                                                  int how, uint32_t *idx_out, conef_stream stream)
+{
+    if (how < CONEF_SELECT_NORMAL || how > CONEF_SELECT_HALF)
+        return CONEF_ERR_INVALID_ARG;
+    return write_indices(seed, tensor, step, d, k, how, idx_out, stream);
 }

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
     uint32_t *tileoff = V.tileoff + L.tileoff_off;
     uint16_t *wordoff = V.wordoff + L.wordoff_off;
     const bool windowed = d > (uint32_t)kSelShortTensor;
+    const uint32_t cap = V.sel_how == CONEF_SELECT_FULL ? 1u : L.cand_cap;
 
     S.hist[tid] = 0;   // the bins of select_threshold
     if (tid < 8)
@@ -111,13 +112,13 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
             const uint32_t word = lo ? ~not_below & exist : 0u;
             for (uint32_t m = ~above & ~word & exist; m; m &= m - 1) {   // the few inside the window
                 const uint32_t j = j0 + (uint32_t)__ffs(m) - 1u;
-                const uint2 e = make_uint2(hash32(st, j), j);
+                const uint2 e = make_uint2(hash32(st, j), V.sel_how == CONEF_SELECT_STALE ? 0xFFFFFFFFu : j);
                 const uint32_t pos = atomicAdd(&s_n, 1u);
                 if (pos < (uint32_t)kSelList) {
                     ((uint2 *)S.keys)[pos] = e;
                 } else {   // (not expected: the list of a CTA holds several times the usual number)
                     const uint32_t g = select_claim(ctr, 1u);
-                    if (g < L.cand_cap)
+                    if (g < cap)
                         list[g] = e;
                 }
             }
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
             tileoff[tile0 + tid] = s_cnt[tid];
         __syncthreads();
         for (uint32_t x = tid; x < n; x += kSelThreads)
-            if (s_base + x < L.cand_cap)
+            if (s_base + x < cap)
                 list[s_base + x] = ((uint2 *)S.keys)[x];
     }
     __threadfence();
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
     const uint32_t k = (uint32_t)L.k, nlist = s_listed;
     const SelectWindow W{lo, hi, d, k, L.sel_scale, V.status};
     uint32_t total = 0xFFFFFFFFu;
-    if (windowed && nlist <= L.cand_cap)
+    if (windowed && nlist <= cap && V.sel_how != CONEF_SELECT_MISS)
         total = ntiles <= (uint32_t)kSelTailTiles
                     ? select_finish_short(S, W, list, nlist, bits, tileoff, wordoff, ntiles)
                     : select_finish<kHistTile>(S, W, list, nlist, tileoff, ntiles,

@@ -43,3 +43,38 @@ def test_window_longer_than_shared_memory():
 
 def test_several_tiles_per_cta():
     _check([(5000, 8100), (33, 77), (2, 8192), (1200, 1111)], 1, 1000, steps=(5,))
+
+
+# sizes in tiles of 8192 elements, a selection's, and of 2048, the allocation-free call's: two, the most that
+# the last CTA finishes alone and one more, and beyond the counts it holds in shared memory
+RECOVERY = [(1, 1025), (3, 999), (2, 8192), (16, 8192), (1, 16 * 8192 + 1), (17, 8190), (1281, 2048), (1281, 8192 + 3)]
+
+
+@pytest.mark.parametrize("how", ["MISS", "FULL", "STALE"])
+@pytest.mark.parametrize("k_num,k_den", [(1, 100), (2, 3)])
+def test_selections_whose_window_fails(how, k_num, k_den):
+    """A window without the threshold, a list without room and a list that holds something else end in the
+    same index sets, messages and stored errors; only the last is reported."""
+    from paper_2312_08538_b200 import binding as b
+    seed, code = 41, getattr(b, "SELECT_" + how)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    g = [torch.randn(sum(r * c for r, c in RECOVERY), device="cuda", generator=gen)]
+    outs = []
+    for x in (b.SELECT_NORMAL, code):
+        eng = b.ConEF([(r, c, 1) for r, c in RECOVERY], 1, dict(kind="randk", k_num=k_num, k_den=k_den, seed=seed),
+                      dict(kind="int8", block=256), 0.1)
+        eng.set_select(x)
+        for t in (0, 1):   # (the second on what the first left in the bitmap and the counters)
+            msg = eng.full_step(t, g)[b.MSG_VALUES]
+        outs.append([msg, eng.decompress_error(0)] + [eng.indices(l).clone() for l in range(len(RECOVERY))])
+        assert eng.last_status() == (1 if x == b.SELECT_STALE else 0)
+    for u, v in zip(*outs):
+        assert torch.equal(u, v)
+    for l, (r, c) in enumerate(RECOVERY):
+        d, k = r * c, max(1, r * c * k_num // k_den)
+        want = orc.randk_indices(seed, l, 1, d, k)
+        assert np.array_equal(outs[1][2 + l].cpu().numpy().view(np.uint32), want), (r, c)
+        out = torch.empty(k, dtype=torch.int32, device="cuda")
+        b.conef_randk_indices_noalloc_select(seed, l, 1, d, k, code, out)
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), want), (r, c)

@@ -82,5 +82,7 @@ def test_init_rejects_bad_workspaces_on_the_host(b):
     assert b.lib.conef_step(None, 0, None, 0, None) == b.ERR_INVALID_ARG
     assert b.lib.conef_reduce_messages(None, 0, None, None) == b.ERR_INVALID_ARG
     assert b.lib.conef_decompress_error(None, 0, None, None) == b.ERR_INVALID_ARG
+    assert b.lib.conef_set_select(None, b.SELECT_NORMAL) == b.ERR_INVALID_ARG
+    assert b.lib.conef_randk_indices_noalloc_select(1, 0, 0, 10, 1, 5, 256, None) == b.ERR_INVALID_ARG
     assert b.lib.conef_message_elems(None, 0) == -1
     assert b.lib.conef_error_string(b.ERR_BAD_PHASE).decode().startswith("calls out of order")

@@ -65,3 +65,18 @@ def test_noalloc_rejects_what_its_fixed_scratch_cannot_hold():
     from oracle import conef_oracle as orc
     assert np.array_equal(idx, orc.randk_indices(7, 2, 5, d, k))      # (the failure mark 0xFFFFFFFF would show here)
     assert int(out[k].item()) == -1, "nothing is written past the k entries"
+
+
+def test_a_call_between_another_calls_kernels():
+    """Its threshold is not found (its CTAs are counted on top of the other call's), so it marks its output and
+    writes nothing else; the call after it is right again."""
+    from paper_2312_08538_b200 import binding as b
+    from oracle import conef_oracle as orc
+    d, k = 70000, 700
+    out = torch.full((k,), -2, dtype=torch.int32, device="cuda")
+    big = torch.empty(16, dtype=torch.int32, device="cuda")
+    b.conef_randk_indices_noalloc_select(3, 0, 1, b.NOALLOC_MAX_ELEMS, 16, b.SELECT_HALF, big)
+    b.conef_randk_indices_noalloc(9, 4, 1, d, k, out)
+    assert out[0].item() == -1 and bool((out[1:] == -2).all())
+    b.conef_randk_indices_noalloc(9, 4, 1, d, k, out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), orc.randk_indices(9, 4, 1, d, k))

@@ -91,8 +91,8 @@ struct Plan {
     size_t csk_smem = 0;        // ... with this much shared memory per CTA (two windows of the widest run)
     std::vector<int> il_groups; // count sketch, workers interleaved: first tensor of every group, then n_tensors
     bool il_direct = true;      // ... or each on its own state
+    bool il_second = false;     // ... and whether the result is left in the second sketch
     std::vector<int64_t> il_fill;   // ... the records of every group
-    int64_t il_records = 0;     // ... and of the largest
     int64_t msg_elems[4] = {0, 0, 0, 0};
     int64_t err_elems = 0;
     int64_t state_stride = 0;  // bytes per worker
@@ -105,7 +105,7 @@ struct Plan {
     // byte offsets in the workspace
     size_t off_layers = 0, off_pfx = 0, off_status = 0, off_sel = 0, off_idx = 0, off_wordoff = 0, off_tileoff = 0, off_selbits = 0,
            off_pbar = 0, off_phat = 0, off_qprev = 0, off_state = 0, off_state_new = 0,
-           off_msgv = 0, off_msgp = 0, off_msgq = 0, off_msg1d = 0, off_part = 0, off_ppart = 0, off_rs = 0, off_cand = 0, off_il = 0,
+           off_msgv = 0, off_msgp = 0, off_msgq = 0, off_msg1d = 0, off_part = 0, off_ppart = 0, off_rs = 0, off_cand = 0,
            off_ev[2] = {0, 0}, off_wordoff2[2] = {0, 0}, off_tileoff2[2] = {0, 0}, off_selbits2[2] = {0, 0},   // iConEF-v2
            off_fu_units = 0, off_fu_groups = 0, off_fu_hint = 0, off_fu_ctr = 0, off_fu_scratch = 0, off_fu_q = 0,   // fused passes 2 + 3
            total = 0;
@@ -325,7 +325,6 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 }
                 L.sk_off = il_fill;
                 P.il_fill.back() = il_fill += rec;
-                P.il_records = std::max(P.il_records, il_fill);
             }
             if (q->kind != CONEF_Q_LOWRANK) {
                 L.msgv_off = P.msg_elems[CONEF_MSG_VALUES];
@@ -491,8 +490,10 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     if (!P.il_groups.empty())
         P.il_groups.push_back(n_tensors);
     P.il_direct = il_width(n_workers) == 1 || P.err_elems * n_workers < kIlDirect;
-    if (!P.il_direct)   // the old and the new records of one group
-        P.off_il = take((size_t)P.il_records * 4 * il_width(n_workers) * 2);
+    for (int64_t rec : P.il_fill)   // (slices of records are counted in 32 bits)
+        if (il_at_once(n_workers, rec, P.state_stride * n_workers) == 0 && rec > 0xFFFFFF00LL)
+            P.il_direct = true;
+    P.il_second = !P.il_direct && P.il_fill.size() == 1 && il_second(n_workers, P.il_fill[0], P.state_stride * n_workers);
     if (c->iconef == 2)   // two value buffers per worker and the structures of two more draws of Q
         for (int x = 0; x < 2; ++x) {
             P.off_ev[x] = take((size_t)P.msg_stride[CONEF_MSG_VALUES] * 4 * n_workers);
@@ -733,22 +734,21 @@ int launch_flat(conef_ctx *ctx, DevView V, cudaStream_t s, int table = T_FLAT)
     return CONEF_OK;
 }
 
-// the step on a whole-tensor count sketch, all workers together (conef_ilsketch.cuh)
-template <int QK>
+// the step on a whole-tensor count sketch, all workers together (conef_ilsketch.cuh), in the memory of the second sketch
 int launch_il(conef_ctx *ctx, const DevView &V, cudaStream_t s)
 {
     const Plan &P = ctx->plan;
     const int32_t *pfx = table_ptr(ctx, T_IL), *epfx = table_ptr(ctx, T_ILT);
-    float *records = (float *)(ctx->ws + P.off_il);
     if (P.il_direct) {
-        il_launch_direct<QK>(V, pfx, tiles_of(ctx, T_IL), s);
-        LAUNCH_CHECK(ctx);
+        ctx->launches += il_launch_direct(ctx->q.kind, V, pfx, tiles_of(ctx, T_IL), s);
+        CK_CUDA(cudaGetLastError());
         return CONEF_OK;
     }
     for (size_t k = 0; k + 1 < P.il_groups.size(); ++k) {
         const int l0 = P.il_groups[k], l1 = P.il_groups[k + 1];
         const int e0 = P.pfx[T_IL][l0], en = P.pfx[T_IL][l1] - e0, t0 = P.pfx[T_ILT][l0], tn = P.pfx[T_ILT][l1] - t0;
-        ctx->launches += il_launch<QK>(V, pfx, e0, en, epfx, t0, tn, P.il_fill[k], records, s);
+        ctx->launches += il_launch(ctx->q.kind, V, pfx, e0, en, epfx, t0, tn, P.il_fill[k], (float *)V.state_new,
+                                   P.state_stride * ctx->n_workers, P.il_second, s);
         CK_CUDA(cudaGetLastError());
     }
     return CONEF_OK;
@@ -859,14 +859,14 @@ template <class F>
 int with_new_sketch(conef_ctx *ctx, const DevView &V, cudaStream_t s, F body)
 {
     const bool sk = ctx->c.kind == CONEF_C_COUNTSKETCH || ctx->c.kind == CONEF_C_ROWSKETCH;
-    // built by atomic adds; the row sketch, the run-by-run step where it takes every tensor, and the
-    // step on interleaved workers write every entry themselves
+    // built by atomic adds; the row sketch and the run-by-run step where it takes every tensor write every
+    // entry themselves; the step on interleaved workers mostly leaves its result where the old sketch was
     const bool all_csk = ctx->fast && ctx->plan.any_csk && tiles_of(ctx, T_NOFV) == 0 && ctx->q.kind != CONEF_Q_LOWRANK;
     const bool all_il = ctx->fast && tiles_of(ctx, T_IL) > 0 && !ctx->plan.il_direct;
     if (ctx->c.kind == CONEF_C_COUNTSKETCH && !all_csk && !all_il)
         CK_CUDA(cudaMemsetAsync(V.state_new, 0, (size_t)ctx->plan.state_stride * ctx->n_workers, s));
     int rc = body();
-    if (rc == CONEF_OK && sk)
+    if (rc == CONEF_OK && sk && (!all_il || ctx->plan.il_second))
         ctx->sketch_cur ^= 1;
     return rc;
 }
@@ -1270,7 +1270,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             return CONEF_OK;
         }
         if (ctx->fast && tiles_of(ctx, T_IL) > 0)
-            return launch_il<QK>(ctx, V, s);
+            return launch_il(ctx, V, s);
         if (!fv && !csk)
             return launch_flat<QK>(ctx, V, s);
         if (fv) {

@@ -10,13 +10,20 @@
 // four workers and a pair of lanes' for eight (the two 16-byte accesses of a pair make one request).
 //
 // The state stays one contiguous sketch per worker: a group of tensors is interleaved into a scratch
-// (k_sketch_swap, which also clears the new sketch), stepped, and written back.  Groups are as many
-// tensors as keep the scratch inside L2, or one larger tensor.
+// (k_sketch_swap, which also clears the new sketch), stepped, and written back to where it was.  Groups
+// are as many tensors as keep the scratch inside L2, or one larger tensor.  The scratch is the memory of
+// the second sketch, which one worker at a time needs and this does not.  Where the old and the new
+// records of a group do not fit it together (a group with more than half of a model), the workers go in
+// batches of eight where that is enough; else the states themselves lend the other half (IlForm), at
+// the price of one or two more passes over the sketch.
 //
 // Transformer-big list (210 M elements), 5 x d/10 buckets, eight workers: 90 ms per step one worker at a
 // time, 25.3 ms now, of which interleaving takes 3.3; the requests still bound it, ten per element.
 // Three CTAs per SM (80 registers); with four (spills) 24.8 ms instead of 23.0 for k_sketch_il.
 #pragma once
+#include <algorithm>
+#include <type_traits>
+
 #include "conef_common.cuh"
 
 namespace conef {
@@ -35,11 +42,55 @@ constexpr int64_t kIlGroupBytes = 40ll << 20;
 constexpr int64_t kIlTogether = 100ll << 20;
 // Below this many elements over all workers the two kernels that interleave cost more than they save.
 constexpr int64_t kIlDirect = 1ll << 20;
-// workers per bucket record: 1, 2, 4 or a multiple of 8
-__host__ __device__ inline int il_width(int n_workers)
+// workers of a batch, and of a whole bucket record: 1, 2, 4 or a multiple of 8
+inline int il_batch(int n_workers) { return n_workers <= 1 ? 1 : n_workers <= 2 ? 2 : n_workers <= 4 ? 4 : 8; }
+inline int il_width(int n_workers) { return (n_workers + il_batch(n_workers) - 1) / il_batch(n_workers) * il_batch(n_workers); }
+// Batches stepped together in a scratch of `bytes`; 0: one batch of 8, 4, 2 or 1 workers at a time, with
+// records in the states too.
+inline int il_at_once(int n_workers, int64_t n_records, int64_t bytes)
 {
-    return n_workers <= 1 ? 1 : n_workers <= 2 ? 2 : n_workers <= 4 ? 4 : (n_workers + 7) / 8 * 8;
+    return (int)std::min<int64_t>(il_width(n_workers) / il_batch(n_workers), bytes / (n_records * 8 * il_batch(n_workers)));
 }
+
+// Whether a group that is the whole model ends in the second sketch (SPLIT, all workers in one batch)
+inline bool il_second(int n_workers, int64_t n_records, int64_t bytes)
+{
+    return il_at_once(n_workers, n_records, bytes) == 0 && (n_workers == 2 || n_workers == 4 || n_workers == 8) &&
+           n_records * 8 * n_workers <= kIlTogether;
+}
+// Where the records are:
+//   SCRATCH  all in the scratch, next to one another or apart (kIlTogether)
+//   SPLIT    old ones in the scratch, new ones in the place of the states; for groups inside L2
+//   FOLD     a tensor beyond L2, old next to new: the first half of the entries in the scratch, the second in
+//            the place of the states.  On the way in and out a record of the scratch carries the entry of
+//            the second half in the slot that is not in use, which frees the states.
+// 5 x d/10 buckets of one 8192 x 8192 matrix: two, four, eight workers 16.2, 17.5, 17.6 ms with room for all
+// records, 19.4, 23.1, 27.0 under SPLIT, 16.9, 18.4, 18.0 under FOLD.  Three and five workers go as 2 + 1 and
+// 4 + 1 (30.5 and 32.0 ms) where records of four and eight fit and take 17.4 with room for them: no
+// form holds more records than two sketches per worker have room for.
+enum IlForm { IL_SCRATCH, IL_SPLIT, IL_FOLD };
+
+// Where record e (of F floats) of a batch lies among its states: in slice e / (c / F) of the c floats (a
+// multiple of 64) of each, counted from the first
+struct IlSlices {
+    uint32_t per, magic;   // records per slice
+    int64_t stride;        // floats from state to state
+    __device__ __forceinline__ IlSlices(uint32_t n, uint32_t F, int64_t state_stride)
+    {
+        per = (n + 63u) / 64u * (64u / F);
+        magic = 0xFFFFFFFFu / per;
+        stride = state_stride / 4;
+    }
+    __device__ __forceinline__ int64_t at(uint32_t e, uint32_t F) const
+    {
+        uint32_t q = __umulhi(e, magic), r = e - q * per;   // e / per or one less
+        if (r >= per) {
+            r -= per;
+            ++q;
+        }
+        return q * stride + (int64_t)r * F;
+    }
+};
 
 template <int W>
 struct IlVec {
@@ -75,11 +126,12 @@ __device__ __forceinline__ void il_add(float *p, const IlVec<W> &a)
 // The old values of a sketch entry are `stride` floats apart from entry to entry, groups of GW = W * LP
 // workers (blockIdx.y) follow one another within an entry; the new values lie newoff floats after the old.
 //
-// VR sketch rows (0: V.cs_rows, up to 7); W workers per lane, LP lanes per element.  GW = 1: no records,
-// the states themselves.
-template <int QK, int VR, int W, int LP>
+// VR sketch rows (0: V.cs_rows, up to 7); W workers per lane, LP lanes per element, the first of them
+// worker0.  GW = 1 in SCRATCH form: no records, the states themselves.
+template <int QK, int VR, int W, int LP, int FORM>
 __global__ void __launch_bounds__(kIlThreads, W == 4 ? 3 : 4)
-k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, int first, float *records, uint32_t stride, int64_t newoff)
+k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, int first, int worker0, float *records, uint32_t stride,
+            int64_t newoff)
 {
     constexpr int VM = VR ? VR : 7, GW = W * LP;
     const int v = VR ? VR : V.cs_rows;
@@ -90,12 +142,17 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
     const uint32_t j0 = (uint32_t)(tile - pfx[li]) * (uint32_t)kIlTile;
     const uint32_t left = min(d - j0, (uint32_t)kIlTile);   // elements of this tile
     const int sub = threadIdx.x & (LP - 1);
-    const int w0 = blockIdx.y * GW + sub * W;               // this lane's first worker
+    const int w0 = worker0 + blockIdx.y * GW + sub * W;     // this lane's first worker
     if (GW == 1)
         stride = 1u;
     const float *So;
     float *Sn;
-    if (GW == 1) {
+    const IlSlices slices((uint32_t)(FORM != IL_SCRATCH ? v * w : 1u), FORM == IL_FOLD ? 2 * GW : GW, V.state_stride);
+    const uint32_t half = ((uint32_t)v * w + 1u) / 2u;   // FOLD: entries in the scratch
+    if (FORM != IL_SCRATCH) {
+        So = records + L.sk_off * stride + sub * W;
+        Sn = (float *)(V.state + worker0 * V.state_stride + L.a_off) + sub * W;
+    } else if (GW == 1) {
         So = (const float *)(V.state + w0 * V.state_stride + L.a_off);
         Sn = (float *)(V.state_new + w0 * V.state_stride + L.a_off);
     } else {
@@ -125,7 +182,11 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
                 const uint64_t u = h64(keys[i], j);
                 bk[i] = (uint32_t)(((u >> 32) * (uint64_t)w) >> 32);
                 sign |= (uint32_t)(u & 1) << i;
-                rec[i] = il_load<W>(So + ((uint64_t)i * w + bk[i]) * stride);
+                const uint32_t e = (uint32_t)i * w + bk[i];
+                if (FORM == IL_FOLD)
+                    rec[i] = il_load<W>(e < half ? So + (uint64_t)e * (2 * GW) : Sn + slices.at(e - half, 2 * GW));
+                else
+                    rec[i] = il_load<W>(So + ((uint64_t)i * w + bk[i]) * stride);
             }
         }
         float gv[W];
@@ -173,30 +234,40 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
 #pragma unroll
                     for (int x = 0; x < W; ++x)
                         a.v[x] = __uint_as_float(__float_as_uint(val.v[x]) ^ (((sign >> i) & 1u) << 31));
-                    il_add<W>(Sn + ((uint64_t)i * w + bk[i]) * stride, a);
+                    const uint32_t e = (uint32_t)i * w + bk[i];
+                    if (FORM == IL_FOLD)
+                        il_add<W>((e < half ? records + sub * W + (uint64_t)e * (2 * GW) : Sn + slices.at(e - half, 2 * GW)) + GW, a);
+                    else if (FORM == IL_SPLIT && GW > 1)
+                        il_add<W>(Sn + slices.at(e, GW), a);
+                    else
+                        il_add<W>(Sn + ((uint64_t)i * w + bk[i]) * stride, a);
                 }
         }
     }
 }
 
-// IN: states -> old values of the records, new ones cleared; else: new values -> states.  A thread has one
-// entry of all GW workers (coalesced over the entries of a worker); the records, exchanged through
-// shared memory, are accessed 16 bytes per lane over contiguous memory.
-template <int GW, bool IN>
+// IN: states -> old values of the records, and the new ones cleared (SPLIT: the states, whose place they
+// take); else: new values -> states (SPLIT: from their slices to one sketch after the other in `records`, or
+// to the second sketch, padding included, with newoff < 0).  A thread has one entry of all GW workers (coalesced over the entries of a worker); the records,
+// exchanged through shared memory, are accessed 16 bytes per lane over contiguous memory.
+template <int GW, bool IN, bool SPLIT>
 __global__ void __launch_bounds__(kIlThreads) k_sketch_swap(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
-                                                            int first, float *__restrict__ records, uint32_t stride, int64_t newoff)
+                                                            int first, int worker0, float *__restrict__ records, uint32_t stride,
+                                                            int64_t newoff)
 {
-    constexpr int PW = GW == 2 ? 2 : 4, H = GW / PW;   // floats per piece, pieces of a record's old (or new) values
+    constexpr int PW = GW < 4 ? GW : 4, H = GW / PW;   // floats per piece, pieces of a record's old (or new) values
     constexpr int PITCH = GW == 8 ? 9 : GW;            // (entries of a warp in different banks)
-    using Piece = typename std::conditional<PW == 2, float2, float4>::type;
+    using Piece = typename std::conditional<PW == 1, float, typename std::conditional<PW == 2, float2, float4>::type>::type;
     __shared__ float buf[kIlThreads * PITCH];
     const int tile = first + (int)blockIdx.x;
     const int li = find_layer(pfx, V.n_layers, tile);
     const LayerDesc &L = V.layers[li];
     const int64_t n = (int64_t)V.cs_rows * L.w;
     const int64_t e0 = (int64_t)(tile - pfx[li]) * kIlEntries;
-    const int w0 = blockIdx.y * GW, t = threadIdx.x;
-    uint8_t *base = IN ? V.state : V.state_new;
+    const int w0 = worker0 + blockIdx.y * GW, t = threadIdx.x;
+    float *const states = (float *)(V.state + w0 * V.state_stride + L.a_off);
+    const int64_t pitch = V.state_stride / 4;
+    const IlSlices slices((uint32_t)(SPLIT ? n : 1), GW, V.state_stride);
     for (int q = 0; q < kIlEntries / kIlThreads; ++q) {
         const int64_t b = e0 + q * kIlThreads, e = b + t;
         if (b >= n)
@@ -206,8 +277,12 @@ __global__ void __launch_bounds__(kIlThreads) k_sketch_swap(const __grid_constan
         float r[GW];
         if (IN) {
 #pragma unroll
-            for (int x = 0; x < GW; ++x)
-                r[x] = t < have && w0 + x < V.n_workers ? __ldcs((const float *)(base + (int64_t)(w0 + x) * V.state_stride + L.a_off) + e) : 0.f;
+            for (int x = 0; x < GW; ++x) {
+                const bool in = t < have && w0 + x < V.n_workers;
+                r[x] = in ? __ldcs(states + x * pitch + e) : 0.f;
+                if (SPLIT && in)
+                    states[x * pitch + e] = 0.f;
+            }
         }
         if (q)
             __syncthreads();
@@ -229,12 +304,14 @@ __global__ void __launch_bounds__(kIlThreads) k_sketch_swap(const __grid_constan
                     for (int x = 0; x < PW; ++x)
                         zf[x] = p[x];
                     *(Piece *)at = z;
+                    if (!SPLIT) {
 #pragma unroll
-                    for (int x = 0; x < PW; ++x)
-                        zf[x] = 0.f;
-                    *(Piece *)(at + newoff) = z;
+                        for (int x = 0; x < PW; ++x)
+                            zf[x] = 0.f;
+                        *(Piece *)(at + newoff) = z;
+                    }
                 } else {
-                    z = *(const Piece *)(at + newoff);
+                    z = *(const Piece *)(SPLIT ? states + slices.at((uint32_t)(b + en), GW) + part * PW : at + newoff);
 #pragma unroll
                     for (int x = 0; x < PW; ++x)
                         p[x] = zf[x];
@@ -246,54 +323,27 @@ __global__ void __launch_bounds__(kIlThreads) k_sketch_swap(const __grid_constan
             if (t < have) {
 #pragma unroll
                 for (int x = 0; x < GW; ++x)
-                    if (w0 + x < V.n_workers)
-                        __stcs((float *)(base + (int64_t)(w0 + x) * V.state_stride + L.a_off) + e, buf[t * PITCH + x]);
+                    if (SPLIT && newoff < 0)
+                        ((float *)(V.state_new + (w0 + x) * V.state_stride + L.a_off))[e] = buf[t * PITCH + x];
+                    else if (SPLIT)
+                        records[x * newoff + L.sk_off + e] = buf[t * PITCH + x];
+                    else if (w0 + x < V.n_workers)
+                        __stcs(states + x * pitch + e, buf[t * PITCH + x]);
+            } else if (SPLIT && newoff < 0 && e < (n + 63) / 64 * 64) {
+#pragma unroll
+                for (int x = 0; x < GW; ++x)
+                    ((float *)(V.state_new + (w0 + x) * V.state_stride + L.a_off))[e] = 0.f;
             }
         }
     }
 }
 
-template <int QK, int W, int LP>
-inline void il_step(const DevView &V, const int32_t *pfx, int first, int tiles, int groups, float *records, uint32_t stride, int64_t newoff, cudaStream_t s)
-{
-    const dim3 grid(tiles, groups);
-    if (V.cs_rows == 5)
-        k_sketch_il<QK, 5, W, LP><<<grid, kIlThreads, 0, s>>>(V, pfx, first, records, stride, newoff);
-    else if (V.cs_rows == 3)
-        k_sketch_il<QK, 3, W, LP><<<grid, kIlThreads, 0, s>>>(V, pfx, first, records, stride, newoff);
-    else
-        k_sketch_il<QK, 0, W, LP><<<grid, kIlThreads, 0, s>>>(V, pfx, first, records, stride, newoff);
-}
-// the step on the states themselves, one worker per blockIdx.y, all tensors
-template <int QK>
-inline void il_launch_direct(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
-{
-    il_step<QK, 1, 1>(V, pfx, 0, tiles, V.n_workers, nullptr, 1, 0, s);
-}
-// the step of a group of tensors: tiles [first, first + tiles) of elements, [efirst, efirst + etiles) of
-// sketch entries.  Returns the number of kernels launched.
-template <int QK>
-inline int il_launch(const DevView &V, const int32_t *pfx, int first, int tiles, const int32_t *epfx, int efirst, int etiles,
-                     int64_t n_records, float *records, cudaStream_t s)
-{
-    const int NW = il_width(V.n_workers);
-    const bool together = n_records * 8 * NW > kIlTogether;
-    const uint32_t stride = (uint32_t)(together ? 2 * NW : NW);
-    const int64_t newoff = together ? std::min(NW, 8) : n_records * NW;
-#define CONEF_IL_CASE(W, LP)                                                                                        \
-    {                                                                                                               \
-        const int groups = NW / (W * LP);                                                                           \
-        k_sketch_swap<W * LP, true><<<dim3(etiles, groups), kIlThreads, 0, s>>>(V, epfx, efirst, records, stride, newoff);          \
-        il_step<QK, W, LP>(V, pfx, first, tiles, groups, records, stride, newoff, s);                                               \
-        k_sketch_swap<W * LP, false><<<dim3(etiles, groups), kIlThreads, 0, s>>>(V, epfx, efirst, records, stride, newoff);         \
-        return 3;                                                                                                   \
-    }
-    if (NW == 2)
-        CONEF_IL_CASE(2, 1)
-    if (NW == 4)
-        CONEF_IL_CASE(4, 1)
-    CONEF_IL_CASE(4, 2)
-#undef CONEF_IL_CASE
-}
+// launchers (conef_ilsketch.cu), each of which returns the number of kernels launched: the step on the states themselves,
+// one worker per blockIdx.y, all tensors; and the step of a group of n_records records: tiles [first, first + tiles) of
+// elements, [efirst, efirst + etiles) of sketch entries, in a scratch of `bytes`; second: the result of a group that
+// il_second accepts is left in V.state_new.
+int il_launch_direct(int qkind, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s);
+int il_launch(int qkind, const DevView &V, const int32_t *pfx, int first, int tiles, const int32_t *epfx, int efirst, int etiles,
+              int64_t n_records, float *records, int64_t bytes, bool second, cudaStream_t s);
 
 }  // namespace conef

@@ -68,6 +68,16 @@ def test_state_sizes_match_the_memory_saving_arithmetic(b):
     assert dense - small == pytest.approx(d * 4 - d * (0.5 + 2 / 128), abs=4096)
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 9, 64])
+@pytest.mark.parametrize("tensors", [[(8192, 8192, 1)], [(4096, 4096, 1), (4096, 4096, 1), (4096, 1, 0), (999, 4096, 1)], [(1024, 4096, 1)] * 60])
+def test_the_count_sketch_takes_two_sketches_per_worker_and_no_scratch_of_its_own(b, tensors, n):
+    got = b.conef_workspace_bytes(tensors, n, dict(kind="randblock", k_num=1, k_den=100), dict(kind="countsketch", cs_rows=5, cs_col_div=10))
+    sketch = sum(4 * 5 * (r * c // 10) for r, c, k in tensors if k)
+    messages = sum(4 * (r * c // 100) if k else 4 * r * c for r, c, k in tensors)
+    indices = sum(4 * (r * c // 100) for r, c, k in tensors if k)
+    assert got <= n * (2 * sketch + messages) + indices + 256 * (4 * n + 20) * len(tensors) + 65536
+
+
 def test_init_rejects_bad_workspaces_on_the_host(b):
     t = b.make_tensors([(8, 8, 1)])
     q = b.make_q(dict(kind="randk", k_num=1, k_den=2, seed=1), None)

@@ -11,14 +11,14 @@ static void launch(int pass, int unit, const DevView &V, const int32_t *pfx, int
         k_gen_pass<1, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
     else if (pass == 2)
         k_gen_pass<2, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else if (unit == 32)
-        k_gen_pass<3, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else if (unit == 64)
-        k_gen_pass<3, CK, R, 2><<<grid, kGenThreads, 0, s>>>(V, pfx);
+    else if (unit == 256)
+        k_gen_pass<3, CK, R, 8><<<grid, kGenThreads, 0, s>>>(V, pfx);
     else if (unit == 128)
         k_gen_pass<3, CK, R, 4><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else
-        k_gen_pass<3, CK, R, 8><<<grid, kGenThreads, 0, s>>>(V, pfx);
+    else if (CK == CONEF_C_INT4 || unit == 64)   // (int4 blocks are 64 or more)
+        k_gen_pass<3, CK, R, 2><<<grid, kGenThreads, 0, s>>>(V, pfx);
+    else if constexpr (CK == CONEF_C_INT8)
+        k_gen_pass<3, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
 }
 
 cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)

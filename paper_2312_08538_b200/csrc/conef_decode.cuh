@@ -15,7 +15,9 @@ constexpr int kDecThreads = 256;
 constexpr int kDecBatch = 4;
 __host__ __device__ constexpr int dec_tile(int batch) { return kDecThreads * 4 * batch; }   // elements per CTA
 constexpr int kDecTile = dec_tile(kDecBatch);
-// Below about four CTAs of the large kind per SM a launch takes the time of its slowest CTA, not of its bytes.
+// Below about four CTAs of the large kind per SM a launch takes the time of its slowest CTA, not of its bytes:
+// one worker, int8, one vector and four vectors per thread, captured calls: 32 k elements 1.56, 1.85 us; 0.5 M
+// 1.93, 2.30; 1 M 2.38, 2.38; 2 M 3.03, 3.36 (int4 the same within 0.2).
 inline int dec_batch(int64_t elements) { return elements < (int64_t)dec_tile(kDecBatch) * kPlanSMs * 4 ? 1 : kDecBatch; }
 
 // four codes, element 0 in the low bits, times the scale; each product is rounded once

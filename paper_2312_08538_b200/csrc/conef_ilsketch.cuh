@@ -40,8 +40,10 @@ constexpr int64_t kIlGroupBytes = 40ll << 20;
 // workers, Transformer-big: 25.0 ms with this line, 26.8 always side by side, 28.0 always apart; four
 // workers, 16 M elements in L2: 476 us apart, 728 side by side.
 constexpr int64_t kIlTogether = 100ll << 20;
-// Below this many elements over all workers the two kernels that interleave cost more than they save.
-constexpr int64_t kIlDirect = 1ll << 20;
+// Below this many elements over all workers the two kernels that interleave cost more than they save: 5 x d/10
+// buckets, steps on the states and on records, two, four and eight workers: 256 k elements 29.7, 27.7, 27.7 and
+// 32.8, 30.8, 36.5 us; 512 k 45.4, 42.0, 40.0 and 40.9, 32.8, 38.7; 1 M 66.0, 63.5, 60.6 and 53.4, 42.3, 41.0.
+constexpr int64_t kIlDirect = 3ll << 17;
 // workers of a batch, and of a whole bucket record: 1, 2, 4 or a multiple of 8
 inline int il_batch(int n_workers) { return n_workers <= 1 ? 1 : n_workers <= 2 ? 2 : n_workers <= 4 ? 4 : 8; }
 inline int il_width(int n_workers) { return (n_workers + il_batch(n_workers) - 1) / il_batch(n_workers) * il_batch(n_workers); }

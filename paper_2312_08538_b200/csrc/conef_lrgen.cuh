@@ -35,7 +35,10 @@ constexpr int kGenCtas = kPlanSMs * 6;   // CTAs a pass should have at least, wh
 struct GenPlan {
     int nr = 4, it = 16;
 };
-// rows: matrix rows of all workers, chunks: 256-element chunks
+// rows: matrix rows of all workers, chunks: 256-element chunks.  Four rows share a row of Q, one row makes four
+// times the warps.  Steps with one and with four rows per warp, int4, rank 2: 3000 x 651 69.1 and 73.0 us,
+// 13000 x 651 91.3 and 92.5, 4001 x 6003 173 and 291; four matrices 40000 x 47 139 and 113, of four workers 444
+// and 323; 60000 x 333 of four workers 577 and 540.
 inline GenPlan gen_plan(int64_t rows, int64_t chunks)
 {
     GenPlan G;

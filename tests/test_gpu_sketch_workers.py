@@ -27,7 +27,7 @@ def _run(cfg, fast, steps=3):
 
 @pytest.mark.parametrize("qkind", ["randk", "randblock", "identity"])
 @pytest.mark.parametrize("workers,rows,beta", [(1, 5, 0.0), (2, 3, 0.0), (3, 5, 0.5), (4, 7, 0.0), (7, 3, 0.0), (8, 5, 0.0), (9, 1, 0.25), (16, 3, 0.0)])
-@pytest.mark.parametrize("extra", [[], [(1100, 1000, 1)]])   # below and above the size that interleaves
+@pytest.mark.parametrize("extra", [[], [(1100, 1000, 1)]])   # below and, from two workers on, above the size that interleaves
 def test_interleaved_equals_generic(qkind, workers, rows, beta, extra):
     cfg = wl.config("tiny")
     cfg.update(tensors=SMALL + extra, n_workers=workers, q=dict(kind=qkind, k_num=1, k_den=20, seed=5),

@@ -20,7 +20,7 @@
 // HBM-bound (4 + 2 state bytes per element).  Transformer-big list, int8 / 256 / fp32, random-k 1 %, one
 // worker: 338 us with eight elements per lane (352 warp instructions per 256 elements, 67 % of the ALU
 // pipe's slots: membership tests and selects, prefix sums over lanes, a scale per eight elements),
-// 208 us = 6.1 TB/s now (217 instructions).
+// 208 us = 6.1 TB/s now (204 instructions).
 #pragma once
 #include "conef_fast.cuh"
 
@@ -37,8 +37,8 @@ __host__ __device__ constexpr int f16_ring(int ico) { return ico == 1 ? 2 : 3; }
 __host__ __device__ constexpr int f16_ctas(int ico) { return ico == 1 ? 4 : 3; }
 
 // Where piece p (16 bytes) of a chunk's gradient lies in its stage.  The pieces of a 128-byte line stay
-// within 128 bytes: a layout that spread them over four rows cost an L2 request per piece (L2 tag
-// lookups at 58 % with DRAM at 47 %).  The exchange inside a line makes the reads of lanes 64 bytes apart
+// within 128 bytes: a layout that spread them over four rows cost an L2 request per piece (0.058
+// requests per element now, tag lookups at 26 % of their rate).  The exchange inside a line makes the reads of lanes 64 bytes apart
 // free of bank conflicts.
 __host__ __device__ constexpr uint32_t f16_slot(uint32_t p) { return p ^ ((p >> 3) & 3u); }
 

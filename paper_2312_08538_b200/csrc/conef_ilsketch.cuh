@@ -3,11 +3,12 @@
 //
 // Every element reads v buckets of the old sketch and adds to the same v buckets of the new one, at
 // random places of arrays that do not fit an SM.  The buckets depend on the element only, not on the
-// worker.  What bounds the step is the number of requests that cross from the SMs to L2 (83 % of the
-// peak rate with one worker at a time, L2 tag lookups 76 %, DRAM 3 %), so the workers of a context are
-// handled together: their sketches are interleaved, workers innermost, and one request of up to 32
-// bytes reads, and one adds to, the bucket of up to eight workers.  An element is one lane's for up to
-// four workers and a pair of lanes' for eight (the two 16-byte accesses of a pair make one request).
+// worker.  What bounds the step is the number of random requests, ten per element: to L2 where a group of
+// tensors fits it, to DRAM beyond (about 64 bytes each).  Their rate hardly depends on their width, so
+// the workers of a context are handled together: their sketches are interleaved, workers innermost, and
+// one request of up to 32 bytes reads, and one adds to, the bucket of up to eight workers.  An element is
+// one lane's for up to four workers and a pair of lanes' for eight (the two 16-byte accesses of a pair
+// make one request).
 //
 // The state stays one contiguous sketch per worker: a group of tensors is interleaved into a scratch
 // (k_sketch_swap, which also clears the new sketch), stepped, and written back to where it was.  Groups

@@ -10,8 +10,8 @@
 // Neighbouring lanes always have neighbouring elements, so that every load is a run of contiguous memory
 // whatever the width of the matrix, and no load depends on 16-byte alignment.  The rank is a template
 // parameter, the factors' rows come as vectors through L1, and every warp has 8 to 16 independent loads in
-// flight.  Bound by instruction issue and the L1 pipe (15 to 21 instructions per element, four L1
-// wavefronts per 32 elements for the rank-4 factor).
+// flight.  Bound by instruction issue and latency (rank 2, int4: 32, 31 and 47 thread instructions per element,
+// issue slots 46, 45 and 74 % busy, DRAM at a quarter of its rate).
 //
 // The order of every sum is part of the result: a factor that moves by one rounding moves a stored int4
 // code by a whole quantum now and then, and the steps that follow amplify it (a reversed sum over the row

@@ -13,7 +13,7 @@
 // Consumers read the bitmap (bit i of word w: element 32 w + i is a member) and
 //   slot(j) = tileoff[j / 8192] + wordoff[j / 32] + members of j's word below j.
 //
-// Bound by the integer pipe: about 25 instructions per element, eight of them multiplies, no memory
+// Bound by the integer pipe: 28 instructions per element (issue slots 69 % busy), eight of them multiplies, no memory
 // traffic to speak of.  Transformer-big list (210 M elements): a three-level radix select that hashed
 // everything three times took 1.26 ms in ten launches; this takes 0.25 ms in two (the hashing loop
 // alone, without anything around it, 0.17 ms).  One 256 x 512 matrix: 35 us in eleven launches -> 11 us.

@@ -19,7 +19,7 @@
 // the price of one or two more passes over the sketch.
 //
 // Transformer-big list (210 M elements), 5 x d/10 buckets, eight workers: 90 ms per step one worker at a
-// time, 25.3 ms now, of which interleaving takes 3.3; the requests still bound it, ten per element.
+// time, 25.2 ms now, of which interleaving takes 3.2; the requests still bound it, ten per element.
 // Three CTAs per SM (80 registers); with four (spills) 24.8 ms instead of 23.0 for k_sketch_il.
 #pragma once
 #include <algorithm>

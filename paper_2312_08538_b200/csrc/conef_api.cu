@@ -563,6 +563,13 @@ struct conef_ctx {
     cudaStream_t aux[kMaxFastClasses] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kMaxFastClasses] = {};
     int n_aux = 0;
+    bool joined = false;   // the caller's stream waits for an event of a side stream: the next launch on it is not a chained one (launch())
+    bool chain()
+    {
+        const bool c = !joined;
+        joined = false;
+        return c;
+    }
     ~conef_ctx()
     {
         for (int k = 0; k < n_aux; ++k) {
@@ -706,9 +713,9 @@ int launch_rowsketch(conef_ctx *ctx, const DevView &V, cudaStream_t s)
         return CONEF_OK;
     dim3 grid(n, ctx->n_workers);
     if (ctx->c.cs_rows == 1)
-        k_rowsketch<QK, true><<<grid, kRsThreads, 0, s>>>(V);
+        launch(ctx->chain(), k_rowsketch<QK, true>, grid, kRsThreads, 0, s, V);
     else
-        k_rowsketch<QK, false><<<grid, kRsThreads, 0, s>>>(V);
+        launch(ctx->chain(), k_rowsketch<QK, false>, grid, kRsThreads, 0, s, V);
     LAUNCH_CHECK(ctx);
     return CONEF_OK;
 }
@@ -793,15 +800,34 @@ int launch_pass2(conef_ctx *ctx, DevView V, cudaStream_t s, int table = T_P2)
 }
 
 // second stage of pass 2: sums the per-tile partials of every tensor in tile order
-int launch_pass2_reduce(conef_ctx *ctx, DevView V, cudaStream_t s, bool skip_fused = false)
+int launch_pass2_reduce(conef_ctx *ctx, DevView V, cudaStream_t s, bool skip_fused)
 {
     const int table = skip_fused ? T_Q2_NF : T_Q2;
     if (tiles_of(ctx, table) == 0)
         return CONEF_OK;
     V.pfx_q2 = table_ptr(ctx, table);
     dim3 grid2(tiles_of(ctx, table), ctx->n_workers);
-    k_lr_pass2_reduce<<<grid2, 256, 0, s>>>(V);
+    launch(ctx->chain(), k_lr_pass2_reduce, grid2, 256, 0, s, V);
     LAUNCH_CHECK(ctx);
+    return CONEF_OK;
+}
+
+// pass 1 of the tensors that take a row per lane, and the sums of the others' row partials
+int launch_p1_rest(conef_ctx *ctx, const DevView &V, cudaStream_t s)
+{
+    if (tiles_of(ctx, T_RP1) > 0) {
+        CK_CUDA(rows_p1_launch<4>(V, table_ptr(ctx, T_RP1), tiles_of(ctx, T_RP1), s, ctx->chain()));
+        LAUNCH_CHECK(ctx);
+    }
+    if (tiles_of(ctx, T_RP1_R8) > 0) {
+        CK_CUDA(rows_p1_launch<8>(V, table_ptr(ctx, T_RP1_R8), tiles_of(ctx, T_RP1_R8), s, ctx->chain()));
+        LAUNCH_CHECK(ctx);
+    }
+    if (tiles_of(ctx, T_FAST_P1) > 0) {
+        // P_i = sum of the per-segment row partials
+        CK_CUDA(fast_launch_p1_combine(ctx->q.rank, V, table_ptr(ctx, T_FAST_P1), tiles_of(ctx, T_FAST_P1), s, ctx->chain()));
+        LAUNCH_CHECK(ctx);
+    }
     return CONEF_OK;
 }
 
@@ -829,7 +855,7 @@ int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool
         const size_t stage = fast_stage_bytes(pass, ctx->q.rank, P.fast_it[pass - 1], P.fast_subs[k], P.fast_threads[k],
                                               P.fast_unit, V.scale_half ? 2 : 4);
         CK_CUDA(fast_launch(pass, ctx->c.kind, ctx->q.rank, V.scale_half, V, table_ptr(ctx, table), n, P.fast_threads[k], sk,
-                            P.short_tiles, P.fast_narrow[k] != 0, stage));
+                            !off_main && ctx->chain(), P.short_tiles, P.fast_narrow[k] != 0, stage));
         LAUNCH_CHECK(ctx);
         if (off_main) {
             CK_CUDA(cudaEventRecord(ctx->ev_join[used], sk));
@@ -838,20 +864,8 @@ int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool
     }
     for (int k = 0; k < used; ++k)
         CK_CUDA(cudaStreamWaitEvent(s, ctx->ev_join[k], 0));
-    if (pass == 1 && tiles_of(ctx, T_RP1) > 0) {
-        CK_CUDA(rows_p1_launch<4>(V, table_ptr(ctx, T_RP1), tiles_of(ctx, T_RP1), s));
-        LAUNCH_CHECK(ctx);
-    }
-    if (pass == 1 && tiles_of(ctx, T_RP1_R8) > 0) {
-        CK_CUDA(rows_p1_launch<8>(V, table_ptr(ctx, T_RP1_R8), tiles_of(ctx, T_RP1_R8), s));
-        LAUNCH_CHECK(ctx);
-    }
-    if (pass == 1 && tiles_of(ctx, T_FAST_P1) > 0) {
-        // P_i = sum of the per-segment row partials
-        CK_CUDA(fast_launch_p1_combine(ctx->q.rank, V, table_ptr(ctx, T_FAST_P1), tiles_of(ctx, T_FAST_P1), s));
-        LAUNCH_CHECK(ctx);
-    }
-    return CONEF_OK;
+    ctx->joined = ctx->joined || used > 0;
+    return pass == 1 ? launch_p1_rest(ctx, V, s) : CONEF_OK;
 }
 
 // zero the sketch being built, run `body`, then swap the two sketch buffers
@@ -1058,10 +1072,10 @@ int launch_randk_select(conef_ctx *ctx, const DevView &V, cudaStream_t s)
     const int nh = tiles_of(ctx, T_HIST), no = tiles_of(ctx, T_SEL_OFFS);
     if (nh == 0)
         return CONEF_OK;
-    k_rk_select<<<nh, kSelThreads, 0, s>>>(V);
+    launch(ctx->chain(), k_rk_select, dim3(nh), kSelThreads, 0, s, V);
     LAUNCH_CHECK(ctx);
     if (no > 0) {
-        k_rk_offsets<<<no, kSelThreads, 0, s>>>(V, table_ptr(ctx, T_SEL_OFFS));
+        launch(ctx->chain(), k_rk_offsets, dim3(no), kSelThreads, 0, s, V, table_ptr(ctx, T_SEL_OFFS));
         LAUNCH_CHECK(ctx);
     }
     return CONEF_OK;
@@ -1253,7 +1267,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
 
     if (phase == 0 && tiles_of(ctx, T_PASS) > 0) {
         dim3 grid(tiles_of(ctx, T_PASS), ctx->n_workers);
-        k_passthrough<<<grid, 256, 0, s>>>(V);
+        launch(ctx->chain(), k_passthrough, grid, 256, 0, s, V);
         LAUNCH_CHECK(ctx);
     }
     // single-phase compressors: the tuned fused step where a tensor allows it, the generic kernel elsewhere
@@ -1264,7 +1278,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
         if (ctx->fast && ctx->c.kind == CONEF_C_IDENTITY && ctx->c.iconef == 0) {
             const int n = tiles_of(ctx, T_DECODE);
             if (n > 0) {
-                k_flat_dense<QK><<<dim3(n, ctx->n_workers), kDecThreads, 0, s>>>(V, table_ptr(ctx, T_DECODE));
+                launch(ctx->chain(), k_flat_dense<QK>, dim3(n, ctx->n_workers), kDecThreads, 0, s, V, table_ptr(ctx, T_DECODE));
                 LAUNCH_CHECK(ctx);
             }
             return CONEF_OK;
@@ -1332,7 +1346,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
             if (n == 0)
                 return CONEF_OK;
-            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s));
+            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->chain()));
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };
@@ -1342,12 +1356,12 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                 return CONEF_OK;
             dim3 grid(n, ctx->n_workers);
             if (pass == 1) {
-                k_rs_pass12<1><<<grid, kRsThreads, 0, s>>>(V, table_ptr(ctx, T_RS_P12));
+                launch(ctx->chain(), k_rs_pass12<1>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
                 LAUNCH_CHECK(ctx);
                 dim3 gridc(tiles_of(ctx, T_RS_P1C), ctx->n_workers);
-                k_rs_p1_combine<<<gridc, 256, 0, s>>>(V, table_ptr(ctx, T_RS_P1C));
+                launch(ctx->chain(), k_rs_p1_combine, gridc, 256, 0, s, V, table_ptr(ctx, T_RS_P1C));
             } else {
-                k_rs_pass12<2><<<grid, kRsThreads, 0, s>>>(V, table_ptr(ctx, T_RS_P12));
+                launch(ctx->chain(), k_rs_pass12<2>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
             }
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
@@ -1420,8 +1434,8 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
         int64_t blocks = ceil_div(len, 256);
         if (blocks > (int64_t)ctx->sm_count * 16)
             blocks = (int64_t)ctx->sm_count * 16;
-        k_reduce_workers<<<(int)blocks, 256, 0, s>>>(base, stride, ctx->n_workers, len, out_sum,
-                                                     mean_out, V.n_workers_f);
+        launch(ctx->chain(), k_reduce_workers, dim3((unsigned)blocks), 256, 0, s, base, stride, ctx->n_workers, len, out_sum, mean_out,
+               V.n_workers_f);
         LAUNCH_CHECK(ctx);
         return CONEF_OK;
     };
@@ -1470,9 +1484,9 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
                     continue;
                 cudaStream_t sk = pick();
                 if (ctx->q.rank <= 4)
-                    CK_CUDA(gs_launch<4>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk));
+                    CK_CUDA(gs_launch<4>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk, sk == s && ctx->chain()));
                 else
-                    CK_CUDA(gs_launch<8>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk));
+                    CK_CUDA(gs_launch<8>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk, sk == s && ctx->chain()));
                 LAUNCH_CHECK(ctx);
                 done(sk);
             }
@@ -1486,6 +1500,7 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
             }
             for (int k = 0; k < used; ++k)
                 CK_CUDA(cudaStreamWaitEvent(s, ctx->ev_join[k], 0));
+            ctx->joined = ctx->joined || used > 0;
         } else if (tiles_of(ctx, T_GS) > 0) {
             k_gram_schmidt<<<tiles_of(ctx, T_GS), 1024, 0, s>>>(V, out_sum);
             LAUNCH_CHECK(ctx);

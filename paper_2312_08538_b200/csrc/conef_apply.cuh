@@ -150,9 +150,16 @@ __global__ void __launch_bounds__(kApplyThreads, R == 8 ? 2 : 3)
 k_apply(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, float *__restrict__ x,
         const float *__restrict__ sum_values, const float *__restrict__ sum_dense1d)
 {
-    const int li = find_layer(pfx, V.n_layers, blockIdx.x);
+    grid_release();
+    int li = find_layer(pfx, V.n_layers, blockIdx.x);
+    if (R >= 0)
+        grid_wait(li);
     const LayerDesc &L = V.layers[li];
     const uint32_t tile = blockIdx.x - pfx[li];
+    if (R < 0)
+        grid_wait();
+    sum_values = fresh(sum_values);
+    sum_dense1d = fresh(sum_dense1d);
     float *__restrict__ xs = x + L.g_off;
     const float nw = V.n_workers_f;
     if (!L.compressed || (R < 0 && V.qkind == CONEF_Q_IDENTITY)) {
@@ -229,12 +236,12 @@ inline void apply_launch(int qkind, int rank, const DevView &V, const int32_t *p
 {
     const int r = qkind != CONEF_Q_LOWRANK ? -1 : rank == 1 || rank == 2 || rank == 4 || rank == 8 ? rank : 0;
     switch (r) {
-    case -1: k_apply<-1><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
-    case 1: k_apply<1><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
-    case 2: k_apply<2><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
-    case 4: k_apply<4><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
-    case 8: k_apply<8><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d); break;
-    default: k_apply<0><<<tiles, kApplyThreads, 0, s>>>(V, pfx, x, sum_values, sum_dense1d);
+    case -1: launch(true, k_apply<-1>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 1: launch(true, k_apply<1>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 2: launch(true, k_apply<2>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 4: launch(true, k_apply<4>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 8: launch(true, k_apply<8>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    default: launch(true, k_apply<0>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d);
     }
 }
 

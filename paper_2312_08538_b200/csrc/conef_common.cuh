@@ -10,18 +10,44 @@
 
 namespace conef {
 
-// last tensor l with pfx[l] <= bid (prefix tables have n + 1 entries)
+// Last tensor l with pfx[l] <= bid (prefix tables have n + 1 entries), by a whole warp: 32 entries per
+// round, so two dependent loads for up to 1024 tensors.  A binary search was eight to ten of them, each a
+// trip to L2 at the start of a kernel.
 __device__ __forceinline__ int find_layer(const int32_t *__restrict__ pfx, int n, int bid)
 {
-    int lo = 0, hi = n;  // invariant: pfx[lo] <= bid < pfx[hi]
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (__ldg(pfx + mid) <= bid)
-            lo = mid;
-        else
-            hi = mid;
+    const int lane = threadIdx.x & 31;
+    int lo = 0;   // pfx[lo] <= bid, and the tensor is one of the n from lo on
+    while (n > 1) {
+        const int step = (n + 31) >> 5, at = lane * step;
+        const bool le = at < n && __ldg(pfx + lo + at) <= bid;
+        const int skip = (__popc(__ballot_sync(0xffffffffu, le)) - 1) * step;
+        lo += skip;
+        n = min(step, n - skip);
     }
     return lo;
+}
+
+// For kernels launched by launch(true, ...) (conef_internal.h).  The kernel ahead in the stream is done and what it
+// wrote is visible:
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and a pointer to what it wrote, so that no load through it (loads of constant memory, as __ldg is taken
+// for, may pass a memory clobber) comes before the wait:
+template <class T>
+__device__ __forceinline__ T *fresh(T *p)
+{
+    asm volatile("" : "+l"(p));
+    return p;
+}
+// ... or, of a kernel whose registers do not allow that, the tensor, before anything is computed from it:
+__device__ __forceinline__ void grid_wait(int &li) { asm volatile("griddepcontrol.wait;" : "+r"(li) : : "memory"); }
+// The kernel behind may come onto the SMs before this one's CTAs leave them.  For grids that leave room on the SMs
+// only: CTAs that wait hold registers and shared memory.  Released always, the count sketch over whole tensors
+// took 36 ms instead of 24; never, the index sets of 54 convolutions 499 us instead of 408 (one CTA per SM; with two or
+// eight 430).
+__device__ __forceinline__ void grid_release()
+{
+    if (gridDim.x * gridDim.y <= (unsigned)kPlanSMs)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Loads of what other CTAs of the same launch wrote before a ticket or a flag: past L1, and volatile with

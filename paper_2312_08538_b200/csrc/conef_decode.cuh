@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kDecThreads) k_decode(const __grid_constant__ 
                                                         int worker, float *__restrict__ out)
 {
     constexpr int kTile = dec_tile(BATCH);
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
@@ -50,6 +51,7 @@ __global__ void __launch_bounds__(kDecThreads) k_decode(const __grid_constant__ 
     const uint32_t d = (uint32_t)L.d, j0 = (blockIdx.x - pfx[li]) * (uint32_t)kTile;
     float *__restrict__ o = out + L.e_off;
     const uint32_t n = min(d - j0, (uint32_t)kTile);
+    grid_wait();
     if (n == (uint32_t)kTile && ((uintptr_t)(o + j0) & 15) == 0) {
         uint32_t w[2][BATCH];
         float s[2][BATCH];
@@ -110,12 +112,9 @@ template <int BATCH>
 inline void decode_launch_batch(bool int4, bool second, const DevView &V, const int32_t *pfx, int tiles, int worker, float *out,
                                 cudaStream_t s)
 {
-    if (int4)
-        second ? k_decode<true, true, BATCH><<<tiles, kDecThreads, 0, s>>>(V, pfx, worker, out)
-               : k_decode<true, false, BATCH><<<tiles, kDecThreads, 0, s>>>(V, pfx, worker, out);
-    else
-        second ? k_decode<false, true, BATCH><<<tiles, kDecThreads, 0, s>>>(V, pfx, worker, out)
-               : k_decode<false, false, BATCH><<<tiles, kDecThreads, 0, s>>>(V, pfx, worker, out);
+    auto *k = int4 ? (second ? k_decode<true, true, BATCH> : k_decode<true, false, BATCH>)
+                   : (second ? k_decode<false, true, BATCH> : k_decode<false, false, BATCH>);
+    launch(true, k, dim3(tiles), kDecThreads, 0, s, V, pfx, worker, out);
 }
 inline void decode_launch(int batch, bool int4, bool second, const DevView &V, const int32_t *pfx, int tiles, int worker, float *out,
                           cudaStream_t s)

@@ -93,9 +93,11 @@ __device__ __forceinline__ void dense_tile(const DevView &V, const LayerDesc &L,
 template <int QK>
 __global__ void __launch_bounds__(kDecThreads) k_flat_dense(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t j0 = (blockIdx.x - pfx[li]) * (uint32_t)kDecTile, n = min((uint32_t)L.d - j0, (uint32_t)kDecTile);
+    grid_wait();
     if (n == (uint32_t)kDecTile && ((uintptr_t)(V.grads[blockIdx.y] + L.g_off) & 15) == 0)
         dense_tile<QK, 4>(V, L, li, j0, n);
     else

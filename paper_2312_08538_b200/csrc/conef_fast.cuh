@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(kFastMaxWarps * 32, min_ctas(PASS, R))
 k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc *Lp = V.layers + li;
     // everything the loop needs goes to registers first
@@ -349,9 +350,10 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
             p1_dstA = ppart + ((size_t)(wg - ((sub * m) >> 8)) * n_rows + sub) * R;
     }
 
+    grid_wait();
     float frag[8][R];   // pass 1: Q_{t-1}[col..col+7][:]; pass 2: accumulators of Q_i[col..col+7][:]; pass 3: Q_i[...]
     if (PASS == 1) {
-        const float *qp = V.qprev + Lp->msgq_off;
+        const float *qp = fresh(V.qprev + Lp->msgq_off);
 #pragma unroll
         for (int q = 0; q < 8; ++q)
 #pragma unroll
@@ -366,7 +368,7 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
             for (int c = 0; c < R; ++c)
                 frag[q][c] = 0.f;
     } else {
-        const float *qi = V.msgq + worker * V.msgq_stride + Lp->msgq_off;
+        const float *qi = fresh(V.msgq + worker * V.msgq_stride + Lp->msgq_off);
 #pragma unroll
         for (int q = 0; q < 8; ++q)
 #pragma unroll
@@ -661,7 +663,7 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
         if (PASS != 1) {
             const uint32_t n4 = (c1 - c0) * subs * (R / 4), n4pad = cpad * subs * (R / 4);
             const int64_t have4 = (n_rows - (int64_t)c0 * subs) * (R / 4);
-            const float4 *src = (const float4 *)(V.phat + Lp->msgp_off + (size_t)c0 * subs * R);
+            const float4 *src = fresh((const float4 *)(V.phat + Lp->msgp_off + (size_t)c0 * subs * R));
             for (uint32_t i = tid; i < n4pad; i += bd) {
                 const float4 v = (i < n4 && (int64_t)i < have4) ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
                 if (PAIR) {
@@ -736,8 +738,10 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 template <int R>
 __global__ void __launch_bounds__(256) k_fast_p1_combine(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc *Lp = V.layers + li;
+    grid_wait();
     const int worker = blockIdx.y;
     const int64_t n = Lp->rows;
     const int64_t q = (int64_t)(blockIdx.x - pfx[li]) * 256 + threadIdx.x;   // (row, c) pair
@@ -757,9 +761,9 @@ __global__ void __launch_bounds__(256) k_fast_p1_combine(const __grid_constant__
 // ------------------------------------------------------------------ launch helpers (conef_fast.cu)
 // PASS: 1, 2 or 3.  Returns cudaErrorNotSupported for a configuration that has no tuned kernel.
 // short_tiles: the plan's tile lengths are below the limits (small models); narrow: the launch's
-// tensors have rows shorter than a warp's 256 elements (pass 1 sums several rows per warp)
+// tensors have rows shorter than a warp's 256 elements (pass 1 sums several rows per warp); chained: see launch()
 cudaError_t fast_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx,
-                        int tiles, int threads, cudaStream_t s, bool short_tiles, bool narrow, size_t stage);
-cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s);
+                        int tiles, int threads, cudaStream_t s, bool chained, bool short_tiles, bool narrow, size_t stage);
+cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained);
 
 }  // namespace conef

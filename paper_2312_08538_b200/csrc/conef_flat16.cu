@@ -4,15 +4,14 @@
 namespace conef {
 
 template <int QK, int CK, bool HALF, int ICO>
-static cudaError_t launch(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
+static cudaError_t flat16(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
 {
     constexpr size_t smem = (size_t)(kF16Threads / 32) * f16_ring(ICO) * sizeof(F16Stage<CK, ICO>);
     static int done[64];
     const cudaError_t e = opt_in_smem(k_flat16<QK, CK, HALF, ICO>, smem, done);
     if (e != cudaSuccess)
         return e;
-    k_flat16<QK, CK, HALF, ICO><<<dim3(tiles, V.n_workers), kF16Threads, smem, s>>>(V, pfx);
-    return cudaSuccess;
+    return launch(true, k_flat16<QK, CK, HALF, ICO>, dim3(tiles, V.n_workers), kF16Threads, smem, s, V, pfx);
 }
 
 cudaError_t flat16_launch(int qkind, int ckind, int half, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
@@ -21,7 +20,7 @@ cudaError_t flat16_launch(int qkind, int ckind, int half, const DevView &V, cons
         return cudaSuccess;
 #define CONEF_F16_CASE(QV, CKV, HV, IV)                                                     \
     if (qkind == QV && ckind == CKV && (half != 0) == HV && (V.iconef == 1) == (IV == 1))   \
-        return launch<QV, CKV, HV, IV>(V, pfx, tiles, s);
+        return flat16<QV, CKV, HV, IV>(V, pfx, tiles, s);
 #define CONEF_F16_Q(QV)                          \
     CONEF_F16_CASE(QV, CONEF_C_INT8, false, 0)   \
     CONEF_F16_CASE(QV, CONEF_C_INT8, true, 0)    \

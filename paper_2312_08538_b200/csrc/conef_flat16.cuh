@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(kF16Threads, f16_ctas(ICO)) k_flat16(const __g
     constexpr int NW = INT4 ? 2 : 4, SB = HALF ? 2 : 4, NS = ICO == 1 ? 2 : 1;
     using Stage = F16Stage<CK, ICO>;
     extern __shared__ __align__(128) uint8_t f16_smem[];
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const int worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -469,6 +470,7 @@ __global__ void __launch_bounds__(kF16Threads, f16_ctas(ICO)) k_flat16(const __g
             }
         }
     };
+    grid_wait();
 #pragma unroll
     for (int i = 0; i < kF16Ring - 1; ++i)
         issue(c0 + i * 8, i);

@@ -47,6 +47,7 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
     __shared__ double warp_part[32][R];
     __shared__ double cta_part[2][R];            // double-buffered by column parity
 #endif
+    grid_release();
     const int tile = blockIdx.x / csize;         // one cluster per tensor of this launch
     const int li = find_layer(pfx, V.n_layers, tile);
     const LayerDesc *Lp = V.layers + li;
@@ -58,6 +59,7 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
     const int64_t row_lo = crank * rows_per_cta;
     const int64_t row_hi = min(n, row_lo + rows_per_cta);
 
+    grid_wait();
     // P_bar = ((P_0 + P_1) + P_2) + ... in worker order.  All of a worker's values are loaded
     // before any is used and nothing is stored until the sum is complete, so that the loads of a
     // round are in flight together (one round trip to L2 per worker instead of one per value).
@@ -69,7 +71,7 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
             v[k][c] = 0.f;
     constexpr int KB = R > 4 ? 2 : 8;   // rows loaded per round (registers)
     for (int i = 0; i < V.n_workers; ++i) {
-        const float *__restrict__ src = V.msgp + i * V.msgp_stride + off;
+        const float *__restrict__ src = fresh(V.msgp + i * V.msgp_stride + off);
 #pragma unroll
         for (int k0 = 0; k0 < kGsRows; k0 += KB) {
             float x[KB][R];
@@ -303,37 +305,12 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
 // Launch over `tiles` tensors (prefix table pfx) with the given cluster size.
 template <int R>
 inline cudaError_t gs_launch(const DevView &V, const int32_t *pfx, int tiles, int cluster_size, float *out_sum,
-                             cudaStream_t s)
+                             cudaStream_t s, bool chained)
 {
     if (tiles <= 0)
         return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(tiles * cluster_size), 1, 1);
-    cfg.blockDim = dim3(kGsThreads, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    if (cluster_size > 8) {   // above the portable limit: opt in once
-        static bool allowed[64] = {};   // per device: function attributes are set per device
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess)
-            return e;
-        if (dev < 0 || dev >= 64 || !allowed[dev]) {
-            e = cudaFuncSetAttribute(k_gs_cluster<R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess)
-                return e;
-            if (dev >= 0 && dev < 64)
-                allowed[dev] = true;
-        }
-    }
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cluster_size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gs_cluster<R>, V, pfx, out_sum);
+    static bool allowed[64] = {};
+    return launch_cluster(chained, k_gs_cluster<R>, tiles, cluster_size, kGsThreads, s, allowed, V, pfx, out_sum);
 }
 
 }  // namespace conef

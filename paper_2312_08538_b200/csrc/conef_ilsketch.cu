@@ -10,9 +10,11 @@ static __global__ void __launch_bounds__(kIlThreads) k_sketch_back(const __grid_
                                                                    int first, int worker0, const float *__restrict__ records,
                                                                    int64_t n_records)
 {
+    grid_release();
     const int tile = first + (int)blockIdx.x;
     const int li = find_layer(pfx, V.n_layers, tile);
     const LayerDesc &L = V.layers[li];
+    grid_wait();
     const int64_t n = (int64_t)V.cs_rows * L.w, room = (n + 63) / 64 * 64;
     const int64_t e0 = (int64_t)(tile - pfx[li]) * kIlEntries + threadIdx.x;
     const float *__restrict__ src = records + blockIdx.y * n_records + L.sk_off;
@@ -37,7 +39,9 @@ static __global__ void __launch_bounds__(kIlThreads) k_sketch_fold(const __grid_
     constexpr int F = 2 * GW, PITCH = F + 1, PW = GW < 4 ? GW : 4;   // floats per record and per piece
     using Piece = typename std::conditional<PW == 2, float2, float4>::type;
     __shared__ float buf[PART == 0 || PART == 3 ? kIlThreads * PITCH : 1];
+    grid_release();
     const LayerDesc &L = V.layers[find_layer(pfx, V.n_layers, first)];
+    grid_wait();
     const uint32_t n = (uint32_t)(V.cs_rows * L.w), half = (n + 1u) / 2u, t = threadIdx.x;
     float *const states = (float *)(V.state + worker0 * V.state_stride + L.a_off);
     const int64_t pitch = V.state_stride / 4;
@@ -122,11 +126,11 @@ static void step(const DevView &V, const int32_t *pfx, int first, int tiles, int
 {
     const dim3 grid(tiles, groups);
     if (V.cs_rows == 5)
-        k_sketch_il<QK, 5, W, LP, FORM><<<grid, kIlThreads, 0, s>>>(V, pfx, first, worker0, records, stride, newoff);
+        launch(true, k_sketch_il<QK, 5, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
     else if (V.cs_rows == 3)
-        k_sketch_il<QK, 3, W, LP, FORM><<<grid, kIlThreads, 0, s>>>(V, pfx, first, worker0, records, stride, newoff);
+        launch(true, k_sketch_il<QK, 3, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
     else
-        k_sketch_il<QK, 0, W, LP, FORM><<<grid, kIlThreads, 0, s>>>(V, pfx, first, worker0, records, stride, newoff);
+        launch(true, k_sketch_il<QK, 0, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
 }
 
 // a group of tensors
@@ -152,9 +156,9 @@ static int together(const Group &G, int worker0, int batches)
     const uint32_t stride = (uint32_t)(near ? 2 * NW : NW);
     const int64_t newoff = near ? GW : G.n_records * NW;
     const dim3 egrid(G.etiles, batches);
-    k_sketch_swap<GW, true, false><<<egrid, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
+    launch(true, k_sketch_swap<GW, true, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
     step<QK, W, LP, IL_SCRATCH>(G.V, G.pfx, G.first, G.tiles, worker0, batches, G.records, stride, newoff, G.s);
-    k_sketch_swap<GW, false, false><<<egrid, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
+    launch(true, k_sketch_swap<GW, false, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
     return 3;
 }
 template <int QK, int W, int LP>
@@ -164,22 +168,22 @@ static int split(const Group &G, int worker0)
     if constexpr (GW > 1) {
         if (G.n_records * 8 * GW > kIlTogether) {   // (one tensor: a group of several is at most 2 kIlGroupBytes)
             const int tiles = (int)(((G.n_records + 1) / 2 + kIlEntries - 1) / kIlEntries);
-            k_sketch_fold<GW, 0><<<tiles, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records);
-            k_sketch_fold<GW, 1><<<tiles, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(true, k_sketch_fold<GW, 0>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(true, k_sketch_fold<GW, 1>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
             step<QK, W, LP, IL_FOLD>(G.V, G.pfx, G.first, G.tiles, worker0, 1, G.records, GW, 0, G.s);
-            k_sketch_fold<GW, 2><<<tiles, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records);
-            k_sketch_fold<GW, 3><<<tiles, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(true, k_sketch_fold<GW, 2>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(true, k_sketch_fold<GW, 3>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
             return 5;
         }
     }
-    k_sketch_swap<GW, true, true><<<G.etiles, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records, GW, 0);
+    launch(true, k_sketch_swap<GW, true, true>, dim3(G.etiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, GW, 0);
     step<QK, W, LP, IL_SPLIT>(G.V, G.pfx, G.first, G.tiles, worker0, 1, G.records, GW, 0, G.s);
     if (GW == 1)   // (its one slice is the state)
         return 2;
-    k_sketch_swap<GW, false, true><<<G.etiles, kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records, GW, G.second ? -1 : G.n_records);
+    launch(true, k_sketch_swap<GW, false, true>, dim3(G.etiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, GW, G.second ? -1 : G.n_records);
     if (G.second)
         return 3;
-    k_sketch_back<<<dim3(G.etiles, GW), kIlThreads, 0, G.s>>>(G.V, G.epfx, G.efirst, worker0, G.records, G.n_records);
+    launch(true, k_sketch_back, dim3(dim3(G.etiles, GW)), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, G.n_records);
     return 4;
 }
 

@@ -138,6 +138,7 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
 {
     constexpr int VM = VR ? VR : 7, GW = W * LP;
     const int v = VR ? VR : V.cs_rows;
+    grid_release();
     const int tile = first + (int)blockIdx.x;
     const int li = find_layer(pfx, V.n_layers, tile);
     const LayerDesc &L = V.layers[li];
@@ -166,6 +167,7 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
     if (threadIdx.x < 7)
         keys[threadIdx.x] = stream_key(V.seed_c, (uint64_t)li, (uint64_t)threadIdx.x);
     __syncthreads();
+    grid_wait();
     uint32_t blk_start = 0;
     if (QK == CONEF_Q_RANDBLOCK)
         blk_start = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step), d, (uint32_t)L.k);
@@ -262,9 +264,11 @@ __global__ void __launch_bounds__(kIlThreads) k_sketch_swap(const __grid_constan
     constexpr int PITCH = GW == 8 ? 9 : GW;            // (entries of a warp in different banks)
     using Piece = typename std::conditional<PW == 1, float, typename std::conditional<PW == 2, float2, float4>::type>::type;
     __shared__ float buf[kIlThreads * PITCH];
+    grid_release();
     const int tile = first + (int)blockIdx.x;
     const int li = find_layer(pfx, V.n_layers, tile);
     const LayerDesc &L = V.layers[li];
+    grid_wait();
     const int64_t n = (int64_t)V.cs_rows * L.w;
     const int64_t e0 = (int64_t)(tile - pfx[li]) * kIlEntries;
     const int w0 = worker0 + blockIdx.y * GW, t = threadIdx.x;

@@ -190,6 +190,64 @@ cudaError_t fused_config(int ckind, int rank, int half, int ctas_per_sm, int n_s
 // cooperative launch (all CTAs co-resident: tasks wait on results of earlier tasks)
 cudaError_t fused_launch(int ckind, int rank, int half, int ctas_per_sm, const FusedParams &P, int n_ctas, size_t smem, cudaStream_t s);
 
+// Launch that may start before the kernel ahead of it in the stream has ended (programmatic stream
+// serialization): its CTAs come onto the SMs as the last ones of that kernel leave them, or earlier where that
+// kernel lets them (grid_release), and look up their tensor meanwhile.  The kernel has to call grid_wait()
+// (conef_common.cuh) in every thread before it touches anything but the tables of the plan, its parameters and
+// its own shared memory.  chained = false: an ordinary launch, after an event of another stream.
+// One small layer on two workers 25.9 -> 15.9 us per step and update (four kernels), index sets of 54 convolutions
+// 733 -> 552 us (two kernels each), iConEF-v1 behind an odd layer 159 -> 137 us, ResNet-50's random block 250 -> 233 us.
+template <class... P, class... A>
+inline cudaError_t launch(bool chained, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
+}
+
+// The same with thread-block clusters; sizes above 8 (the portable limit) opt the kernel in once per device:
+// `allowed` is the caller's per-kernel record.
+template <class... P, class... A>
+inline cudaError_t launch_cluster(bool chained, void (*kernel)(P...), int tiles, int cluster_size, int threads, cudaStream_t s,
+                                  bool (&allowed)[64], A &&...args)
+{
+    if (cluster_size > 8) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess)
+            return e;
+        if (dev < 0 || dev >= 64 || !allowed[dev]) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess)
+                return e;
+            if (dev >= 0 && dev < 64)
+                allowed[dev] = true;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * cluster_size), 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster_size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chained ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
+}
+
 // Opt a kernel in to `bytes` of dynamic shared memory, once per device and kernel: `done` is the
 // caller's per-kernel record (largest size set so far on each device).  Sizes up to the default
 // 48 KB need no call.

@@ -14,12 +14,14 @@ namespace conef {
 // ------------------------------------------------------------------ 1-D pass-through
 __global__ void __launch_bounds__(256) k_passthrough(const __grid_constant__ DevView V)
 {
+    grid_release();
     const int li = find_layer(V.pfx_pass, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const int worker = blockIdx.y;
     const int64_t j0 = (int64_t)(blockIdx.x - V.pfx_pass[li]) * kPassTile;
     const float *__restrict__ g = V.grads[worker] + L.g_off;
     float *__restrict__ out = V.msg1d + worker * V.msg1d_stride + L.msg1d_off;
+    grid_wait();
     for (int q = threadIdx.x; q < kPassTile; q += 256) {
         int64_t j = j0 + q;
         if (j < L.d)
@@ -478,8 +480,10 @@ __global__ void __launch_bounds__(kP2ColsPerCta) k_lr_pass2(const __grid_constan
 constexpr int kQ2PerCta = 1024;
 __global__ void __launch_bounds__(256) k_lr_pass2_reduce(const __grid_constant__ DevView V)
 {
+    grid_release();
     const int li = find_layer(V.pfx_q2, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
+    grid_wait();
     const int worker = blockIdx.y;
     const int64_t mr = L.cols * L.rank;
     const int64_t q = ((int64_t)(blockIdx.x - V.pfx_q2[li]) * 256 + threadIdx.x) * 4;
@@ -525,6 +529,9 @@ __global__ void __launch_bounds__(256) k_reduce_workers(const float *__restrict_
                                                         float *__restrict__ out,
                                                         float *__restrict__ mean_out, float nf)
 {
+    grid_release();
+    grid_wait();
+    base = fresh(base);
     for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < len; j += (int64_t)gridDim.x * 256) {
         float acc = base[j];
         for (int i = 1; i < n_workers; ++i)

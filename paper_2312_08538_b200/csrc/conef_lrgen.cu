@@ -4,35 +4,36 @@
 namespace conef {
 
 template <int CK, int R>
-static void launch(int pass, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
+static cudaError_t pass_launch(int pass, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained)
 {
     const dim3 grid(tiles, V.n_workers);
     if (pass == 1)
-        k_gen_pass<1, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else if (pass == 2)
-        k_gen_pass<2, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else if (unit == 256)
-        k_gen_pass<3, CK, R, 8><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else if (unit == 128)
-        k_gen_pass<3, CK, R, 4><<<grid, kGenThreads, 0, s>>>(V, pfx);
-    else if (CK == CONEF_C_INT4 || unit == 64)   // (int4 blocks are 64 or more)
-        k_gen_pass<3, CK, R, 2><<<grid, kGenThreads, 0, s>>>(V, pfx);
+        return launch(chained, k_gen_pass<1, CK, R, 1>, grid, kGenThreads, 0, s, V, pfx);
+    if (pass == 2)
+        return launch(chained, k_gen_pass<2, CK, R, 1>, grid, kGenThreads, 0, s, V, pfx);
+    if (unit == 256)
+        return launch(chained, k_gen_pass<3, CK, R, 8>, grid, kGenThreads, 0, s, V, pfx);
+    if (unit == 128)
+        return launch(chained, k_gen_pass<3, CK, R, 4>, grid, kGenThreads, 0, s, V, pfx);
+    if (CK == CONEF_C_INT4 || unit == 64)   // (int4 blocks are 64 or more)
+        return launch(chained, k_gen_pass<3, CK, R, 2>, grid, kGenThreads, 0, s, V, pfx);
     else if constexpr (CK == CONEF_C_INT8)
-        k_gen_pass<3, CK, R, 1><<<grid, kGenThreads, 0, s>>>(V, pfx);
+        return launch(chained, k_gen_pass<3, CK, R, 1>, grid, kGenThreads, 0, s, V, pfx);
+    return cudaErrorNotSupported;
 }
 
-cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
+cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained)
 {
     if (tiles <= 0)
         return cudaSuccess;
 #define CONEF_GEN_CK(CKV)                                                                  \
     if (ckind == CKV) {                                                                    \
         switch (rank) {                                                                    \
-        case 1: launch<CKV, 1>(pass, unit, V, pfx, tiles, s); return cudaSuccess;          \
-        case 2: launch<CKV, 2>(pass, unit, V, pfx, tiles, s); return cudaSuccess;          \
-        case 4: launch<CKV, 4>(pass, unit, V, pfx, tiles, s); return cudaSuccess;          \
-        case 8: launch<CKV, 8>(pass, unit, V, pfx, tiles, s); return cudaSuccess;          \
-        default: launch<CKV, 0>(pass, unit, V, pfx, tiles, s); return cudaSuccess;         \
+        case 1: return pass_launch<CKV, 1>(pass, unit, V, pfx, tiles, s, chained); \
+        case 2: return pass_launch<CKV, 2>(pass, unit, V, pfx, tiles, s, chained); \
+        case 4: return pass_launch<CKV, 4>(pass, unit, V, pfx, tiles, s, chained); \
+        case 8: return pass_launch<CKV, 8>(pass, unit, V, pfx, tiles, s, chained); \
+        default: return pass_launch<CKV, 0>(pass, unit, V, pfx, tiles, s, chained); \
         }                                                                                  \
     }
     CONEF_GEN_CK(CONEF_C_INT8)

@@ -110,9 +110,9 @@ __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L
     const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
     const uint32_t row0 = (tile * 8u + warp) * NR;
-    const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
+    const uint8_t *__restrict__ st = fresh(V.state + worker * V.state_stride);
     const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
-    const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ Q = V.qprev + L.msgq_off;
+    const float *__restrict__ g = fresh(V.grads[worker] + L.g_off), *__restrict__ Q = fresh(V.qprev + L.msgq_off);
     const int shift = 31 - __clz(L.unit);
     const bool half = V.scale_half != 0;
     const float lr = V.lr, omb = V.omb;
@@ -187,9 +187,9 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
     const uint32_t r_lo = rt * (uint32_t)kP2RowsPerTile, r_hi = min(n, r_lo + (uint32_t)kP2RowsPerTile);
     if (r_lo >= n)
         return;   // (no CTA-wide barrier below)
-    const uint8_t *__restrict__ st = V.state + worker * V.state_stride;
+    const uint8_t *__restrict__ st = fresh(V.state + worker * V.state_stride);
     const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
-    const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ ph = V.phat + L.msgp_off;
+    const float *__restrict__ g = fresh(V.grads[worker] + L.g_off), *__restrict__ ph = fresh(V.phat + L.msgp_off);
     const int shift = 31 - __clz(L.unit);
     const bool half = V.scale_half != 0;
     const float lr = V.lr, omb = V.omb;
@@ -260,8 +260,8 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
     uint8_t *st = V.state + worker * V.state_stride;
     uint32_t *codes = (uint32_t *)(st + L.a_off);
     uint8_t *scales = st + L.b_off;
-    const float *__restrict__ g = V.grads[worker] + L.g_off, *__restrict__ ph = V.phat + L.msgp_off;
-    const float *__restrict__ Q = V.msgq + worker * V.msgq_stride + L.msgq_off;
+    const float *__restrict__ g = fresh(V.grads[worker] + L.g_off), *__restrict__ ph = fresh(V.phat + L.msgp_off);
+    const float *__restrict__ Q = fresh(V.msgq + worker * V.msgq_stride + L.msgq_off);
     const bool half = V.scale_half != 0;
     const float lr = V.lr, omb = V.omb, beta = V.beta;
     uint8_t *mine = bytes + warp * kGenChunk;
@@ -426,9 +426,11 @@ template <int PASS, int CK, int R, int KB>
 __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3 : 4) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     __shared__ __align__(16) uint8_t bytes[PASS == 3 ? 8 * kGenChunk : 16];
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t tile = blockIdx.x - pfx[li];
+    grid_wait();
     constexpr int VW = R == 8 ? 4 : R ? R : 1;   // floats per vector load
     const bool exact = R != 0 && L.rank == R && ((L.msgp_off | L.msgq_off) & (VW - 1)) == 0;
     if (PASS == 1) {
@@ -455,6 +457,6 @@ __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3
 }
 
 // launcher (conef_lrgen.cu)
-cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s);
+cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained);
 
 }  // namespace conef

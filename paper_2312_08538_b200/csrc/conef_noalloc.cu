@@ -53,12 +53,10 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
     __shared__ uint32_t s_n, s_base, s_cnt, s_last, s_listed;
     const int tid = threadIdx.x;
     const bool windowed = a.d > (uint32_t)kSelShortTensor;
+    grid_release();
     S.hist[tid] = 0;   // the bins of select_threshold
-    if (tid == 0) {
+    if (tid == 0)
         s_n = s_cnt = 0;
-        if (blockIdx.x == 0)
-            a.ctr[NA_K] = 0;   // (before this CTA's ticket, so before the last CTA's result)
-    }
     __syncthreads();
     if (windowed) {
         const uint32_t j0 = blockIdx.x * kNaTile + tid * kNaPer;
@@ -77,6 +75,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
             if (pos < (uint32_t)kSelList) {
                 ((uint2 *)S.keys)[pos] = e;
             } else {
+                grid_wait();
                 const uint32_t g = select_claim(a.ctr, 1u);
                 if (g < a.cap)
                     a.list[g] = e;
@@ -86,6 +85,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
         below = __reduce_add_sync(0xffffffffu, below);
         if ((tid & 31) == 0 && below)
             atomicAdd(&s_cnt, below);
+        grid_wait();   // (all of that while the kernel ahead ends)
         __syncthreads();
         const uint32_t n = min(s_n, (uint32_t)kSelList);
         if (tid == 0) {
@@ -96,7 +96,11 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
         for (uint32_t x = tid; x < n; x += kSelThreads)
             if (s_base + x < a.cap)
                 a.list[s_base + x] = ((uint2 *)S.keys)[x];
+    } else {
+        grid_wait();
     }
+    if (tid == 0 && blockIdx.x == 0)
+        a.ctr[NA_K] = 0;   // (before this CTA's ticket, so before the last CTA's result)
     __threadfence();
     __syncthreads();
     if (tid == 0)
@@ -157,6 +161,12 @@ __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32
     __shared__ uint32_t wsum[kSelThreads / 32], s_own, s_first;
     __shared__ uint64_t s_tau;
     const uint32_t j0 = blockIdx.x * kNaTile + threadIdx.x * kNaPer;
+    grid_release();
+    uint32_t h[kNaPer];   // (while the first kernel ends)
+#pragma unroll
+    for (uint32_t q = 0; q < kNaPer; ++q)
+        h[q] = hash32(a.stream, j0 + q);
+    grid_wait();
     if (threadIdx.x == 0) {   // (one thread reads them: a CTA has to agree on whether it goes on)
         const uint2 tau = *(const uint2 *)(a.ctr + NA_TAU_LO);
         const uint4 of = *(const uint4 *)(a.ctr + NA_STREAM_LO);
@@ -166,10 +176,6 @@ __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32
         if (blockIdx.x == 0)
             a.ctr[NA_DONE] = a.ctr[NA_LISTED] = 0;   // (no CTA of this kernel reads them)
     }
-    uint32_t h[kNaPer];   // (while those loads are under way)
-#pragma unroll
-    for (uint32_t q = 0; q < kNaPer; ++q)
-        h[q] = hash32(a.stream, j0 + q);
     __syncthreads();
     if (!s_own) {
         if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -230,9 +236,9 @@ int write_indices(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_
     if (how == CONEF_SELECT_FULL)
         a.cap = 1;
     a.ntiles = (uint32_t)((d + kNaTile - 1) / kNaTile);
-    k_na_select<<<a.ntiles, kSelThreads, 0, s>>>(a);
+    launch(true, k_na_select, dim3(a.ntiles), kSelThreads, 0, s, a);
     if (how != CONEF_SELECT_HALF)
-        k_na_write<<<a.ntiles, kSelThreads, 0, s>>>(a, idx_out);
+        launch(true, k_na_write, dim3(a.ntiles), kSelThreads, 0, s, a, idx_out);
     return cudaGetLastError() == cudaSuccess ? CONEF_OK : CONEF_ERR_CUDA;
 }
 

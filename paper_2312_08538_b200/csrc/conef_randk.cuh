@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
 {
     __shared__ SelectShared S;
     __shared__ uint32_t s_n, s_base, s_cnt[8], s_last, s_listed;
+    grid_release();
     const int li = find_layer(V.pfx_hist, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t d = (uint32_t)L.d, lo = L.sel_lo, hi = L.sel_hi, T = (uint32_t)V.sel_tiles;
@@ -117,14 +118,18 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
                 if (pos < (uint32_t)kSelList) {
                     ((uint2 *)S.keys)[pos] = e;
                 } else {   // (not expected: the list of a CTA holds several times the usual number)
+                    grid_wait();
                     const uint32_t g = select_claim(ctr, 1u);
                     if (g < cap)
                         list[g] = e;
                 }
             }
+            if (i == 0)
+                grid_wait();   // (the first tile is hashed while the kernel ahead ends)
             bits[w] = word;
             cnt += __popc(word);
         }
+        grid_wait();
         cnt = __reduce_add_sync(0xffffffffu, cnt);
         if (lane == 0 && cnt)
             atomicAdd(&s_cnt[(warp * T) >> 3], cnt);   // a warp's words lie in one tile
@@ -138,6 +143,8 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
         for (uint32_t x = tid; x < n; x += kSelThreads)
             if (s_base + x < cap)
                 list[s_base + x] = ((uint2 *)S.keys)[x];
+    } else {
+        grid_wait();
     }
     __threadfence();
     __syncthreads();
@@ -200,8 +207,10 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
 // word offsets of the tensors with more than kSelTailTiles tiles: a warp per tile
 __global__ void __launch_bounds__(kSelThreads) k_rk_offsets(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
+    grid_wait();
     const uint32_t tile = (blockIdx.x - pfx[li]) * (kSelThreads / 32) + (threadIdx.x >> 5);
     if ((int64_t)tile * kHistTile < L.d)
         select_offsets(V.selbits + L.selbits_off, V.wordoff + L.wordoff_off, tile);

@@ -67,7 +67,7 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
         blk_start = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step), d, (uint32_t)L.k);
     const int r = L.rank;
     float qreg[VEC][RK];   // Q_i[b..b+VEC-1][:], fixed for the thread
-    const float *__restrict__ phat = V.phat + L.msgp_off;
+    const float *__restrict__ phat = fresh(V.phat + L.msgp_off);
     if (QK == CONEF_Q_LOWRANK) {
         const float *qi = V.msgq + worker * V.msgq_stride + L.msgq_off;
 #pragma unroll
@@ -239,9 +239,11 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
 template <int QK, bool V1>   // V1: one sketch row (the usual setting), no median
 __global__ void __launch_bounds__(kRsThreads) k_rowsketch(const __grid_constant__ DevView V)
 {
+    grid_release();
     const int li = find_layer(V.pfx_rs, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t local = blockIdx.x - V.pfx_rs[li];
+    grid_wait();
     constexpr int RKG = QK == CONEF_Q_LOWRANK ? 8 : 4;   // the rank only matters to the low-rank Q
     if (L.rs_vec == 4 && V.rs_vec_ok) {
         if (QK == CONEF_Q_LOWRANK && L.rank == 4 && (L.msgp_off & 3) == 0)
@@ -290,7 +292,7 @@ __device__ __forceinline__ void rs12_body(const DevView &V, const int32_t *__res
     const void *__restrict__ T = V.state + worker * V.state_stride + L.a_off;
     const bool th = V.scale_half != 0;
     const float *__restrict__ g = V.grads[worker] + L.g_off;
-    const float *__restrict__ phat = V.phat + L.msgp_off;
+    const float *__restrict__ phat = fresh(V.phat + L.msgp_off);
     const int r = L.rank;
 
     float q[VEC][RK];   // pass 1: Q_{t-1}[b..b+3][:]; pass 2: accumulators of Q_i[b..b+3][:]
@@ -387,8 +389,10 @@ __device__ __forceinline__ void rs12_body(const DevView &V, const int32_t *__res
 template <int PASS>
 __global__ void __launch_bounds__(kRsThreads) k_rs_pass12(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
+    grid_wait();
     if (L.rank == 4 && (L.msgp_off & 3) == 0)
         rs12_body<PASS, 4>(V, pfx, li, L);
     else
@@ -398,8 +402,10 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_pass12(const __grid_constant_
 // P_i[a][c] = sum over the (column slab, warp) partials of pass 1, in slab-major order
 __global__ void __launch_bounds__(256) k_rs_p1_combine(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
+    grid_wait();
     const int worker = blockIdx.y;
     const int64_t nr = L.rows * L.rank;
     const int64_t qi = (int64_t)(blockIdx.x - pfx[li]) * 256 + threadIdx.x;

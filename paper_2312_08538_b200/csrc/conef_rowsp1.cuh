@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(kRpThreads, CONEF_RP_MINB) k_rows_p1(const __g
     static_assert(sizeof(Stage) % 16 == 0, "stages stay 16-byte aligned");
     extern __shared__ __align__(16) unsigned char rp_smem[];
     Stage *st = (Stage *)rp_smem;
+    grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const int worker = blockIdx.y;
@@ -98,6 +99,7 @@ __global__ void __launch_bounds__(kRpThreads, CONEF_RP_MINB) k_rows_p1(const __g
         for (int c = 0; c < R; ++c)
             acc[rr][c] = 0.f;
 
+    grid_wait();
     // kRpStages buffers, one barrier per stage.  The first kRpStages stages are issued up front; from
     // stage 1 on, stage s + kRpStages - 1 is issued while stage s is worked on, into the buffer of
     // stage s - 1, which every warp left before the barrier of this iteration.  One group of copies
@@ -220,7 +222,7 @@ inline bool rows_p1_takes(const LayerDesc &L)
 }
 
 template <int R>
-inline cudaError_t rows_p1_launch(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
+inline cudaError_t rows_p1_launch(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained)
 {
     if (tiles <= 0)
         return cudaSuccess;
@@ -230,14 +232,12 @@ inline cudaError_t rows_p1_launch(const DevView &V, const int32_t *pfx, int tile
         const cudaError_t e = opt_in_smem(k_rows_p1<R, true>, smem, done_partial);
         if (e != cudaSuccess)
             return e;
-        k_rows_p1<R, true><<<dim3(tiles, V.n_workers), kRpThreads, smem, s>>>(V, pfx);
-        return cudaSuccess;
+        return launch(chained, k_rows_p1<R, true>, dim3(tiles, V.n_workers), kRpThreads, smem, s, V, pfx);
     }
     const cudaError_t e = opt_in_smem(k_rows_p1<R, false>, smem, done_plain);
     if (e != cudaSuccess)
         return e;
-    k_rows_p1<R, false><<<dim3(tiles, V.n_workers), kRpThreads, smem, s>>>(V, pfx);
-    return cudaSuccess;
+    return launch(chained, k_rows_p1<R, false>, dim3(tiles, V.n_workers), kRpThreads, smem, s, V, pfx);
 }
 
 }  // namespace conef

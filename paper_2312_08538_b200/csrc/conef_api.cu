@@ -33,7 +33,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 33 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 34 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -43,6 +43,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_CSK,                                               // count sketch applied run by run: one tile per run
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
        T_SEL_OFFS,                                          // random-k: word offsets of the tensors too large for the selection's last CTA
+       T_SEL_CLUSTER,                                       // random-k where every tensor is selected by a cluster: one per tensor
        T_DECODE,                                            // tiles of the stored error expanded (dec_batch) or of the step on a dense error (kDecTile elements)
        T_IL, T_ILT,                                         // count sketch, workers interleaved: tiles of elements, of sketch entries
        T_GEN1, T_GEN2, T_GEN3,                              // low-rank passes for any shape
@@ -85,6 +86,7 @@ struct Plan {
     bool any_fv = false;        // some tensor takes the tuned fused step (conef_flatvec.cuh)
     int fv_tiles = 1;           // ... with this many selection tiles per CTA
     int sel_tiles = 1;          // random-k selection: tiles hashed per CTA
+    int sel_cluster = 1;        // ... or CTAs per cluster where every tensor is selected by one, else 0
     bool any_fused = false;     // some tensor takes the fused passes 2 + 3 (conef_fused.cu)
     int n_fused = 0;
     bool any_csk = false;       // some tensor takes the shared-memory step of the chunk-wise count sketch
@@ -309,6 +311,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 L.cand_off = P.cand_pairs;
                 select_window(L.d, L.k, L.sel_lo, L.sel_hi, L.cand_cap, L.sel_scale);
                 P.cand_pairs += L.cand_cap;
+                tiles[T_SEL_CLUSTER] = 1;
+                while (P.sel_cluster > 0 && P.sel_cluster < ceil_div(L.d, kHistTile))
+                    P.sel_cluster = P.sel_cluster < kSelClusterTiles ? P.sel_cluster * 2 : 0;
                 if (ceil_div(L.d, kHistTile) > kSelTailTiles)
                     tiles[T_SEL_OFFS] = (int)ceil_div(L.d, (int64_t)kHistTile * (kSelThreads / 32));
                 tiles[T_HIST] = (int)ceil_div(L.d, (int64_t)kHistTile * P.sel_tiles);
@@ -1072,6 +1077,13 @@ int launch_randk_select(conef_ctx *ctx, const DevView &V, cudaStream_t s)
     const int nh = tiles_of(ctx, T_HIST), no = tiles_of(ctx, T_SEL_OFFS);
     if (nh == 0)
         return CONEF_OK;
+    if (ctx->plan.sel_cluster > 0 && (V.sel_how == CONEF_SELECT_NORMAL || V.sel_how == CONEF_SELECT_MISS)) {   // (the others have no list)
+        static bool allowed[64] = {};
+        launch_cluster(ctx->chain(), k_rk_select_cluster, tiles_of(ctx, T_SEL_CLUSTER), ctx->plan.sel_cluster, kSelThreads, s, allowed, V,
+                       table_ptr(ctx, T_SEL_CLUSTER));
+        LAUNCH_CHECK(ctx);
+        return CONEF_OK;
+    }
     launch(ctx->chain(), k_rk_select, dim3(nh), kSelThreads, 0, s, V);
     LAUNCH_CHECK(ctx);
     if (no > 0) {

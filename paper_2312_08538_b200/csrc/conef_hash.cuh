@@ -28,10 +28,10 @@ __host__ __device__ __forceinline__ uint64_t h64(uint64_t st, uint64_t j)
 }
 __device__ __forceinline__ uint32_t hash32(uint64_t st, uint64_t j) { return (uint32_t)(h64(st, j) >> 32); }
 // hash32 without the mixer's last step, which can only flip the lowest bit: comparisons with an even
-// bound (x < even) come out the same
-__device__ __forceinline__ uint32_t hash32_but_lowest(uint64_t st, uint64_t j)
+// bound (x < even) come out the same.  z: st + kGolden * (j + 1), which a caller with a run of consecutive j
+// steps along by additions of constants (left to the compiler it was three multiplies per element)
+__device__ __forceinline__ uint32_t hash32_but_lowest_of(uint64_t z)
 {
-    uint64_t z = st + kGolden * (j + 1);
     z ^= z >> 30;
     z *= 0xBF58476D1CE4E5B9ULL;
     z ^= z >> 27;

@@ -49,7 +49,7 @@ struct NaArgs {
 // below the window and lists those inside; the last CTA finds the threshold and the tiles' offsets.
 __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
 {
-    __shared__ SelectShared S;
+    __shared__ SelectSharedTiles S;
     __shared__ uint32_t s_n, s_base, s_cnt, s_last, s_listed;
     const int tid = threadIdx.x;
     const bool windowed = a.d > (uint32_t)kSelShortTensor;
@@ -61,9 +61,10 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
     if (windowed) {
         const uint32_t j0 = blockIdx.x * kNaTile + tid * kNaPer;
         uint32_t below = 0, upto = 0;
+        const uint64_t z0 = a.stream + kGolden * ((uint64_t)j0 + 1);
 #pragma unroll
         for (uint32_t q = 0; q < kNaPer; ++q) {
-            const uint32_t h = hash32_but_lowest(a.stream, j0 + q);
+            const uint32_t h = hash32_but_lowest_of(z0 + kGolden * q);
             below |= h < a.lo ? 1u << q : 0u;
             upto |= h <= a.hi ? 1u << q : 0u;
         }
@@ -196,6 +197,28 @@ __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32
             idx_out[slot] = j0 + (uint32_t)__ffs(in) - 1u;
 }
 
+// Tensors of at most kNaClusterTiles tiles of 8192: one cluster does all of it, without the scratch
+// (one launch, and nothing kept between calls).  54 convolutions, of which 20 are that small: 552 -> 408 us with it and
+// with the first kernel's hashing ahead of its wait.
+constexpr int kNaClusterTiles = 8;
+__global__ void __launch_bounds__(kSelThreads) k_na_cluster(const NaArgs a, uint32_t *__restrict__ idx_out)
+{
+    __shared__ SelectCluster S;
+    grid_release();
+    const SelectResult R = select_in_cluster(S, a.stream, a.d, a.k, a.lo, a.hi, a.scale, a.how != CONEF_SELECT_NORMAL);
+    grid_wait();
+    if (R.failed || R.total != a.k) {
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            idx_out[0] = 0xFFFFFFFFu;
+        return;
+    }
+    const uint32_t j0 = blockIdx.x * (uint32_t)kHistTile + threadIdx.x * 32u;
+    uint32_t all, slot = R.first + block_exclusive(__popc(R.word), S.wsum, all);
+    for (uint32_t m = R.word; m; m &= m - 1, ++slot)
+        if (slot < a.k)
+            idx_out[slot] = j0 + (uint32_t)__ffs(m) - 1u;
+}
+
 // device address of the scratch on each device, resolved once per device
 std::mutex g_mu;
 uint32_t *g_scratch_ptr[64] = {nullptr};
@@ -235,6 +258,13 @@ int write_indices(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_
     a.how = (uint32_t)how;
     if (how == CONEF_SELECT_FULL)
         a.cap = 1;
+    const int64_t ctas = (d + kHistTile - 1) / kHistTile;
+    if (ctas <= kNaClusterTiles && how != CONEF_SELECT_HALF) {
+        static bool allowed[64] = {};
+        const int size = ctas <= 1 ? 1 : ctas <= 2 ? 2 : ctas <= 4 ? 4 : kNaClusterTiles;
+        launch_cluster(true, k_na_cluster, 1, size, kSelThreads, s, allowed, a, idx_out);
+        return cudaGetLastError() == cudaSuccess ? CONEF_OK : CONEF_ERR_CUDA;
+    }
     a.ntiles = (uint32_t)((d + kNaTile - 1) / kNaTile);
     launch(true, k_na_select, dim3(a.ntiles), kSelThreads, 0, s, a);
     if (how != CONEF_SELECT_HALF)

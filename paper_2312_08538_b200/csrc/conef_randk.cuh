@@ -7,7 +7,7 @@ namespace conef {
 // select_finish for a tensor of at most kSelTailTiles tiles, word offsets included: its bitmap is
 // completed in shared memory (16 words per thread), so that nothing but the list and the bitmap
 // itself is waited for
-__device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
+__device__ __forceinline__ uint32_t select_finish_short(SelectSharedTiles &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
                                                         uint32_t *bits, uint32_t *tileoff, uint16_t *wordoff, uint32_t ntiles)
 {
     constexpr int PER = kSelTailWords / kSelThreads;   // a tile is 16 threads' words
@@ -28,9 +28,10 @@ __device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const S
             }
         }
     }
-    if (select_threshold(S, W, list, nlist, below) == 0xFFFFFFFFu)
+    const auto get = [list](uint32_t x) { return load_cg(&list[x]); };
+    if (select_threshold(S, W, get, nlist, below) == 0xFFFFFFFFu)
         return 0xFFFFFFFFu;
-    select_listed(S, W, list, nlist, [&](uint32_t j) { atomicOr(&S.words[j >> 5], 1u << (j & 31u)); });
+    select_listed(S, W, get, nlist, [&](uint32_t j) { atomicOr(&S.words[j >> 5], 1u << (j & 31u)); });
     __syncthreads();
     uint32_t word[PER], cnt = 0, total;
 #pragma unroll
@@ -66,7 +67,7 @@ __device__ __forceinline__ uint32_t select_finish_short(SelectShared &S, const S
 // at a time.
 __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_constant__ DevView V)
 {
-    __shared__ SelectShared S;
+    __shared__ SelectSharedTiles S;
     __shared__ uint32_t s_n, s_base, s_cnt[8], s_last, s_listed;
     grid_release();
     const int li = find_layer(V.pfx_hist, V.n_layers, blockIdx.x);
@@ -98,20 +99,9 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
             if (w * 32ull >= d)
                 break;
             const uint32_t j0 = w * 32u;
-            // not_below, above: bit q is the carry of h + (2^32 - bound), i.e. h >= bound; the lowest bit of
-            // the hash does not matter to the (even) bounds
-            uint32_t not_below = 0, above = 0;
-            const uint32_t nlo = 0u - lo, nhi = 0u - (hi + 1u);
-#pragma unroll
-            for (int q = 31; q >= 0; --q) {
-                const uint32_t h = hash32_but_lowest(st, (uint64_t)j0 + q);
-                asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %2, %3;\n\taddc.u32 %0, %0, %0;\n\t"
-                    "add.cc.u32 t, %2, %4;\n\taddc.u32 %1, %1, %1;\n\t}"
-                    : "+r"(not_below), "+r"(above) : "r"(h), "r"(nlo), "r"(nhi));
-            }
-            const uint32_t exist = d - j0 >= 32u ? 0xFFFFFFFFu : (1u << (d - j0)) - 1u;
-            const uint32_t word = lo ? ~not_below & exist : 0u;
-            for (uint32_t m = ~above & ~word & exist; m; m &= m - 1) {   // the few inside the window
+            uint32_t inside;
+            const uint32_t word = select_word(st, j0, d, lo, hi, inside);
+            for (uint32_t m = inside; m; m &= m - 1) {   // the few inside the window
                 const uint32_t j = j0 + (uint32_t)__ffs(m) - 1u;
                 const uint2 e = make_uint2(hash32(st, j), V.sel_how == CONEF_SELECT_STALE ? 0xFFFFFFFFu : j);
                 const uint32_t pos = atomicAdd(&s_n, 1u);
@@ -202,6 +192,35 @@ __global__ void __launch_bounds__(kSelThreads, 5) k_rk_select(const __grid_const
             atomicOr(V.status, ST_COUNT_MISMATCH);
         ctr[0] = ctr[1] = 0;
     }
+}
+
+// The same for models all of whose tensors have at most kSelClusterTiles tiles: a cluster per tensor, no counters,
+// one pass.
+static __global__ void __launch_bounds__(kSelThreads) k_rk_select_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+{
+    __shared__ SelectCluster S;
+    grid_release();
+    const uint32_t csize = cooperative_groups::this_cluster().num_blocks(), rank = cooperative_groups::this_cluster().block_rank();
+    const int li = find_layer(pfx, V.n_layers, blockIdx.x / csize);
+    const LayerDesc &L = V.layers[li];
+    const uint32_t d = (uint32_t)L.d, k = (uint32_t)L.k;
+    const uint64_t st = stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step);
+    const SelectResult R = select_in_cluster(S, st, d, k, L.sel_lo, L.sel_hi, L.sel_scale, V.sel_how == CONEF_SELECT_MISS);
+    grid_wait();
+    if (rank == 0 && threadIdx.x == 0) {
+        if (R.failed)
+            atomicOr(V.status, ST_SELECT_FAILED);
+        if (R.total != k)
+            atomicOr(V.status, ST_COUNT_MISMATCH);
+    }
+    if (rank * (uint32_t)kHistTile >= d)
+        return;
+    uint32_t all;
+    const uint32_t before = block_exclusive(__popc(R.word), S.wsum, all), w = rank * (kHistTile / 32) + threadIdx.x;
+    V.selbits[L.selbits_off + w] = R.word;   // (the arrays cover whole tiles; words past the tensor are zero)
+    V.wordoff[L.wordoff_off + w] = (uint16_t)before;
+    if (threadIdx.x == 0)
+        V.tileoff[L.tileoff_off + rank] = R.first;
 }
 
 // word offsets of the tensors with more than kSelTailTiles tiles: a warp per tile

@@ -13,11 +13,11 @@
 // Consumers read the bitmap (bit i of word w: element 32 w + i is a member) and
 //   slot(j) = tileoff[j / 8192] + wordoff[j / 32] + members of j's word below j.
 //
-// Bound by the integer pipe: 28 instructions per element (issue slots 69 % busy), eight of them multiplies, no memory
-// traffic to speak of.  Transformer-big list (210 M elements): a three-level radix select that hashed
-// everything three times took 1.26 ms in ten launches; this takes 0.25 ms in two (the hashing loop
-// alone, without anything around it, 0.17 ms).  One 256 x 512 matrix: 35 us in eleven launches -> 11 us.
+// Bound by the integer pipe, no memory traffic to speak of.  Transformer-big list (210 M elements): a three-level radix
+// select that hashed everything three times took 1.26 ms in ten launches; this takes 0.2 ms in two.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "conef_common.cuh"
 
 namespace conef {
@@ -30,17 +30,20 @@ constexpr int kSelList = 2304;          // window entries a CTA holds in shared 
 constexpr int kSelTiles = 1280;         // tile counts it holds there
 constexpr int kSelTailWords = kSelTailTiles * kHistTile / 32;
 
-// shared memory of the CTA that finishes a tensor
+// shared memory of the CTA that finds a tensor's threshold
 struct SelectShared {
     uint32_t hist[kSelBins];
     uint64_t keys[kSelList];
+    uint32_t wsum[kSelThreads / 32], wsum2[kSelThreads / 32];
+    uint64_t tau;
+    uint32_t bin, rem, n, bad;
+};
+// ... and of the CTA that finishes a tensor
+struct SelectSharedTiles : SelectShared {
     union {
         uint32_t tiles[kSelTiles];
         uint32_t words[kSelTailWords];
     };
-    uint32_t wsum[kSelThreads / 32], wsum2[kSelThreads / 32];
-    uint64_t tau;
-    uint32_t bin, rem, n, bad;
 };
 
 // A tensor's counters, one 64-bit word: listed elements in the low half, CTAs that have finished in the high
@@ -56,6 +59,27 @@ __device__ __forceinline__ bool select_ticket(uint32_t *ctr, uint32_t ncta, uint
         return false;
     __threadfence();   // (with the barrier that follows, for the whole CTA)
     return true;
+}
+
+// The 32 elements from j0 on (a multiple of 32, below d): bits of those whose hash is below the window [lo, hi],
+// and of those inside it.  lo is even and hi odd, so the lowest bit of the hash does not matter.
+__device__ __forceinline__ uint32_t select_word(uint64_t st, uint32_t j0, uint32_t d, uint32_t lo, uint32_t hi, uint32_t &inside)
+{
+    // bit q is the carry of h + (2^32 - bound), i.e. h >= bound
+    uint32_t not_below = 0, above = 0;
+    const uint32_t nlo = 0u - lo, nhi = 0u - (hi + 1u);
+    const uint64_t z0 = st + kGolden * ((uint64_t)j0 + 1);
+#pragma unroll
+    for (int q = 31; q >= 0; --q) {
+        const uint32_t h = hash32_but_lowest_of(z0 + kGolden * (uint64_t)q);
+        asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %2, %3;\n\taddc.u32 %0, %0, %0;\n\t"
+            "add.cc.u32 t, %2, %4;\n\taddc.u32 %1, %1, %1;\n\t}"
+            : "+r"(not_below), "+r"(above) : "r"(h), "r"(nlo), "r"(nhi));
+    }
+    const uint32_t exist = d - j0 >= 32u ? 0xFFFFFFFFu : (1u << (d - j0)) - 1u;
+    const uint32_t word = lo ? ~not_below & exist : 0u;
+    inside = ~above & ~word & exist;
+    return word;
 }
 
 // exclusive prefix over the CTA's threads of v; total: the sum over all threads; FRESH: wsum is not in use
@@ -153,12 +177,12 @@ struct SelectWindow {
     }
 };
 
-// The threshold among the window's elements.  `below_mine`: the calling thread's share of the number of
-// elements below the window.  The caller has zeroed S.hist[0 .. kSelThreads) and synchronised.  Returns
+// The threshold among the window's elements, get(x) for x < nlist.  `below_mine`: the calling thread's share of the
+// number of elements below the window.  The caller has zeroed S.hist[0 .. kSelThreads) and synchronised.  Returns
 // the number of elements below the window, or 0xFFFFFFFF where the window does not hold the threshold;
 // S.tau is the threshold key (0 when no listed element belongs).
-__device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
-                                                     uint32_t below_mine)
+template <class Get>
+__device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const SelectWindow &W, Get get, uint32_t nlist, uint32_t below_mine)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lo = W.lo, k = W.k;
@@ -169,7 +193,7 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const Sele
         auto bin_of = [&](uint32_t h) { return (uint32_t)(((uint64_t)(h - lo) * W.scale) >> 32); };
 #pragma unroll 4
         for (uint32_t x = tid; x < nlist; x += kSelThreads) {
-            const uint2 e = load_cg(&list[x]);
+            const uint2 e = get(x);
             S.keys[x] = ((uint64_t)e.x << 32) | e.y;
             if (W.holds(e))
                 atomicAdd(&S.hist[bin_of(e.x)], 1u);
@@ -251,7 +275,7 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const Sele
         return below;
 #pragma unroll 8
     for (uint32_t x = tid; x < nlist; x += kSelThreads) {
-        const uint2 e = load_cg(&list[x]);
+        const uint2 e = get(x);
         if (W.holds(e))
             atomicAdd(&S.hist[bin_of(e.x)], 1u);
         else
@@ -268,7 +292,7 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const Sele
     __syncthreads();
 #pragma unroll 8
     for (uint32_t x = tid; x < nlist; x += kSelThreads) {
-        const uint2 e = load_cg(&list[x]);
+        const uint2 e = get(x);
         if (bin_of(e.x) == bin) {
             const uint32_t pos = atomicAdd(&S.n, 1u);
             if (pos < (uint32_t)kSelList)
@@ -282,8 +306,8 @@ __device__ __forceinline__ uint32_t select_threshold(SelectShared &S, const Sele
 
 // calls f(j) for the listed elements that belong to the set; j < d, also where the list changed after
 // select_threshold looked at it
-template <class F>
-__device__ __forceinline__ void select_listed(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist, F f)
+template <class Get, class F>
+__device__ __forceinline__ void select_listed(SelectShared &S, const SelectWindow &W, Get get, uint32_t nlist, F f)
 {
     const uint64_t tau = S.tau;
     if (nlist <= (uint32_t)kSelList) {
@@ -293,7 +317,7 @@ __device__ __forceinline__ void select_listed(SelectShared &S, const SelectWindo
     } else {
 #pragma unroll 4
         for (uint32_t x = threadIdx.x; x < nlist; x += kSelThreads) {
-            const uint2 e = load_cg(&list[x]);
+            const uint2 e = get(x);
             if ((((uint64_t)e.x << 32) | e.y) <= tau && e.y < W.d)
                 f(e.y);
         }
@@ -342,6 +366,168 @@ static __device__ __noinline__ void select_exact(SelectShared &S, uint64_t st, u
     select_key(S, rank);
 }
 
+// ---- a tensor of at most kSelClusterTiles tiles: a cluster, one tile per CTA
+// Without it a selection is a chain of trips to L2 (a place in the list, a fence, the ticket, the bitmap and the list read
+// back) whatever the tensor's size.
+// Everything is exchanged through the CTAs' shared memory, and nothing in global memory is touched before the
+// result is written, so that all of it can run while the kernel ahead in the stream ends.
+constexpr int kSelClusterTiles = 16;
+constexpr int kSelMine = 1024;   // window elements of a CTA: expected 607 at most (d = 8192, k = d / 2), or a whole short tensor
+struct SelectCluster : SelectShared {
+    uint2 mine[kSelMine];
+    uint32_t words[kSelThreads];
+    uint32_t n_mine, below;                                       // this CTA's elements inside the window and below it
+    uint32_t base[kSelClusterTiles + 1], cnt[kSelClusterTiles];   // of the CTA that finds the threshold: the lists' places, members listed
+    uint64_t r_tau;                                               // what that CTA writes into all of them: the threshold key,
+    uint32_t r_first, r_total, r_found;                           // members before this CTA's tile and in all, whether the window held
+};
+struct SelectResult {
+    uint32_t word, first, total;   // this thread's 32 elements, members before this CTA's tile, members of the tensor
+    bool failed;
+};
+__device__ __forceinline__ SelectResult select_in_cluster(SelectCluster &S, uint64_t st, uint32_t d, uint32_t k, uint32_t lo, uint32_t hi,
+                                                          uint64_t scale, bool miss)
+{
+    static_assert(kHistTile == 32 * kSelThreads, "a word per thread");
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const uint32_t rank = cluster.block_rank(), csize = cluster.num_blocks();
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (d <= (uint32_t)kSelShortTensor) {   // the window is everything
+        lo = 0u;
+        hi = 0xFFFFFFFFu;
+        scale = 256u;
+    }
+    const SelectWindow W{lo, hi, d, k, scale, nullptr};
+    S.hist[tid] = 0;   // the bins of select_threshold
+    if (tid == 0)
+        S.n_mine = S.below = 0;
+    __syncthreads();
+    const uint32_t j0 = rank * (uint32_t)kHistTile + tid * 32u;
+    uint32_t word = 0;
+    if (j0 < d) {
+        uint32_t inside;
+        word = select_word(st, j0, d, lo, hi, inside);
+        for (; inside; inside &= inside - 1) {
+            const uint32_t j = j0 + (uint32_t)__ffs(inside) - 1u, pos = atomicAdd(&S.n_mine, 1u);
+            if (pos < (uint32_t)kSelMine)
+                S.mine[pos] = make_uint2(hash32(st, j), j);
+        }
+    }
+    const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(word));
+    if (lane == 0 && c)
+        atomicAdd(&S.below, c);
+    cluster.sync();
+    if (rank == 0) {
+        uint32_t below = 0, n = 0;
+        if (tid < 32) {   // (a CTA per lane)
+            if ((uint32_t)tid < csize) {
+                n = *cluster.map_shared_rank(&S.n_mine, tid);
+                below = *cluster.map_shared_rank(&S.below, tid);
+            }
+            const bool full = __any_sync(0xffffffffu, n > (uint32_t)kSelMine);
+            uint32_t inc = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o)
+                    inc += t;
+            }
+            if (tid < kSelClusterTiles) {
+                S.base[tid] = inc - n;
+                S.cnt[tid] = 0;
+            }
+            if (tid == kSelClusterTiles - 1) {
+                S.base[kSelClusterTiles] = inc;
+                S.r_found = !full && !miss;
+            }
+        }
+        __syncthreads();
+        const uint32_t nlist = S.base[kSelClusterTiles];
+        auto owner = [&](uint32_t x) {   // the CTA that listed entry x
+            uint32_t r = 0;
+#pragma unroll
+            for (uint32_t o = kSelClusterTiles / 2; o; o /= 2)
+                r += x >= S.base[r + o] ? o : 0u;
+            return r;
+        };
+        auto get = [&](uint32_t x) {
+            const uint32_t r = owner(x);
+            return cluster.map_shared_rank(S.mine, r)[x - S.base[r]];
+        };
+        const bool found = S.r_found && select_threshold(S, W, get, nlist, below) != 0xFFFFFFFFu;
+        __syncthreads();
+        if (found) {
+            const uint64_t tau = S.tau;
+            for (uint32_t x = tid; x < nlist; x += kSelThreads) {
+                uint64_t key;
+                if (nlist <= (uint32_t)kSelList) {
+                    key = S.keys[x];
+                } else {
+                    const uint2 e = get(x);
+                    key = ((uint64_t)e.x << 32) | e.y;
+                }
+                if (key <= tau)
+                    atomicAdd(&S.cnt[owner(x)], 1u);
+            }
+            __syncthreads();
+        } else {
+            select_exact(S, st, d, k);
+            __syncthreads();
+        }
+        if (tid < 32) {
+            const uint32_t m = found && (uint32_t)tid < csize ? below + S.cnt[tid & (kSelClusterTiles - 1)] : 0u;
+            uint32_t inc = m;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o)
+                    inc += t;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+            if ((uint32_t)tid < csize) {
+                SelectCluster *to = cluster.map_shared_rank(&S, tid);
+                to->r_tau = found || !S.bad ? S.tau : 0u;
+                to->r_first = inc - m;
+                to->r_total = total;
+                to->r_found = found ? 1u : S.bad ? 2u : 0u;
+            }
+        }
+    }
+    cluster.sync();
+    SelectResult R;
+    const uint64_t tau = S.r_tau;
+    R.failed = S.r_found == 2u;
+    if (S.r_found == 1u) {
+        S.words[tid] = word;
+        __syncthreads();
+        for (uint32_t x = tid; x < S.n_mine; x += kSelThreads) {
+            const uint2 e = S.mine[x];
+            if ((((uint64_t)e.x << 32) | e.y) <= tau)
+                atomicOr(&S.words[(e.y >> 5) & (kSelThreads - 1)], 1u << (e.y & 31u));
+        }
+        __syncthreads();
+        R.word = S.words[tid];
+        R.first = S.r_first;
+        R.total = S.r_total;
+    } else {   // the threshold is known, but not from the window: every element once more
+        word = 0;
+        for (uint32_t q = 0; q < 32 && j0 < d && j0 + q < d; ++q)
+            if ((((uint64_t)hash32(st, j0 + q) << 32) | (j0 + q)) <= tau)
+                word |= 1u << q;
+        R.word = word;
+        uint32_t mine;
+        block_exclusive(__popc(word), S.wsum, mine);
+        if (tid == 0)
+            S.below = mine;
+        cluster.sync();
+        uint32_t n = (uint32_t)lane < csize ? *cluster.map_shared_rank(&S.below, lane) : 0u;
+        R.total = __reduce_add_sync(0xffffffffu, n);
+        R.first = __reduce_add_sync(0xffffffffu, (uint32_t)lane < rank ? n : 0u);
+        cluster.sync();   // (no CTA leaves while its shared memory may still be read)
+    }
+    return R;
+}
+
 // exclusive scan of n counts in place by the CTA; returns the total
 __device__ __forceinline__ uint32_t scan_counts(uint32_t *cnt, int64_t n, uint32_t *wsum)
 {
@@ -371,7 +557,7 @@ __device__ __forceinline__ uint32_t scan_counts(uint32_t *cnt, int64_t n, uint32
 // into exclusive offsets, in place.  Returns the number of members, or 0xFFFFFFFF where the window
 // does not hold the threshold (nothing is marked then).
 template <uint32_t TILE, class Mark>
-__device__ __forceinline__ uint32_t select_finish(SelectShared &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
+__device__ __forceinline__ uint32_t select_finish(SelectSharedTiles &S, const SelectWindow &W, const uint2 *list, uint32_t nlist,
                                                   uint32_t *cnt, uint32_t ntiles, Mark mark)
 {
     const int tid = threadIdx.x;
@@ -384,9 +570,10 @@ __device__ __forceinline__ uint32_t select_finish(SelectShared &S, const SelectW
             S.tiles[t] = c;
         mine += c;
     }
-    if (select_threshold(S, W, list, nlist, mine) == 0xFFFFFFFFu)
+    const auto get = [list](uint32_t x) { return load_cg(&list[x]); };
+    if (select_threshold(S, W, get, nlist, mine) == 0xFFFFFFFFu)
         return 0xFFFFFFFFu;
-    select_listed(S, W, list, nlist, [&](uint32_t j) {
+    select_listed(S, W, get, nlist, [&](uint32_t j) {
         mark(j);
         atomicAdd(shared ? &S.tiles[j / TILE] : &cnt[j / TILE], 1u);
     });

@@ -14,7 +14,7 @@ constexpr int kApplySparse = 1024;    // message values per CTA where it is spar
 // rows; a thread keeps its columns' rows of Q in registers and walks ap_rpt rows, ap_ty apart.
 inline void apply_classify(LayerDesc &L)
 {
-    L.ap_vec = (L.cols % 4 == 0 && L.g_off % 4 == 0) ? 4 : 1;
+    L.ap_vec = ((L.cols | L.g_off) & 3) == 0 ? 4 : ((L.cols | L.g_off) & 1) == 0 ? 2 : 1;
     const int64_t ncg = (L.cols + L.ap_vec - 1) / L.ap_vec;
     // column tiles of equal width: as few as leave at most 7 % of the threads idle, else the best of eight
     const int64_t ct0 = (ncg + kApplyThreads - 1) / kApplyThreads;
@@ -51,7 +51,8 @@ inline int64_t apply_tiles(LayerDesc &L, int qkind)
 // of the factors lie on 16-byte boundaries.  HBM-bound (8 bytes per element).  GPT-2-XL list, rank 4:
 // one column per thread and 16 rows one after the other took 3.76 ms (3.3 TB/s); four columns and
 // eight rows in flight take 2.09 ms (6.0 TB/s); four rows in flight 2.21 ms, eight under a
-// 64-register cap (spills) 3.1 ms.  GPT-2-small list, rank 8: 324 -> 193 us.
+// 64-register cap (spills) 3.1 ms.  GPT-2-small list, rank 8: 324 -> 193 us.  Odd recurrent layers (33279 x 650 among
+// them), rank 2: one column per thread 60 us, two where rows lie on 8-byte boundaries 48 us.
 template <int RK, int VEC, int B, bool FV>
 __device__ __forceinline__ void apply_lowrank(const DevView &V, const LayerDesc &L, uint32_t tile, float *__restrict__ xs,
                                               bool aligned)
@@ -89,6 +90,9 @@ __device__ __forceinline__ void apply_lowrank(const DevView &V, const LayerDesc 
         if (VEC == 4 && aligned) {
             const float4 t = *(const float4 *)p;
             xv[0] = t.x; xv[1 % VEC] = t.y; xv[2 % VEC] = t.z; xv[3 % VEC] = t.w;
+        } else if (VEC == 2 && aligned) {
+            const float2 t = *(const float2 *)p;
+            xv[0] = t.x; xv[1 % VEC] = t.y;
         } else {
 #pragma unroll
             for (int v = 0; v < VEC; ++v)
@@ -107,6 +111,8 @@ __device__ __forceinline__ void apply_lowrank(const DevView &V, const LayerDesc 
         }
         if (VEC == 4 && aligned) {
             *(float4 *)p = make_float4(xv[0], xv[1 % VEC], xv[2 % VEC], xv[3 % VEC]);
+        } else if (VEC == 2 && aligned) {
+            *(float2 *)p = make_float2(xv[0], xv[1 % VEC]);
         } else {
 #pragma unroll
             for (int v = 0; v < VEC; ++v)
@@ -213,7 +219,7 @@ k_apply(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, floa
         // Tensors thinner than the configured rank take the run-time rank.
         const bool exact = R > 0 && L.rank == R;
         const bool fv = ((L.msgp_off | L.msgq_off) & 3) == 0;
-        const bool aligned = ((uintptr_t)xs & 15) == 0;
+        const bool aligned = ((uintptr_t)xs & (L.ap_vec == 2 ? 7 : 15)) == 0;
         constexpr int RX = R > 0 ? R : 0;
         if (L.ap_vec == 4) {
             if (exact && R >= 4 && fv)
@@ -222,6 +228,11 @@ k_apply(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, floa
                 apply_lowrank<RX, 4, 4, false>(V, L, tile, xs, aligned);
             else
                 apply_lowrank<0, 4, 1, false>(V, L, tile, xs, aligned);
+        } else if (L.ap_vec == 2) {
+            if (exact)
+                apply_lowrank<RX, 2, 8, false>(V, L, tile, xs, aligned);
+            else
+                apply_lowrank<0, 2, 2, false>(V, L, tile, xs, aligned);
         } else {
             if (exact)
                 apply_lowrank<RX, 1, 8, false>(V, L, tile, xs, false);

@@ -78,3 +78,33 @@ def test_free_running_lowrank_update_is_close():
     o.apply_update(xh, res)
     eng.apply_update(xd, out)
     assert pu.frob_err(xd.cpu().numpy(), xh) <= pu.FROB
+
+
+@pytest.mark.parametrize("rank", [1, 2, 3, 8])
+def test_lowrank_update_of_even_widths_and_offsets(rank):
+    """Two columns per thread where a matrix's rows lie on 8-byte boundaries, one elsewhere."""
+    from paper_2312_08538_b200 import binding as b
+    tensors = [(37, 54, 1), (9, 2, 1), (129, 650, 1), (5, 1, 0), (64, 30, 1), (33, 102, 1)]
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    q0 = torch.randn(sum(c * min(rank, r, c) for r, c, k in tensors if k), generator=gen, device="cuda")
+    eng = b.ConEF(tensors, 1, dict(kind="lowrank", rank=rank), dict(kind="int8", block=256), 0.1, q_init=q0)
+    total = sum(r * c for r, c, _ in tensors)
+    g = [torch.randn(total, generator=gen, device="cuda")]
+    for shift in (0, 1):   # (the parameters themselves may lie off that boundary)
+        x = torch.randn(total + 1, generator=gen, device="cuda")[shift:total + shift]
+        before = x.clone()
+        sums = eng.full_step(shift, g)
+        eng.apply_update(x, sums)
+        off = 0
+        for l, (r, c, k) in enumerate(tensors):
+            want = before[off:off + r * c].view(r, c)
+            if k:
+                f = eng.factors(l, 0)
+                d = torch.zeros(r, c, dtype=torch.float64, device="cuda")
+                for a in range(f["rank"]):   # an fma chain over ascending columns: one rounding per term
+                    d = (f["p_hat"][:, a:a + 1].double() * f["q_prev"][:, a].double() + d).float().double()
+                # (the chain above rounds twice, to double and to float: now and then one unit in the last place off)
+                bound = 2.0 ** -22 * (want.abs() + d.abs().float())
+                assert bool(((x[off:off + r * c].view(r, c) - (want - d.float())).abs() <= bound).all()), (shift, l)
+            off += r * c

@@ -404,7 +404,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                     L.p2_rows_fast = groups;
                     L.f_j = (int32_t)(slabs * (kRsThreads / 32));
                     tiles[T_RS_P12] = (int)(groups * slabs);
-                    tiles[T_RS_P1C] = (int)ceil_div(L.rows * r, 256);
+                    tiles[T_RS_P1C] = (int)ceil_div(L.rows * r, 1024);
                     L.pp_off = P.ppart_stride;
                     P.ppart_stride += (int64_t)L.f_j * L.rows * r;
                 } else if (L.fast) {

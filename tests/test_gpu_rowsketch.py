@@ -121,3 +121,18 @@ def test_half_precision_sketch_lowrank_teacher_forced():
     cfg["n_workers"] = 2
     cfg["c"] = dict(kind="rowsketch", cs_rows=1, cs_col_div=4, seed=5, beta=0.9, scale_dtype="fp16")
     lowrank_teacher_forced(cfg, 3, fast=True)
+
+
+@pytest.mark.parametrize("q", [dict(kind="lowrank", rank=4), dict(kind="lowrank", rank=3), dict(kind="randk", k_num=3, k_den=100, seed=4),
+                               dict(kind="randblock", k_num=1, k_den=10, seed=4), dict(kind="identity")])
+@pytest.mark.parametrize("div,scale", [(10, "fp32"), (60, "fp16")])
+def test_walk_over_buckets(q, div, scale):
+    """More rows in eight buckets than are staged at a time, buckets without rows, more bucket groups than are added
+    singly, columns that end inside a CTA."""
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=[(900, 516, 1), (7, 1, 0), (2700, 36, 1), (12, 1028, 1)], n_workers=2, q=q, grad="normal1e-3",
+               c=dict(kind="rowsketch", cs_rows=1, cs_col_div=div, seed=3, beta=0.9, scale_dtype=scale))
+    if q["kind"] == "lowrank":
+        lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)
+    else:
+        run_single_phase(cfg, 3, exact_values=True)

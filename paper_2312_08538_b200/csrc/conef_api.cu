@@ -366,7 +366,6 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 L.p2_rows_generic = rtiles;
                 tiles[T_P1] = (int)ceil_div(L.rows, kP1RowsPerCta);
                 tiles[T_P2] = (int)(rtiles * ceil_div(L.cols, kP2ColsPerCta));
-                tiles[T_Q2] = (int)ceil_div(L.cols * r, kQ2PerCta);
                 const int64_t gs_cta = gs_rows_per_cta(q->rank <= 4 ? 4 : 8);
                 if (L.rows <= gs_cta)
                     tiles[T_GS_ONE] = 1;
@@ -447,6 +446,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                     tiles[T_SLOW_P1] = tiles[T_P1];
                     tiles[T_SLOW_P2] = tiles[T_P2];
                 }
+                // (many partials: fewer entries per CTA)
+                L.q2_per = std::max(L.p2_rows_generic, L.p2_rows_fast) >= kQ2Many ? kQ2Few : kQ2PerCta;
+                tiles[T_Q2] = (int)ceil_div(L.cols * r, L.q2_per);
                 if (!L.f_fused)
                     tiles[T_Q2_NF] = tiles[T_Q2];
                 L.part_off = P.part_stride;

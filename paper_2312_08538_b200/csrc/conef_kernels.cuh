@@ -478,6 +478,72 @@ __global__ void __launch_bounds__(kP2ColsPerCta) k_lr_pass2(const __grid_constan
 // Q_i = sum over the row tiles' partials, in tile order: four consecutive (column, c) entries per
 // thread, 16-byte loads where the tensor's offsets allow, the loads of four tiles in flight
 constexpr int kQ2PerCta = 1024;
+// A tensor with many tiles (tall ones; the bucket groups of a row sketch): the chain of sums is long, and the few CTAs
+// that kQ2PerCta leaves it waited for four loads at a time.  A CTA then takes kQ2Few entries; its warps bring 64 tiles at
+// a time into shared memory, the next ones while one thread per entry adds those.
+// GPT-2-small list on a row sketch (628 bucket groups for the embedding): 77 -> 17 us; odd recurrent layers (131 tiles) 20 -> 7.
+constexpr int kQ2Many = 32, kQ2Few = 128;
+__device__ __forceinline__ void q2_reduce_many(const DevView &V, const LayerDesc &L, int64_t q0)
+{
+    constexpr int ROUND = 64, PER = ROUND / 8;   // tiles at a time, of which a thread brings PER
+    __shared__ __align__(16) float sum[ROUND][kQ2Few];
+    const int worker = blockIdx.y, tid = threadIdx.x;
+    const int64_t mr = L.cols * L.rank;
+    const int64_t ntiles = (V.fast_on && L.fast) ? L.p2_rows_fast : L.p2_rows_generic;
+    const float *__restrict__ part = V.part + worker * V.part_stride + L.part_off;
+    float *__restrict__ out = V.msgq + worker * V.msgq_stride + L.msgq_off;
+    const int n = (int)min((int64_t)kQ2Few, mr - q0);
+    if (mr % 4 != 0 || ((V.part_stride | L.part_off) & 3) != 0) {
+        if (tid < n) {
+            float acc = part[q0 + tid];
+#pragma unroll 8
+            for (int64_t t = 1; t < ntiles; ++t)
+                acc = __fadd_rn(acc, part[t * mr + q0 + tid]);
+            out[q0 + tid] = acc;
+        }
+        return;
+    }
+    const int c4 = (tid & 31) * 4, ty = tid >> 5;
+    float4 v[PER];
+    auto fetch = [&](int64_t t0) {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int64_t t = t0 + ty + 8 * u;
+            v[u] = t < ntiles && c4 < n ? __ldcs((const float4 *)(part + t * mr + q0 + c4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    fetch(0);
+    float acc = 0.f;
+    for (int64_t t0 = 0; t0 < ntiles; t0 += ROUND) {
+        if (t0)
+            __syncthreads();   // (the previous tiles are added)
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            *(float4 *)&sum[ty + 8 * u][c4] = v[u];
+        __syncthreads();
+        if (t0 + ROUND < ntiles)
+            fetch(t0 + ROUND);
+        if (tid < kQ2Few) {
+            const int have = (int)min((int64_t)ROUND, ntiles - t0);
+            int t = 0;
+            if (t0 == 0)
+                acc = sum[t++][tid];
+            for (; t + 8 <= have; t += 8) {
+                float x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    x[u] = sum[t + u][tid];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    acc = __fadd_rn(acc, x[u]);
+            }
+            for (; t < have; ++t)
+                acc = __fadd_rn(acc, sum[t][tid]);
+        }
+    }
+    if (tid < n)
+        out[q0 + tid] = acc;
+}
 __global__ void __launch_bounds__(256) k_lr_pass2_reduce(const __grid_constant__ DevView V)
 {
     grid_release();
@@ -486,6 +552,10 @@ __global__ void __launch_bounds__(256) k_lr_pass2_reduce(const __grid_constant__
     grid_wait();
     const int worker = blockIdx.y;
     const int64_t mr = L.cols * L.rank;
+    if (L.q2_per == kQ2Few) {
+        q2_reduce_many(V, L, (int64_t)(blockIdx.x - V.pfx_q2[li]) * kQ2Few);
+        return;
+    }
     const int64_t q = ((int64_t)(blockIdx.x - V.pfx_q2[li]) * 256 + threadIdx.x) * 4;
     if (q >= mr)
         return;

@@ -19,6 +19,7 @@
 #include "conef_decode.cuh"
 #include "conef_dense.cuh"
 #include "conef_fast.cuh"
+#include "conef_fastmulti.cuh"
 #include "conef_lrgen.cuh"
 #include "conef_gs.cuh"
 #include "conef_flat16.cuh"
@@ -33,7 +34,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 34 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 39 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -47,6 +48,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_DECODE,                                            // tiles of the stored error expanded (dec_batch) or of the step on a dense error (kDecTile elements)
        T_IL, T_ILT,                                         // count sketch, workers interleaved: tiles of elements, of sketch entries
        T_GEN1, T_GEN2, T_GEN3,                              // low-rank passes for any shape
+       T_MULTI1, T_MULTI2, T_MULTI3, T_MULTINF2, T_MULTINF3, // passes over all tensors in one launch; 2, 3 without the fused kernel's tensors
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -83,6 +85,8 @@ struct Plan {
     int fast_unit = 256;            // elements per quantisation block
     bool any_fast = false, any_slow = false, any_rs12 = false, any_gen = false;
     bool short_tiles = false;   // tile lengths of the tuned passes below their limits
+    bool multi = false;         // one launch per pass takes all tensors (conef_fastmulti.cuh)
+    size_t multi_smem[3] = {2048, 2048, 2048};   // ... with this much shared memory per CTA
     bool any_fv = false;        // some tensor takes the tuned fused step (conef_flatvec.cuh)
     int fv_tiles = 1;           // ... with this many selection tiles per CTA
     int sel_tiles = 1;          // random-k selection: tiles hashed per CTA
@@ -458,6 +462,34 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
         tiles[T_APPLY] = (int)apply_tiles(L, q->kind);
         for (int k = 0; k < kNumTables; ++k)
             P.pfx[k][l + 1] = P.pfx[k][l] + tiles[k];
+    }
+    if (P.short_tiles && P.any_fast) {
+        P.multi = true;
+        const int sb = scale_bytes, cw = c->kind == CONEF_C_INT4 ? 1 : 2;
+        for (int l = 0; l < n_tensors; ++l) {
+            LayerDesc &L = P.layers[l];
+            int t[5] = {0, 0, 0, 0, 0};
+            if (!L.compressed) {
+                t[0] = P.pfx[T_PASS][l + 1] - P.pfx[T_PASS][l];
+            } else if (L.fast == 1) {
+                multi_classify(L, c->kind, sb);
+                const int rt[3] = {L.f_rt1, L.f_rt2, L.f_rt3}, its[3] = {L.f_it1, L.f_it2, L.f_it3};
+                for (int p = 0; p < 3; ++p) {
+                    if (p > 0 || P.pfx[T_FAST_P1][l + 1] > P.pfx[T_FAST_P1][l]) {   // (else pass 1 has a row per lane)
+                        t[p] = (int)ceil_div((int64_t)rt[p] * L.f_ncg, L.f_nsub);
+                        P.multi_smem[p] = std::max(P.multi_smem[p], L.f_nsub * multi_tile_bytes(p + 1, L.rank, cw, sb, its[p], L.f_subs, L.f_threads, L.unit));
+                    }
+                    if (p > 0 && !L.f_fused)
+                        t[2 + p] = t[p];
+                }
+            } else if (L.fast == 3) {
+                t[0] = L.g_t1;
+                t[1] = t[3] = L.g_t2;
+                t[2] = t[4] = L.g_t3 * L.g_groups;
+            }
+            for (int p = 0; p < 5; ++p)
+                P.pfx[T_MULTI1 + p][l + 1] = P.pfx[T_MULTI1 + p][l] + t[p];
+        }
     }
     P.state_stride = state_off;
     for (int k = 0; k < 4; ++k)
@@ -842,6 +874,15 @@ int launch_p1_rest(conef_ctx *ctx, const DevView &V, cudaStream_t s)
 int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool skip_fused = false)
 {
     const Plan &P = ctx->plan;
+    if (P.multi) {
+        const int table = skip_fused && pass >= 2 ? T_MULTINF2 + pass - 2 : T_MULTI1 + pass - 1;
+        if (tiles_of(ctx, table) > 0) {
+            CK_CUDA(multi_launch(pass, ctx->c.kind, ctx->q.rank, V.scale_half, V, table_ptr(ctx, table), tiles_of(ctx, table), s, ctx->chain(),
+                                 P.multi_smem[pass - 1]));
+            LAUNCH_CHECK(ctx);
+        }
+        return pass == 1 ? launch_p1_rest(ctx, V, s) : CONEF_OK;
+    }
     // The classes touch different tensors: all but the first go to side streams that fork from
     // and join back into the caller's stream, so that their (often small) grids share the GPU.
     const bool side = ctx->n_aux > 0 && P.fast_threads.size() > 1;
@@ -1279,7 +1320,8 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
     const bool fast = (ctx->fast && (ctx->plan.any_fast ? aligned32 : ctx->plan.any_gen)) || rs12;
     int rc = CONEF_OK;
 
-    if (phase == 0 && tiles_of(ctx, T_PASS) > 0) {
+    const bool multi = lowrank && fast && !rs12 && ctx->plan.multi;   // (its pass 1 takes the 1-D tensors along)
+    if (phase == 0 && tiles_of(ctx, T_PASS) > 0 && !multi) {
         dim3 grid(tiles_of(ctx, T_PASS), ctx->n_workers);
         launch(ctx->chain(), k_passthrough, grid, 256, 0, s, V);
         LAUNCH_CHECK(ctx);
@@ -1358,7 +1400,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             rc = launch_fused(ctx, V, s, phase == 4);
         auto launch_gen = [&](int pass) -> int {
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
-            if (n == 0)
+            if (n == 0 || multi)
                 return CONEF_OK;
             CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->chain()));
             LAUNCH_CHECK(ctx);

@@ -79,6 +79,29 @@ __device__ __forceinline__ void load_cg(const uint32_t *p, uint32_t (&v)[8])   /
                  : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p + 4) : "memory");
 }
 
+// one tile of a 1-D tensor that passes through, by 256 threads: message eta g
+__device__ __forceinline__ void pass_tile(const DevView &V, const LayerDesc &L, int tile)
+{
+    constexpr int PER = kPassTile / 256;
+    const int worker = blockIdx.y;
+    const int64_t j0 = (int64_t)tile * kPassTile;
+    const float *__restrict__ g = V.grads[worker] + L.g_off + j0;
+    float *__restrict__ out = V.msg1d + worker * V.msg1d_stride + L.msg1d_off + j0;
+    const int n = (int)min((int64_t)kPassTile, L.d - j0);
+    float v[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int q = u * 256 + threadIdx.x;
+        v[u] = q < n ? __ldcs(g + q) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int q = u * 256 + threadIdx.x;
+        if (q < n)
+            out[q] = __fmul_rn(V.lr, v[u]);
+    }
+}
+
 __device__ __forceinline__ float warp_max(float v)
 {
 #pragma unroll

@@ -100,15 +100,19 @@ constexpr int kFastMaxWarps = 8;     // warps per CTA, passes 2 and 3
 // even an iteration ahead, they held the warp for an L2 round trip per iteration (a wait on the
 // scoreboard such a load shares ends only when the youngest load on it has returned).
 constexpr int kFastStageIt = 64;
+// In the launch over all tensors (conef_fastmulti.cuh), whose CTAs hold several tiles with a stage each: a quarter, so that
+// three CTAs share an SM (ResNet-50 list, tiles of 16 iterations: 481 -> 458 us per step)
+constexpr int kMultiStageIt = 16;
 #ifndef CONEF_PAIRS
 #define CONEF_PAIRS 1
 #endif
 __host__ __device__ constexpr bool pairs_pass(int pass) { return CONEF_PAIRS != 0 && pass == 3; }
 // bytes of that stage: per iteration `subs` rows of P_hat (passes 2, 3) and threads * 8 / unit scales
-inline size_t fast_stage_bytes(int pass, int rank, int it, int subs, int threads, int unit, int scale_bytes)
+__host__ __device__ inline size_t fast_stage_bytes(int pass, int rank, int it, int subs, int threads, int unit, int scale_bytes,
+                                                             int stage_it = kFastStageIt)
 {
     const size_t ph = pass == 1 ? 0 : (size_t)subs * rank * 4 * (pairs_pass(pass) ? 2 : 1);
-    return (size_t)std::min(it, kFastStageIt) * (ph + (size_t)(threads * kFastE / unit) * scale_bytes) + 16;
+    return (size_t)(it < stage_it ? it : stage_it) * (ph + (size_t)(threads * kFastE / unit) * scale_bytes) + 16;
 }
 
 inline int64_t gcd64(int64_t a, int64_t b)
@@ -245,14 +249,13 @@ __device__ __forceinline__ void static_for(F &&f)
 // usual 160-thread CTAs share an SM; rank 8 keeps its 128 registers.
 // PARTIAL: partial error feedback, Alg. 4: p = eta g + (1 - beta) e with the product rounded first,
 // and the stored error is C(beta e + r).  A template parameter so that Alg. 2 pays nothing for it.
-template <int PASS, int CK, int R, bool HALF, bool SHORT, bool NARROW, bool PARTIAL = false>
-__global__ void __launch_bounds__(kFastMaxWarps * 32, min_ctas(PASS, R))
-k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+// Tile `local` of a tensor by the bd threads of a CTA, or with MULTI by bd of its threads, which meet at barrier
+// `bar` of the CTA and have smem_raw for themselves.
+template <int PASS, int CK, int R, bool HALF, bool SHORT, bool NARROW, bool PARTIAL, bool MULTI>
+__device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp, const uint32_t local, const int tid, const int bd,
+                                          uint8_t *smem_raw, const int bar)
 {
-    extern __shared__ __align__(128) uint8_t smem_raw[];
-    grid_release();
-    const int li = find_layer(pfx, V.n_layers, blockIdx.x);
-    const LayerDesc *Lp = V.layers + li;
+    constexpr int kStageIt = MULTI ? kMultiStageIt : kFastStageIt;
     // everything the loop needs goes to registers first
     const uint32_t m = (uint32_t)Lp->cols, d = (uint32_t)Lp->d, P = (uint32_t)Lp->f_lcm;
     const uint32_t subs = (uint32_t)Lp->f_subs, ncg = (uint32_t)Lp->f_ncg;
@@ -260,8 +263,13 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     const int unit_shift = 31 - __clz(Lp->unit);
     const int lpb = Lp->unit >> 3;   // lanes per quantisation block
     const int worker = blockIdx.y;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int bd = blockDim.x;
+    const int lane = tid & 31;
+    auto meet = [&] {
+        if (MULTI)
+            asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(bd) : "memory");
+        else
+            __syncthreads();
+    };
     // tile length: a constant for large models (faster than the same value read from the table),
     // the table's value for small ones
     const uint32_t IT = SHORT ? (uint32_t)(PASS == 1 ? Lp->f_it1 : PASS == 2 ? Lp->f_it2 : Lp->f_it3)
@@ -270,7 +278,6 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     constexpr int NI = iters_per_step(PASS, R);                   // iterations a thread works on at once
     constexpr int CW = (CK == CONEF_C_INT4) ? 1 : 2;        // code words per thread and iteration
     constexpr int SB = HALF ? 2 : 4;                        // bytes per scale
-    const uint32_t local = blockIdx.x - pfx[li];
     const uint32_t cg = local % ncg, rt = local / ncg;
     const uint32_t off = cg * (uint32_t)Lp->f_cw + (uint32_t)tid * kFastE;   // within the period
     const uint32_t sub = off / m, col = off - sub * m;
@@ -298,10 +305,10 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     // yields two ready operands
     constexpr bool PAIR = pairs_pass(PASS) && !PARTIAL && HALF;   // (fp32 scales: the two-step decode made it slower)
     constexpr int PHW = PAIR ? 2 : 1;   // staged floats per element of a row of P_hat
-    // the rows of P_hat and the block scales of kFastStageIt iterations at a time, staged by the CTA behind the ring
+    // the rows of P_hat and the block scales of kStageIt iterations at a time, staged by the CTA behind the ring
     const uint32_t st_nb = ((uint32_t)bd * kFastE) >> unit_shift;               // blocks a CTA covers per iteration
     float *st_ph = (float *)(smem_raw + (size_t)kRing23 * bd * (32 + 4 * CW));
-    uint8_t *st_sc = (uint8_t *)(st_ph + (PASS == 1 ? 0 : (size_t)min(IT, (uint32_t)kFastStageIt) * subs * R * PHW));
+    uint8_t *st_sc = (uint8_t *)(st_ph + (PASS == 1 ? 0 : (size_t)min(IT, (uint32_t)kStageIt) * subs * R * PHW));
 
     // pass 1: where this warp's row sums go.  rowA = the row (within the period) of the warp's first
     // lane; a warp straddles when its last lane is in the next row.  The totals of warp_reduce_many
@@ -652,13 +659,13 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     for (int s = 0; s < kRing23 - NI; ++s)
         issue(it0 + s, s);
     static_assert(kRing23 % NI == 0 && kRing23 > NI - 1, "steps tile the ring");
-    static_assert(kFastStageIt % kRing23 == 0, "chunks end on a ring boundary");
+    static_assert(kStageIt % kRing23 == 0, "chunks end on a ring boundary");
     // iterations [c0, c1) of the tile: their rows of P_hat (contiguous; rows past the matrix read as
     // zero) and their st_nb block scales each (blocks past the tensor read as zero).  A step of NI
     // iterations may reach past c1 at the end of the tile: those iterations are staged as zeros
     // (pass 2 multiplies its zero p by them).
     auto stage = [&](uint32_t c0, uint32_t c1) {
-        __syncthreads();   // every thread is done with the previous chunk
+        meet();   // every thread is done with the previous chunk
         const uint32_t cpad = (c1 - c0 + NI - 1) / NI * NI;
         if (PASS != 1) {
             const uint32_t n4 = (c1 - c0) * subs * (R / 4), n4pad = cpad * subs * (R / 4);
@@ -687,7 +694,7 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
             else
                 ((float *)st_sc)[i] = have ? ((const float *)sbase)[blk] : 0.f;
         }
-        __syncthreads();
+        meet();
         st_scp = st_sc + (((uint32_t)tid * kFastE) >> unit_shift) * SB;
         st_php = st_ph + sub * R * PHW;
     };
@@ -695,7 +702,7 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     uint32_t cend = it0;
     do {
         const uint32_t c0 = cend;
-        cend = min(c0 + (uint32_t)kFastStageIt, it1);
+        cend = min(c0 + (uint32_t)kStageIt, it1);
         stage(c0, cend);
         const uint32_t lim = min(it_full, cend);
         if constexpr (ring_unrolled(PASS, R)) {
@@ -732,6 +739,16 @@ k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
             for (int c = 0; c < R; c += 4)
                 *(float4 *)(part + q * R + c) = make_float4(frag[q][c], frag[q][c + 1], frag[q][c + 2], frag[q][c + 3]);
     }
+}
+
+template <int PASS, int CK, int R, bool HALF, bool SHORT, bool NARROW, bool PARTIAL = false>
+__global__ void __launch_bounds__(kFastMaxWarps * 32, min_ctas(PASS, R))
+k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+{
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    grid_release();
+    const int li = find_layer(pfx, V.n_layers, blockIdx.x);
+    fast_tile<PASS, CK, R, HALF, SHORT, NARROW, PARTIAL, false>(V, V.layers + li, blockIdx.x - pfx[li], threadIdx.x, blockDim.x, smem_raw, 0);
 }
 
 // P_i[row][c] = sum over the warps that meet the row, in warp order

@@ -1,0 +1,59 @@
+// One launch per low-rank pass over all tensors of a model of small or middling size (int8 / int4 error state).
+//
+// The tuned passes (conef_fast.cuh) take CTAs whose size follows from a tensor's width, so a model of many widths
+// took a launch per size on side streams, forked and joined by events, and a further launch for the tensors of
+// any other shape; with short tiles these cost as much as the passes.  Here every CTA has 256 threads: it holds
+// as many tiles of its tensor as fit (f_nsub, each with its own part of shared memory and its own barrier), or
+// one tile of the passes for any shape (conef_lrgen.cuh), or, in pass 1, of a 1-D tensor that passes through.
+// What a tile computes, and the order of its sums, is that of those kernels.
+// ResNet-50 list (seven widths and one odd convolution), int8, rank 4, four workers: 550 -> 440 us per step and update; six
+// aligned matrices of 17 M elements, int4, eight workers: 803 -> 750 us.  (64 registers, four CTAs per SM, spill: 577 us on the
+// first list; two CTAs: 485 us.)
+#pragma once
+#include "conef_fast.cuh"
+#include "conef_lrgen.cuh"
+
+namespace conef {
+
+constexpr int kMultiThreads = 256;
+constexpr size_t kMultiSmem = 72 * 1024;   // shared memory of a CTA's tiles, where more than one shares it: three CTAs per SM
+// Iterations per tile of passes 1 and 3 at most (pass 2's are part of the order of its sums): longer tiles leave the last
+// wave of CTAs nearly empty.  (ResNet-50 list: 8 iterations 554 us, 16 481, 32 457.)
+constexpr int kMultiIt = 32;
+constexpr int multi_ctas(int pass, int rank) { return rank == 4 ? 3 : min_ctas(pass, rank); }
+
+// bytes of shared memory of one tile
+__host__ __device__ inline size_t multi_tile_bytes(int pass, int rank, int code_words, int scale_bytes, int it, int subs, int threads, int unit)
+{
+    const size_t b = (size_t)ring_depth(pass, rank) * threads * (32 + 4 * code_words) + fast_stage_bytes(pass, rank, it, subs, threads, unit, scale_bytes, kMultiStageIt);
+    return (b + 127) / 128 * 128;
+}
+
+// Warps per tile (any divisor of the warps of a period) so that the CTAs are as full as possible, then as many as possible;
+// a tile's iterations stay those of the plan.
+inline void multi_classify(LayerDesc &L, int ckind, int scale_bytes)
+{
+    const int64_t nw = L.f_lcm / 256;
+    int best = 1;
+    for (int w = 1; w <= kFastMaxWarps; ++w)
+        if (nw % w == 0 && kFastMaxWarps / w * w >= kFastMaxWarps / best * best)
+            best = w;
+    L.f_cw = best * 256;
+    L.f_threads = best * 32;
+    L.f_ncg = (int32_t)(nw / best);
+    L.f_it1 = std::min(L.f_it1, kMultiIt);
+    L.f_it3 = std::min(L.f_it3, kMultiIt);
+    L.f_rt1 = (int32_t)((L.f_niter + L.f_it1 - 1) / L.f_it1);
+    L.f_rt3 = (int32_t)((L.f_niter + L.f_it3 - 1) / L.f_it3);
+    size_t most = 1;
+    const int its[3] = {L.f_it1, L.f_it2, L.f_it3};
+    for (int pass = 1; pass <= 3; ++pass)
+        most = std::max(most, multi_tile_bytes(pass, L.rank, ckind == CONEF_C_INT4 ? 1 : 2, scale_bytes, its[pass - 1], L.f_subs, L.f_threads, L.unit));
+    L.f_nsub = (int32_t)std::max<size_t>(1, std::min<size_t>(kMultiThreads / L.f_threads, kMultiSmem / most));
+}
+
+// the launch of one pass: conef_fastmulti.cu.  smem: the most that a CTA's tiles need
+cudaError_t multi_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s,
+                         bool chained, size_t smem);
+
+}  // namespace conef

@@ -72,6 +72,7 @@ struct LayerDesc {
     int32_t f_cw;        // elements of a super-row covered by one CTA
     int32_t f_threads;   // f_cw / 8
     int32_t f_ncg;       // column groups = f_lcm / f_cw
+    int32_t f_nsub;      // tiles that share a CTA of the launch over all tensors (conef_fastmulti.cuh)
     int32_t q2_per;      // entries of Q_i per CTA of the sum over pass 2's partials
     int32_t f_subs;      // rows per super-row
     int32_t f_rt1, f_rt2, f_rt3;  // row tiles of the three passes

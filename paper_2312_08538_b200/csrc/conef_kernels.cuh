@@ -12,21 +12,12 @@
 namespace conef {
 
 // ------------------------------------------------------------------ 1-D pass-through
-__global__ void __launch_bounds__(256) k_passthrough(const __grid_constant__ DevView V)
+static __global__ void __launch_bounds__(256) k_passthrough(const __grid_constant__ DevView V)
 {
     grid_release();
     const int li = find_layer(V.pfx_pass, V.n_layers, blockIdx.x);
-    const LayerDesc &L = V.layers[li];
-    const int worker = blockIdx.y;
-    const int64_t j0 = (int64_t)(blockIdx.x - V.pfx_pass[li]) * kPassTile;
-    const float *__restrict__ g = V.grads[worker] + L.g_off;
-    float *__restrict__ out = V.msg1d + worker * V.msg1d_stride + L.msg1d_off;
     grid_wait();
-    for (int q = threadIdx.x; q < kPassTile; q += 256) {
-        int64_t j = j0 + q;
-        if (j < L.d)
-            out[j] = __fmul_rn(V.lr, g[j]);
-    }
+    pass_tile(V, V.layers[li], blockIdx.x - V.pfx_pass[li]);
 }
 
 // ------------------------------------------------------------------ quantiser (S5, C1)

@@ -248,7 +248,9 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
 template <int CK, int R, int KB>
 __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L, uint32_t tile, uint8_t *bytes)
 {
-    constexpr int RM = R ? R : CONEF_MAX_RANK, K = kGenChunk / 32, NB = K / KB;   // KB * 32 elements per block
+    constexpr int RM = R ? R : CONEF_MAX_RANK, K = kGenChunk / 32;
+    const int bs = KB ? (KB == 8 ? 3 : KB == 4 ? 2 : KB == 2 ? 1 : 0) : 26 - __clz(L.unit);   // 32 << bs elements per block (KB << 5, or as configured)
+    const int NB = K >> bs;
     constexpr bool INT4 = CK == CONEF_C_INT4;
     constexpr int NW = INT4 ? 1 : 2;   // code words per lane
     const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -317,7 +319,7 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
                 raw = __shfl_sync(0xffffffffu, w[0], 4 * k + (lane >> 3)) >> (4 * (lane & 7));
             else
                 raw = __shfl_sync(0xffffffffu, w[NW == 2 ? k / 4 : 0], 8 * (k & 3) + (lane >> 2)) >> (8 * (lane & 3));
-            const float s = __shfl_sync(0xffffffffu, sv, k / KB);
+            const float s = __shfl_sync(0xffffffffu, sv, k >> bs);
             ek[k] = __fmul_rn(code_value<CK>(raw), s);
             res[k] = __fmaf_rn(lr, gv[k], __fmul_rn(omb, ek[k]));   // Alg. 2 (4) line 5
         }
@@ -365,14 +367,23 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
         }
         // block maxima: lane b takes block b's
         float amax = 0.f;
+        if constexpr (KB != 0) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            float x = 0.f;
+            for (int b = 0; b < K / KB; ++b) {
+                float x = 0.f;
 #pragma unroll
-            for (int k = 0; k < KB; ++k)
-                x = fmaxf(x, fabsf(res[b * KB + k]));
-            const float y = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));   // (not negative: ordered like integers)
-            amax = lane == b ? y : amax;
+                for (int k = 0; k < KB; ++k)
+                    x = fmaxf(x, fabsf(res[b * KB + k]));
+                const float y = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));   // (not negative: ordered like integers)
+                amax = lane == b ? y : amax;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float x = fmaxf(0.f, fabsf(res[k]));   // (a NaN counts as nothing, as above)
+                const float y = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+                amax = lane == k >> bs ? fmaxf(amax, y) : amax;
+            }
         }
         float s, inv;
         unsigned short hb = 0;
@@ -384,7 +395,7 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
         const bool clamp = __any_sync(0xffffffffu, !(__fmul_rn(amax, inv) < qm + 0.49f));   // (see quant_pack8)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            float x = __fmul_rn(res[k], __shfl_sync(0xffffffffu, inv, k / KB));
+            float x = __fmul_rn(res[k], __shfl_sync(0xffffffffu, inv, k >> bs));
             if (clamp)
                 x = fminf(fmaxf(x, -qm), qm);
             mine[32 * k + lane] = (uint8_t)__float_as_uint(__fadd_rn(x, 12582912.0f));   // the low byte is the code

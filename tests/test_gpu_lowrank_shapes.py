@@ -78,3 +78,16 @@ def test_order_of_sums(rank, c, many):
                     assert torch.equal(x[k], y[k]), (t, l, i, k)
         for e in both:
             e.reduce_messages(b.MSG_Q)
+
+
+@pytest.mark.parametrize("rank,c", [(4, dict(kind="int8", block=256)), (8, dict(kind="int4", block=128, scale_dtype="fp16")),
+                                    (4, dict(kind="int4", block=64, scale_dtype="fp16", beta=0.9)), (8, dict(kind="int8", block=32, scale_dtype="fp16"))])
+def test_all_widths_in_one_launch(rank, c):
+    """One launch per pass over narrow, middling and wide matrices (tiles that share a CTA, with a remainder), 1-D
+    tensors, and shapes that only the passes for any shape take; more tiles of a factor's sum than are added singly."""
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=[(41, 32, 1), (64, 1, 0), (33, 96, 1), (130, 256, 1), (2065, 320, 1), (21, 576, 1), (11, 1152, 1), (70, 147, 1),
+                        (2100, 1, 0), (301, 2048, 1), (3, 4608, 1), (8500, 37, 1)],
+               n_workers=2, q=dict(kind="lowrank", rank=rank), c=c, grad="normal1e-3")
+    from tests.test_gpu_parity import lowrank_teacher_forced
+    lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)

@@ -40,7 +40,11 @@ k_fast_multi(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
                     gen_p1_body<CK, 0, 1>(V, L, tile * (uint32_t)L.g_nr + x);
             }
         } else if (PASS == 2) {
-            if (exact)
+            if (L.g_coop && exact)
+                gen_p2_cta<CK, R>(V, L, tile, (float *)smem_raw);
+            else if (L.g_coop)
+                gen_p2_cta<CK, 0>(V, L, tile, (float *)smem_raw);
+            else if (exact)
                 gen_p2_body<CK, R>(V, L, tile);
             else
                 gen_p2_body<CK, 0>(V, L, tile);

@@ -82,8 +82,8 @@ struct LayerDesc {
     int64_t pp_off;      // floats, within a worker's pass-1 partial buffer
     int64_t f_niter;     // super-rows in the tensor
     // low-rank passes for any shape (conef_lrgen.cuh): rows per warp and CTAs of pass 1, CTAs of pass 2, steps
-    // per tile, chunks per step, CTAs per step and row of tiles of pass 3
-    int32_t g_nr, g_t1, g_t2, g_it, g_step, g_groups, g_t3;
+    // per tile, chunks per step, CTAs per step and row of tiles of pass 3; whether a CTA takes a tile of pass 2
+    int32_t g_nr, g_t1, g_t2, g_it, g_step, g_groups, g_t3, g_coop;
     // row sketch: uint32 words in the bucket tables (see DevView::rs)
     int64_t rs_info_off; // [v][rows]: bucket of a row | sign << 31
     int64_t rs_ptr_off;  // [v][w + 1]: start of each bucket's row list

@@ -31,17 +31,24 @@ constexpr int kGenCols = 32;     // pass 2: columns per warp
 constexpr int kGenChunk = 256;   // pass 3: elements per warp and step
 constexpr int kGenCtas = kPlanSMs * 6;   // CTAs a pass should have at least, where tiles can be made smaller
 
-// tile sizes for a model: rows per warp of pass 1 (4 or 1), steps per tile of pass 3
+// tile sizes for a model: rows per warp of pass 1 (4 or 1), steps per tile of pass 3, and whether a whole CTA takes a
+// tile of pass 2 (gen_p2_cta)
 struct GenPlan {
-    int nr = 4, it = 16;
+    int nr = 4, it = 16, coop = 0;
 };
+// Below this many warps of pass 2 a CTA takes a tile.  Steps without and with it, int8 / int4, ranks 1, 2 and 4: 20 k to 1 M
+// elements over all workers (50 to 270 warps) 48.6 -> 38.9, 44.9 -> 34.0, 54.8 -> 38.2 us, 5.1 M (1026 warps) 102 -> 83 us;
+// 15 M (2040) 135 -> 137 us, 45 M (4900) 420 -> 451, 50 M (7300) 447 -> 474.
+constexpr int64_t kGenCoop = kPlanSMs * 12;
 // rows: matrix rows of all workers, chunks: 256-element chunks.  Four rows share a row of Q, one row makes four
 // times the warps.  Steps with one and with four rows per warp, int4, rank 2: 3000 x 651 69.1 and 73.0 us,
 // 13000 x 651 91.3 and 92.5, 4001 x 6003 173 and 291; four matrices 40000 x 47 139 and 113, of four workers 444
 // and 323; 60000 x 333 of four workers 577 and 540.
-inline GenPlan gen_plan(int64_t rows, int64_t chunks)
+// tiles2: warps of pass 2.
+inline GenPlan gen_plan(int64_t rows, int64_t chunks, int64_t tiles2)
 {
     GenPlan G;
+    G.coop = tiles2 < kGenCoop;
     if (rows / 32 < kGenCtas)
         G.nr = 1;
     while (G.it > 1 && chunks / (8 * G.it) < kGenCtas)
@@ -60,7 +67,10 @@ inline void gen_classify(LayerDesc &L, const GenPlan &G)
     L.g_groups = (int32_t)((L.g_step + 7) / 8);
     const int64_t nc = (L.d + kGenChunk - 1) / kGenChunk;
     L.g_t1 = (int32_t)((L.rows + 8 * L.g_nr - 1) / (8 * L.g_nr));
-    L.g_t2 = (int32_t)((((L.rows + kP2RowsPerTile - 1) / kP2RowsPerTile) * ((L.cols + kGenCols - 1) / kGenCols) + 7) / 8);
+    L.g_coop = G.coop;
+    L.g_t2 = (int32_t)(((L.rows + kP2RowsPerTile - 1) / kP2RowsPerTile) * ((L.cols + kGenCols - 1) / kGenCols));
+    if (!G.coop)
+        L.g_t2 = (L.g_t2 + 7) / 8;
     L.g_t3 = (int32_t)((nc + (int64_t)L.g_step * L.g_it - 1) / ((int64_t)L.g_step * L.g_it));
 }
 
@@ -243,6 +253,64 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
                 if (R || c < r)
                     part[(size_t)(c0 + 32 * k) * r + c] = acc[k][c];
         }
+}
+
+// The same tile by a whole CTA, for models whose tiles do not fill the SMs: the eight warps form p of 32 rows each in shared
+// memory, then a warp per column of the factor adds down the rows, in the order of gen_p2_body.  There a warp walks the
+// 256 rows eight at a time, 32 waits for memory one after the other, however small the model.
+constexpr size_t kGenCoopSmem = (size_t)kP2RowsPerTile * (32 + CONEF_MAX_RANK) * 4;
+template <int CK, int R>
+__device__ __forceinline__ void gen_p2_cta(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
+{
+    constexpr int U = 16;   // rows in flight per warp
+    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
+    const uint32_t ct = (m + kGenCols - 1) / kGenCols, rt = tile / ct, c0 = (tile - rt * ct) * kGenCols + lane;
+    const uint32_t r_lo = rt * (uint32_t)kP2RowsPerTile, have = min(n - r_lo, (uint32_t)kP2RowsPerTile);
+    const uint8_t *__restrict__ st = fresh(V.state + worker * V.state_stride);
+    const uint8_t *__restrict__ codes = st + L.a_off, *__restrict__ scales = st + L.b_off;
+    const float *__restrict__ g = fresh(V.grads[worker] + L.g_off), *__restrict__ ph = fresh(V.phat + L.msgp_off) + (size_t)r_lo * r;
+    const int shift = 31 - __clz(L.unit);
+    const bool half = V.scale_half != 0;
+    const float lr = V.lr, omb = V.omb;
+    float *const p = smem, *const phs = smem + kP2RowsPerTile * 32;   // [row][column], [row][c]
+    for (uint32_t x = threadIdx.x; x < have * r; x += kGenThreads)
+        phs[x] = __ldg(ph + x);
+    const uint32_t col = min(c0, m - 1);   // (columns past the end repeat the last one and are not stored)
+    for (uint32_t a0 = warp; a0 < have; a0 += 8 * U) {
+        float gv[U], sc[U];
+        uint32_t w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {   // (rows past the end repeat the last one)
+            const uint32_t j = (r_lo + min(a0 + 8 * u, have - 1)) * m + col;
+            gv[u] = __ldg(g + j);
+            w[u] = code_raw<CK>(codes, j);
+            sc[u] = gen_scale(scales, j >> shift, half);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (a0 + 8 * u < have)
+                p[(a0 + 8 * u) * 32 + lane] = __fmaf_rn(lr, gv[u], __fmul_rn(omb, __fmul_rn(code_value<CK>(w[u]), sc[u])));
+    }
+    __syncthreads();
+    if (warp < r && c0 < m) {
+        float acc = 0.f;
+        uint32_t a = 0;
+        for (; a + 8 <= have; a += 8) {
+            float x[8], y[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                x[u] = p[(a + u) * 32 + lane];
+                y[u] = phs[(a + u) * r + warp];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                acc = __fmaf_rn(x[u], y[u], acc);
+        }
+        for (; a < have; ++a)
+            acc = __fmaf_rn(p[a * 32 + lane], phs[a * r + warp], acc);
+        V.part[worker * V.part_stride + L.part_off + ((size_t)rt * m + c0) * r + warp] = acc;
+    }
 }
 
 template <int CK, int R, int KB>
@@ -437,6 +505,7 @@ template <int PASS, int CK, int R, int KB>
 __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3 : 4) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     __shared__ __align__(16) uint8_t bytes[PASS == 3 ? 8 * kGenChunk : 16];
+    extern __shared__ __align__(16) float gen_smem[];
     grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
@@ -455,10 +524,16 @@ __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3
                 gen_p1_body<CK, 0, 1>(V, L, tile * (uint32_t)L.g_nr + x);
         }
     } else if (PASS == 2) {
-        if (R && exact)
+        if (L.g_coop) {
+            if (R && exact)
+                gen_p2_cta<CK, R>(V, L, tile, gen_smem);
+            else
+                gen_p2_cta<CK, 0>(V, L, tile, gen_smem);
+        } else if (R && exact) {
             gen_p2_body<CK, R>(V, L, tile);
-        else
+        } else {
             gen_p2_body<CK, 0>(V, L, tile);
+        }
     } else {
         if (R && exact)
             gen_p3_body<CK, R, KB>(V, L, tile, bytes);
@@ -467,7 +542,7 @@ __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3
     }
 }
 
-// launcher (conef_lrgen.cu)
-cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained);
+// launcher (conef_lrgen.cu); coop: the plan's
+cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained, bool coop);
 
 }  // namespace conef

@@ -78,3 +78,26 @@ def test_selections_whose_window_fails(how, k_num, k_den):
         out = torch.empty(k, dtype=torch.int32, device="cuda")
         b.conef_randk_indices_noalloc_select(seed, l, 1, d, k, code, out)
         assert np.array_equal(out.cpu().numpy().view(np.uint32), want), (r, c)
+
+
+# models whose tensors all have at most 16 tiles: one cluster per tensor, of as many CTAs as the largest has tiles
+@pytest.mark.parametrize("shapes", [[(1, 2), (32, 32), (1, 1025), (3, 999)], [(1, 8193), (5, 205)], [(3, 8192), (1, 4 * 8192)], [(16, 8192), (7, 9)]])
+@pytest.mark.parametrize("k_num,k_den", [(1, 100), (1, 2), (1, 1)])
+@pytest.mark.parametrize("how", ["NORMAL", "MISS"])
+def test_small_models_by_a_cluster(shapes, k_num, k_den, how):
+    from paper_2312_08538_b200 import binding as b
+    seed = 19
+    eng = b.ConEF([(r, c, 1) for r, c in shapes], 1, dict(kind="randk", k_num=k_num, k_den=k_den, seed=seed),
+                  dict(kind="int8", block=256), 0.1)
+    eng.set_select(getattr(b, "SELECT_" + how))
+    g = [torch.ones(sum(r * c for r, c in shapes), device="cuda")]
+    for step in (2, 3):
+        eng.step(step, g, 0)
+        for l, (r, c) in enumerate(shapes):
+            d, k = r * c, max(1, r * c * k_num // k_den)
+            want = orc.randk_indices(seed, l, step, d, k)
+            assert np.array_equal(eng.indices(l).cpu().numpy().view(np.uint32), want), (step, r, c)
+            out = torch.empty(k, dtype=torch.int32, device="cuda")
+            b.conef_randk_indices_noalloc_select(seed, l, step, d, k, getattr(b, "SELECT_" + how), out)
+            assert np.array_equal(out.cpu().numpy().view(np.uint32), want), (step, r, c)
+    assert eng.last_status() == 0

@@ -34,7 +34,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxFastClasses = 8;
-constexpr int kNumTables = 39 + 5 * kMaxFastClasses;
+constexpr int kNumTables = 40 + 5 * kMaxFastClasses;
 enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P1, T_SLOW_P2, T_FAST_P1,
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
@@ -49,6 +49,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_IL, T_ILT,                                         // count sketch, workers interleaved: tiles of elements, of sketch entries
        T_GEN1, T_GEN2, T_GEN3,                              // low-rank passes for any shape
        T_MULTI1, T_MULTI2, T_MULTI3, T_MULTINF2, T_MULTINF3, // passes over all tensors in one launch; 2, 3 without the fused kernel's tensors
+       T_DENSE,                                             // the step on a dense error: T_DECODE's tiles and those of 1-D tensors
        T_Q2_NF,                                             // pass-2 reduce over the tensors the fused passes 2 + 3 do not take
        T_FAST_CLASS0,                                       // + 3 c + {0, 1, 2}: tuned passes 1, 2, 3 of CTA-size class c
        T_FASTNF_CLASS0 = T_FAST_CLASS0 + 3 * kMaxFastClasses };   // + 2 c + {0, 1}: passes 2, 3 without the fused kernel's tensors
@@ -249,6 +250,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             L.msg1d_off = P.msg_elems[CONEF_MSG_DENSE1D];
             P.msg_elems[CONEF_MSG_DENSE1D] += L.d;
             tiles[T_PASS] = (int)ceil_div(L.d, kPassTile);
+            // 1-D tensors go along with the kernels that can take them (a launch of their own took 4 to 9 us)
+            tiles[T_FV] = c->iconef == 2 ? 0 : tiles[T_PASS];
+            tiles[T_DENSE] = tiles[T_GEN1] = tiles[T_PASS];
         } else {
             L.cidx = P.n_comp++;
             L.unit = unit;
@@ -291,7 +295,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             }
             tiles[T_FLAT] = (int)ceil_div(L.nunits, kFlatUnitsPerCta);
             tiles[T_GS] = 1;
-            tiles[T_DECODE] = (int)ceil_div(L.d, c->kind == CONEF_C_IDENTITY ? kDecTile : dec_tile(P.dec_batch));
+            tiles[T_DECODE] = tiles[T_DENSE] = (int)ceil_div(L.d, c->kind == CONEF_C_IDENTITY ? kDecTile : dec_tile(P.dec_batch));
             if (q->kind == CONEF_Q_IDENTITY) {
                 L.k = L.d;
             } else if (q->kind == CONEF_Q_RANDBLOCK) {
@@ -1324,8 +1328,12 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
     const bool fast = (ctx->fast && (ctx->plan.any_fast ? aligned32 : ctx->plan.any_gen)) || rs12;
     int rc = CONEF_OK;
 
-    const bool multi = lowrank && fast && !rs12 && ctx->plan.multi;   // (its pass 1 takes the 1-D tensors along)
-    if (phase == 0 && tiles_of(ctx, T_PASS) > 0 && !multi) {
+    const bool multi = lowrank && fast && !rs12 && ctx->plan.multi;
+    const bool dense = ctx->fast && ctx->c.kind == CONEF_C_IDENTITY && ctx->c.iconef == 0;
+    // whether one of the kernels below takes the 1-D tensors along
+    const bool with_1d = lowrank ? fast && !rs12   // (pass 1: the launch over all tensors, or that for any shape)
+                                 : dense || (ctx->fast && ctx->plan.any_fv && ctx->c.iconef != 2);
+    if (phase == 0 && tiles_of(ctx, T_PASS) > 0 && !with_1d) {
         dim3 grid(tiles_of(ctx, T_PASS), ctx->n_workers);
         launch(ctx->chain(), k_passthrough, grid, 256, 0, s, V);
         LAUNCH_CHECK(ctx);
@@ -1335,10 +1343,10 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
     const bool csk = ctx->fast && ctx->plan.any_csk;
     auto flat_step = [&](auto qk) -> int {
         constexpr int QK = decltype(qk)::value;
-        if (ctx->fast && ctx->c.kind == CONEF_C_IDENTITY && ctx->c.iconef == 0) {
-            const int n = tiles_of(ctx, T_DECODE);
+        if (dense) {
+            const int n = tiles_of(ctx, T_DENSE);
             if (n > 0) {
-                launch(ctx->chain(), k_flat_dense<QK>, dim3(n, ctx->n_workers), kDecThreads, 0, s, V, table_ptr(ctx, T_DECODE));
+                launch(ctx->chain(), k_flat_dense<QK>, dim3(n, ctx->n_workers), kDecThreads, 0, s, V, table_ptr(ctx, T_DENSE));
                 LAUNCH_CHECK(ctx);
             }
             return CONEF_OK;
@@ -1404,7 +1412,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             rc = launch_fused(ctx, V, s, phase == 4);
         auto launch_gen = [&](int pass) -> int {
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
-            if (n == 0 || multi)
+            if (n == 0 || multi || rs12)   // (the table may hold 1-D tensors alone, of a model on a row sketch)
                 return CONEF_OK;
             CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->chain(), ctx->plan.gen_coop));
             LAUNCH_CHECK(ctx);

@@ -96,6 +96,11 @@ __global__ void __launch_bounds__(kDecThreads) k_flat_dense(const __grid_constan
     grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
+    if (!L.compressed) {   // (a 1-D tensor: its message in the same launch)
+        grid_wait();
+        pass_tile(V, L, blockIdx.x - pfx[li]);
+        return;
+    }
     const uint32_t j0 = (blockIdx.x - pfx[li]) * (uint32_t)kDecTile, n = min((uint32_t)L.d - j0, (uint32_t)kDecTile);
     grid_wait();
     if (n == (uint32_t)kDecTile && ((uintptr_t)(V.grads[blockIdx.y] + L.g_off) & 15) == 0)

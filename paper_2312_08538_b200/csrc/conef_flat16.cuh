@@ -125,6 +125,11 @@ __global__ void __launch_bounds__(kF16Threads, f16_ctas(ICO)) k_flat16(const __g
     grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
+    if (!L.compressed) {   // (a 1-D tensor: its message in the same launch)
+        grid_wait();
+        pass_tile(V, L, blockIdx.x - pfx[li]);
+        return;
+    }
     const int worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t d = (uint32_t)L.d;
     const uint32_t tile0 = (blockIdx.x - pfx[li]) * (uint32_t)V.fv_tiles;

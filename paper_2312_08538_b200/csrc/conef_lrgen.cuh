@@ -511,6 +511,10 @@ __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3
     const LayerDesc &L = V.layers[li];
     const uint32_t tile = blockIdx.x - pfx[li];
     grid_wait();
+    if (PASS == 1 && !L.compressed) {   // (a 1-D tensor: its message in the same launch)
+        pass_tile(V, L, tile);
+        return;
+    }
     constexpr int VW = R == 8 ? 4 : R ? R : 1;   // floats per vector load
     const bool exact = R != 0 && L.rank == R && ((L.msgp_off | L.msgq_off) & (VW - 1)) == 0;
     if (PASS == 1) {

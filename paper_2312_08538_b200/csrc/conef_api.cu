@@ -92,7 +92,7 @@ struct Plan {
     bool any_fv = false;        // some tensor takes the tuned fused step (conef_flatvec.cuh)
     int fv_tiles = 1;           // ... with this many selection tiles per CTA
     int sel_tiles = 1;          // random-k selection: tiles hashed per CTA
-    int sel_cluster = 1;        // ... or CTAs per cluster where every tensor is selected by one, else 0
+    int sel_cluster = 1;        // ... or CTAs per cluster where every tensor is selected by one (kSelClusterTiles, kSelClusterIdle), else 0
     bool any_fused = false;     // some tensor takes the fused passes 2 + 3 (conef_fused.cu)
     int n_fused = 0;
     bool any_csk = false;       // some tensor takes the shared-memory step of the chunk-wise count sketch
@@ -230,7 +230,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     P.gen_coop = gen.coop != 0;
     P.fast_it[0] = it1, P.fast_it[1] = it2, P.fast_it[2] = it3;
     P.fast_unit = unit;
-    int64_t g_off = 0, state_off = 0, il_fill = 0;
+    int64_t g_off = 0, state_off = 0, il_fill = 0, hist_tiles = 0;
     for (int l = 0; l < n_tensors; ++l) {
         const conef_tensor &t = tensors[l];
         if (t.rows <= 0 || t.cols <= 0)
@@ -323,6 +323,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 select_window(L.d, L.k, L.sel_lo, L.sel_hi, L.cand_cap, L.sel_scale);
                 P.cand_pairs += L.cand_cap;
                 tiles[T_SEL_CLUSTER] = 1;
+                hist_tiles += ceil_div(L.d, kHistTile);
                 while (P.sel_cluster > 0 && P.sel_cluster < ceil_div(L.d, kHistTile))
                     P.sel_cluster = P.sel_cluster < kSelClusterTiles ? P.sel_cluster * 2 : 0;
                 if (ceil_div(L.d, kHistTile) > kSelTailTiles)
@@ -469,6 +470,11 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
         tiles[T_APPLY] = (int)apply_tiles(L, q->kind);
         for (int k = 0; k < kNumTables; ++k)
             P.pfx[k][l + 1] = P.pfx[k][l] + tiles[k];
+    }
+    if (P.sel_cluster > 1) {   // (all clusters have the size that the largest tensor needs)
+        const int64_t ctas = (int64_t)P.pfx[T_SEL_CLUSTER][n_tensors] * P.sel_cluster, idle = ctas - hist_tiles;
+        if (ctas > kSelClusterCtas || idle > kSelClusterIdle)
+            P.sel_cluster = 0;
     }
     if (P.short_tiles && P.any_fast) {
         P.multi = true;

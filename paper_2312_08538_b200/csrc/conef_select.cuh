@@ -372,6 +372,13 @@ static __device__ __noinline__ void select_exact(SelectShared &S, uint64_t st, u
 // Everything is exchanged through the CTAs' shared memory, and nothing in global memory is touched before the
 // result is written, so that all of it can run while the kernel ahead in the stream ends.
 constexpr int kSelClusterTiles = 16;
+// All clusters of a launch have the size that the largest tensor needs, so small tensors beside a large one leave most of
+// their CTAs idle, and those of many tensors do not fit the SMs together.  Selection and step of one worker on the GPU, clusters
+// and k_rk_select, one tensor of 16 tiles beside small ones: 11 (176 CTAs idle) 11.5 and 15.1 us, 19 (285) 14.4 and 15.4, 23
+// (345) 14.2 and 15.7, 31 (465) 18.6 and 15.6, 300 (4500) 76.7 and 20.8; of 8 tiles: 39 (273) 12.3 and 13.8, 43 (301) 14.8 and
+// 14.0, 1000 (7000) 116 and 37.  Tensors of 16 tiles, none idle: 20 (320 CTAs) 20.5 and 23.0, 40 (640) 30.8 and 33.4, 60 (960)
+// 40.5 and 39.3, 200 (3200) 110 and 94.  Clusters of one CTA are faster throughout (1000 tensors 38.4 and 40.0).
+constexpr int64_t kSelClusterIdle = kPlanSMs * 2, kSelClusterCtas = kPlanSMs * 5;
 constexpr int kSelMine = 1024;   // window elements of a CTA: expected 607 at most (d = 8192, k = d / 2), or a whole short tensor
 struct SelectCluster : SelectShared {
     uint2 mine[kSelMine];

@@ -101,3 +101,33 @@ def test_small_models_by_a_cluster(shapes, k_num, k_den, how):
             b.conef_randk_indices_noalloc_select(seed, l, step, d, k, getattr(b, "SELECT_" + how), out)
             assert np.array_equal(out.cpu().numpy().view(np.uint32), want), (step, r, c)
     assert eng.last_status() == 0
+
+
+# one launch of clusters or the selection through the scratch: small tensors beside a larger one, on both sides of the
+# number of idle CTAs that a launch of clusters may have, and of the number of its CTAs
+@pytest.mark.parametrize("shapes", [[(64, 64)] * 19 + [(256, 512)], [(64, 64)] * 24 + [(256, 512)], [(3, 5)] * 150 + [(2, 8192)],
+                                    [(33, 77)] * 300 + [(2, 8192)], [(256, 512)] * 46, [(255, 512)] * 47])
+def test_models_around_the_limit_of_a_launch_of_clusters(shapes):
+    _check(shapes, 1, 100, steps=(3, 4))
+
+
+def test_small_tensors_beside_a_larger_one_take_no_clusters_of_its_size():
+    """300 tensors of one tile, alone and beside one of 16 tiles: with clusters of 16 CTAs for all of them the step
+    took 4.7 times as long as without the larger tensor, through the scratch 1.3 times."""
+    from paper_2312_08538_b200 import binding as b
+    best = []
+    for shapes in ([(64, 64, 1)] * 300, [(64, 64, 1)] * 300 + [(256, 512, 1)]):
+        eng = b.ConEF(shapes, 1, dict(kind="randk", k_num=1, k_den=100, seed=3), dict(kind="int8", block=256), 0.1)
+        g = [torch.ones(sum(r * c for r, c, _ in shapes), device="cuda")]
+        times, t = [], 0
+        for _ in range(6):
+            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            start.record()
+            for _ in range(100):
+                eng.step(t, g, 0)
+                t += 1
+            end.record()
+            end.synchronize()
+            times.append(start.elapsed_time(end))
+        best.append(min(times))
+    assert best[1] < 2.5 * best[0], best

@@ -50,6 +50,40 @@ __device__ __forceinline__ void grid_release()
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Loads of what the kernel itself does not write: as free to be moved and batched as __ldg (they depend on the address
+// alone, which has to come from behind grid_wait(), by fresh() or through the tensor), but not by the non-coherent path, which
+// is for memory that nobody writes while the grid lives: a chained kernel's CTAs live while the one ahead writes its results.
+__device__ __forceinline__ float load_global(const float *p)
+{
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 load_global(const float2 *p)
+{
+    float2 v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 load_global(const float4 *p)
+{
+    float4 v;
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t load_global(const uint8_t *p)
+{
+    uint32_t v;
+    asm("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned short load_global(const unsigned short *p)
+{
+    unsigned short v;
+    asm("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
 // Loads of what other CTAs of the same launch wrote before a ticket or a flag: past L1, and volatile with
 // a memory clobber, so that the compiler may not move them ahead of it (it may move __ldcg, whose
 // result depends on its address alone).

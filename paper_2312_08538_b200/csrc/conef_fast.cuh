@@ -365,7 +365,7 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
         for (int q = 0; q < 8; ++q)
 #pragma unroll
             for (int c = 0; c < R; c += 4) {
-                const float4 t = __ldg((const float4 *)(qp + (size_t)(col + q) * R + c));
+                const float4 t = load_global((const float4 *)(qp + (size_t)(col + q) * R + c));
                 frag[q][c] = t.x; frag[q][c + 1] = t.y; frag[q][c + 2] = t.z; frag[q][c + 3] = t.w;
             }
     } else if (PASS == 2) {
@@ -380,7 +380,7 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
         for (int q = 0; q < 8; ++q)
 #pragma unroll
             for (int c = 0; c < R; c += 4) {
-                const float4 t = __ldg((const float4 *)(qi + (size_t)(col + q) * R + c));
+                const float4 t = load_global((const float4 *)(qi + (size_t)(col + q) * R + c));
                 frag[q][c] = t.x; frag[q][c + 1] = t.y; frag[q][c + 2] = t.z; frag[q][c + 3] = t.w;
             }
     }
@@ -672,7 +672,7 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
             const int64_t have4 = (n_rows - (int64_t)c0 * subs) * (R / 4);
             const float4 *src = fresh((const float4 *)(V.phat + Lp->msgp_off + (size_t)c0 * subs * R));
             for (uint32_t i = tid; i < n4pad; i += bd) {
-                const float4 v = (i < n4 && (int64_t)i < have4) ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 v = (i < n4 && (int64_t)i < have4) ? load_global(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
                 if (PAIR) {
                     ((float4 *)st_ph)[2 * i] = make_float4(-v.x, -v.x, -v.y, -v.y);
                     ((float4 *)st_ph)[2 * i + 1] = make_float4(-v.z, -v.z, -v.w, -v.w);

@@ -84,7 +84,7 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
                     for (int c = 0; c < R; c += 4) {
                         float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (a < row_hi)
-                            t = __ldg((const float4 *)(src + a * R + c));
+                            t = load_global((const float4 *)(src + a * R + c));
                         x[k][c] = t.x; x[k][c + 1] = t.y; x[k][c + 2] = t.z; x[k][c + 3] = t.w;
                     }
                 }
@@ -94,7 +94,7 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
                     const int64_t a = row_lo + (int64_t)(k0 + k) * kGsThreads + tid;
 #pragma unroll
                     for (int c = 0; c < R; ++c)
-                        x[k][c] = (a < row_hi && c < r) ? __ldg(src + a * r + c) : 0.f;
+                        x[k][c] = (a < row_hi && c < r) ? load_global(src + a * r + c) : 0.f;
                 }
             }
 #pragma unroll

@@ -7,7 +7,7 @@ namespace conef {
 // SPLIT's last step: `records`, one sketch after the other (n_records floats apart), -> states, whose padding
 // (to 64 floats) is cleared again.  blockIdx.y: worker of the batch.
 static __global__ void __launch_bounds__(kIlThreads) k_sketch_back(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
-                                                                   int first, int worker0, const float *__restrict__ records,
+                                                                   int first, int worker0, const float *records,
                                                                    int64_t n_records)
 {
     grid_release();
@@ -17,7 +17,7 @@ static __global__ void __launch_bounds__(kIlThreads) k_sketch_back(const __grid_
     grid_wait();
     const int64_t n = (int64_t)V.cs_rows * L.w, room = (n + 63) / 64 * 64;
     const int64_t e0 = (int64_t)(tile - pfx[li]) * kIlEntries + threadIdx.x;
-    const float *__restrict__ src = records + blockIdx.y * n_records + L.sk_off;
+    const float *src = records + blockIdx.y * n_records + L.sk_off;
     float *__restrict__ dst = (float *)(V.state + (worker0 + (int)blockIdx.y) * V.state_stride + L.a_off);
 #pragma unroll
     for (int q = 0; q < kIlEntries / kIlThreads; ++q) {
@@ -34,7 +34,7 @@ static __global__ void __launch_bounds__(kIlThreads) k_sketch_back(const __grid_
 //   3  scratch -> states, whose padding is cleared again
 template <int GW, int PART>
 static __global__ void __launch_bounds__(kIlThreads) k_sketch_fold(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
-                                                                   int first, int worker0, float *__restrict__ records)
+                                                                   int first, int worker0, float *records)
 {
     constexpr int F = 2 * GW, PITCH = F + 1, PW = GW < 4 ? GW : 4;   // floats per record and per piece
     using Piece = typename std::conditional<PW == 2, float2, float4>::type;

@@ -257,7 +257,7 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
 // exchanged through shared memory, are accessed 16 bytes per lane over contiguous memory.
 template <int GW, bool IN, bool SPLIT>
 __global__ void __launch_bounds__(kIlThreads) k_sketch_swap(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
-                                                            int first, int worker0, float *__restrict__ records, uint32_t stride,
+                                                            int first, int worker0, float *records, uint32_t stride,
                                                             int64_t newoff)
 {
     constexpr int PW = GW < 4 ? GW : 4, H = GW / PW;   // floats per piece, pieces of a record's old (or new) values

@@ -81,18 +81,18 @@ __device__ __forceinline__ void factor_row(const float *__restrict__ p, int r, f
     if constexpr (R == 4 || R == 8) {
 #pragma unroll
         for (int c = 0; c < R; c += 4) {
-            const float4 t = __ldg((const float4 *)(p + c));
+            const float4 t = load_global((const float4 *)(p + c));
             out[c] = t.x; out[c + 1] = t.y; out[c + 2] = t.z; out[c + 3] = t.w;
         }
     } else if constexpr (R == 2) {
-        const float2 t = __ldg((const float2 *)p);
+        const float2 t = load_global((const float2 *)p);
         out[0] = t.x; out[1] = t.y;
     } else if constexpr (R == 1) {
-        out[0] = __ldg(p);
+        out[0] = load_global(p);
     } else {
 #pragma unroll
         for (int c = 0; c < CONEF_MAX_RANK; ++c)
-            out[c] = c < r ? __ldg(p + c) : 0.f;
+            out[c] = c < r ? load_global(p + c) : 0.f;
     }
 }
 // float(code) from a code's byte or nibble
@@ -106,11 +106,11 @@ __device__ __forceinline__ float code_value(uint32_t raw)
 template <int CK>
 __device__ __forceinline__ uint32_t code_raw(const uint8_t *__restrict__ codes, uint32_t j)
 {
-    return CK == CONEF_C_INT4 ? (uint32_t)__ldg(codes + (j >> 1)) >> (4 * (j & 1u)) : (uint32_t)__ldg(codes + j);
+    return CK == CONEF_C_INT4 ? (uint32_t)load_global(codes + (j >> 1)) >> (4 * (j & 1u)) : (uint32_t)load_global(codes + j);
 }
 __device__ __forceinline__ float gen_scale(const uint8_t *__restrict__ b, uint32_t blk, bool half)
 {
-    return half ? __half2float(__ushort_as_half(__ldg((const unsigned short *)b + blk))) : __ldg((const float *)b + blk);
+    return half ? __half2float(__ushort_as_half(load_global((const unsigned short *)b + blk))) : load_global((const float *)b + blk);
 }
 
 template <int CK, int R, int NR>   // NR: rows per warp
@@ -145,7 +145,7 @@ __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L
 #pragma unroll
             for (int i = 0; i < NR; ++i) {
                 const uint32_t j = jb[i] + col + u * 32;
-                gv[u][i] = __ldg(g + j);
+                gv[u][i] = load_global(g + j);
                 w[u][i] = code_raw<CK>(codes, j);
                 sc[u][i] = gen_scale(scales, j >> shift, half);
             }
@@ -222,7 +222,7 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 const uint32_t j = (a + u) * m + col[k];
-                gv[u][k] = __ldg(g + j);
+                gv[u][k] = load_global(g + j);
                 w[u][k] = code_raw<CK>(codes, j);
                 sc[u][k] = gen_scale(scales, j >> shift, half);
             }
@@ -275,7 +275,7 @@ __device__ __forceinline__ void gen_p2_cta(const DevView &V, const LayerDesc &L,
     const float lr = V.lr, omb = V.omb;
     float *const p = smem, *const phs = smem + kP2RowsPerTile * 32;   // [row][column], [row][c]
     for (uint32_t x = threadIdx.x; x < have * r; x += kGenThreads)
-        phs[x] = __ldg(ph + x);
+        phs[x] = load_global(ph + x);
     const uint32_t col = min(c0, m - 1);   // (columns past the end repeat the last one and are not stored)
     for (uint32_t a0 = warp; a0 < have; a0 += 8 * U) {
         float gv[U], sc[U];
@@ -283,7 +283,7 @@ __device__ __forceinline__ void gen_p2_cta(const DevView &V, const LayerDesc &L,
 #pragma unroll
         for (int u = 0; u < U; ++u) {   // (rows past the end repeat the last one)
             const uint32_t j = (r_lo + min(a0 + 8 * u, have - 1)) * m + col;
-            gv[u] = __ldg(g + j);
+            gv[u] = load_global(g + j);
             w[u] = code_raw<CK>(codes, j);
             sc[u] = gen_scale(scales, j >> shift, half);
         }

@@ -205,7 +205,7 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
                 } else {
                     float ph[RK];
                     if (RK == 4) {
-                        const float4 t = __ldg((const float4 *)(phat + (size_t)a * 4));
+                        const float4 t = load_global((const float4 *)(phat + (size_t)a * 4));
                         ph[0] = t.x; ph[1] = t.y; ph[2] = t.z; ph[3] = t.w;
                     } else {
 #pragma unroll

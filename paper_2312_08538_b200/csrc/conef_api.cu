@@ -87,7 +87,8 @@ struct Plan {
     bool any_fast = false, any_slow = false, any_rs12 = false, any_gen = false;
     bool gen_coop = false;      // pass 2 for any shape: a CTA per tile
     bool short_tiles = false;   // tile lengths of the tuned passes below their limits
-    bool multi = false;         // one launch per pass takes all tensors (conef_fastmulti.cuh)
+    bool multi = false;         // one launch per pass takes tensors of all widths (conef_fastmulti.cuh)
+    bool multi_gen = false;     // ... those of any other shape and 1-D ones included
     size_t multi_smem[3] = {2048, 2048, 2048};   // ... with this much shared memory per CTA
     bool any_fv = false;        // some tensor takes the tuned fused step (conef_flatvec.cuh)
     int fv_tiles = 1;           // ... with this many selection tiles per CTA
@@ -478,11 +479,18 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     }
     if (P.short_tiles && P.any_fast) {
         P.multi = true;
+        int64_t gen_elems = 0;
+        for (const LayerDesc &L : P.layers)
+            if (L.compressed && L.fast == 3)
+                gen_elems += L.d;
+        P.multi_gen = gen_elems * n_workers <= multi_gen(q->rank);
         const int sb = scale_bytes, cw = c->kind == CONEF_C_INT4 ? 1 : 2;
         for (int l = 0; l < n_tensors; ++l) {
             LayerDesc &L = P.layers[l];
             int t[5] = {0, 0, 0, 0, 0};
-            if (!L.compressed) {
+            if (!P.multi_gen && (!L.compressed || L.fast == 3)) {
+                // (the launches for any shape take them)
+            } else if (!L.compressed) {
                 t[0] = P.pfx[T_PASS][l + 1] - P.pfx[T_PASS][l];
             } else if (L.fast == 1) {
                 multi_classify(L, c->kind, sb);
@@ -1418,7 +1426,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             rc = launch_fused(ctx, V, s, phase == 4);
         auto launch_gen = [&](int pass) -> int {
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
-            if (n == 0 || multi || rs12)   // (the table may hold 1-D tensors alone, of a model on a row sketch)
+            if (n == 0 || (multi && ctx->plan.multi_gen) || rs12)   // (the table may hold 1-D tensors alone, of a model on a row sketch)
                 return CONEF_OK;
             CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->chain(), ctx->plan.gen_coop));
             LAUNCH_CHECK(ctx);

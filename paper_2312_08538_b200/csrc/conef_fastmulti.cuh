@@ -4,7 +4,7 @@
 // took a launch per size on side streams, forked and joined by events, and a further launch for the tensors of
 // any other shape; with short tiles these cost as much as the passes.  Here every CTA has 256 threads: it holds
 // as many tiles of its tensor as fit (f_nsub, each with its own part of shared memory and its own barrier), or
-// one tile of the passes for any shape (conef_lrgen.cuh), or, in pass 1, of a 1-D tensor that passes through.
+// one tile of the passes for any shape (conef_lrgen.cuh; up to multi_gen elements), or, in pass 1, of a 1-D tensor that passes through.
 // What a tile computes, and the order of its sums, is that of those kernels.
 // ResNet-50 list (seven widths and one odd convolution), int8, rank 4, four workers: 550 -> 440 us per step and update; six
 // aligned matrices of 17 M elements, int4, eight workers: 803 -> 750 us.  (64 registers, four CTAs per SM, spill: 577 us on the
@@ -20,6 +20,14 @@ constexpr size_t kMultiSmem = 72 * 1024;   // shared memory of a CTA's tiles, wh
 // Iterations per tile of passes 1 and 3 at most (pass 2's are part of the order of its sums): longer tiles leave the last
 // wave of CTAs nearly empty.  (ResNet-50 list: 8 iterations 554 us, 16 481, 32 457.)
 constexpr int kMultiIt = 32;
+// Tensors of any other shape share these launches up to this many of their elements (all workers).  Beyond, they and the 1-D
+// tensors have launches of their own (k_gen_pass), with four CTAs per SM instead of three at rank 4, three instead of two at rank 8,
+// the block size as a constant in pass 3 and all of L1.  Step and update, one 1024 x 512 matrix beside an odd one of two workers,
+// shared and on their own.  Rank 8, int4: 10 M elements 193 and 186 us, 16 M 274 and 267, 20 M 359 and 305, 28 M 412 and 342, 36 M 485
+// and 467, 80 M 1032 and 841; int8: 16 M 259 and 287, 24 M 380 and 353, 36 M 451 and 512, 80 M 940 and 893; sixteen odd ones of eight
+// workers, 167 M: 1827 and 1479, 1681 and 1586.  Rank 4, int4: 20 M 204 and 215, 40 M 332 and 365, 120 M 846 and 869; int8: 40 M 324 and
+// 358, 120 M 820 and 830; those sixteen: 1045 and 1054, 1027 and 976.  (Ups and downs are waves of CTAs.)
+constexpr int64_t multi_gen(int rank) { return rank == 8 ? 18'000'000 : 160'000'000; }
 constexpr int multi_ctas(int pass, int rank) { return rank == 4 ? 3 : min_ctas(pass, rank); }
 
 // bytes of shared memory of one tile

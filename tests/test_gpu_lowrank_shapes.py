@@ -91,3 +91,39 @@ def test_all_widths_in_one_launch(rank, c):
                n_workers=2, q=dict(kind="lowrank", rank=rank), c=c, grad="normal1e-3")
     from tests.test_gpu_parity import lowrank_teacher_forced
     lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)
+
+
+@pytest.mark.parametrize("c", [dict(kind="int8", block=256), dict(kind="int4", block=64, scale_dtype="fp16", beta=0.9)])
+def test_many_elements_of_other_shapes_beside_a_tuned_matrix(c):
+    """Up to 18 M elements at rank 8 they share its launches, beyond that each pass has one of their own: three more
+    launches, the same bits."""
+    from paper_2312_08538_b200 import binding as b
+    launches = []
+    for rows in (2252, 2254):   # 18 M elements of eight workers between them
+        cfg = wl.config("resnet50-mini")
+        cfg.update(tensors=[(512, 256, 1), (77, 1, 0), (rows, 999, 1)], n_workers=8, q=dict(kind="lowrank", rank=8), c=c, grad="normal1e-3")
+        q0 = wl.q_init(cfg, "cuda")
+        both = [pu.make_gpu(cfg, q_init=q0, fast=f) for f in (True, False)]
+        for t in range(2):
+            gd, _ = pu.grads_both(cfg, t)
+            for e, f in zip(both, (True, False)):
+                before = e.launch_count()
+                e.step(t, gd, 0)
+                e.set_fast_path(True)   # (the same Gram-Schmidt)
+                e.reduce_messages(b.MSG_P)
+                e.set_fast_path(f)
+                e.step(t, gd, 2)
+                e.step(t, gd, 3)
+                if f and t == 1:
+                    launches.append(e.launch_count() - before)
+            dense = [e.reduce_messages(b.MSG_DENSE1D) for e in both]
+            assert torch.equal(*dense)
+            for i in range(8):
+                x, y = (e.factors(2, i) for e in both)
+                for k in ("p_i", "q_i"):
+                    assert torch.equal(x[k], y[k]), (rows, t, i, k)
+                u, v = (e.decompress_error(i)[512 * 256:] for e in both)
+                assert torch.equal(u, v), (rows, t, i)
+            for e in both:
+                e.reduce_messages(b.MSG_Q)
+    assert launches[1] == launches[0] + 3

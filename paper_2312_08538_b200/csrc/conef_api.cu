@@ -624,13 +624,6 @@ struct conef_ctx {
     cudaStream_t aux[kMaxFastClasses] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kMaxFastClasses] = {};
     int n_aux = 0;
-    bool joined = false;   // the caller's stream waits for an event of a side stream: the next launch on it is not a chained one (launch())
-    bool chain()
-    {
-        const bool c = !joined;
-        joined = false;
-        return c;
-    }
     ~conef_ctx()
     {
         for (int k = 0; k < n_aux; ++k) {
@@ -774,9 +767,9 @@ int launch_rowsketch(conef_ctx *ctx, const DevView &V, cudaStream_t s)
         return CONEF_OK;
     dim3 grid(n, ctx->n_workers);
     if (ctx->c.cs_rows == 1)
-        launch(ctx->chain(), k_rowsketch<QK, true>, grid, kRsThreads, 0, s, V);
+        launch(k_rowsketch<QK, true>, grid, kRsThreads, 0, s, V);
     else
-        launch(ctx->chain(), k_rowsketch<QK, false>, grid, kRsThreads, 0, s, V);
+        launch(k_rowsketch<QK, false>, grid, kRsThreads, 0, s, V);
     LAUNCH_CHECK(ctx);
     return CONEF_OK;
 }
@@ -868,7 +861,7 @@ int launch_pass2_reduce(conef_ctx *ctx, DevView V, cudaStream_t s, bool skip_fus
         return CONEF_OK;
     V.pfx_q2 = table_ptr(ctx, table);
     dim3 grid2(tiles_of(ctx, table), ctx->n_workers);
-    launch(ctx->chain(), k_lr_pass2_reduce, grid2, 256, 0, s, V);
+    launch(k_lr_pass2_reduce, grid2, 256, 0, s, V);
     LAUNCH_CHECK(ctx);
     return CONEF_OK;
 }
@@ -877,16 +870,16 @@ int launch_pass2_reduce(conef_ctx *ctx, DevView V, cudaStream_t s, bool skip_fus
 int launch_p1_rest(conef_ctx *ctx, const DevView &V, cudaStream_t s)
 {
     if (tiles_of(ctx, T_RP1) > 0) {
-        CK_CUDA(rows_p1_launch<4>(V, table_ptr(ctx, T_RP1), tiles_of(ctx, T_RP1), s, ctx->chain()));
+        CK_CUDA(rows_p1_launch<4>(V, table_ptr(ctx, T_RP1), tiles_of(ctx, T_RP1), s));
         LAUNCH_CHECK(ctx);
     }
     if (tiles_of(ctx, T_RP1_R8) > 0) {
-        CK_CUDA(rows_p1_launch<8>(V, table_ptr(ctx, T_RP1_R8), tiles_of(ctx, T_RP1_R8), s, ctx->chain()));
+        CK_CUDA(rows_p1_launch<8>(V, table_ptr(ctx, T_RP1_R8), tiles_of(ctx, T_RP1_R8), s));
         LAUNCH_CHECK(ctx);
     }
     if (tiles_of(ctx, T_FAST_P1) > 0) {
         // P_i = sum of the per-segment row partials
-        CK_CUDA(fast_launch_p1_combine(ctx->q.rank, V, table_ptr(ctx, T_FAST_P1), tiles_of(ctx, T_FAST_P1), s, ctx->chain()));
+        CK_CUDA(fast_launch_p1_combine(ctx->q.rank, V, table_ptr(ctx, T_FAST_P1), tiles_of(ctx, T_FAST_P1), s));
         LAUNCH_CHECK(ctx);
     }
     return CONEF_OK;
@@ -899,7 +892,7 @@ int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool
     if (P.multi) {
         const int table = skip_fused && pass >= 2 ? T_MULTINF2 + pass - 2 : T_MULTI1 + pass - 1;
         if (tiles_of(ctx, table) > 0) {
-            CK_CUDA(multi_launch(pass, ctx->c.kind, ctx->q.rank, V.scale_half, V, table_ptr(ctx, table), tiles_of(ctx, table), s, ctx->chain(),
+            CK_CUDA(multi_launch(pass, ctx->c.kind, ctx->q.rank, V.scale_half, V, table_ptr(ctx, table), tiles_of(ctx, table), s,
                                  P.multi_smem[pass - 1]));
             LAUNCH_CHECK(ctx);
         }
@@ -925,7 +918,7 @@ int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool
         const size_t stage = fast_stage_bytes(pass, ctx->q.rank, P.fast_it[pass - 1], P.fast_subs[k], P.fast_threads[k],
                                               P.fast_unit, V.scale_half ? 2 : 4);
         CK_CUDA(fast_launch(pass, ctx->c.kind, ctx->q.rank, V.scale_half, V, table_ptr(ctx, table), n, P.fast_threads[k], sk,
-                            !off_main && ctx->chain(), P.short_tiles, P.fast_narrow[k] != 0, stage));
+                            P.short_tiles, P.fast_narrow[k] != 0, stage));
         LAUNCH_CHECK(ctx);
         if (off_main) {
             CK_CUDA(cudaEventRecord(ctx->ev_join[used], sk));
@@ -934,7 +927,6 @@ int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool
     }
     for (int k = 0; k < used; ++k)
         CK_CUDA(cudaStreamWaitEvent(s, ctx->ev_join[k], 0));
-    ctx->joined = ctx->joined || used > 0;
     return pass == 1 ? launch_p1_rest(ctx, V, s) : CONEF_OK;
 }
 
@@ -1144,15 +1136,15 @@ int launch_randk_select(conef_ctx *ctx, const DevView &V, cudaStream_t s)
         return CONEF_OK;
     if (ctx->plan.sel_cluster > 0 && (V.sel_how == CONEF_SELECT_NORMAL || V.sel_how == CONEF_SELECT_MISS)) {   // (the others have no list)
         static bool allowed[64] = {};
-        launch_cluster(ctx->chain(), k_rk_select_cluster, tiles_of(ctx, T_SEL_CLUSTER), ctx->plan.sel_cluster, kSelThreads, s, allowed, V,
+        launch_cluster(k_rk_select_cluster, tiles_of(ctx, T_SEL_CLUSTER), ctx->plan.sel_cluster, kSelThreads, s, allowed, V,
                        table_ptr(ctx, T_SEL_CLUSTER));
         LAUNCH_CHECK(ctx);
         return CONEF_OK;
     }
-    launch(ctx->chain(), k_rk_select, dim3(nh), kSelThreads, 0, s, V);
+    launch(k_rk_select, dim3(nh), kSelThreads, 0, s, V);
     LAUNCH_CHECK(ctx);
     if (no > 0) {
-        launch(ctx->chain(), k_rk_offsets, dim3(no), kSelThreads, 0, s, V, table_ptr(ctx, T_SEL_OFFS));
+        launch(k_rk_offsets, dim3(no), kSelThreads, 0, s, V, table_ptr(ctx, T_SEL_OFFS));
         LAUNCH_CHECK(ctx);
     }
     return CONEF_OK;
@@ -1349,7 +1341,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                                  : dense || (ctx->fast && ctx->plan.any_fv && ctx->c.iconef != 2);
     if (phase == 0 && tiles_of(ctx, T_PASS) > 0 && !with_1d) {
         dim3 grid(tiles_of(ctx, T_PASS), ctx->n_workers);
-        launch(ctx->chain(), k_passthrough, grid, 256, 0, s, V);
+        launch(k_passthrough, grid, 256, 0, s, V);
         LAUNCH_CHECK(ctx);
     }
     // single-phase compressors: the tuned fused step where a tensor allows it, the generic kernel elsewhere
@@ -1360,7 +1352,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
         if (dense) {
             const int n = tiles_of(ctx, T_DENSE);
             if (n > 0) {
-                launch(ctx->chain(), k_flat_dense<QK>, dim3(n, ctx->n_workers), kDecThreads, 0, s, V, table_ptr(ctx, T_DENSE));
+                launch(k_flat_dense<QK>, dim3(n, ctx->n_workers), kDecThreads, 0, s, V, table_ptr(ctx, T_DENSE));
                 LAUNCH_CHECK(ctx);
             }
             return CONEF_OK;
@@ -1428,7 +1420,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
             if (n == 0 || (multi && ctx->plan.multi_gen) || rs12)   // (the table may hold 1-D tensors alone, of a model on a row sketch)
                 return CONEF_OK;
-            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->chain(), ctx->plan.gen_coop));
+            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->plan.gen_coop));
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };
@@ -1438,12 +1430,12 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
                 return CONEF_OK;
             dim3 grid(n, ctx->n_workers);
             if (pass == 1) {
-                launch(ctx->chain(), k_rs_pass12<1>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
+                launch(k_rs_pass12<1>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
                 LAUNCH_CHECK(ctx);
                 dim3 gridc(tiles_of(ctx, T_RS_P1C), ctx->n_workers);
-                launch(ctx->chain(), k_rs_p1_combine, gridc, 256, 0, s, V, table_ptr(ctx, T_RS_P1C));
+                launch(k_rs_p1_combine, gridc, 256, 0, s, V, table_ptr(ctx, T_RS_P1C));
             } else {
-                launch(ctx->chain(), k_rs_pass12<2>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
+                launch(k_rs_pass12<2>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
             }
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
@@ -1516,7 +1508,7 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
         int64_t blocks = ceil_div(len, 256);
         if (blocks > (int64_t)ctx->sm_count * 16)
             blocks = (int64_t)ctx->sm_count * 16;
-        launch(ctx->chain(), k_reduce_workers, dim3((unsigned)blocks), 256, 0, s, base, stride, ctx->n_workers, len, out_sum, mean_out,
+        launch(k_reduce_workers, dim3((unsigned)blocks), 256, 0, s, base, stride, ctx->n_workers, len, out_sum, mean_out,
                V.n_workers_f);
         LAUNCH_CHECK(ctx);
         return CONEF_OK;
@@ -1566,9 +1558,9 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
                     continue;
                 cudaStream_t sk = pick();
                 if (ctx->q.rank <= 4)
-                    CK_CUDA(gs_launch<4>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk, sk == s && ctx->chain()));
+                    CK_CUDA(gs_launch<4>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk));
                 else
-                    CK_CUDA(gs_launch<8>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk, sk == s && ctx->chain()));
+                    CK_CUDA(gs_launch<8>(V, table_ptr(ctx, tabs[k]), n, csz[k], out_sum, sk));
                 LAUNCH_CHECK(ctx);
                 done(sk);
             }
@@ -1582,7 +1574,6 @@ int conef_reduce_messages(conef_ctx *ctx, int which, float *out_sum, conef_strea
             }
             for (int k = 0; k < used; ++k)
                 CK_CUDA(cudaStreamWaitEvent(s, ctx->ev_join[k], 0));
-            ctx->joined = ctx->joined || used > 0;
         } else if (tiles_of(ctx, T_GS) > 0) {
             k_gram_schmidt<<<tiles_of(ctx, T_GS), 1024, 0, s>>>(V, out_sum);
             LAUNCH_CHECK(ctx);

@@ -259,12 +259,12 @@ inline void apply_launch(int qkind, int rank, const DevView &V, const int32_t *p
 {
     const int r = qkind != CONEF_Q_LOWRANK ? -1 : rank == 1 || rank == 2 || rank == 4 || rank == 8 ? rank : 0;
     switch (r) {
-    case -1: launch(true, k_apply<-1>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
-    case 1: launch(true, k_apply<1>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
-    case 2: launch(true, k_apply<2>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
-    case 4: launch(true, k_apply<4>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
-    case 8: launch(true, k_apply<8>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
-    default: launch(true, k_apply<0>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d);
+    case -1: launch(k_apply<-1>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 1: launch(k_apply<1>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 2: launch(k_apply<2>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 4: launch(k_apply<4>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    case 8: launch(k_apply<8>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d); break;
+    default: launch(k_apply<0>, dim3(tiles), kApplyThreads, 0, s, V, pfx, x, sum_values, sum_dense1d);
     }
 }
 

@@ -27,7 +27,7 @@ __device__ __forceinline__ int find_layer(const int32_t *__restrict__ pfx, int n
     return lo;
 }
 
-// For kernels launched by launch(true, ...) (conef_internal.h).  The kernel ahead in the stream is done and what it
+// For kernels launched by launch() (conef_internal.h).  The kernel ahead in the stream is done and what it
 // wrote is visible:
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // ... and a pointer to what it wrote, so that no load through it (loads of constant memory, as __ldg is taken

@@ -114,7 +114,7 @@ inline void decode_launch_batch(bool int4, bool second, const DevView &V, const 
 {
     auto *k = int4 ? (second ? k_decode<true, true, BATCH> : k_decode<true, false, BATCH>)
                    : (second ? k_decode<false, true, BATCH> : k_decode<false, false, BATCH>);
-    launch(true, k, dim3(tiles), kDecThreads, 0, s, V, pfx, worker, out);
+    launch(k, dim3(tiles), kDecThreads, 0, s, V, pfx, worker, out);
 }
 inline void decode_launch(int batch, bool int4, bool second, const DevView &V, const int32_t *pfx, int tiles, int worker, float *out,
                           cudaStream_t s)

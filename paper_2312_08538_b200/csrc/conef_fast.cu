@@ -5,35 +5,35 @@ namespace conef {
 
 template <int PASS, int CK, int R, bool HALF, bool SHORT, bool NARROW = false, bool PARTIAL = false>
 inline cudaError_t fast_launch_pass23(const DevView &V, const int32_t *pfx, int tiles, int threads, cudaStream_t s,
-                                      bool chained, size_t stage)
+                                      size_t stage)
 {
     const size_t smem = (size_t)ring_depth(PASS, R) * threads * (32 + (CK == CONEF_C_INT4 ? 4 : 8)) + stage;
     static int done[64];
     const cudaError_t e = opt_in_smem(k_fast_pass<PASS, CK, R, HALF, SHORT, NARROW, PARTIAL>, smem, done);
     if (e != cudaSuccess)
         return e;
-    return launch(chained, k_fast_pass<PASS, CK, R, HALF, SHORT, NARROW, PARTIAL>, dim3(tiles, V.n_workers), threads, smem, s, V, pfx);
+    return launch(k_fast_pass<PASS, CK, R, HALF, SHORT, NARROW, PARTIAL>, dim3(tiles, V.n_workers), threads, smem, s, V, pfx);
 }
 
 cudaError_t fast_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx,
-                               int tiles, int threads, cudaStream_t s, bool chained, bool short_tiles, bool narrow, size_t stage)
+                               int tiles, int threads, cudaStream_t s, bool short_tiles, bool narrow, size_t stage)
 {
     if (tiles <= 0)
         return cudaSuccess;
 #define CONEF_FAST_CASE_P(CKV, RV, HV, PV)                                                                \
     if (ckind == CKV && rank == RV && (half != 0) == HV && (V.beta != 0.f) == PV) {                       \
         if (pass == 1 && narrow) {                                                                        \
-            if (short_tiles) return fast_launch_pass23<1, CKV, RV, HV, true, true, PV>(V, pfx, tiles, threads, s, chained, stage);  \
-            return fast_launch_pass23<1, CKV, RV, HV, false, true, PV>(V, pfx, tiles, threads, s, chained, stage);        \
+            if (short_tiles) return fast_launch_pass23<1, CKV, RV, HV, true, true, PV>(V, pfx, tiles, threads, s, stage);  \
+            return fast_launch_pass23<1, CKV, RV, HV, false, true, PV>(V, pfx, tiles, threads, s, stage);        \
         }                                                                                                 \
         if (short_tiles) {                                                                                \
-            if (pass == 1) return fast_launch_pass23<1, CKV, RV, HV, true, false, PV>(V, pfx, tiles, threads, s, chained, stage);    \
-            if (pass == 2) return fast_launch_pass23<2, CKV, RV, HV, true, false, PV>(V, pfx, tiles, threads, s, chained, stage);    \
-            return fast_launch_pass23<3, CKV, RV, HV, true, false, PV>(V, pfx, tiles, threads, s, chained, stage);        \
+            if (pass == 1) return fast_launch_pass23<1, CKV, RV, HV, true, false, PV>(V, pfx, tiles, threads, s, stage);    \
+            if (pass == 2) return fast_launch_pass23<2, CKV, RV, HV, true, false, PV>(V, pfx, tiles, threads, s, stage);    \
+            return fast_launch_pass23<3, CKV, RV, HV, true, false, PV>(V, pfx, tiles, threads, s, stage);        \
         }                                                                                                 \
-        if (pass == 1) return fast_launch_pass23<1, CKV, RV, HV, false, false, PV>(V, pfx, tiles, threads, s, chained, stage);       \
-        if (pass == 2) return fast_launch_pass23<2, CKV, RV, HV, false, false, PV>(V, pfx, tiles, threads, s, chained, stage);       \
-        return fast_launch_pass23<3, CKV, RV, HV, false, false, PV>(V, pfx, tiles, threads, s, chained, stage);           \
+        if (pass == 1) return fast_launch_pass23<1, CKV, RV, HV, false, false, PV>(V, pfx, tiles, threads, s, stage);       \
+        if (pass == 2) return fast_launch_pass23<2, CKV, RV, HV, false, false, PV>(V, pfx, tiles, threads, s, stage);       \
+        return fast_launch_pass23<3, CKV, RV, HV, false, false, PV>(V, pfx, tiles, threads, s, stage);           \
     }
 #define CONEF_FAST_CASE(CKV, RV, HV) CONEF_FAST_CASE_P(CKV, RV, HV, false) CONEF_FAST_CASE_P(CKV, RV, HV, true)
     CONEF_FAST_CASE(CONEF_C_INT4, 4, true)
@@ -49,11 +49,11 @@ cudaError_t fast_launch(int pass, int ckind, int rank, int half, const DevView &
     return cudaErrorNotSupported;
 }
 
-cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained)
+cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
 {
     if (tiles <= 0)
         return cudaSuccess;
-    return launch(chained, rank == 4 ? k_fast_p1_combine<4> : k_fast_p1_combine<8>, dim3(tiles, V.n_workers), 256, 0, s, V, pfx);
+    return launch(rank == 4 ? k_fast_p1_combine<4> : k_fast_p1_combine<8>, dim3(tiles, V.n_workers), 256, 0, s, V, pfx);
 }
 
 }  // namespace conef

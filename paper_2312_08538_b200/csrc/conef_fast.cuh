@@ -778,9 +778,9 @@ __global__ void __launch_bounds__(256) k_fast_p1_combine(const __grid_constant__
 // ------------------------------------------------------------------ launch helpers (conef_fast.cu)
 // PASS: 1, 2 or 3.  Returns cudaErrorNotSupported for a configuration that has no tuned kernel.
 // short_tiles: the plan's tile lengths are below the limits (small models); narrow: the launch's
-// tensors have rows shorter than a warp's 256 elements (pass 1 sums several rows per warp); chained: see launch()
+// tensors have rows shorter than a warp's 256 elements (pass 1 sums several rows per warp)
 cudaError_t fast_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx,
-                        int tiles, int threads, cudaStream_t s, bool chained, bool short_tiles, bool narrow, size_t stage);
-cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained);
+                        int tiles, int threads, cudaStream_t s, bool short_tiles, bool narrow, size_t stage);
+cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s);
 
 }  // namespace conef

@@ -60,25 +60,25 @@ k_fast_multi(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 }
 
 template <int PASS, int CK, int R, bool HALF, bool PARTIAL>
-static cudaError_t multi(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained, size_t smem)
+static cudaError_t multi(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem)
 {
     static int done[64];
     const cudaError_t e = opt_in_smem(k_fast_multi<PASS, CK, R, HALF, PARTIAL>, smem, done);
     if (e != cudaSuccess)
         return e;
-    return launch(chained, k_fast_multi<PASS, CK, R, HALF, PARTIAL>, dim3(tiles, V.n_workers), kMultiThreads, smem, s, V, pfx);
+    return launch(k_fast_multi<PASS, CK, R, HALF, PARTIAL>, dim3(tiles, V.n_workers), kMultiThreads, smem, s, V, pfx);
 }
 
 cudaError_t multi_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s,
-                         bool chained, size_t smem)
+                         size_t smem)
 {
     if (tiles <= 0)
         return cudaSuccess;
 #define CONEF_MULTI_CASE_P(CKV, RV, HV, PV)                                                 \
     if (ckind == CKV && rank == RV && (half != 0) == HV && (V.beta != 0.f) == PV)           \
-        return pass == 1   ? multi<1, CKV, RV, HV, PV>(V, pfx, tiles, s, chained, smem)     \
-               : pass == 2 ? multi<2, CKV, RV, HV, PV>(V, pfx, tiles, s, chained, smem)     \
-                           : multi<3, CKV, RV, HV, PV>(V, pfx, tiles, s, chained, smem);
+        return pass == 1   ? multi<1, CKV, RV, HV, PV>(V, pfx, tiles, s, smem)     \
+               : pass == 2 ? multi<2, CKV, RV, HV, PV>(V, pfx, tiles, s, smem)     \
+                           : multi<3, CKV, RV, HV, PV>(V, pfx, tiles, s, smem);
 #define CONEF_MULTI_CASE(CKV, RV, HV) CONEF_MULTI_CASE_P(CKV, RV, HV, false) CONEF_MULTI_CASE_P(CKV, RV, HV, true)
     CONEF_MULTI_CASE(CONEF_C_INT4, 4, true)
     CONEF_MULTI_CASE(CONEF_C_INT4, 8, true)

@@ -62,6 +62,6 @@ inline void multi_classify(LayerDesc &L, int ckind, int scale_bytes)
 
 // the launch of one pass: conef_fastmulti.cu.  smem: the most that a CTA's tiles need
 cudaError_t multi_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s,
-                         bool chained, size_t smem);
+                         size_t smem);
 
 }  // namespace conef

@@ -11,7 +11,7 @@ static cudaError_t flat16(const DevView &V, const int32_t *pfx, int tiles, cudaS
     const cudaError_t e = opt_in_smem(k_flat16<QK, CK, HALF, ICO>, smem, done);
     if (e != cudaSuccess)
         return e;
-    return launch(true, k_flat16<QK, CK, HALF, ICO>, dim3(tiles, V.n_workers), kF16Threads, smem, s, V, pfx);
+    return launch(k_flat16<QK, CK, HALF, ICO>, dim3(tiles, V.n_workers), kF16Threads, smem, s, V, pfx);
 }
 
 cudaError_t flat16_launch(int qkind, int ckind, int half, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)

@@ -305,12 +305,12 @@ k_gs_cluster(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx,
 // Launch over `tiles` tensors (prefix table pfx) with the given cluster size.
 template <int R>
 inline cudaError_t gs_launch(const DevView &V, const int32_t *pfx, int tiles, int cluster_size, float *out_sum,
-                             cudaStream_t s, bool chained)
+                             cudaStream_t s)
 {
     if (tiles <= 0)
         return cudaSuccess;
     static bool allowed[64] = {};
-    return launch_cluster(chained, k_gs_cluster<R>, tiles, cluster_size, kGsThreads, s, allowed, V, pfx, out_sum);
+    return launch_cluster(k_gs_cluster<R>, tiles, cluster_size, kGsThreads, s, allowed, V, pfx, out_sum);
 }
 
 }  // namespace conef

@@ -126,11 +126,11 @@ static void step(const DevView &V, const int32_t *pfx, int first, int tiles, int
 {
     const dim3 grid(tiles, groups);
     if (V.cs_rows == 5)
-        launch(true, k_sketch_il<QK, 5, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
+        launch(k_sketch_il<QK, 5, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
     else if (V.cs_rows == 3)
-        launch(true, k_sketch_il<QK, 3, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
+        launch(k_sketch_il<QK, 3, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
     else
-        launch(true, k_sketch_il<QK, 0, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
+        launch(k_sketch_il<QK, 0, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
 }
 
 // a group of tensors
@@ -156,9 +156,9 @@ static int together(const Group &G, int worker0, int batches)
     const uint32_t stride = (uint32_t)(near ? 2 * NW : NW);
     const int64_t newoff = near ? GW : G.n_records * NW;
     const dim3 egrid(G.etiles, batches);
-    launch(true, k_sketch_swap<GW, true, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
+    launch(k_sketch_swap<GW, true, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
     step<QK, W, LP, IL_SCRATCH>(G.V, G.pfx, G.first, G.tiles, worker0, batches, G.records, stride, newoff, G.s);
-    launch(true, k_sketch_swap<GW, false, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
+    launch(k_sketch_swap<GW, false, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
     return 3;
 }
 template <int QK, int W, int LP>
@@ -168,22 +168,22 @@ static int split(const Group &G, int worker0)
     if constexpr (GW > 1) {
         if (G.n_records * 8 * GW > kIlTogether) {   // (one tensor: a group of several is at most 2 kIlGroupBytes)
             const int tiles = (int)(((G.n_records + 1) / 2 + kIlEntries - 1) / kIlEntries);
-            launch(true, k_sketch_fold<GW, 0>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
-            launch(true, k_sketch_fold<GW, 1>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(k_sketch_fold<GW, 0>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(k_sketch_fold<GW, 1>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
             step<QK, W, LP, IL_FOLD>(G.V, G.pfx, G.first, G.tiles, worker0, 1, G.records, GW, 0, G.s);
-            launch(true, k_sketch_fold<GW, 2>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
-            launch(true, k_sketch_fold<GW, 3>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(k_sketch_fold<GW, 2>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
+            launch(k_sketch_fold<GW, 3>, dim3(tiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records);
             return 5;
         }
     }
-    launch(true, k_sketch_swap<GW, true, true>, dim3(G.etiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, GW, 0);
+    launch(k_sketch_swap<GW, true, true>, dim3(G.etiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, GW, 0);
     step<QK, W, LP, IL_SPLIT>(G.V, G.pfx, G.first, G.tiles, worker0, 1, G.records, GW, 0, G.s);
     if (GW == 1)   // (its one slice is the state)
         return 2;
-    launch(true, k_sketch_swap<GW, false, true>, dim3(G.etiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, GW, G.second ? -1 : G.n_records);
+    launch(k_sketch_swap<GW, false, true>, dim3(G.etiles), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, GW, G.second ? -1 : G.n_records);
     if (G.second)
         return 3;
-    launch(true, k_sketch_back, dim3(dim3(G.etiles, GW)), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, G.n_records);
+    launch(k_sketch_back, dim3(dim3(G.etiles, GW)), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, G.n_records);
     return 4;
 }
 

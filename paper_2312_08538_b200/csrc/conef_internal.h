@@ -196,11 +196,16 @@ cudaError_t fused_launch(int ckind, int rank, int half, int ctas_per_sm, const F
 // serialization): its CTAs come onto the SMs as the last ones of that kernel leave them, or earlier where that
 // kernel lets them (grid_release), and look up their tensor meanwhile.  The kernel has to call grid_wait()
 // (conef_common.cuh) in every thread before it touches anything but the tables of the plan, its parameters and
-// its own shared memory.  chained = false: an ordinary launch, after an event of another stream.
+// its own shared memory.
+// The attribute relaxes the order towards the kernel ahead in the same stream only ("opportunistically allow the grid's
+// execution to overlap with the previous kernel in the stream", cudaLaunchAttributeProgrammaticStreamSerialization).  What
+// an event holds the stream back for is over before the launch begins: cudaStreamWaitEvent "makes all future work submitted
+// to stream wait for all work captured in event".  So a caller may order a call by events, and the launches behind the
+// passes' side streams and those on them are no exception.
 // One small layer on two workers 25.9 -> 15.9 us per step and update (four kernels), index sets of 54 convolutions
 // 733 -> 552 us (two kernels each), iConEF-v1 behind an odd layer 159 -> 137 us, ResNet-50's random block 250 -> 233 us.
 template <class... P, class... A>
-inline cudaError_t launch(bool chained, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A &&...args)
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -211,14 +216,14 @@ inline cudaError_t launch(bool chained, void (*kernel)(P...), dim3 grid, int thr
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = chained ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
 }
 
 // The same with thread-block clusters; sizes above 8 (the portable limit) opt the kernel in once per device:
 // `allowed` is the caller's per-kernel record.
 template <class... P, class... A>
-inline cudaError_t launch_cluster(bool chained, void (*kernel)(P...), int tiles, int cluster_size, int threads, cudaStream_t s,
+inline cudaError_t launch_cluster(void (*kernel)(P...), int tiles, int cluster_size, int threads, cudaStream_t s,
                                   bool (&allowed)[64], A &&...args)
 {
     if (cluster_size > 8) {
@@ -246,7 +251,7 @@ inline cudaError_t launch_cluster(bool chained, void (*kernel)(P...), int tiles,
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = chained ? 2 : 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
 }
 

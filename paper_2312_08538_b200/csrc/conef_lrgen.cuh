@@ -547,6 +547,6 @@ __global__ void __launch_bounds__(kGenThreads, PASS == 2 || R == 8 || R == 0 ? 3
 }
 
 // launcher (conef_lrgen.cu); coop: the plan's
-cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained, bool coop);
+cudaError_t gen_launch(int pass, int ckind, int rank, int unit, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool coop);
 
 }  // namespace conef

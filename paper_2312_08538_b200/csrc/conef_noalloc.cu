@@ -262,13 +262,13 @@ int write_indices(uint64_t seed, int64_t tensor, int64_t step, int64_t d, int64_
     if (ctas <= kNaClusterTiles && how != CONEF_SELECT_HALF) {
         static bool allowed[64] = {};
         const int size = ctas <= 1 ? 1 : ctas <= 2 ? 2 : ctas <= 4 ? 4 : kNaClusterTiles;
-        launch_cluster(true, k_na_cluster, 1, size, kSelThreads, s, allowed, a, idx_out);
+        launch_cluster(k_na_cluster, 1, size, kSelThreads, s, allowed, a, idx_out);
         return cudaGetLastError() == cudaSuccess ? CONEF_OK : CONEF_ERR_CUDA;
     }
     a.ntiles = (uint32_t)((d + kNaTile - 1) / kNaTile);
-    launch(true, k_na_select, dim3(a.ntiles), kSelThreads, 0, s, a);
+    launch(k_na_select, dim3(a.ntiles), kSelThreads, 0, s, a);
     if (how != CONEF_SELECT_HALF)
-        launch(true, k_na_write, dim3(a.ntiles), kSelThreads, 0, s, a, idx_out);
+        launch(k_na_write, dim3(a.ntiles), kSelThreads, 0, s, a, idx_out);
     return cudaGetLastError() == cudaSuccess ? CONEF_OK : CONEF_ERR_CUDA;
 }
 

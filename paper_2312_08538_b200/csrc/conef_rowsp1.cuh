@@ -228,7 +228,7 @@ inline bool rows_p1_takes(const LayerDesc &L)
 }
 
 template <int R>
-inline cudaError_t rows_p1_launch(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, bool chained)
+inline cudaError_t rows_p1_launch(const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s)
 {
     if (tiles <= 0)
         return cudaSuccess;
@@ -238,12 +238,12 @@ inline cudaError_t rows_p1_launch(const DevView &V, const int32_t *pfx, int tile
         const cudaError_t e = opt_in_smem(k_rows_p1<R, true>, smem, done_partial);
         if (e != cudaSuccess)
             return e;
-        return launch(chained, k_rows_p1<R, true>, dim3(tiles, V.n_workers), kRpThreads, smem, s, V, pfx);
+        return launch(k_rows_p1<R, true>, dim3(tiles, V.n_workers), kRpThreads, smem, s, V, pfx);
     }
     const cudaError_t e = opt_in_smem(k_rows_p1<R, false>, smem, done_plain);
     if (e != cudaSuccess)
         return e;
-    return launch(chained, k_rows_p1<R, false>, dim3(tiles, V.n_workers), kRpThreads, smem, s, V, pfx);
+    return launch(k_rows_p1<R, false>, dim3(tiles, V.n_workers), kRpThreads, smem, s, V, pfx);
 }
 
 }  // namespace conef

@@ -918,7 +918,7 @@ int launch_fast(conef_ctx *ctx, int pass, const DevView &V, cudaStream_t s, bool
         const size_t stage = fast_stage_bytes(pass, ctx->q.rank, P.fast_it[pass - 1], P.fast_subs[k], P.fast_threads[k],
                                               P.fast_unit, V.scale_half ? 2 : 4);
         CK_CUDA(fast_launch(pass, ctx->c.kind, ctx->q.rank, V.scale_half, V, table_ptr(ctx, table), n, P.fast_threads[k], sk,
-                            P.short_tiles, P.fast_narrow[k] != 0, stage));
+                            P.fast_narrow[k] != 0, stage));
         LAUNCH_CHECK(ctx);
         if (off_main) {
             CK_CUDA(cudaEventRecord(ctx->ev_join[used], sk));

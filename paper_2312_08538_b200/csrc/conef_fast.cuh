@@ -251,7 +251,7 @@ __device__ __forceinline__ void static_for(F &&f)
 // and the stored error is C(beta e + r).  A template parameter so that Alg. 2 pays nothing for it.
 // Tile `local` of a tensor by the bd threads of a CTA, or with MULTI by bd of its threads, which meet at barrier
 // `bar` of the CTA and have smem_raw for themselves.
-template <int PASS, int CK, int R, bool HALF, bool SHORT, bool NARROW, bool PARTIAL, bool MULTI>
+template <int PASS, int CK, int R, bool HALF, bool NARROW, bool PARTIAL, bool MULTI>
 __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp, const uint32_t local, const int tid, const int bd,
                                           uint8_t *smem_raw, const int bar)
 {
@@ -272,7 +272,7 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
     };
     // tile length: a constant for large models (faster than the same value read from the table),
     // the table's value for small ones
-    const uint32_t IT = SHORT ? (uint32_t)(PASS == 1 ? Lp->f_it1 : PASS == 2 ? Lp->f_it2 : Lp->f_it3)
+    const uint32_t IT = MULTI ? (uint32_t)(PASS == 1 ? Lp->f_it1 : PASS == 2 ? Lp->f_it2 : Lp->f_it3)
                               : (uint32_t)(PASS == 1 ? kFastIt1 : PASS == 2 ? kFastIt2 : kFastIt3);
     constexpr int kRing23 = ring_depth(PASS, R);
     constexpr int NI = iters_per_step(PASS, R);                   // iterations a thread works on at once
@@ -741,14 +741,14 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
     }
 }
 
-template <int PASS, int CK, int R, bool HALF, bool SHORT, bool NARROW, bool PARTIAL = false>
+template <int PASS, int CK, int R, bool HALF, bool NARROW, bool PARTIAL = false>
 __global__ void __launch_bounds__(kFastMaxWarps * 32, min_ctas(PASS, R))
 k_fast_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
-    fast_tile<PASS, CK, R, HALF, SHORT, NARROW, PARTIAL, false>(V, V.layers + li, blockIdx.x - pfx[li], threadIdx.x, blockDim.x, smem_raw, 0);
+    fast_tile<PASS, CK, R, HALF, NARROW, PARTIAL, false>(V, V.layers + li, blockIdx.x - pfx[li], threadIdx.x, blockDim.x, smem_raw, 0);
 }
 
 // P_i[row][c] = sum over the warps that meet the row, in warp order
@@ -777,10 +777,10 @@ __global__ void __launch_bounds__(256) k_fast_p1_combine(const __grid_constant__
 
 // ------------------------------------------------------------------ launch helpers (conef_fast.cu)
 // PASS: 1, 2 or 3.  Returns cudaErrorNotSupported for a configuration that has no tuned kernel.
-// short_tiles: the plan's tile lengths are below the limits (small models); narrow: the launch's
+// narrow: the launch's
 // tensors have rows shorter than a warp's 256 elements (pass 1 sums several rows per warp)
 cudaError_t fast_launch(int pass, int ckind, int rank, int half, const DevView &V, const int32_t *pfx,
-                        int tiles, int threads, cudaStream_t s, bool short_tiles, bool narrow, size_t stage);
+                        int tiles, int threads, cudaStream_t s, bool narrow, size_t stage);
 cudaError_t fast_launch_p1_combine(int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s);
 
 }  // namespace conef

@@ -22,9 +22,9 @@ k_fast_multi(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
         uint8_t *mine = smem_raw + sub * multi_tile_bytes(PASS, R, CK == CONEF_C_INT4 ? 1 : 2, HALF ? 2 : 4, it, L.f_subs, bd, L.unit);
         const int tid = threadIdx.x - sub * bd;
         if (PASS == 1 && L.cols < 256)
-            fast_tile<PASS, CK, R, HALF, true, PASS == 1, PARTIAL, true>(V, &L, local, tid, bd, mine, sub + 1);
+            fast_tile<PASS, CK, R, HALF, PASS == 1, PARTIAL, true>(V, &L, local, tid, bd, mine, sub + 1);
         else
-            fast_tile<PASS, CK, R, HALF, true, false, PARTIAL, true>(V, &L, local, tid, bd, mine, sub + 1);
+            fast_tile<PASS, CK, R, HALF, false, PARTIAL, true>(V, &L, local, tid, bd, mine, sub + 1);
         return;
     }
     grid_wait();

@@ -1134,7 +1134,7 @@ int launch_randk_select(conef_ctx *ctx, const DevView &V, cudaStream_t s)
     const int nh = tiles_of(ctx, T_HIST), no = tiles_of(ctx, T_SEL_OFFS);
     if (nh == 0)
         return CONEF_OK;
-    if (ctx->plan.sel_cluster > 0 && (V.sel_how == CONEF_SELECT_NORMAL || V.sel_how == CONEF_SELECT_MISS)) {   // (the others have no list)
+    if (ctx->plan.sel_cluster > 0 && V.sel_how != CONEF_SELECT_STALE) {   // (clusters leave no list to be found changed)
         static bool allowed[64] = {};
         launch_cluster(k_rk_select_cluster, tiles_of(ctx, T_SEL_CLUSTER), ctx->plan.sel_cluster, kSelThreads, s, allowed, V,
                        table_ptr(ctx, T_SEL_CLUSTER));

@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_select(const NaArgs a)
     __shared__ SelectSharedTiles S;
     __shared__ uint32_t s_n, s_base, s_cnt, s_last, s_listed;
     const int tid = threadIdx.x;
-    const bool windowed = a.d > (uint32_t)kSelShortTensor;
+    const bool windowed = a.d > (uint32_t)kSelShortTensor;   // (shorter ones come here with CONEF_SELECT_HALF only: see k_na_cluster)
     grid_release();
     S.hist[tid] = 0;   // the bins of select_threshold
     if (tid == 0)
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kSelThreads) k_na_cluster(const NaArgs a, uint
 {
     __shared__ SelectCluster S;
     grid_release();
-    const SelectResult R = select_in_cluster(S, a.stream, a.d, a.k, a.lo, a.hi, a.scale, a.how != CONEF_SELECT_NORMAL);
+    const SelectResult R = select_in_cluster(S, a.stream, a.d, a.k, a.lo, a.hi, a.scale, (int)a.how);
     grid_wait();
     if (R.failed || R.total != a.k) {
         if (blockIdx.x == 0 && threadIdx.x == 0)

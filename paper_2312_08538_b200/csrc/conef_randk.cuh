@@ -205,7 +205,7 @@ static __global__ void __launch_bounds__(kSelThreads) k_rk_select_cluster(const 
     const LayerDesc &L = V.layers[li];
     const uint32_t d = (uint32_t)L.d, k = (uint32_t)L.k;
     const uint64_t st = stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step);
-    const SelectResult R = select_in_cluster(S, st, d, k, L.sel_lo, L.sel_hi, L.sel_scale, V.sel_how == CONEF_SELECT_MISS);
+    const SelectResult R = select_in_cluster(S, st, d, k, L.sel_lo, L.sel_hi, L.sel_scale, V.sel_how);
     grid_wait();
     if (rank == 0 && threadIdx.x == 0) {
         if (R.failed)

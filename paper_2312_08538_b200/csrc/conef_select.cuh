@@ -392,8 +392,9 @@ struct SelectResult {
     uint32_t word, first, total;   // this thread's 32 elements, members before this CTA's tile, members of the tensor
     bool failed;
 };
+// how: CONEF_SELECT_*; with STALE, of which there is nothing here (no list outlives the call), as with MISS
 __device__ __forceinline__ SelectResult select_in_cluster(SelectCluster &S, uint64_t st, uint32_t d, uint32_t k, uint32_t lo, uint32_t hi,
-                                                          uint64_t scale, bool miss)
+                                                          uint64_t scale, int how)
 {
     static_assert(kHistTile == 32 * kSelThreads, "a word per thread");
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
@@ -405,6 +406,7 @@ __device__ __forceinline__ SelectResult select_in_cluster(SelectCluster &S, uint
         scale = 256u;
     }
     const SelectWindow W{lo, hi, d, k, scale, nullptr};
+    const uint32_t room = how == CONEF_SELECT_FULL ? 1u : (uint32_t)kSelMine;
     S.hist[tid] = 0;   // the bins of select_threshold
     if (tid == 0)
         S.n_mine = S.below = 0;
@@ -416,7 +418,7 @@ __device__ __forceinline__ SelectResult select_in_cluster(SelectCluster &S, uint
         word = select_word(st, j0, d, lo, hi, inside);
         for (; inside; inside &= inside - 1) {
             const uint32_t j = j0 + (uint32_t)__ffs(inside) - 1u, pos = atomicAdd(&S.n_mine, 1u);
-            if (pos < (uint32_t)kSelMine)
+            if (pos < room)
                 S.mine[pos] = make_uint2(hash32(st, j), j);
         }
     }
@@ -431,7 +433,7 @@ __device__ __forceinline__ SelectResult select_in_cluster(SelectCluster &S, uint
                 n = *cluster.map_shared_rank(&S.n_mine, tid);
                 below = *cluster.map_shared_rank(&S.below, tid);
             }
-            const bool full = __any_sync(0xffffffffu, n > (uint32_t)kSelMine);
+            const bool full = __any_sync(0xffffffffu, n > room);
             uint32_t inc = n;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -445,7 +447,7 @@ __device__ __forceinline__ SelectResult select_in_cluster(SelectCluster &S, uint
             }
             if (tid == kSelClusterTiles - 1) {
                 S.base[kSelClusterTiles] = inc;
-                S.r_found = !full && !miss;
+                S.r_found = !full && (how == CONEF_SELECT_NORMAL || how == CONEF_SELECT_FULL);
             }
         }
         __syncthreads();

@@ -83,7 +83,7 @@ def test_selections_whose_window_fails(how, k_num, k_den):
 # models whose tensors all have at most 16 tiles: one cluster per tensor, of as many CTAs as the largest has tiles
 @pytest.mark.parametrize("shapes", [[(1, 2), (32, 32), (1, 1025), (3, 999)], [(1, 8193), (5, 205)], [(3, 8192), (1, 4 * 8192)], [(16, 8192), (7, 9)]])
 @pytest.mark.parametrize("k_num,k_den", [(1, 100), (1, 2), (1, 1)])
-@pytest.mark.parametrize("how", ["NORMAL", "MISS"])
+@pytest.mark.parametrize("how", ["NORMAL", "MISS", "FULL"])
 def test_small_models_by_a_cluster(shapes, k_num, k_den, how):
     from paper_2312_08538_b200 import binding as b
     seed = 19

@@ -26,18 +26,17 @@ namespace conef {
 #ifndef CONEF_RS_ROWS
 #define CONEF_RS_ROWS 2
 #endif
-// Rows of a bucket whose loads are issued together.  Measured on the two-block GPT-2-XL list with a
-// low-rank Q (pass 3 on the row sketch), on an earlier version of the loop body: 2 rows 1.05 ms,
-// 4 rows 1.16 ms, 8 rows 1.24 ms (registers against occupancy); the current body with 2 rows takes
-// 0.87 ms.  A per-thread ring of asynchronous copies 8 rows deep over the concatenated row lists,
-// without and with the lists in shared memory, was also built: 0.86 and 0.96 ms with almost twice
-// the instructions, so the simple form stays.
+// Rows of a bucket whose loads are issued together.  Measured with a low-rank Q and one sketch row, which rs_walk takes now
+// where 16-byte loads line up, on the two-block GPT-2-XL list: 2 rows 1.05 ms, 4 rows 1.16 ms, 8 rows 1.24 ms (registers
+// against occupancy).
 constexpr int kRsRows = CONEF_RS_ROWS;
 
+// The single-phase compressors, and the low-rank residual with several sketch rows or where 16-byte loads do not line up.
 // VEC columns per thread (4: 16-byte loads; needs cols % 4 == 0 and 16-byte aligned gradients; 1: any shape).  The CTA covers kRsThreads * VEC columns of kRsBuckets
 // buckets of one sketch row.
-// RK: 4 when the tensor's rank is exactly 4 (one 16-byte load per row of P_hat), else 8 (any rank).
-template <int QK, int VEC, bool V1, int RK>
+// A low-rank Q has room for any rank: a body for rank 4 with one 16-byte load per row of P_hat takes as long (two matrices of
+// 4 M elements, two workers, rank 4, three sketch rows: 399 us in binary16 with both, 394 and 403 us in fp32 without and with it).
+template <int QK, int VEC, bool V1>
 __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, const int li, uint32_t local)
 {
     const int worker = blockIdx.y;
@@ -67,6 +66,7 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
     if (QK == CONEF_Q_RANDBLOCK)
         blk_start = randblock_start(stream_key(V.seed_q, (uint64_t)li, (uint64_t)V.step), d, (uint32_t)L.k);
     const int r = L.rank;
+    constexpr int RK = QK == CONEF_Q_LOWRANK ? CONEF_MAX_RANK : 1;
     float qreg[VEC][RK];   // Q_i[b..b+VEC-1][:], fixed for the thread
     const float *__restrict__ phat = fresh(V.phat + L.msgp_off);
     if (QK == CONEF_Q_LOWRANK) {
@@ -204,20 +204,15 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
                     }
                 } else {
                     float ph[RK];
-                    if (RK == 4) {
-                        const float4 t = load_global((const float4 *)(phat + (size_t)a * 4));
-                        ph[0] = t.x; ph[1] = t.y; ph[2] = t.z; ph[3] = t.w;
-                    } else {
 #pragma unroll
-                        for (int c = 0; c < RK; ++c)
-                            ph[c] = c < r ? phat[(size_t)a * r + c] : 0.f;
-                    }
+                    for (int c = 0; c < RK; ++c)
+                        ph[c] = c < r ? phat[(size_t)a * r + c] : 0.f;
 #pragma unroll
                     for (int x = 0; x < VEC; ++x) {
                         res[x] = p[x];
 #pragma unroll
                         for (int c = 0; c < RK; ++c)
-                            if (RK == 4 || c < r)
+                            if (c < r)
                                 res[x] = __fmaf_rn(-ph[c], qreg[x][c], res[x]);   // r = p - P_hat Q_i^T
                     }
                 }
@@ -244,7 +239,6 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
     const int li = find_layer(V.pfx_rs, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
     const uint32_t local = blockIdx.x - V.pfx_rs[li];
-    constexpr int RKG = QK == CONEF_Q_LOWRANK ? 8 : 4;   // the rank only matters to the low-rank Q
     const bool vec = L.rs_vec == 4 && V.rs_vec_ok;
     if constexpr (V1 && QK == CONEF_Q_LOWRANK) {
         __shared__ RwShared S;
@@ -258,7 +252,7 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
     }
     grid_wait();
     if (!(V1 && QK == CONEF_Q_LOWRANK) && vec)
-        rs_body<QK, 4, V1, RKG>(V, L, li, local);
+        rs_body<QK, 4, V1>(V, L, li, local);
     else if (L.rs_vec == 4) {
         // 16-byte loads are not possible with this call's gradient pointers: the same tiles,
         // four scalar slabs per vector slab
@@ -266,9 +260,9 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
         const uint32_t slabs1 = (uint32_t)((L.cols + kRsThreads - 1) / kRsThreads);
         const uint32_t slab = local % slabs4, rest = local / slabs4;
         for (uint32_t s = slab * 4; s < min(slabs1, slab * 4 + 4); ++s)
-            rs_body<QK, 1, V1, RKG>(V, L, li, rest * slabs1 + s);
+            rs_body<QK, 1, V1>(V, L, li, rest * slabs1 + s);
     } else
-        rs_body<QK, 1, V1, RKG>(V, L, li, local);
+        rs_body<QK, 1, V1>(V, L, li, local);
 }
 
 // ------------------------------------------------------------------ low-rank passes 1 and 2 on a row-sketch state

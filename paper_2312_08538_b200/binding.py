@@ -281,7 +281,7 @@ class ConEF:
         _check(lib.conef_set_select(self.h, int(how)), "conef_set_select")
 
     def set_fused(self, enable: bool, tile_periods: int = 0, ctas_per_sm: int = 0) -> None:
-        """Low-rank phase 1 in one persistent kernel (default on); tile_periods = 0: default tile
+        """Low-rank phase 1 in one persistent kernel (default off); tile_periods = 0: default tile
         length; ctas_per_sm 0 (default) or 2..4."""
         _check(lib.conef_set_fused(self.h, int(enable), int(tile_periods), int(ctas_per_sm)), "conef_set_fused")
 

@@ -611,7 +611,7 @@ struct conef_ctx {
     int fast = 1;
     int sm_count = kPlanSMs;   // of the device the context was created on (read in conef_init)
     int64_t launches = 0;
-    // fused passes 2 + 3 (conef_fused.cu): on by default where the device allows
+    // fused passes 2 + 3 (conef_fused.cu): off by default
     int fused = 0, fused_tile_periods = kFuTilePeriods, fused_ctas_per_sm = 2;
     bool fused_ready = false;       // configuration and task list exist for this device
     bool fused_dirty = false;       // the tables on the device are older than the host's

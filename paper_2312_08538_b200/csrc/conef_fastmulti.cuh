@@ -7,7 +7,7 @@
 // one tile of the passes for any shape (conef_lrgen.cuh; up to multi_gen elements), or, in pass 1, of a 1-D tensor that passes through.
 // What a tile computes, and the order of its sums, is that of those kernels.
 // ResNet-50 list (seven widths and one odd convolution), int8, rank 4, four workers: 550 -> 440 us per step and update; six
-// aligned matrices of 17 M elements, int4, eight workers: 803 -> 750 us.  (64 registers, four CTAs per SM, spill: 577 us on the
+// aligned matrices of 16 M elements together, int4, one worker 220 -> 182 us, eight workers 500 -> 492.  (64 registers, four CTAs per SM, spill: 577 us on the
 // first list; two CTAs: 485 us.)
 #pragma once
 #include "conef_fast.cuh"
@@ -17,8 +17,9 @@ namespace conef {
 
 constexpr int kMultiThreads = 256;
 constexpr size_t kMultiSmem = 72 * 1024;   // shared memory of a CTA's tiles, where more than one shares it: three CTAs per SM
-// Iterations per tile of passes 1 and 3 at most (pass 2's are part of the order of its sums): longer tiles leave the last
-// wave of CTAs nearly empty.  (ResNet-50 list: 8 iterations 554 us, 16 481, 32 457.)
+// Iterations per tile of passes 1 and 3 at most (pass 2's are part of the order of its sums).  Shorter tiles are slower, longer ones
+// no faster at rank 4.  ResNet-50 list, four workers, int8, 8, 16, 32, 64 iterations and no limit: rank 4 532, 462, 443, 441, 441 us, rank 8
+// 731, 606, 563, 554, 555; six matrices of 16 M elements together, eight workers, int4, rank 4: 553, 508, 496, 497, 496.
 constexpr int kMultiIt = 32;
 // Tensors of any other shape share these launches up to this many of their elements (all workers).  Beyond, they and the 1-D
 // tensors have launches of their own (k_gen_pass), with four CTAs per SM instead of three at rank 4, three instead of two at rank 8,

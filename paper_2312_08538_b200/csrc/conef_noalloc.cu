@@ -198,8 +198,10 @@ __global__ void __launch_bounds__(kSelThreads) k_na_write(const NaArgs a, uint32
 }
 
 // Tensors of at most kNaClusterTiles tiles of 8192: one cluster does all of it, without the scratch
-// (one launch, and nothing kept between calls).  54 convolutions, of which 20 are that small: 552 -> 408 us with it and
-// with the first kernel's hashing ahead of its wait.
+// (one launch, and nothing kept between calls).  54 convolutions, of which 19 are that small: 552 -> 408 us with it and
+// with the first kernel's hashing ahead of its wait.  Eight calls in a row, a cluster and two kernels, k = d / 100: 1 tile 37 and 58
+// us, 8 tiles 37 and 65, 16 tiles 38 and 69 (k = d / 2: 38 and 68, 38 and 80, 38 and 85), so the line is not where the cluster gets
+// slower: eight CTAs are what a cluster may have on every device without opting in.
 constexpr int kNaClusterTiles = 8;
 __global__ void __launch_bounds__(kSelThreads) k_na_cluster(const NaArgs a, uint32_t *__restrict__ idx_out)
 {

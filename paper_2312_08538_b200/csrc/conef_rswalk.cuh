@@ -8,7 +8,7 @@
 //
 // Before, every thread loaded entries, rows of P_hat and sketch entries when they were due, two rows at a time: a chain of
 // trips to L2.  GPT-2-small list, rank 4, binary16 sketch, one worker: passes 204 / 183 / 239 us, now 169 / 148 / 177 us
-// (4.4 B per element: 3.1 - 3.7 TB/s).  Bound by instruction issue and by 20 warps per SM (94 registers).  With single loads
+// (4.4 B per element: 3.1 - 3.7 TB/s).  Bound by latency: 17 warps per SM (94 registers), issue slots 35 to 44 % busy.  With single loads
 // four rows ahead instead of batches the waits ran to the youngest load: 266 / 246 / 259 us.  The single-phase compressors
 // have no such chain in their step and stay with rs_body (3 % slower here).
 #pragma once

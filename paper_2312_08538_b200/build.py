@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libconef.so")
-SOURCES = ["conef_api.cu", "conef_fast.cu", "conef_fastmulti.cu", "conef_flat16.cu", "conef_flatvec.cu", "conef_fused.cu", "conef_ilsketch.cu", "conef_lrgen.cu", "conef_noalloc.cu"]
+SOURCES = ["conef_api.cu", "conef_fast.cu", "conef_fastmulti.cu", "conef_flat16.cu", "conef_flatvec.cu", "conef_fused.cu", "conef_ilsketch.cu", "conef_lrgen.cu", "conef_lrgen_int8.cu", "conef_lrgen_int4.cu", "conef_noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-fmad=false", "-Xcompiler", "-fPIC"]
 

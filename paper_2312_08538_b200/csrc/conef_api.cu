@@ -85,7 +85,7 @@ struct Plan {
     int fast_it[3] = {kFastIt1, kFastIt2, kFastIt3};   // iterations per tile of the tuned passes
     int fast_unit = 256;            // elements per quantisation block
     bool any_fast = false, any_slow = false, any_rs12 = false, any_gen = false;
-    bool gen_coop = false;      // pass 2 for any shape: a CTA per tile
+    size_t gen_smem2 = 0;       // shared memory of a CTA of pass 2 for any shape
     bool short_tiles = false;   // tile lengths of the tuned passes below their limits
     bool multi = false;         // one launch per pass takes tensors of all widths (conef_fastmulti.cuh)
     bool multi_gen = false;     // ... those of any other shape and 1-D ones included
@@ -202,7 +202,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
     int it1 = kFastIt1, it2 = kFastIt2, it3 = kFastIt3;
     GenPlan gen;
     if (q->kind == CONEF_Q_LOWRANK) {
-        int64_t cta_iters = 0, rows = 0, chunks = 0, tiles2 = 0;
+        int64_t cta_iters = 0, rows = 0, elems = 0, tiles2 = 0;
         for (int l = 0; l < n_tensors; ++l) {
             LayerDesc T{};
             T.rows = tensors[l].rows;
@@ -215,10 +215,10 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
             if (T.fast)
                 cta_iters += T.f_niter * T.f_ncg;
             rows += T.rows;
-            chunks += ceil_div(T.d, kGenChunk);
+            elems += T.d;
             tiles2 += ceil_div(T.rows, kP2RowsPerTile) * ceil_div(T.cols, kGenCols);
         }
-        gen = gen_plan(rows * n_workers, chunks * n_workers, tiles2 * n_workers);
+        gen = gen_plan(q->rank, rows * n_workers, elems * n_workers, tiles2 * n_workers);
         cta_iters *= n_workers;
         it1 = fast_tile_iters(kFastIt1, cta_iters);
         it2 = fast_tile_iters(kFastIt2, cta_iters);
@@ -228,7 +228,6 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
         else
             it1 = kFastIt1, it2 = kFastIt2, it3 = kFastIt3;
     }
-    P.gen_coop = gen.coop != 0;
     P.fast_it[0] = it1, P.fast_it[1] = it2, P.fast_it[2] = it3;
     P.fast_unit = unit;
     int64_t g_off = 0, state_off = 0, il_fill = 0, hist_tiles = 0;
@@ -448,7 +447,8 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                 } else if (c->iconef == 0 && gen_takes(L, c->kind)) {
                     L.fast = 3;
                     P.any_gen = true;
-                    gen_classify(L, gen);
+                    gen_classify(L, gen, q->rank);
+                    P.gen_smem2 = std::max(P.gen_smem2, gen_p2_smem(L, q->rank));
                     L.p2_rows_fast = rtiles;
                     tiles[T_GEN1] = L.g_t1;
                     tiles[T_GEN2] = L.g_t2;
@@ -504,7 +504,9 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                         t[2 + p] = t[p];
                 }
             } else if (L.fast == 3) {
-                P.multi_smem[1] = std::max(P.multi_smem[1], kGenCoopSmem);
+                P.multi_smem[0] = std::max(P.multi_smem[0], kGenP1Smem);
+                P.multi_smem[1] = std::max(P.multi_smem[1], gen_p2_smem(L, q->rank));
+                P.multi_smem[2] = std::max(P.multi_smem[2], kGenP3Smem);
                 t[0] = L.g_t1;
                 t[1] = t[3] = L.g_t2;
                 t[2] = t[4] = L.g_t3 * L.g_groups;
@@ -1420,7 +1422,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
             if (n == 0 || (multi && ctx->plan.multi_gen) || rs12)   // (the table may hold 1-D tensors alone, of a model on a row sketch)
                 return CONEF_OK;
-            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.fast_unit, V, table_ptr(ctx, table), n, s, ctx->plan.gen_coop));
+            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, V, table_ptr(ctx, table), n, s, ctx->plan.gen_smem2));
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };

@@ -71,6 +71,18 @@ __device__ __forceinline__ float4 load_global(const float4 *p)
     asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
+__device__ __forceinline__ uint32_t load_global(const uint32_t *p)
+{
+    uint32_t v;
+    asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 load_global(const uint2 *p)
+{
+    uint2 v;
+    asm("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint32_t load_global(const uint8_t *p)
 {
     uint32_t v;
@@ -82,6 +94,43 @@ __device__ __forceinline__ unsigned short load_global(const unsigned short *p)
     unsigned short v;
     asm("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
     return v;
+}
+
+// ... OFF bytes behind p
+template <int OFF>
+__device__ __forceinline__ float load_global_at(const float *p)
+{
+    float v;
+    asm("ld.global.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ float2 load_global_at(const float2 *p)
+{
+    float2 v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "l"(p), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ float4 load_global_at(const float4 *p)
+{
+    float4 v;
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4+%5];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "n"(OFF));
+    return v;
+}
+
+template <int OFF>   // ... of what is not read again
+__device__ __forceinline__ float load_stream_at(const float *p)
+{
+    float v;
+    asm("ld.global.cs.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(OFF));
+    return v;
+}
+
+template <int OFF>   // ... where `in` says so, without a branch; v stays what it is elsewhere
+__device__ __forceinline__ void load_stream_if(float &v, const float *p, uint32_t in)
+{
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.global.cs.f32 %0, [%1+%2];\n\t}" : "+f"(v) : "l"(p), "n"(OFF), "r"(in));
 }
 
 // Loads of what other CTAs of the same launch wrote before a ticket or a flag: past L1, and volatile with

@@ -29,31 +29,7 @@ k_fast_multi(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     }
     grid_wait();
     if (L.fast == 3) {
-        const bool exact = L.rank == R && ((L.msgp_off | L.msgq_off) & 3) == 0;
-        if (PASS == 1) {
-            if (exact && L.g_nr == 4) {
-                gen_p1_body<CK, R, 4>(V, L, tile);
-            } else if (exact) {
-                gen_p1_body<CK, R, 1>(V, L, tile);
-            } else {
-                for (int x = 0; x < L.g_nr; ++x)
-                    gen_p1_body<CK, 0, 1>(V, L, tile * (uint32_t)L.g_nr + x);
-            }
-        } else if (PASS == 2) {
-            if (L.g_coop && exact)
-                gen_p2_cta<CK, R>(V, L, tile, (float *)smem_raw);
-            else if (L.g_coop)
-                gen_p2_cta<CK, 0>(V, L, tile, (float *)smem_raw);
-            else if (exact)
-                gen_p2_body<CK, R>(V, L, tile);
-            else
-                gen_p2_body<CK, 0>(V, L, tile);
-        } else {
-            if (exact)
-                gen_p3_body<CK, R, 0>(V, L, tile, smem_raw);
-            else
-                gen_p3_body<CK, 0, 0>(V, L, tile, smem_raw);
-        }
+        gen_tile<PASS, CK, HALF, PARTIAL, R>(V, L, tile, (float *)smem_raw);
     } else if (PASS == 1 && !L.compressed) {
         pass_tile(V, L, tile);
     }

@@ -82,17 +82,18 @@ struct LayerDesc {
     int64_t pp_off;      // floats, within a worker's pass-1 partial buffer
     int64_t f_niter;     // super-rows in the tensor
     // low-rank passes for any shape (conef_lrgen.cuh): rows per warp and CTAs of pass 1, CTAs of pass 2, steps
-    // per tile, chunks per step, CTAs per step and row of tiles of pass 3; whether a CTA takes a tile of pass 2
-    int32_t g_nr, g_t1, g_t2, g_it, g_step, g_groups, g_t3, g_coop;
+    // per tile, chunks per step, CTAs per step and row of tiles of pass 3; threads per tile of pass 2 (0: a CTA, gen_p2_cta)
+    int32_t g_nr, g_t1, g_t2, g_it, g_step, g_groups, g_t3, g_p2t;
     // row sketch: uint32 words in the bucket tables (see DevView::rs)
     int64_t rs_info_off; // [v][rows]: bucket of a row | sign << 31
     int64_t rs_ptr_off;  // [v][w + 1]: start of each bucket's row list
     int64_t rs_row_off;  // [v][rows]: rows by bucket, ascending within a bucket, | sign << 31
     // model update of a low-rank tensor (conef_apply.cuh): columns per thread, threads across and down, rows
     // per thread, column tiles
-    int32_t ap_vec, ap_tx, ap_ty, ap_rpt, ap_ct, ap_pad;
+    int32_t ap_vec, ap_tx, ap_ty, ap_rpt, ap_ct;
+    int32_t g_chunk;     // elements per warp and step of pass 3 for any shape
     int32_t rs_vec;      // columns per thread of the row-sketch kernel (4 or 1)
-    int32_t rs_pad;
+    int32_t g_p2w;       // columns per tile of pass 2 for any shape
 };
 
 // Device-side view of a context; passed to kernels by value.

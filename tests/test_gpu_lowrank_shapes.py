@@ -80,6 +80,45 @@ def test_order_of_sums(rank, c, many):
             e.reduce_messages(b.MSG_Q)
 
 
+# what tall models take beside it: rows of one word per lane and more, tiles of 32, 64 and 128 columns on and off whole words, chunks
+# of pass 3 that hold one, two and many rows, and row counts around a stage and a tile
+BIG = [(60011, 97, 1), (3, 1, 0), (1001, 57, 1), (1003, 58, 1), (1005, 25, 1), (257, 26, 1), (255, 121, 1), (256, 122, 1), (273, 128, 1),
+       (271, 136, 1), (77, 511, 1), (5, 1, 0), (33, 512, 1), (65, 513, 1), (19, 1023, 1), (15, 2000, 1), (1, 999, 1), (2, 130, 1)]
+
+
+@pytest.mark.parametrize("rank,c", [(1, dict(kind="int4", block=64)), (2, dict(kind="int8", block=32, scale_dtype="fp16")),
+                                    (3, dict(kind="int4", block=128, scale_dtype="fp16")), (4, dict(kind="int8", block=256, beta=0.3)),
+                                    (8, dict(kind="int4", block=256, scale_dtype="fp16")), (8, dict(kind="int8", block=128, scale_dtype="fp16", beta=0.9))])
+def test_tall_models_give_the_bits_of_the_kernels_for_every_codec(rank, c):
+    from paper_2312_08538_b200 import binding as b
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=BIG, n_workers=2, q=dict(kind="lowrank", rank=rank), c=c, grad="normal1e-3")
+    q0 = wl.q_init(cfg, "cuda")
+    both = [pu.make_gpu(cfg, q_init=q0, fast=f) for f in (True, False)]
+    # the second gradient buffer is off every vector alignment
+    room = torch.empty(sum(r * k for r, k, _ in BIG) + 1, device="cuda")
+    for t in range(3):
+        gd, _ = pu.grads_both(cfg, t)
+        room[1:].copy_(gd[1])
+        gd = [gd[0], room[1:]]
+        for e, f in zip(both, (True, False)):
+            e.step(t, gd, 0)
+            e.set_fast_path(True)   # (the same Gram-Schmidt)
+            e.reduce_messages(b.MSG_P)
+            e.set_fast_path(f)
+            e.step(t, gd, 1)
+        for l in [l for l, x in enumerate(BIG) if x[2]]:
+            for i in range(2):
+                x, y = (e.factors(l, i) for e in both)
+                for k in ("p_i", "q_i"):
+                    assert torch.equal(x[k], y[k]), (t, l, i, k)
+        for i in range(2):
+            x, y = (e.decompress_error(i) for e in both)
+            assert torch.equal(x, y), (t, i)
+        for e in both:
+            e.reduce_messages(b.MSG_Q)
+
+
 @pytest.mark.parametrize("rank,c", [(4, dict(kind="int8", block=256)), (8, dict(kind="int4", block=128, scale_dtype="fp16")),
                                     (4, dict(kind="int4", block=64, scale_dtype="fp16", beta=0.9)), (8, dict(kind="int8", block=32, scale_dtype="fp16"))])
 def test_all_widths_in_one_launch(rank, c):

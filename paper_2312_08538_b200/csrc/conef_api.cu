@@ -1426,20 +1426,33 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };
-        auto launch_rs12 = [&](int pass) -> int {
-            const int n = tiles_of(ctx, T_RS_P12);
+        auto launch_rs12 = [&](int pass) -> int {   // (pass 3: of a model whose tensors all take it)
+            const int table = pass == 3 ? T_RS : T_RS_P12, n = tiles_of(ctx, table);
             if (n == 0)
                 return CONEF_OK;
             dim3 grid(n, ctx->n_workers);
+            const int32_t *pfx = table_ptr(ctx, table);
+            auto by_rank = [&](auto rank) {
+                constexpr int RK = decltype(rank)::value;
+                if (pass == 1)
+                    launch(k_rs_pass<1, RK>, grid, kRsThreads, 0, s, V, pfx);
+                else if (pass == 2)
+                    launch(k_rs_pass<2, RK>, grid, kRsThreads, 0, s, V, pfx);
+                else
+                    launch(k_rs_pass<3, RK>, grid, kRsThreads, 0, s, V, pfx);
+            };
+            if (ctx->q.rank == 4)
+                by_rank(IntC<4>());
+            else if (ctx->q.rank == 2)
+                by_rank(IntC<2>());
+            else
+                by_rank(IntC<CONEF_MAX_RANK>());
+            LAUNCH_CHECK(ctx);
             if (pass == 1) {
-                launch(k_rs_pass12<1>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
-                LAUNCH_CHECK(ctx);
                 dim3 gridc(tiles_of(ctx, T_RS_P1C), ctx->n_workers);
                 launch(k_rs_p1_combine, gridc, 256, 0, s, V, table_ptr(ctx, T_RS_P1C));
-            } else {
-                launch(k_rs_pass12<2>, grid, kRsThreads, 0, s, V, table_ptr(ctx, T_RS_P12));
+                LAUNCH_CHECK(ctx);
             }
-            LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };
         if (phase == 0) {
@@ -1467,7 +1480,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
         if (rc == CONEF_OK && (phase == 1 || phase == 3 || phase == 4)) {
             rc = with_new_sketch(ctx, V, s, [&] {
                 if (ctx->c.kind == CONEF_C_ROWSKETCH)
-                    return launch_rowsketch<CONEF_Q_LOWRANK>(ctx, V, s);
+                    return rs12 && !ctx->plan.any_slow ? launch_rs12(3) : launch_rowsketch<CONEF_Q_LOWRANK>(ctx, V, s);
                 int r2 = fast ? launch_fast(ctx, 3, V, s, fused) : CONEF_OK;
                 if (r2 == CONEF_OK && fast)
                     r2 = launch_gen(3);

@@ -243,10 +243,7 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
     if constexpr (V1 && QK == CONEF_Q_LOWRANK) {
         __shared__ RwShared S;
         if (vec) {
-            if (L.rank == 4 && (L.msgp_off & 3) == 0)
-                rs_walk<3, 4>(V, L, local, S);
-            else
-                rs_walk<3, 8>(V, L, local, S);
+            rs_walk<3, 8>(V, L, local, S);
             return;
         }
     }
@@ -276,17 +273,21 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
 //           order by k_lr_pass2_reduce.
 // Sums over rows and columns run in bucket order, not index order: like the other factor kernels
 // they match the oracle to rounding (fp32, fixed order), not bit for bit.
-template <int PASS>
-__global__ void __launch_bounds__(kRsThreads, 5) k_rs_pass12(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+// RK: the configured rank (2, 4; 8: another one); tensors that rs_exact does not accept take the walk for any rank.
+// PASS 3 is the step's last, of models whose tensors all take the walk (else: k_rowsketch).
+// CTAs per SM: rank 4 with six, seven and eight (64 registers) on the GPT-2-small list 136 / 115 / 135, 134 / 117 / 127, 142 / 117 / 129 us;
+// rank 2 with seven and eight 65 / 62 / 74, 63 / 59 / 69.
+template <int PASS, int RK>
+__global__ void __launch_bounds__(kRsThreads, RK == 2 ? 8 : RK == 4 ? 7 : 5) k_rs_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     __shared__ RwShared S;
     grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
-    if (L.rank == 4 && (L.msgp_off & 3) == 0)
-        rs_walk<PASS, 4>(V, L, blockIdx.x - pfx[li], S);
+    if (RK < CONEF_MAX_RANK && rs_exact(L, RK))
+        rs_walk<PASS, RK>(V, L, blockIdx.x - pfx[li], S);
     else
-        rs_walk<PASS, 8>(V, L, blockIdx.x - pfx[li], S);
+        rs_walk<PASS, CONEF_MAX_RANK>(V, L, blockIdx.x - pfx[li], S);
 }
 
 // P_i[a][c] = sum over the (column slab, warp) partials of pass 1, in slab-major order; four consecutive entries per thread
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(256) k_rs_p1_combine(const __grid_constant__ D
         return;
     const float *__restrict__ ppart = V.ppart + worker * V.ppart_stride + L.pp_off;
     float *__restrict__ out = V.msgp + worker * V.msgp_stride + L.msgp_off;
-    if (L.rank % 4 == 0 && ((L.pp_off | L.msgp_off) & 3) == 0) {
+    if (nr % 4 == 0 && ((L.pp_off | L.msgp_off) & 3) == 0) {
         float4 acc = *(const float4 *)(ppart + q);
 #pragma unroll 4
         for (int j = 1; j < L.f_j; ++j) {

@@ -136,3 +136,15 @@ def test_walk_over_buckets(q, div, scale):
         lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)
     else:
         run_single_phase(cfg, 3, exact_values=True)
+
+
+@pytest.mark.parametrize("rank", [1, 2, 4, 8])
+@pytest.mark.parametrize("div,scale", [(10, "fp16"), (60, "fp32")])
+def test_walk_with_the_rank_as_a_constant(rank, div, scale):
+    """Ranks 2 and 4 as constants, tensors thinner than them and behind those (factors off their vectors' boundaries), warps
+    without a column, fewer rows than a batch, more than the ring holds and than are staged at a time."""
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=[(900, 768, 1), (7, 1, 0), (1, 132, 1), (2700, 36, 1), (3, 520, 1), (64, 4, 1), (129, 1152, 1)], n_workers=2,
+               q=dict(kind="lowrank", rank=rank), grad="normal1e-3",
+               c=dict(kind="rowsketch", cs_rows=1, cs_col_div=div, seed=3, beta=0.9, scale_dtype=scale))
+    lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)

@@ -120,17 +120,17 @@ static __global__ void __launch_bounds__(kIlThreads) k_sketch_fold(const __grid_
     }
 }
 
-template <int QK, int W, int LP, int FORM>
+template <int QK, int W, int LP, int FORM, int WALK = 0>
 static void step(const DevView &V, const int32_t *pfx, int first, int tiles, int worker0, int groups, float *records, uint32_t stride,
-                 int64_t newoff, cudaStream_t s)
+                 int64_t newoff, cudaStream_t s, float *resid = nullptr)
 {
     const dim3 grid(tiles, groups);
     if (V.cs_rows == 5)
-        launch(k_sketch_il<QK, 5, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
+        launch(k_sketch_il<QK, 5, W, LP, FORM, WALK>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff, resid);
     else if (V.cs_rows == 3)
-        launch(k_sketch_il<QK, 3, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
+        launch(k_sketch_il<QK, 3, W, LP, FORM, WALK>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff, resid);
     else
-        launch(k_sketch_il<QK, 0, W, LP, FORM>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff);
+        launch(k_sketch_il<QK, 0, W, LP, FORM, WALK>, dim3(grid), kIlThreads, 0, s, V, pfx, first, worker0, records, stride, newoff, resid);
 }
 
 // a group of tensors
@@ -148,18 +148,24 @@ struct Group {
 
 // `batches` batches of W * LP workers from worker0 on
 template <int QK, int W, int LP>
-static int together(const Group &G, int worker0, int batches)
+static int together(const Group &G, int worker0, int batches, int64_t bytes)
 {
     constexpr int GW = W * LP;
     const int NW = GW * batches;
-    const bool near = G.n_records * 8 * NW > kIlTogether;
+    const bool two = il_two_walks(G.n_records, G.tiles, NW, bytes), near = !two && G.n_records * 8 * NW > kIlTogether;
     const uint32_t stride = (uint32_t)(near ? 2 * NW : NW);
     const int64_t newoff = near ? GW : G.n_records * NW;
     const dim3 egrid(G.etiles, batches);
     launch(k_sketch_swap<GW, true, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
-    step<QK, W, LP, IL_SCRATCH>(G.V, G.pfx, G.first, G.tiles, worker0, batches, G.records, stride, newoff, G.s);
+    if (two) {
+        float *const resid = G.records + G.n_records * 2 * NW;
+        step<QK, W, LP, IL_SCRATCH, 1>(G.V, G.pfx, G.first, G.tiles, worker0, batches, G.records, stride, newoff, G.s, resid);
+        step<QK, W, LP, IL_SCRATCH, 2>(G.V, G.pfx, G.first, G.tiles, worker0, batches, G.records, stride, newoff, G.s, resid);
+    } else {
+        step<QK, W, LP, IL_SCRATCH>(G.V, G.pfx, G.first, G.tiles, worker0, batches, G.records, stride, newoff, G.s);
+    }
     launch(k_sketch_swap<GW, false, false>, dim3(egrid), kIlThreads, 0, G.s, G.V, G.epfx, G.efirst, worker0, G.records, stride, newoff);
-    return 3;
+    return two ? 4 : 3;
 }
 template <int QK, int W, int LP>
 static int split(const Group &G, int worker0)
@@ -195,7 +201,7 @@ static int group(const Group &G, int64_t bytes)
     int launched = 0;
     for (int b = 0; at_once > 0 && b < all; b += at_once) {
         const int now = std::min(at_once, all - b);
-        launched += batch == 2 ? together<QK, 2, 1>(G, 0, now) : batch == 4 ? together<QK, 4, 1>(G, 0, now) : together<QK, 4, 2>(G, 8 * b, now);
+        launched += batch == 2 ? together<QK, 2, 1>(G, 0, now, bytes) : batch == 4 ? together<QK, 4, 1>(G, 0, now, bytes) : together<QK, 4, 2>(G, 8 * b, now, bytes);
     }
     for (int w = 0; at_once == 0 && w < n;) {
         const int left = n - w, now = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;

@@ -19,7 +19,7 @@
 // the price of one or two more passes over the sketch.
 //
 // Transformer-big list (210 M elements), 5 x d/10 buckets, eight workers: 90 ms per step one worker at a
-// time, 25.2 ms now, of which interleaving takes 3.2; the requests still bound it, ten per element.
+// time, 23.2 ms now, of which interleaving takes 3.1; the requests still bound it, ten per element.
 // Three CTAs per SM (80 registers); with four (spills) 24.8 ms instead of 23.0 for k_sketch_il.
 #pragma once
 #include <algorithm>
@@ -38,9 +38,20 @@ constexpr int64_t kIlGroupBytes = 40ll << 20;
 // A group whose records are larger than this (one tensor that does not fit L2) has the old and the new
 // values of an entry side by side, so that the addition finds in L2 what the read brought; in a group
 // that fits they are apart, since an addition next to a read of the same sector waits for it.  Eight
-// workers, Transformer-big: 25.0 ms with this line, 26.8 always side by side, 28.0 always apart; four
+// workers, Transformer-big, in one walk: 25.0 ms with this line, 26.8 always side by side, 28.0 always apart; four
 // workers, 16 M elements in L2: 476 us apart, 728 side by side.
 constexpr int64_t kIlTogether = 100ll << 20;
+// ... unless the old values alone, and then the new ones, mostly stay in L2, and the scratch has room for r: then the sketch is read in one
+// walk over the elements and added to in a second, for a write and a read of r and a second hash of the elements.  Steps of models
+// of five or six such tensors, 5 x d/10 buckets, one walk and two: eight workers, 4 M elements (64 MB of old values) 2728 and 2345 us,
+// 4.8 M (77 MB) 3702 and 3031, 5.9 M (94 MB) 5319 and 4533; four workers, 8 M (64 MB) 5307 and 3102, 12 M (96 MB) 9322 and 6211; two
+// workers, 16 M (64 MB) 8853 and 4358.  Above L2: eight workers, 6.9 M (110 MB) 5720 and 5155, 9 M (144 MB) 8505 and 8475; two workers,
+// 30 M (120 MB) 20.5 and 13.6 ms.  Transformer-big list, eight workers 24.6 and 23.2 ms.
+constexpr int64_t kIlOneSide = 150ll << 20;
+inline bool il_two_walks(int64_t n_records, int64_t tiles, int n, int64_t bytes)
+{
+    return n_records * 8 * n > kIlTogether && n_records * 4 * n <= kIlOneSide && (n_records * 8 + tiles * kIlTile * 4) * n <= bytes;
+}
 // Below this many elements over all workers the two kernels that interleave cost more than they save: 5 x d/10
 // buckets, steps on the states and on records, two, four and eight workers: 256 k elements 29.7, 27.7, 27.7 and
 // 32.8, 30.8, 36.5 us; 512 k 45.4, 42.0, 40.0 and 40.9, 32.8, 38.7; 1 M 66.0, 63.5, 60.6 and 53.4, 42.3, 41.0.
@@ -114,6 +125,32 @@ __device__ __forceinline__ IlVec<W> il_load(const float *p)
     }
     return r;
 }
+// r of an element, between the two walks
+template <int W>
+__device__ __forceinline__ IlVec<W> il_load_once(const float *p)
+{
+    IlVec<W> r;
+    if constexpr (W == 4) {
+        const float4 t = __ldcs((const float4 *)p);
+        r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
+    } else if constexpr (W == 2) {
+        const float2 t = __ldcs((const float2 *)p);
+        r.v[0] = t.x; r.v[1] = t.y;
+    } else {
+        r.v[0] = __ldcs(p);
+    }
+    return r;
+}
+template <int W>
+__device__ __forceinline__ void il_store_once(float *p, const IlVec<W> &a)
+{
+    if constexpr (W == 4)
+        __stcs((float4 *)p, make_float4(a.v[0], a.v[1], a.v[2], a.v[3]));
+    else if constexpr (W == 2)
+        __stcs((float2 *)p, make_float2(a.v[0], a.v[1]));
+    else
+        __stcs(p, a.v[0]);
+}
 template <int W>
 __device__ __forceinline__ void il_add(float *p, const IlVec<W> &a)
 {
@@ -131,10 +168,12 @@ __device__ __forceinline__ void il_add(float *p, const IlVec<W> &a)
 //
 // VR sketch rows (0: V.cs_rows, up to 7); W workers per lane, LP lanes per element, the first of them
 // worker0.  GW = 1 in SCRATCH form: no records, the states themselves.
-template <int QK, int VR, int W, int LP, int FORM>
+//
+// WALK 0: the whole step; 1: without the additions, r to `resid` (GW floats per element, elements by tile); 2: the additions.
+template <int QK, int VR, int W, int LP, int FORM, int WALK>
 __global__ void __launch_bounds__(kIlThreads, W == 4 ? 3 : 4)
 k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, int first, int worker0, float *records, uint32_t stride,
-            int64_t newoff)
+            int64_t newoff, float *resid)
 {
     constexpr int VM = VR ? VR : 7, GW = W * LP;
     const int v = VR ? VR : V.cs_rows;
@@ -175,6 +214,8 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
     const uint32_t kept = (uint32_t)L.k;
     const int64_t goff = L.g_off, moff = L.msgv_off;
     const float lr = V.lr, omb = V.omb, beta = V.beta;
+    if (WALK != 0)
+        resid += ((uint64_t)blockIdx.y * gridDim.x + blockIdx.x) * (kIlTile * GW) + sub * W;
     for (uint32_t q = threadIdx.x / LP; q < left; q += kIlThreads / LP) {
         const uint32_t j = j0 + q;
         uint32_t bk[VM];    // bucket
@@ -188,45 +229,55 @@ k_sketch_il(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx, 
                 bk[i] = (uint32_t)(((u >> 32) * (uint64_t)w) >> 32);
                 sign |= (uint32_t)(u & 1) << i;
                 const uint32_t e = (uint32_t)i * w + bk[i];
+                if (WALK == 2)
+                    continue;
                 if (FORM == IL_FOLD)
                     rec[i] = il_load<W>(e < half ? So + (uint64_t)e * (2 * GW) : Sn + slices.at(e - half, 2 * GW));
                 else
                     rec[i] = il_load<W>(So + ((uint64_t)i * w + bk[i]) * stride);
             }
         }
-        float gv[W];
-#pragma unroll
-        for (int x = 0; x < W; ++x)
-            gv[x] = w0 + x < V.n_workers ? __ldcs(V.grads[w0 + x] + goff + j) : 0.f;
-        bool sel = QK == CONEF_Q_IDENTITY;
-        uint32_t slot = j;
-        if (QK == CONEF_Q_RANDK) {
-            const uint32_t word = bits[j >> 5];
-            sel = (word >> (j & 31u)) & 1u;
-            if (sel)
-                slot = draw_slot(L, V.wordoff, V.tileoff, word, j);
-        } else if (QK == CONEF_Q_RANDBLOCK) {
-            slot = j - blk_start;   // wraps to a large value below the block
-            sel = slot < kept;
-        }
         IlVec<W> val;
+        if (WALK == 2) {
+            val = il_load_once<W>(resid + q * GW);
+        } else {
+            float gv[W];
 #pragma unroll
-        for (int x = 0; x < W; ++x) {
-            float est[VM];
+            for (int x = 0; x < W; ++x)
+                gv[x] = w0 + x < V.n_workers ? __ldcs(V.grads[w0 + x] + goff + j) : 0.f;
+            bool sel = QK == CONEF_Q_IDENTITY;
+            uint32_t slot = j;
+            if (QK == CONEF_Q_RANDK) {
+                const uint32_t word = bits[j >> 5];
+                sel = (word >> (j & 31u)) & 1u;
+                if (sel)
+                    slot = draw_slot(L, V.wordoff, V.tileoff, word, j);
+            } else if (QK == CONEF_Q_RANDBLOCK) {
+                slot = j - blk_start;   // wraps to a large value below the block
+                sel = slot < kept;
+            }
 #pragma unroll
-            for (int i = 0; i < VM; ++i)
-                est[i] = (VR || i < v) ? __uint_as_float(__float_as_uint(rec[i].v[x]) ^ (((sign >> i) & 1u) << 31)) : 0.f;
-            const float e = median_small(est, v);
-            const float p = __fmaf_rn(lr, gv[x], __fmul_rn(omb, e));   // Alg. 2 line 5 (Alg. 4 line 5 with beta)
-            if (sel && w0 + x < V.n_workers)
-                V.msgv[(w0 + x) * V.msgv_stride + moff + slot] = p;
-            // r = p - Delta (zero on a transmitted coordinate); Alg. 4 line 9 keeps beta e as well
-            val.v[x] = sel ? 0.f : p;
-            if (beta != 0.f)
-                val.v[x] = __fmaf_rn(beta, e, val.v[x]);
+            for (int x = 0; x < W; ++x) {
+                float est[VM];
+#pragma unroll
+                for (int i = 0; i < VM; ++i)
+                    est[i] = (VR || i < v) ? __uint_as_float(__float_as_uint(rec[i].v[x]) ^ (((sign >> i) & 1u) << 31)) : 0.f;
+                const float e = median_small(est, v);
+                const float p = __fmaf_rn(lr, gv[x], __fmul_rn(omb, e));   // Alg. 2 line 5 (Alg. 4 line 5 with beta)
+                if (sel && w0 + x < V.n_workers)
+                    V.msgv[(w0 + x) * V.msgv_stride + moff + slot] = p;
+                // r = p - Delta (zero on a transmitted coordinate); Alg. 4 line 9 keeps beta e as well
+                val.v[x] = sel ? 0.f : p;
+                if (beta != 0.f)
+                    val.v[x] = __fmaf_rn(beta, e, val.v[x]);
+            }
+            if (QK != CONEF_Q_IDENTITY && sel && w0 == 0)
+                V.idx[L.idx_off + slot] = j;
+            if (WALK == 1) {
+                il_store_once<W>(resid + q * GW, val);
+                continue;
+            }
         }
-        if (QK != CONEF_Q_IDENTITY && sel && w0 == 0)
-            V.idx[L.idx_off + slot] = j;
         bool any = false;
 #pragma unroll
         for (int x = 0; x < W; ++x)

@@ -59,6 +59,18 @@ def test_a_tensor_beyond_the_l2_that_is_the_model(workers):
         assert float(((a - b).double().abs() / torch.maximum(b.double().abs(), rms)).max()) < 1e-5
 
 
+@pytest.mark.parametrize("qkind", ["randk", "randblock", "identity"])
+@pytest.mark.parametrize("workers,rows", [(8, 701), (7, 1021), (3, 1401), (2, 2801)])
+def test_reading_and_adding_in_two_walks(qkind, workers, rows):
+    """Tensors whose old values fit L2 and whose old and new ones do not, in a model with room for r between the walks."""
+    cfg = wl.config("tiny")
+    cfg.update(tensors=[(rows, 1001, 1), (7, 1, 0), (rows, 999, 1), (rows + 3, 1000, 1), (rows, 1003, 1)], n_workers=workers,
+               q=dict(kind=qkind, k_num=1, k_den=20, seed=5), c=dict(kind="countsketch", cs_rows=5, cs_col_div=2, seed=9, beta=0.5))
+    for a, b in zip(_run(cfg, True, 2), _run(cfg, False, 2)):
+        rms = b.double().square().mean().sqrt().clamp_min(1e-30)
+        assert float(((a - b).double().abs() / torch.maximum(b.double().abs(), rms)).max()) < 1e-5
+
+
 # three tensors of a similar size, which fit the scratch with their new records, and one that does not
 @pytest.mark.parametrize("tensors", [[(600, 1000, 1), (300, 1, 0), (601, 1000, 1), (599, 1001, 1)], [(37, 53, 1), (1100, 1001, 1), (64, 1, 0)]])
 @pytest.mark.parametrize("qkind,workers,rows", [("randk", 2, 5), ("randblock", 3, 3), ("randk", 8, 5), ("identity", 9, 7)])

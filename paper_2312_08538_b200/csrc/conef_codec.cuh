@@ -146,6 +146,16 @@ __device__ __forceinline__ void pack_fields8(const uint32_t (&t)[8], uint32_t &w
     }
 }
 
+// max(a, |x|), or NaN where either is one (fmaxf gives the other).  A block's maximum by this is NaN where a residual is, so that
+// the test for the clamp of quant_pack8 catches both; the maximum that makes the scale, without NaNs, is then formed again.
+// (Unclamped, a NaN's bits would be added to the neighbouring fields.)
+__device__ __forceinline__ float absmax_nan(float a, float x)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(fabsf(x)));
+    return r;
+}
+
 template <bool HALF>
 __device__ __forceinline__ float load_scale_g(const uint8_t *scales, uint32_t blk)
 {

@@ -794,16 +794,25 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
         float amax = 0.f;
 #pragma unroll
         for (int x = 0; x < E; ++x)
-            amax = fmaxf(amax, fabsf(res[x >> 3][x & 7]));   // (a NaN counts as nothing)
+            amax = absmax_nan(amax, res[x >> 3][x & 7]);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1)
             if (lpb > o)
-                amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+                amax = absmax_nan(amax, __shfl_xor_sync(0xffffffffu, amax, o));
         float s, inv;
         unsigned short hb = 0;
         block_scale<CK, HALF>(amax, s, inv, hb);
         uint32_t t[E / 4], o[NW];   // (int4: every other word)
         if (__any_sync(0xffffffffu, !(__fmul_rn(amax, inv) < (INT4 ? 7.f : 127.f) + 0.49f))) {   // (see quant_pack8)
+            amax = 0.f;
+#pragma unroll
+            for (int x = 0; x < E; ++x)
+                amax = fmaxf(amax, fabsf(res[x >> 3][x & 7]));   // (a NaN counts as nothing)
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1)
+                if (lpb > o)
+                    amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+            block_scale<CK, HALF>(amax, s, inv, hb);
 #pragma unroll
             for (int x = 0; x < E / 8; ++x)
                 quant_pack8<CK, true>(res[x], inv, t[2 * x], t[2 * x + 1]);

@@ -1,0 +1,54 @@
+"""A residual that is not a number leaves the other codes of its quantisation block, and the block's scale, as they are
+without it.  The kernels for every codec are the reference."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2312_08538_b200 import workloads as wl
+from tests import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+ODD = [(70, 33, 1), (3, 1, 0), (9, 31, 1), (130, 257, 1), (1, 700, 1), (300, 5, 1), (17, 2049, 1)]
+
+
+def _lowrank(tensors, rank, c):
+    """Steps whose Q_i has a NaN in two of its columns' rows: both columns of the residual are NaN throughout."""
+    from paper_2312_08538_b200 import binding as b
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=tensors, n_workers=2, q=dict(kind="lowrank", rank=rank), c=c, grad="normal1e-3")
+    q0 = wl.q_init(cfg, "cuda")
+    eng, ref = (pu.make_gpu(cfg, q_init=q0, fast=f) for f in (True, False))
+    layers = [l for l, t in enumerate(tensors) if t[2]]
+    gd, _ = pu.grads_both(cfg, 0)
+    for e in (eng, ref):
+        e.step(0, gd, 0)
+        e.reduce_messages(b.MSG_P)
+    for l in layers:
+        eng.factors(l, 0)["p_hat"].copy_(ref.factors(l, 0)["p_hat"])
+    for e in (eng, ref):
+        e.step(0, gd, 2)
+    bad = {l: [0, 2 * tensors[l][1] // 3] for l in layers}
+    for l in layers:
+        for i in range(2):
+            q = ref.factors(l, i)["q_i"]
+            q[bad[l]] = float("nan")
+            eng.factors(l, i)["q_i"].copy_(q)
+    for e in (eng, ref):
+        e.step(0, gd, 3)
+    o = pu.make_oracle(cfg, q_init=q0.cpu().numpy())
+    for l in layers:
+        keep = np.ones((tensors[l][0], tensors[l][1]), bool)
+        keep[:, bad[l]] = False
+        for i in range(2):
+            (ca, sa), (cb, sb) = (pu.gpu_state_arrays(e, o, i, l) for e in (eng, ref))
+            assert np.isfinite(sa).all() and np.array_equal(sa, sb), (l, i)
+            assert np.array_equal(ca[keep.ravel()], cb[keep.ravel()]), (l, i)
+
+
+@pytest.mark.parametrize("rank,c", [(2, dict(kind="int4", block=64, scale_dtype="fp16")), (3, dict(kind="int8", block=32)),
+                                    (4, dict(kind="int4", block=256)), (8, dict(kind="int8", block=128, scale_dtype="fp16", beta=0.5))])
+@pytest.mark.parametrize("more", [[], [(2000, 1001, 1)]])   # (eight and sixteen elements per lane)
+def test_lowrank_passes_for_any_shape(rank, c, more):
+    _lowrank(ODD + more, rank, c)
+

@@ -582,7 +582,7 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
                             acc = valid[u] ? acc : 0.f;   // lanes past the end of the tensor add nothing to the block's absmax
                         p[u][q] = acc;
                     }
-                    amax[u] = fmaxf(amax[u], fabsf(acc));
+                    amax[u] = absmax_nan(amax[u], acc);
                 }
             }
             // absmax over the block/8 lanes of the quantisation block
@@ -591,7 +591,7 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
                 if (o <= 2 || lpb > o)
 #pragma unroll
                     for (int u = 0; u < NI; ++u)
-                        amax[u] = fmaxf(amax[u], __shfl_xor_sync(0xffffffffu, amax[u], o));
+                        amax[u] = absmax_nan(amax[u], __shfl_xor_sync(0xffffffffu, amax[u], o));
             float s[NI], inv[NI];
             unsigned short hb[NI];
             bool clamp = false;
@@ -607,8 +607,18 @@ __device__ __forceinline__ void fast_tile(const DevView &V, const LayerDesc *Lp,
             uint32_t c0[NI], c1[NI];
             if (__any_sync(0xffffffffu, clamp)) {
 #pragma unroll
-                for (int u = 0; u < NI; ++u)
+                for (int u = 0; u < NI; ++u) {
+                    amax[u] = 0.f;   // (a NaN counts as nothing)
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        amax[u] = fmaxf(amax[u], fabsf(p[u][q]));
+#pragma unroll
+                    for (int o = 16; o >= 1; o >>= 1)
+                        if (o <= 2 || lpb > o)
+                            amax[u] = fmaxf(amax[u], __shfl_xor_sync(0xffffffffu, amax[u], o));
+                    block_scale<CK, HALF>(amax[u], s[u], inv[u], hb[u]);
                     quant_pack8<CK, true>(p[u], inv[u], c0[u], c1[u]);
+                }
             } else if constexpr (PAIR) {
 #pragma unroll
                 for (int u = 0; u < NI; ++u) {

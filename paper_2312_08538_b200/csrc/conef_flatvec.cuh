@@ -216,21 +216,31 @@ __global__ void __launch_bounds__(kFvThreads, 3) k_flat_vec2(const __grid_consta
         float amax = 0.f;
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-            amax = fmaxf(amax, fabsf(r[q]));
+            amax = absmax_nan(amax, r[q]);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1)
             if (o <= 2 || lpb > o)
-                amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+                amax = absmax_nan(amax, __shfl_xor_sync(0xffffffffu, amax, o));
         float s, inv;
         unsigned short hb = 0;
         uint32_t c0 = 0, c1 = 0;
         {
             block_scale<CK, HALF>(amax, s, inv, hb);
             constexpr float qlim = (CK == CONEF_C_INT8 ? 127.f : 7.f) + 0.49f;
-            if (__any_sync(0xffffffffu, !(__fmul_rn(amax, inv) < qlim)))
+            if (__any_sync(0xffffffffu, !(__fmul_rn(amax, inv) < qlim))) {
+                amax = 0.f;   // (a NaN counts as nothing)
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    amax = fmaxf(amax, fabsf(r[q]));
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1)
+                    if (o <= 2 || lpb > o)
+                        amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+                block_scale<CK, HALF>(amax, s, inv, hb);
                 quant_pack8<CK, true>(r, inv, c0, c1);
-            else
+            } else {
                 quant_pack8<CK, false>(r, inv, c0, c1);
+            }
         }
         if (valid) {
             if ((lane & (lpb - 1)) == 0) {

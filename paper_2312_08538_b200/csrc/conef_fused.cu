@@ -597,32 +597,43 @@ __global__ void __launch_bounds__(kFuThreads, MINB) k_fused23(const __grid_const
                         if (TAIL)
                             acc = ok[x] ? acc : 0.f;
                         p[4 * x + q] = acc;
-                        am[x] = fmaxf(am[x], fabsf(acc));
+                        am[x] = absmax_nan(am[x], acc);
                     }
                 }
-                // block maxima: bit patterns of non-negative floats order like integers
-                float bm[2];
-                if (NBLK == 2) {
-                    bm[0] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am[0])));
-                    bm[1] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am[1])));
-                } else {
-                    bm[0] = bm[1] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(am[0], am[1]))));
-                }
-                float s[2], inv[2];
+                // block maxima: bit patterns of non-negative floats order like integers, a NaN's above them
+                float bm[2], s[2], inv[2];
                 unsigned short hb[2];
+                auto scales_of = [&](const float (&am)[2]) {
+                    if (NBLK == 2) {
+                        bm[0] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am[0])));
+                        bm[1] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am[1])));
+                    } else {
+                        bm[0] = bm[1] = __uint_as_float(__reduce_max_sync(0xffffffffu, max(__float_as_uint(am[0]), __float_as_uint(am[1]))));
+                    }
+#pragma unroll
+                    for (int x = 0; x < NBLK; ++x)
+                        block_scale<CK, HALF>(bm[x], s[x], inv[x], hb[x]);
+                    if (NBLK == 1) {
+                        s[1] = s[0];
+                        inv[1] = inv[0];
+                        hb[1] = hb[0];
+                    }
+                };
+                scales_of(am);
                 bool clamp = false;
 #pragma unroll
-                for (int x = 0; x < NBLK; ++x) {
-                    block_scale<CK, HALF>(bm[x], s[x], inv[x], hb[x]);
+                for (int x = 0; x < NBLK; ++x)
                     clamp = clamp || !(__fmul_rn(bm[x], inv[x]) < qlim);
-                }
-                if (NBLK == 1) {
-                    s[1] = s[0];
-                    inv[1] = inv[0];
-                    hb[1] = hb[0];
-                }
                 uint32_t cw[2];
                 if (clamp) {   // (the same for every lane: the maxima are the warp's)
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        am[x] = 0.f;   // (a NaN counts as nothing)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            am[x] = fmaxf(am[x], fabsf(p[4 * x + q]));
+                    }
+                    scales_of(am);
                     cw[0] = quant_pack4<CK, true>(&p[0], inv[0]);
                     cw[1] = quant_pack4<CK, true>(&p[4], inv[1]);
                 } else {

@@ -39,7 +39,7 @@ enum { T_FLAT = 0, T_PASS, T_P1, T_P2, T_Q2, T_HIST, T_GS, T_SLOW_FLAT, T_SLOW_P
        T_GS_ONE, T_GS_CLUSTER, T_GS_CLUSTER16, T_GS_REST,   // Gram-Schmidt: one CTA / clusters of 8, 16 / generic
        T_RS,                                                // row sketch: (sketch row, bucket group, column slab)
        T_APPLY,                                             // model update
-       T_RS_P12, T_RS_P1C,                                  // low-rank passes 1, 2 on a row-sketch state; pass-1 combine
+       T_RS_P12, T_RS_P1C,                                  // low-rank passes on a row-sketch state; pass-1 combine
        T_FV, T_NOFV,                                        // tuned fused step (identity / random-k Q, int8 / int4 C) and the rest
        T_CSK,                                               // count sketch applied run by run: one tile per run
        T_RP1, T_RP1_R8,                                     // low-rank pass 1 with a matrix row per lane (rank 4, rank 8)
@@ -408,7 +408,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                         P.fast_subs[cls] = std::max(P.fast_subs[cls], (int)L.f_subs);
                 }
                 if (c->kind == CONEF_C_ROWSKETCH && c->cs_rows == 1 && L.rs_vec == 4 && c->beta >= 0.f) {
-                    // bucket-major passes 1 and 2 (conef_rowsketch.cuh)
+                    // bucket-major passes (conef_rowsketch.cuh)
                     L.fast = 2;
                     P.any_rs12 = true;
                     const int64_t groups = ceil_div(L.w, kRsBuckets), slabs = ceil_div(L.cols, kRsThreads * 4);
@@ -1426,7 +1426,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };
-        auto launch_rs12 = [&](int pass) -> int {   // (pass 3: of a model whose tensors all take it)
+        auto launch_rs12 = [&](int pass) -> int {   // (pass 3: all tensors)
             const int table = pass == 3 ? T_RS : T_RS_P12, n = tiles_of(ctx, table);
             if (n == 0)
                 return CONEF_OK;
@@ -1480,7 +1480,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
         if (rc == CONEF_OK && (phase == 1 || phase == 3 || phase == 4)) {
             rc = with_new_sketch(ctx, V, s, [&] {
                 if (ctx->c.kind == CONEF_C_ROWSKETCH)
-                    return rs12 && !ctx->plan.any_slow ? launch_rs12(3) : launch_rowsketch<CONEF_Q_LOWRANK>(ctx, V, s);
+                    return V.rs_vec_ok && ctx->plan.any_rs12 ? launch_rs12(3) : launch_rowsketch<CONEF_Q_LOWRANK>(ctx, V, s);
                 int r2 = fast ? launch_fast(ctx, 3, V, s, fused) : CONEF_OK;
                 if (r2 == CONEF_OK && fast)
                     r2 = launch_gen(3);

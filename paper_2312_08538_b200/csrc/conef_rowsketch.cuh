@@ -231,7 +231,8 @@ __device__ __forceinline__ void rs_body(const DevView &V, const LayerDesc &L, co
     }
 }
 
-// rs_vec of a tensor chooses the body; both live in one kernel so that one launch covers the model
+// rs_vec of a tensor chooses the body; both live in one kernel so that one launch covers the model.  (A low-rank Q on one sketch row
+// comes here where no tensor takes the walk: 16-byte loads are not possible.)
 template <int QK, bool V1>   // V1: one sketch row (the usual setting), no median
 __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 0) k_rowsketch(const __grid_constant__ DevView V)
 {
@@ -240,13 +241,6 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
     const LayerDesc &L = V.layers[li];
     const uint32_t local = blockIdx.x - V.pfx_rs[li];
     const bool vec = L.rs_vec == 4 && V.rs_vec_ok;
-    if constexpr (V1 && QK == CONEF_Q_LOWRANK) {
-        __shared__ RwShared S;
-        if (vec) {
-            rs_walk<3, 8>(V, L, local, S);
-            return;
-        }
-    }
     grid_wait();
     if (!(V1 && QK == CONEF_Q_LOWRANK) && vec)
         rs_body<QK, 4, V1>(V, L, li, local);
@@ -273,9 +267,14 @@ __global__ void __launch_bounds__(kRsThreads, V1 && QK == CONEF_Q_LOWRANK ? 5 : 
 //           order by k_lr_pass2_reduce.
 // Sums over rows and columns run in bucket order, not index order: like the other factor kernels
 // they match the oracle to rounding (fp32, fixed order), not bit for bit.
-// RK: the configured rank (2, 4; 8: another one); tensors that rs_exact does not accept take the walk for any rank.
-// PASS 3 is the step's last, of models whose tensors all take the walk (else: k_rowsketch).
-// CTAs per SM: rank 4 with six, seven and eight (64 registers) on the GPT-2-small list 136 / 115 / 135, 134 / 117 / 127, 142 / 117 / 129 us;
+// RK: the configured rank (2, 4; 8: another one); tensors that rs_exact does not accept take the walk for any rank up to it (with
+// room for eight it spilled under these registers: behind a matrix of one row the GPT-2-small list, rank 4, takes 722 us per step instead of 920,
+// two of 4096 x 4096, rank 2, two workers 282 instead of 522).
+// PASS 3, the step's last, takes the tensors that do not walk along: in a launch of their own behind it they make the step longer (512 x 768,
+// 300 x 333 and 768 x 512, rank 4, two workers 244 -> 262 us).  With the walk for any rank up to 8 beside rs_body in k_rowsketch it was 266, the
+// GPT-2-small list with 300 x 333 behind it 878 instead of 810, two of 4096 x 4096 around 333 x 4097, rank 2, 1107 instead of 1001.
+// CTAs per SM: rank 4 with six, seven and eight (64 registers) on the GPT-2-small list 136 / 115 / 135, 134 / 117 / 127, 142 / 117 / 129 us (with
+// the spilling body beside it; 131 / 114 / 125 now);
 // rank 2 with seven and eight 65 / 62 / 74, 63 / 59 / 69.
 template <int PASS, int RK>
 __global__ void __launch_bounds__(kRsThreads, RK == 2 ? 8 : RK == 4 ? 7 : 5) k_rs_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
@@ -284,10 +283,19 @@ __global__ void __launch_bounds__(kRsThreads, RK == 2 ? 8 : RK == 4 ? 7 : 5) k_r
     grid_release();
     const int li = find_layer(pfx, V.n_layers, blockIdx.x);
     const LayerDesc &L = V.layers[li];
-    if (RK < CONEF_MAX_RANK && rs_exact(L, RK))
-        rs_walk<PASS, RK>(V, L, blockIdx.x - pfx[li], S);
-    else
-        rs_walk<PASS, CONEF_MAX_RANK>(V, L, blockIdx.x - pfx[li], S);
+    const uint32_t local = blockIdx.x - pfx[li];
+    if constexpr (PASS == 3)
+        if (L.rs_vec != 4) {
+            grid_wait();
+            rs_body<CONEF_Q_LOWRANK, 1, true>(V, L, li, local);
+            return;
+        }
+    if constexpr (RK < CONEF_MAX_RANK)
+        if (rs_exact(L, RK)) {
+            rs_walk<PASS, RK, true>(V, L, local, S);
+            return;
+        }
+    rs_walk<PASS, RK, false>(V, L, local, S);
 }
 
 // P_i[a][c] = sum over the (column slab, warp) partials of pass 1, in slab-major order; four consecutive entries per thread

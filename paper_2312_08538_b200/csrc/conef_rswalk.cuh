@@ -4,11 +4,11 @@
 // the bucket lists, as one sequence.  The entries (row, sign) of all its buckets, which are contiguous in the tables, and their
 // rows of P_hat are in shared memory before the walk starts.  The gradient comes by asynchronous copies, a batch of rows ahead, each
 // thread's own, so that it takes no registers and no barrier; the old sketch entry of the next bucket is loaded at the start of the one before.
-// The rank is a constant (2, 4) where it is the configured one.
+// The rank is a constant (2, 4) where it is the configured one; arrays have room for the configured one elsewhere.
 //
 // GPT-2-small list, rank 4, binary16 sketch, one worker: with the gradient in registers, the old entries in shared memory and
 // the body for any rank beside it (94 registers, five CTAs per SM) the passes took 169 / 148 / 177 us, issue slots 40 to 50 % busy;
-// now 131 / 117 / 127 us (72 registers, seven CTAs; step and update 698 -> 587 us), 60 to 72 % busy.  Rank 2, 33 M elements of two
+// now 131 / 114 / 125 us (72 registers, seven CTAs; step and update 698 -> 579 us), 60 to 72 % busy.  Rank 2, 33 M elements of two
 // workers, fp32 sketch: 120 / 98 / 130 -> 64 / 59 / 69 us (eight CTAs).  The single-phase compressors stay with rs_body (3 % slower here).
 #pragma once
 #include "conef_fast.cuh"
@@ -18,7 +18,7 @@ namespace conef {
 
 constexpr int kRwBatch = 4;      // rows of a batch
 // Rows of the gradient under way per thread, in shared memory.  Sixteen leave room for six CTAs per SM: passes 147 / 134 / 145 us instead
-// of 131 / 117 / 127 on the list below.
+// of 131 / 117 / 127 on the list above.
 constexpr int kRwRing = 8;
 constexpr int kRwEntries = 128;  // entries staged at a time (eight buckets of ten rows expect 80)
 constexpr int kRwCols = kRsThreads * 4;
@@ -30,12 +30,13 @@ struct alignas(16) RwShared {
     uint32_t start[kRsBuckets + 1];
 };
 
-// PASS 1, 2, 3: the low-rank passes; 3 writes the new sketch.  RK: 2 or 4 for that rank and rows of the factors on their vector's
-// boundaries, else 8 (any rank).
-template <int PASS, int RK>
+// PASS 1, 2, 3: the low-rank passes; 3 writes the new sketch.  EXACT: rank RK (2, 4) and rows of the factors on their vector's
+// boundaries; else any rank up to RK.
+template <int PASS, int RK, bool EXACT>
 __device__ __forceinline__ void rs_walk(const DevView &V, const LayerDesc &L, const uint32_t local, RwShared &S)
 {
-    constexpr bool NEED_PH = PASS != 1, EXACT = RK < CONEF_MAX_RANK;
+    constexpr bool NEED_PH = PASS != 1;
+    static_assert(!EXACT || RK == 2 || RK == 4, "vectors of a row");
     const int worker = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t m = (uint32_t)L.cols, w = (uint32_t)L.w, slabs = (m + kRwCols - 1) / kRwCols;
     const uint32_t grp = local / slabs, slab = local - grp * slabs, h0 = grp * kRsBuckets, nb = min((uint32_t)kRsBuckets, w - h0);
@@ -83,10 +84,10 @@ __device__ __forceinline__ void rs_walk(const DevView &V, const LayerDesc &L, co
 #pragma unroll
                 for (int c = 0; c < RK; ++c)
                     q[x][c] = 0.f;
-            } else if (RK == 4) {
+            } else if (EXACT && RK == 4) {
                 const float4 t = load_global((const float4 *)qp + x);
                 q[x][0] = t.x; q[x][1] = t.y; q[x][2 % RK] = t.z; q[x][3 % RK] = t.w;
-            } else if (RK == 2) {
+            } else if (EXACT && RK == 2) {
                 const float2 t = load_global((const float2 *)qp + x);
                 q[x][0] = t.x; q[x][1] = t.y;
             } else {
@@ -158,9 +159,9 @@ __device__ __forceinline__ void rs_walk(const DevView &V, const LayerDesc &L, co
             for (uint32_t x = tid; x < n; x += kRsThreads) {
                 const float *src = phat + (size_t)(S.ent[x] & 0x7FFFFFFFu) * r;
                 float *const dst = EXACT ? &S.ph[0][0] + x * RK : S.ph[x];
-                if (RK == 4) {
+                if (EXACT && RK == 4) {
                     cp_async16(dst, src);
-                } else if (RK == 2) {
+                } else if (EXACT && RK == 2) {
                     cp_async_small<8>(dst, src);
                 } else {
                     for (int c = 0; c < r; ++c)
@@ -221,10 +222,10 @@ __device__ __forceinline__ void rs_walk(const DevView &V, const LayerDesc &L, co
                             pr[u][c] = __fmaf_rn(p[y], q[y][c], pr[u][c]);
                 } else {
                     float ph[RK];
-                    if constexpr (RK == 4) {
+                    if constexpr (EXACT && RK == 4) {
                         const float4 t = ((const float4 *)S.ph)[x];
                         ph[0] = t.x; ph[1] = t.y; ph[2] = t.z; ph[3] = t.w;
-                    } else if constexpr (RK == 2) {
+                    } else if constexpr (EXACT && RK == 2) {
                         const float2 t = ((const float2 *)S.ph)[x];
                         ph[0] = t.x; ph[1] = t.y;
                     } else {

@@ -148,3 +148,40 @@ def test_walk_with_the_rank_as_a_constant(rank, div, scale):
                q=dict(kind="lowrank", rank=rank), grad="normal1e-3",
                c=dict(kind="rowsketch", cs_rows=1, cs_col_div=div, seed=3, beta=0.9, scale_dtype=scale))
     lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)
+
+
+def _walks(tensors):
+    """Which compressed tensors have 16-byte loads: their width and their place among the gradients are multiples of four."""
+    off, out = 0, []
+    for r, c, k in tensors:
+        if k:
+            out.append(c % 4 == 0 and off % 4 == 0)
+        off += r * c
+    return out
+
+
+@pytest.mark.parametrize("rank", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("div,scale", [(10, "fp16"), (60, "fp32"), (1, "fp32")])
+def test_all_tensors_walk(rank, div, scale):
+    """One tensor of each sort that the constant ranks take (wide, narrow, of several column slabs, one bucket), then one thinner than rank 4
+    and one of a single row, behind which factors are off their vectors' boundaries; 1-D tensors of lengths that four divides."""
+    tensors = [(900, 768, 1), (8, 1, 0), (2700, 36, 1), (64, 4, 1), (129, 1152, 1), (4, 520, 1), (9, 128, 1), (4, 1, 0), (3, 520, 1), (1, 132, 1),
+               (40, 96, 1), (900, 516, 1)]
+    assert all(_walks(tensors))
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=tensors, n_workers=2, q=dict(kind="lowrank", rank=rank), grad="normal1e-3",
+               c=dict(kind="rowsketch", cs_rows=1, cs_col_div=div, seed=3, beta=0.9, scale_dtype=scale))
+    lowrank_teacher_forced(cfg, 2, fast=True, scale_with_cond=True)
+
+
+@pytest.mark.parametrize("rank", [2, 3, 4, 8])
+@pytest.mark.parametrize("scale", ["fp16", "fp32"])
+@pytest.mark.parametrize("fast", [True, False])
+def test_tensors_that_walk_and_others(rank, scale, fast):
+    """Odd widths and a tensor behind an odd length among those that walk."""
+    tensors = [(900, 768, 1), (2700, 35, 1), (129, 1152, 1), (7, 1, 0), (33, 64, 1), (64, 257, 1), (1, 1, 0), (40, 96, 1), (3, 520, 1), (300, 260, 1)]
+    assert _walks(tensors) == [True, False, True, False, False, True, True, True]
+    cfg = wl.config("resnet50-mini")
+    cfg.update(tensors=tensors, n_workers=2, q=dict(kind="lowrank", rank=rank), grad="normal1e-3",
+               c=dict(kind="rowsketch", cs_rows=1, cs_col_div=10, seed=3, beta=0.9, scale_dtype=scale))
+    lowrank_teacher_forced(cfg, 2, fast=fast, scale_with_cond=True)

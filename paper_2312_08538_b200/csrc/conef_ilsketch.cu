@@ -152,7 +152,7 @@ static int together(const Group &G, int worker0, int batches, int64_t bytes)
 {
     constexpr int GW = W * LP;
     const int NW = GW * batches;
-    const bool two = il_two_walks(G.n_records, G.tiles, NW, bytes), near = !two && G.n_records * 8 * NW > kIlTogether;
+    const bool two = il_two_walks(G.n_records, G.tiles, NW, GW, G.V.cs_rows, bytes), near = !two && G.n_records * 8 * NW > kIlTogether;
     const uint32_t stride = (uint32_t)(near ? 2 * NW : NW);
     const int64_t newoff = near ? GW : G.n_records * NW;
     const dim3 egrid(G.etiles, batches);

@@ -48,9 +48,19 @@ constexpr int64_t kIlTogether = 100ll << 20;
 // workers, 16 M (64 MB) 8853 and 4358.  Above L2: eight workers, 6.9 M (110 MB) 5720 and 5155, 9 M (144 MB) 8505 and 8475; two workers,
 // 30 M (120 MB) 20.5 and 13.6 ms.  Transformer-big list, eight workers 24.6 and 23.2 ms.
 constexpr int64_t kIlOneSide = 150ll << 20;
-inline bool il_two_walks(int64_t n_records, int64_t tiles, int n, int64_t bytes)
+// What is saved are requests (two per sketch row), what it costs are 8 bytes of r per element and worker: with batches of eight workers, whose
+// requests are a sector each, it does not pay beyond half of L2 but at five rows, nor for the general number of rows.  Eight workers, one walk and
+// two, old values in MB: three rows 1.8 M elements, d/5 (58) 986 and 908 us, 6 M, d/10 (58) 2558 and 2240, 2 M, d/2 (96) 1065 and 1088, 6 M, d/5 (115)
+// 2650 and 2709, 13 M, d/10 (125) 8068 and 8395; seven rows 5 M, d/20 (56) 9292 and 9077, 2 M, d/5 (90) 2919 and 3112, 5 M, d/10 (112) 9835 and
+// 11325; one row 7 M, d/2 (112) 1981 and 2357; five rows 3 M, d/5 (96) 1963 and 1756, 7 M, d/10 (112) 6713 and 6128, 7 M, d/20 (56) 4380 and
+// 3382.  Sixteen: three rows 3 M, d/5 (115) 2804 and 2722, 6 M, d/10 (115) 7342 and 7203, seven rows 2 M, d/10 (90) 8073 and 8260.  Two and
+// four workers at one, three, five and seven rows, d/2 to d/20, 60 to 130 MB: 0 to 48 % less time.
+constexpr int64_t kIlOneSide8 = 70ll << 20;
+// n_records of n workers, in batches of gw
+inline bool il_two_walks(int64_t n_records, int64_t tiles, int n, int gw, int cs_rows, int64_t bytes)
 {
-    return n_records * 8 * n > kIlTogether && n_records * 4 * n <= kIlOneSide && (n_records * 8 + tiles * kIlTile * 4) * n <= bytes;
+    const int64_t most = gw < 8 || cs_rows == 5 || (cs_rows == 3 && n > 8) ? kIlOneSide : kIlOneSide8;
+    return n_records * 8 * n > kIlTogether && n_records * 4 * n <= most && (n_records * 8 + tiles * kIlTile * 4) * n <= bytes;
 }
 // Below this many elements over all workers the two kernels that interleave cost more than they save: 5 x d/10
 // buckets, steps on the states and on records, two, four and eight workers: 256 k elements 29.7, 27.7, 27.7 and

@@ -71,6 +71,24 @@ def test_reading_and_adding_in_two_walks(qkind, workers, rows):
         assert float(((a - b).double().abs() / torch.maximum(b.double().abs(), rms)).max()) < 1e-5
 
 
+@pytest.mark.parametrize("qkind", ["randk", "identity"])
+@pytest.mark.parametrize("workers,sketch_rows,rows", [(8, 3, 1201), (9, 3, 701), (16, 3, 701), (9, 7, 301), (16, 1, 1701), (9, 5, 421)])
+def test_two_walks_over_other_sketches_and_batches_of_workers(qkind, workers, sketch_rows, rows):
+    """Three rows, five and the general form, one and two batches of eight workers (the last one not full)."""
+    cfg = wl.config("tiny")
+    cfg.update(tensors=[(rows, 1001, 1), (rows, 999, 1), (rows + 3, 1000, 1), (rows, 1003, 1), (rows + 1, 1002, 1)], n_workers=workers,
+               q=dict(kind=qkind, k_num=1, k_den=20, seed=5),
+               c=dict(kind="countsketch", cs_rows=sketch_rows, cs_col_div=2, seed=9, beta=0.5))
+    if qkind == "identity":   # interleaving, reading, adding, back: four launches per tensor (three in one walk)
+        eng = pu.make_gpu(cfg)
+        before = eng.launch_count()
+        eng.step(0, [wl.gradient(cfg, i, 0, device="cuda") for i in range(workers)], 0)
+        assert eng.launch_count() - before == 4 * len(cfg["tensors"])
+    for a, b in zip(_run(cfg, True, 2), _run(cfg, False, 2)):
+        rms = b.double().square().mean().sqrt().clamp_min(1e-30)
+        assert float(((a - b).double().abs() / torch.maximum(b.double().abs(), rms)).max()) < 1e-5
+
+
 # three tensors of a similar size, which fit the scratch with their new records, and one that does not
 @pytest.mark.parametrize("tensors", [[(600, 1000, 1), (300, 1, 0), (601, 1000, 1), (599, 1001, 1)], [(37, 53, 1), (1100, 1001, 1), (64, 1, 0)]])
 @pytest.mark.parametrize("qkind,workers,rows", [("randk", 2, 5), ("randblock", 3, 3), ("randk", 8, 5), ("identity", 9, 7)])

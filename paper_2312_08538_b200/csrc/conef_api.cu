@@ -85,6 +85,7 @@ struct Plan {
     int fast_it[3] = {kFastIt1, kFastIt2, kFastIt3};   // iterations per tile of the tuned passes
     int fast_unit = 256;            // elements per quantisation block
     bool any_fast = false, any_slow = false, any_rs12 = false, any_gen = false;
+    bool gen_exact = true;      // the tensors of the passes for any shape have the configured rank and aligned factors (conef_lrgen.cuh)
     size_t gen_smem2 = 0;       // shared memory of a CTA of pass 2 for any shape
     bool short_tiles = false;   // tile lengths of the tuned passes below their limits
     bool multi = false;         // one launch per pass takes tensors of all widths (conef_fastmulti.cuh)
@@ -448,6 +449,7 @@ int make_plan(const conef_tensor *tensors, int n_tensors, int n_workers, const c
                     L.fast = 3;
                     P.any_gen = true;
                     gen_classify(L, gen, q->rank);
+                    P.gen_exact = P.gen_exact && gen_exact(L, q->rank);
                     P.gen_smem2 = std::max(P.gen_smem2, gen_p2_smem(L, q->rank));
                     L.p2_rows_fast = rtiles;
                     tiles[T_GEN1] = L.g_t1;
@@ -1422,7 +1424,7 @@ int conef_step(conef_ctx *ctx, int64_t step, const float *const *grads, int phas
             const int table = pass == 1 ? T_GEN1 : pass == 2 ? T_GEN2 : T_GEN3, n = tiles_of(ctx, table);
             if (n == 0 || (multi && ctx->plan.multi_gen) || rs12)   // (the table may hold 1-D tensors alone, of a model on a row sketch)
                 return CONEF_OK;
-            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, V, table_ptr(ctx, table), n, s, ctx->plan.gen_smem2));
+            CK_CUDA(gen_launch(pass, ctx->c.kind, ctx->q.rank, ctx->plan.gen_exact, V, table_ptr(ctx, table), n, s, ctx->plan.gen_smem2));
             LAUNCH_CHECK(ctx);
             return CONEF_OK;
         };

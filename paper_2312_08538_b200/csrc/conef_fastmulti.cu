@@ -29,7 +29,7 @@ k_fast_multi(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
     }
     grid_wait();
     if (L.fast == 3) {
-        gen_tile<PASS, CK, HALF, PARTIAL, R>(V, L, tile, (float *)smem_raw);
+        gen_tile<PASS, CK, HALF, PARTIAL, -R>(V, L, tile, (float *)smem_raw);
     } else if (PASS == 1 && !L.compressed) {
         pass_tile(V, L, tile);
     }

@@ -70,6 +70,8 @@ __host__ __device__ __forceinline__ bool gen_exact(const LayerDesc &L, int rank)
 {
     return (rank == 1 || rank == 2 || rank == 4 || rank == 8) && L.rank == rank && ((L.msgp_off | L.msgq_off) & ((rank == 8 ? 4 : rank) - 1)) == 0;
 }
+// the rank that a configuration's kernels are made for
+__host__ __device__ constexpr int gen_rank(int rank) { return rank <= 2 ? rank : rank <= 4 ? 4 : 8; }
 // Threads per tile of pass 2 and columns per tile: equal tiles whose words (one more than the columns make where a row starts
 // within a word) are two per thread; the largest that leaves as few threads idle as any other, give or take 5 %.
 inline void gen_p2_split(int64_t cols, int32_t &threads, int32_t &width)
@@ -118,9 +120,11 @@ inline void gen_classify(LayerDesc &L, const GenPlan &G, int cfg_rank)
 // bytes of shared memory of a CTA of pass 2
 inline size_t gen_p2_smem(const LayerDesc &L, int cfg_rank);
 
-// a row of a factor; R = 0: any rank
-template <int R, int AT = 0>   // AT: rows behind p (with any rank none)
-__device__ __forceinline__ void factor_row(const float *p, int r, float (&out)[R ? R : CONEF_MAX_RANK])
+// Ranks as template arguments: R > 0 is the rank, R < 0 stands for any up to -R
+__host__ __device__ constexpr int gen_most(int R) { return R < 0 ? -R : R; }
+// a row of a factor
+template <int R, int AT = 0>   // AT: rows behind p
+__device__ __forceinline__ void factor_row(const float *p, int r, float (&out)[gen_most(R)])
 {
     if constexpr (R == 4 || R == 8) {
         const float4 t = load_global_at<AT * R * 4>((const float4 *)p);
@@ -137,7 +141,7 @@ __device__ __forceinline__ void factor_row(const float *p, int r, float (&out)[R
     } else {
         p += (size_t)AT * r;
 #pragma unroll
-        for (int c = 0; c < CONEF_MAX_RANK; ++c)
+        for (int c = 0; c < -R; ++c)
             out[c] = c < r ? load_global(p + c) : 0.f;
     }
 }
@@ -201,7 +205,7 @@ __device__ __forceinline__ float gen_scale(const uint8_t *__restrict__ b, uint32
     return half ? __half2float(__ushort_as_half(load_global((const unsigned short *)b + blk))) : load_global((const float *)b + blk);
 }
 
-// Floats of shared memory per warp of pass 1: a chunk of kGenP1Cols columns of each row, and eight for where it starts
+// Floats of shared memory per warp of pass 1: a chunk of gen_p1_cols columns of each row, and eight for where it starts
 __host__ __device__ constexpr int gen_p1_cols(int nr) { return nr == 4 ? 128 : 256; }
 __host__ __device__ constexpr int gen_p1_floats(int nr) { return nr * (gen_p1_cols(nr) + 8); }
 constexpr size_t kGenP1Smem = 8 * gen_p1_floats(4) * 4;
@@ -235,8 +239,8 @@ __device__ __forceinline__ void gen_p1_store(float (&acc)[NR][RM], float *__rest
 template <int CK, bool HALF, bool PARTIAL, int R, int NR>
 __device__ __forceinline__ void gen_p1_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
-    constexpr int RM = R ? R : CONEF_MAX_RANK, CH = gen_p1_cols(NR), U = CH / 32, PITCH = CH + 8, GR = CH / 8, NG = NR * GR / 32;
-    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int RM = gen_most(R), CH = gen_p1_cols(NR), U = CH / 32, PITCH = CH + 8, GR = CH / 8, NG = NR * GR / 32;
+    const int r = R > 0 ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
     const uint32_t row0 = (tile * 8u + warp) * NR;
     if (row0 >= n)
@@ -395,7 +399,7 @@ constexpr int kGenP2Rows = 16;
 __host__ __device__ constexpr int gen_p2_floats(int t, int rank) { return 2 * kGenP2Rows * (t + 8 + rank); }
 // a row of a factor in shared memory
 template <int R>
-__device__ __forceinline__ void factor_row_smem(const float *p, int r, float (&out)[R ? R : CONEF_MAX_RANK])
+__device__ __forceinline__ void factor_row_smem(const float *p, float (&out)[R])
 {
     if constexpr (R == 4 || R == 8) {
 #pragma unroll
@@ -407,16 +411,14 @@ __device__ __forceinline__ void factor_row_smem(const float *p, int r, float (&o
         const float2 t = *(const float2 *)p;
         out[0] = t.x; out[1] = t.y;
     } else {
-#pragma unroll
-        for (int c = 0; c < (R ? R : CONEF_MAX_RANK); ++c)
-            out[c] = R || c < r ? p[c] : 0.f;
+        out[0] = p[0];
     }
 }
 template <int CK, bool HALF, bool PARTIAL, int R>
 __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
-    constexpr int RM = R ? R : CONEF_MAX_RANK, S = kGenP2Rows, KP = (S * RM + 31) / 32;
-    const int r = R ? R : L.rank, worker = blockIdx.y;
+    constexpr int RM = gen_most(R), S = kGenP2Rows, KP = (S * RM + 31) / 32;
+    const int r = R > 0 ? R : L.rank, worker = blockIdx.y;
     const uint32_t T = (uint32_t)L.g_p2t, lt = 31 - __clz(T);   // threads of a tile
     const uint32_t part_of = threadIdx.x >> lt, tid = threadIdx.x & (T - 1), bar = part_of + 1;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows, wd = (uint32_t)L.g_p2w;
@@ -454,8 +456,14 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
 #pragma unroll
         for (int x = 0; x < KP; ++x) {
             const uint32_t at = tid + x * T;
-            if (at < S * r)
-                phn[x] = a * r + at < have * r ? load_global(ph + a * r + at) : 0.f;
+            if constexpr (R > 0) {
+                if (at < S * R)
+                    phn[x] = a * R + at < have * R ? load_global(ph + a * R + at) : 0.f;
+            } else {   // (rows of RM, so that the walk reads them as vectors)
+                const uint32_t row = a + at / RM, c = at % RM;
+                if (at < S * RM)
+                    phn[x] = row < have && c < r ? load_global(ph + row * r + c) : 0.f;
+            }
         }
     };
     fetch(0);
@@ -470,7 +478,7 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
         gen_decode<CK, HALF, PARTIAL>(w[1], omb, es + put + 8 * pitch, swap);
 #pragma unroll
         for (int x = 0; x < KP; ++x)
-            if (tid + x * T < S * r)
+            if (tid + x * T < S * RM)
                 phs[tid + x * T] = phn[x];
         if (a + S < have)
             fetch(a + S);
@@ -481,7 +489,7 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
                 const float p = __fmaf_rn(lr, gv[u], *ep);   // Alg. 2 (4) line 5
                 ep += pitch;
                 float pr[RM];
-                factor_row_smem<R>(phs + u * r, r, pr);
+                factor_row_smem<RM>(phs + u * RM, pr);
 #pragma unroll
                 for (int c = 0; c < RM; ++c)
                     acc[c] = __fmaf_rn(p, pr[c], acc[c]);
@@ -517,20 +525,20 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
         float *part = V.part + worker * V.part_stride + L.part_off + ((size_t)rt * m + c0 + tid) * r;   // added in order by k_lr_pass2_reduce
 #pragma unroll
         for (int c = 0; c < RM; ++c)
-            if (R || c < r)
+            if (R > 0 || c < r)
                 part[c] = acc[c];
     }
 }
 
-// The same tile by a whole CTA, for models whose tiles do not fill the SMs: the eight warps form p of 32 rows each in shared
-// memory, then a warp per column of the factor adds down the rows, in the order of gen_p2_body.  There a warp walks the
-// 256 rows eight at a time, 32 waits for memory one after the other, however small the model.
+// kP2RowsPerTile rows by kGenCols columns by a whole CTA, for models whose tiles do not fill the SMs: the eight warps form p of 32 rows
+// each in shared memory, then a warp per column of the factor adds down the rows, in the order of gen_p2_body.  There a tile waits for memory
+// at each of its sixteen stages, however small the model (times: kGenCoop).
 constexpr size_t kGenCoopSmem = (size_t)kP2RowsPerTile * (32 + CONEF_MAX_RANK) * 4;
 template <int CK, int R>
 __device__ __forceinline__ void gen_p2_cta(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
     constexpr int U = 16;   // rows in flight per warp
-    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = R > 0 ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows;
     const uint32_t ct = (m + kGenCols - 1) / kGenCols, rt = tile / ct, c0 = (tile - rt * ct) * kGenCols + lane;
     const uint32_t r_lo = rt * (uint32_t)kP2RowsPerTile, have = min(n - r_lo, (uint32_t)kP2RowsPerTile);
@@ -584,7 +592,7 @@ inline size_t gen_p2_smem(const LayerDesc &L, int cfg_rank)
 {
     if (L.g_p2t == 0)
         return kGenCoopSmem;
-    return (size_t)(kGenThreads / L.g_p2t) * gen_p2_floats(L.g_p2t, gen_exact(L, cfg_rank) ? cfg_rank : CONEF_MAX_RANK) * 4;
+    return (size_t)(kGenThreads / L.g_p2t) * gen_p2_floats(L.g_p2t, gen_rank(cfg_rank)) * 4;
 }
 
 // Pass 3 takes 32 * E elements per warp at a time.  E consecutive ones are a lane's where codes are decoded and quantised (a block
@@ -634,10 +642,10 @@ struct GenTurn {
 template <int CK, bool HALF, bool PARTIAL, int R, int E>
 __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
-    constexpr int RM = R ? R : CONEF_MAX_RANK, K = E, NW = GenTurn<CK, E>::NW, CH = 32 * E;
+    constexpr int RM = gen_most(R), K = E, NW = GenTurn<CK, E>::NW, CH = 32 * E;
     constexpr bool INT4 = CK == CONEF_C_INT4;
     const int lpb = L.unit / E;   // lanes per quantisation block
-    const int r = R ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = R > 0 ? R : L.rank, worker = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t m = (uint32_t)L.cols, n = (uint32_t)L.rows, d = (uint32_t)L.d;
     const uint32_t step = L.g_step, groups = L.g_groups, nc = (d + CH - 1) / CH;
     const uint32_t tt = tile / groups, cpos = (tile - tt * groups) * 8 + warp;   // place among the chunks of a step
@@ -725,7 +733,7 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
             float res = __fmaf_rn(lr, gv[k], PARTIAL ? __fmul_rn(omb, e) : e);   // Alg. 2 (4) line 5
 #pragma unroll
             for (int c = 0; c < RM; ++c)
-                if (R || c < r)
+                if (R > 0 || c < r)
                     res = __fmaf_rn(-pr[c], q[c], res);
             if (PARTIAL)
                 res = __fmaf_rn(beta, e, res);
@@ -853,58 +861,66 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
     }
 }
 
-// R: the configured rank (1, 2, 4, 8; 0: another one).  Tensors thinner than it, and those behind them whose
-// factors are off the vector loads' alignment, take the run-time rank.
+// R: the configured rank, or the next of 1, 2, 4 and 8 above it (gen_rank).  Tensors of another rank than R, and those behind them whose
+// factors are off the vector loads' alignment, take the body for any rank up to R.  That was one for any rank up to 8 with a row per warp in pass
+// 1; steps of the recurrent layers of odd widths, before and now: rank 3 608 and 407 us (int8), 596 and 383 (int4), rank 5 641 and 527, rank 7 681 and
+// 551, behind a matrix of one row rank 4, int8, 711 and 444, rank 2, int4, 557 and 338.  As a function that is not inlined
+// it takes no registers from the body with the rank as a constant, but both were slower: rank 3 439, rank 7 651, rank 8 511 instead of 496.
+// R < 0: of models with such tensors (rank -R); R > 0: of those without, whose kernels have the one body alone (rank 2, int8 296 us
+// with both and 288 with one, rank 8, int4 501 and 473).
 template <int PASS, int CK, bool HALF, bool PARTIAL, int R>
 __device__ __forceinline__ void gen_tile(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
-    const bool exact = gen_exact(L, R);
+    constexpr int K = gen_most(R);
+    const bool exact = R > 0 || gen_exact(L, K);
     if constexpr (PASS == 1) {
-        if constexpr (R != 0) {
-            if (exact) {
-                if (L.g_nr > 1 && L.cols <= kGenNarrow)
-                    gen_p1_narrow<CK, HALF, PARTIAL, R, gen_p1_rows(R)>(V, L, tile, smem);
-                else if (L.g_nr > 1)
-                    gen_p1_body<CK, HALF, PARTIAL, R, gen_p1_rows(R)>(V, L, tile, smem);
-                else
-                    gen_p1_body<CK, HALF, PARTIAL, R, 1>(V, L, tile, smem);
-                return;
-            }
+        if (exact) {
+            if (L.g_nr > 1 && L.cols <= kGenNarrow)
+                gen_p1_narrow<CK, HALF, PARTIAL, K, gen_p1_rows(K)>(V, L, tile, smem);
+            else if (L.g_nr > 1)
+                gen_p1_body<CK, HALF, PARTIAL, K, gen_p1_rows(K)>(V, L, tile, smem);
+            else
+                gen_p1_body<CK, HALF, PARTIAL, K, 1>(V, L, tile, smem);
+            return;
         }
-        for (int x = 0; x < L.g_nr; ++x)
-            gen_p1_body<CK, HALF, PARTIAL, 0, 1>(V, L, tile * (uint32_t)L.g_nr + x, smem);
+        if (L.g_nr > 1)
+            gen_p1_body<CK, HALF, PARTIAL, R, gen_p1_rows(K)>(V, L, tile, smem);
+        else
+            gen_p1_body<CK, HALF, PARTIAL, R, 1>(V, L, tile, smem);
     } else if constexpr (PASS == 2) {
         if (L.g_p2t == 0) {
-            if (R && exact)
-                gen_p2_cta<CK, R>(V, L, tile, smem);
+            if (exact)
+                gen_p2_cta<CK, K>(V, L, tile, smem);
             else
-                gen_p2_cta<CK, 0>(V, L, tile, smem);
-        } else if (R && exact) {
-            gen_p2_body<CK, HALF, PARTIAL, R>(V, L, tile, smem);
+                gen_p2_cta<CK, R>(V, L, tile, smem);
+        } else if (exact) {
+            gen_p2_body<CK, HALF, PARTIAL, K>(V, L, tile, smem);
         } else {
-            gen_p2_body<CK, HALF, PARTIAL, 0>(V, L, tile, smem);
+            gen_p2_body<CK, HALF, PARTIAL, R>(V, L, tile, smem);
         }
     } else {
         if (!exact)
-            gen_p3_body<CK, HALF, PARTIAL, 0, 8>(V, L, tile, smem);
-        else if (L.g_chunk == kGenChunk)
-            gen_p3_body<CK, HALF, PARTIAL, R, 16>(V, L, tile, smem);
-        else
             gen_p3_body<CK, HALF, PARTIAL, R, 8>(V, L, tile, smem);
+        else if (L.g_chunk == kGenChunk)
+            gen_p3_body<CK, HALF, PARTIAL, K, 16>(V, L, tile, smem);
+        else
+            gen_p3_body<CK, HALF, PARTIAL, K, 8>(V, L, tile, smem);
     }
 }
 
-// CTAs per SM that the registers have to allow for
+// CTAs per SM that the registers have to allow for.  Pass 3 on int8 with four and with three of them, steps on the recurrent layers of odd widths (28.4 M
+// elements, two workers): rank 1 292 and 289 us, 2 302 and 297, 3 489 and 456, 4 350 and 343 (104 and 16 bytes spilled); rank 8 with
+// three and two 493 and 497.
 __host__ __device__ constexpr int gen_ctas(int pass, int ckind, int rank)
 {
-    if (rank == 0 || pass == 2)
+    if (pass == 2)
         return 3;
     if (pass == 1)
         return rank == 8 ? 3 : 4;
-    return (rank == 8 ? 2 : 3) + (ckind == CONEF_C_INT8);
+    return rank == 8 ? 2 + (ckind == CONEF_C_INT8) : 3;
 }
 template <int PASS, int CK, bool HALF, bool PARTIAL, int R>
-__global__ void __launch_bounds__(kGenThreads, gen_ctas(PASS, CK, R)) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
+__global__ void __launch_bounds__(kGenThreads, gen_ctas(PASS, CK, gen_most(R))) k_gen_pass(const __grid_constant__ DevView V, const int32_t *__restrict__ pfx)
 {
     extern __shared__ __align__(16) float gen_smem[];
     grid_release();
@@ -919,12 +935,12 @@ __global__ void __launch_bounds__(kGenThreads, gen_ctas(PASS, CK, R)) k_gen_pass
     gen_tile<PASS, CK, HALF, PARTIAL, R>(V, L, tile, gen_smem);
 }
 
-// launcher (conef_lrgen.cu, the variants by codec in two more files); smem2: the most that a tensor's CTAs of pass 2 need
-cudaError_t gen_launch(int pass, int ckind, int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem2);
+// launcher (conef_lrgen.cu, the variants by codec in two more files); exact: every tensor is gen_exact; smem2: the most that a tensor's CTAs of pass 2 need
+cudaError_t gen_launch(int pass, int ckind, int rank, bool exact, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem2);
 
 template <int CK>
-cudaError_t gen_launch_codec(int pass, int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem2);
-extern template cudaError_t gen_launch_codec<CONEF_C_INT8>(int, int, const DevView &, const int32_t *, int, cudaStream_t, size_t);
-extern template cudaError_t gen_launch_codec<CONEF_C_INT4>(int, int, const DevView &, const int32_t *, int, cudaStream_t, size_t);
+cudaError_t gen_launch_codec(int pass, int rank, bool exact, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem2);
+extern template cudaError_t gen_launch_codec<CONEF_C_INT8>(int, int, bool, const DevView &, const int32_t *, int, cudaStream_t, size_t);
+extern template cudaError_t gen_launch_codec<CONEF_C_INT4>(int, int, bool, const DevView &, const int32_t *, int, cudaStream_t, size_t);
 
 }  // namespace conef

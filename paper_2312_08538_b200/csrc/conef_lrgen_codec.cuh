@@ -16,16 +16,18 @@ static cudaError_t gen_pass_launch(int pass, const DevView &V, const int32_t *pf
 }
 
 template <int CK>
-cudaError_t gen_launch_codec(int pass, int rank, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem2)
+cudaError_t gen_launch_codec(int pass, int rank, bool exact, const DevView &V, const int32_t *pfx, int tiles, cudaStream_t s, size_t smem2)
 {
     auto by_rank = [&](auto half, auto partial) {
         constexpr bool H = decltype(half)::value != 0, P = decltype(partial)::value != 0;
-        switch (rank) {
+        switch (exact ? gen_rank(rank) : -gen_rank(rank)) {
         case 1: return gen_pass_launch<CK, H, P, 1>(pass, V, pfx, tiles, s, smem2);
         case 2: return gen_pass_launch<CK, H, P, 2>(pass, V, pfx, tiles, s, smem2);
         case 4: return gen_pass_launch<CK, H, P, 4>(pass, V, pfx, tiles, s, smem2);
         case 8: return gen_pass_launch<CK, H, P, 8>(pass, V, pfx, tiles, s, smem2);
-        default: return gen_pass_launch<CK, H, P, 0>(pass, V, pfx, tiles, s, smem2);
+        case -2: return gen_pass_launch<CK, H, P, -2>(pass, V, pfx, tiles, s, smem2);
+        case -4: return gen_pass_launch<CK, H, P, -4>(pass, V, pfx, tiles, s, smem2);
+        default: return gen_pass_launch<CK, H, P, -8>(pass, V, pfx, tiles, s, smem2);
         }
     };
     if (V.beta != 0.f)

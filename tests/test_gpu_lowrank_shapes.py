@@ -119,6 +119,16 @@ def test_tall_models_give_the_bits_of_the_kernels_for_every_codec(rank, c):
             e.reduce_messages(b.MSG_Q)
 
 
+@pytest.mark.parametrize("tensors", [[(1, 97, 1)] + BIG, [(1, 97, 1), (70, 33, 1), (3, 1, 0), (2, 61, 1), (300, 257, 1), (64, 512, 1)]])
+@pytest.mark.parametrize("rank,c", [(2, dict(kind="int8", block=256)), (2, dict(kind="int4", block=64, beta=0.5)), (3, dict(kind="int8", block=64, scale_dtype="fp16")),
+                                    (4, dict(kind="int4", block=128, scale_dtype="fp16")), (5, dict(kind="int8", block=256)), (6, dict(kind="int4", block=256)),
+                                    (7, dict(kind="int8", block=32, beta=0.9)), (8, dict(kind="int4", block=128, scale_dtype="fp16"))])
+def test_ranks_without_kernels_of_their_own(monkeypatch, tensors, rank, c):
+    """Ranks between those that the kernels are made for, and factors off their vectors' boundaries behind a tensor of one row."""
+    monkeypatch.setitem(globals(), "BIG", tensors)
+    test_tall_models_give_the_bits_of_the_kernels_for_every_codec(rank, c)
+
+
 @pytest.mark.parametrize("rank,c", [(4, dict(kind="int8", block=256)), (8, dict(kind="int4", block=128, scale_dtype="fp16")),
                                     (4, dict(kind="int4", block=64, scale_dtype="fp16", beta=0.9)), (8, dict(kind="int8", block=32, scale_dtype="fp16"))])
 def test_all_widths_in_one_launch(rank, c):

@@ -414,7 +414,7 @@ __device__ __forceinline__ void factor_row_smem(const float *p, float (&out)[R])
         out[0] = p[0];
     }
 }
-template <int CK, bool HALF, bool PARTIAL, int R>
+template <int CK, bool HALF, bool PARTIAL, int R, bool PAD = true>   // PAD: with any rank, rows of P_hat on their vectors' boundaries in shared memory
 __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
     constexpr int RM = gen_most(R), S = kGenP2Rows, KP = (S * RM + 31) / 32;
@@ -456,10 +456,10 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
 #pragma unroll
         for (int x = 0; x < KP; ++x) {
             const uint32_t at = tid + x * T;
-            if constexpr (R > 0) {
-                if (at < S * R)
-                    phn[x] = a * R + at < have * R ? load_global(ph + a * R + at) : 0.f;
-            } else {   // (rows of RM, so that the walk reads them as vectors)
+            if constexpr (R > 0 || !PAD) {
+                if (at < S * r)
+                    phn[x] = a * r + at < have * r ? load_global(ph + a * r + at) : 0.f;
+            } else {
                 const uint32_t row = a + at / RM, c = at % RM;
                 if (at < S * RM)
                     phn[x] = row < have && c < r ? load_global(ph + row * r + c) : 0.f;
@@ -478,7 +478,7 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
         gen_decode<CK, HALF, PARTIAL>(w[1], omb, es + put + 8 * pitch, swap);
 #pragma unroll
         for (int x = 0; x < KP; ++x)
-            if (tid + x * T < S * RM)
+            if (tid + x * T < S * (PAD ? RM : r))
                 phs[tid + x * T] = phn[x];
         if (a + S < have)
             fetch(a + S);
@@ -489,7 +489,13 @@ __device__ __forceinline__ void gen_p2_body(const DevView &V, const LayerDesc &L
                 const float p = __fmaf_rn(lr, gv[u], *ep);   // Alg. 2 (4) line 5
                 ep += pitch;
                 float pr[RM];
-                factor_row_smem<RM>(phs + u * RM, pr);
+                if constexpr (R > 0 || PAD) {
+                    factor_row_smem<RM>(phs + u * RM, pr);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < RM; ++c)
+                        pr[c] = c < r ? phs[u * r + c] : 0.f;
+                }
 #pragma unroll
                 for (int c = 0; c < RM; ++c)
                     acc[c] = __fmaf_rn(p, pr[c], acc[c]);
@@ -867,12 +873,28 @@ __device__ __forceinline__ void gen_p3_body(const DevView &V, const LayerDesc &L
 // 551, behind a matrix of one row rank 4, int8, 711 and 444, rank 2, int4, 557 and 338.  As a function that is not inlined
 // it takes no registers from the body with the rank as a constant, but both were slower: rank 3 439, rank 7 651, rank 8 511 instead of 496.
 // R < 0: of models with such tensors (rank -R); R > 0: of those without, whose kernels have the one body alone (rank 2, int8 296 us
-// with both and 288 with one, rank 8, int4 501 and 473).
+// with both and 288 with one, rank 8, int4 501 and 473).  BOTH:
+// rank 8 on int8 alone compiles to slower code in its own kernel, though it spills less (4001 x 6003, four workers, fp16 scales: pass 1 286 instead of 260 us,
+// pass 2 174 instead of 141; steps 883 and 831), so that it keeps the other body beside it, a row per warp and P_hat's rows as they come.
 template <int PASS, int CK, bool HALF, bool PARTIAL, int R>
 __device__ __forceinline__ void gen_tile(const DevView &V, const LayerDesc &L, uint32_t tile, float *smem)
 {
     constexpr int K = gen_most(R);
-    const bool exact = R > 0 || gen_exact(L, K);
+    constexpr bool BOTH = CK == CONEF_C_INT8 && R == 8;
+    const bool exact = (R > 0 && !BOTH) || gen_exact(L, K);
+    if constexpr (BOTH && PASS != 3) {
+        if (!exact) {
+            if constexpr (PASS == 1) {
+                for (int x = 0; x < L.g_nr; ++x)
+                    gen_p1_body<CK, HALF, PARTIAL, -K, 1>(V, L, tile * (uint32_t)L.g_nr + x, smem);
+            } else if (L.g_p2t == 0) {
+                gen_p2_cta<CK, -K>(V, L, tile, smem);
+            } else {
+                gen_p2_body<CK, HALF, PARTIAL, -K, false>(V, L, tile, smem);
+            }
+            return;
+        }
+    }
     if constexpr (PASS == 1) {
         if (exact) {
             if (L.g_nr > 1 && L.cols <= kGenNarrow)
@@ -900,7 +922,7 @@ __device__ __forceinline__ void gen_tile(const DevView &V, const LayerDesc &L, u
         }
     } else {
         if (!exact)
-            gen_p3_body<CK, HALF, PARTIAL, R, 8>(V, L, tile, smem);
+            gen_p3_body<CK, HALF, PARTIAL, -K, 8>(V, L, tile, smem);
         else if (L.g_chunk == kGenChunk)
             gen_p3_body<CK, HALF, PARTIAL, K, 16>(V, L, tile, smem);
         else

@@ -20,7 +20,8 @@ cudaError_t gen_launch_codec(int pass, int rank, bool exact, const DevView &V, c
 {
     auto by_rank = [&](auto half, auto partial) {
         constexpr bool H = decltype(half)::value != 0, P = decltype(partial)::value != 0;
-        switch (exact ? gen_rank(rank) : -gen_rank(rank)) {
+        // (rank 8 on int8: gen_tile, BOTH)
+        switch (exact || (rank == 8 && CK == CONEF_C_INT8) ? gen_rank(rank) : -gen_rank(rank)) {
         case 1: return gen_pass_launch<CK, H, P, 1>(pass, V, pfx, tiles, s, smem2);
         case 2: return gen_pass_launch<CK, H, P, 2>(pass, V, pfx, tiles, s, smem2);
         case 4: return gen_pass_launch<CK, H, P, 4>(pass, V, pfx, tiles, s, smem2);
